@@ -1,4 +1,4 @@
-"""Builds libxkv.so (sm_100a) in-tree with nvcc.  `python -m paper_2503_18893_b200.build`."""
+"""Builds libxkv.so (sm_100a, nvcc) and its Python module _xkv.so (g++) in-tree.  `python -m paper_2503_18893_b200.build`."""
 from __future__ import annotations
 
 import concurrent.futures
@@ -7,11 +7,13 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libxkv.so")
+PYMOD = os.path.join(HERE, "_xkv.so")
 OBJ = os.path.join(HERE, "build")
 
 NVCC_FLAGS = [
@@ -37,7 +39,7 @@ def _stamp() -> str:
     for f in sorted(os.listdir(CSRC)) + ["../../include/xkv.h"]:
         with open(os.path.join(CSRC, f), "rb") as fh:
             h.update(f.encode() + b"\0" + fh.read())
-    h.update(" ".join(NVCC_FLAGS).encode())
+    h.update(" ".join(NVCC_FLAGS + [sysconfig.get_paths()["include"]]).encode())
     return h.hexdigest()
 
 
@@ -46,7 +48,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
     os.makedirs(OBJ, exist_ok=True)
     stamp_file = os.path.join(OBJ, "stamp")
     stamp = _stamp()
-    if not force and not ptxas_info and os.path.exists(LIB) and os.path.exists(stamp_file):
+    if not force and not ptxas_info and os.path.exists(LIB) and os.path.exists(PYMOD) and os.path.exists(stamp_file):
         if open(stamp_file).read() == stamp:
             return LIB
     nvcc = _nvcc()
@@ -71,6 +73,13 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
     if r.returncode != 0:
         sys.stderr.write(r.stdout + r.stderr)
         raise RuntimeError("link failed")
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I", os.path.join(ROOT, "include"),
+           "-I", sysconfig.get_paths()["include"], os.path.join(CSRC, "xkv_py.cpp"), "-o", PYMOD, "-L", HERE, "-lxkv",
+           "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+        raise RuntimeError("building the Python module failed")
     with open(stamp_file, "w") as f:
         f.write(stamp)
     return LIB

@@ -1,0 +1,201 @@
+// CPython module over the C ABI for the calls of a decode step and the other per-prompt calls (argument marshalling
+// only).  A decode step is a handful of kernels of a few microseconds each, so what a call costs on the host is part
+// of its latency: through ctypes and torch.cuda.current_stream() a call spent 4.5 us before its first launch, here
+// 0.7 us.  Tensor arguments are anything with a data_ptr() method (or None, or an integer address); a stream is None
+// (torch's current one), an integer, or an object with a cuda_stream attribute.  Every function returns the status.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <stdint.h>
+
+#include "xkv.h"
+
+namespace {
+
+PyObject *s_data_ptr, *s_cuda_stream;      // interned attribute names
+PyObject *g_get_device, *g_get_stream;     // torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+
+// Cursor over the arguments of a call; `bad` is set (with a Python exception) by the first one that does not convert.
+struct Args {
+  PyObject* const* v;
+  Py_ssize_t n, at;
+  bool bad;
+  Args(PyObject* const* args, Py_ssize_t have, Py_ssize_t want) : v(args), n(have), at(0), bad(false) {
+    if (have != want) {
+      PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, have);
+      bad = true;
+    }
+  }
+  PyObject* next() { return bad ? nullptr : v[at++]; }
+  void* address(PyObject* o) {
+    void* p = PyLong_AsVoidPtr(o);
+    if (!p && PyErr_Occurred()) bad = true;
+    return p;
+  }
+  void* ptr() {
+    PyObject* o = next();
+    if (!o || o == Py_None) return nullptr;
+    if (PyLong_Check(o)) return address(o);
+    PyObject* r = PyObject_CallMethodNoArgs(o, s_data_ptr);
+    if (!r) { bad = true; return nullptr; }
+    void* p = address(r);
+    Py_DECREF(r);
+    return p;
+  }
+  long long i64() {
+    PyObject* o = next();
+    if (!o) return 0;
+    const long long x = PyLong_AsLongLong(o);
+    if (x == -1 && PyErr_Occurred()) bad = true;
+    return x;
+  }
+  int i32() {
+    const long long x = i64();
+    if (!bad && (x < INT32_MIN || x > INT32_MAX)) {
+      PyErr_SetString(PyExc_OverflowError, "integer argument does not fit 32 bits");
+      bad = true;
+    }
+    return (int)x;
+  }
+  void* stream() {
+    PyObject* o = next();
+    if (!o) return nullptr;
+    if (PyLong_Check(o)) return address(o);
+    PyObject* r;
+    if (o == Py_None) {
+      PyObject* dev = PyObject_CallNoArgs(g_get_device);
+      if (!dev) { bad = true; return nullptr; }
+      r = PyObject_CallOneArg(g_get_stream, dev);
+      Py_DECREF(dev);
+    } else {
+      r = PyObject_GetAttr(o, s_cuda_stream);
+    }
+    if (!r) { bad = true; return nullptr; }
+    void* p = address(r);
+    Py_DECREF(r);
+    return p;
+  }
+};
+
+#define XKV_PY(name, want) \
+  PyObject* name(PyObject*, PyObject* const* args, Py_ssize_t nargs) { \
+    Args a(args, nargs, want);
+#define XKV_PY_END(call) \
+    if (a.bad) return nullptr; \
+    int st; \
+    Py_BEGIN_ALLOW_THREADS st = call; \
+    Py_END_ALLOW_THREADS \
+    return PyLong_FromLong(st); \
+  }
+
+XKV_PY(sr_select, 8)
+  xkv_group* g = (xkv_group*)a.ptr();
+  const int l0 = a.i32(), l1 = a.i32();
+  void* q = a.ptr();
+  const int k = a.i32();
+  int32_t* idx = (int32_t*)a.ptr();
+  int32_t* cnt = (int32_t*)a.ptr();
+  void* s = a.stream();
+XKV_PY_END(xkv_sr_select(g, l0, l1, q, k, idx, cnt, s))
+
+XKV_PY(sr_select_static, 15)
+  xkv_select_static_config cfg;
+  cfg.struct_size = sizeof(cfg);
+  cfg.G = a.i32(); cfg.batch = a.i32(); cfg.T = a.i32(); cfg.H_kv = a.i32(); cfg.H_q = a.i32(); cfg.d_h = a.i32();
+  cfg.chunk = a.i32();
+  cfg.landmarks = a.ptr();
+  const int l0 = a.i32(), l1 = a.i32();
+  void* q = a.ptr();
+  const int k = a.i32();
+  int32_t* idx = (int32_t*)a.ptr();
+  int32_t* cnt = (int32_t*)a.ptr();
+  void* s = a.stream();
+XKV_PY_END(xkv_sr_select_static(&cfg, l0, l1, q, k, idx, cnt, s))
+
+XKV_PY(sr_reconstruct_attend, 10)
+  xkv_group* g = (xkv_group*)a.ptr();
+  const int l0 = a.i32(), l1 = a.i32();
+  void* q = a.ptr();
+  const int32_t* idx = (const int32_t*)a.ptr();
+  const int32_t* cnt = (const int32_t*)a.ptr();
+  const int k_cap = a.i32();
+  void* out = a.ptr();
+  float* lse = (float*)a.ptr();
+  void* s = a.stream();
+XKV_PY_END(xkv_sr_reconstruct_attend(g, l0, l1, q, idx, cnt, k_cap, out, lse, s))
+
+XKV_PY(sr_reconstruct_attend_tail, 16)
+  xkv_group* g = (xkv_group*)a.ptr();
+  const int l0 = a.i32(), l1 = a.i32();
+  void* q = a.ptr();
+  const int32_t* idx = (const int32_t*)a.ptr();
+  const int32_t* cnt = (const int32_t*)a.ptr();
+  const int k_cap = a.i32();
+  void* tk = a.ptr();
+  void* tv = a.ptr();
+  const int32_t* len = (const int32_t*)a.ptr();
+  const int cap = a.i32();
+  void* ws = a.ptr();
+  const uint64_t ws_bytes = (uint64_t)a.i64();
+  void* out = a.ptr();
+  float* lse = (float*)a.ptr();
+  void* s = a.stream();
+XKV_PY_END(xkv_sr_reconstruct_attend_tail(g, l0, l1, q, idx, cnt, k_cap, tk, tv, len, cap, ws, ws_bytes, out, lse, s))
+
+XKV_PY(dense_attend, 13)
+  xkv_group* g = (xkv_group*)a.ptr();
+  const int l0 = a.i32(), l1 = a.i32();
+  void* q = a.ptr();
+  void* K = a.ptr();
+  void* V = a.ptr();
+  const int32_t* len = (const int32_t*)a.ptr();
+  const int cap = a.i32();
+  void* ws = a.ptr();
+  const uint64_t ws_bytes = (uint64_t)a.i64();
+  void* out = a.ptr();
+  float* lse = (float*)a.ptr();
+  void* s = a.stream();
+XKV_PY_END(xkv_dense_attend(g, l0, l1, q, K, V, len, cap, ws, ws_bytes, out, lse, s))
+
+XKV_PY(quantize_rtn, 7)
+  void* x = a.ptr();
+  const int64_t rows = a.i64();
+  const int cols = a.i32(), bits = a.i32();
+  void* codes = a.ptr();
+  void* meta = a.ptr();
+  void* s = a.stream();
+XKV_PY_END(xkv_quantize_rtn(x, rows, cols, bits, codes, meta, s))
+
+XKV_PY(dequantize_rtn, 7)
+  void* codes = a.ptr();
+  void* meta = a.ptr();
+  const int64_t rows = a.i64();
+  const int cols = a.i32(), bits = a.i32();
+  void* x = a.ptr();
+  void* s = a.stream();
+XKV_PY_END(xkv_dequantize_rtn(codes, meta, rows, cols, bits, x, s))
+
+// torch_hooks(get_device, get_current_raw_stream): how "the current stream" is found.
+PyObject* torch_hooks(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
+  if (nargs != 2) { PyErr_SetString(PyExc_TypeError, "expected 2 arguments"); return nullptr; }
+  Py_INCREF(args[0]);
+  Py_INCREF(args[1]);
+  Py_XSETREF(g_get_device, args[0]);
+  Py_XSETREF(g_get_stream, args[1]);
+  Py_RETURN_NONE;
+}
+
+#define XKV_DEF(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {XKV_DEF(sr_select), XKV_DEF(sr_select_static), XKV_DEF(sr_reconstruct_attend),
+                         XKV_DEF(sr_reconstruct_attend_tail), XKV_DEF(dense_attend), XKV_DEF(quantize_rtn),
+                         XKV_DEF(dequantize_rtn), XKV_DEF(torch_hooks), {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_xkv", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__xkv(void) {
+  s_data_ptr = PyUnicode_InternFromString("data_ptr");
+  s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
+  if (!s_data_ptr || !s_cuda_stream) return nullptr;
+  return PyModule_Create(&module);
+}

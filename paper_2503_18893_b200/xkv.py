@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libxkv (argument marshalling only; every step runs in the CUDA library).
+"""Thin binding of libxkv (argument marshalling only; every step runs in the CUDA library).  The calls of a decode step
+go through the native module `_xkv` (csrc/xkv_py.cpp), the rest through ctypes.
 
 The functions carry the names of the C ABI (include/xkv.h).  Tensors are torch CUDA tensors used
 for their device memory; the stream is torch's current stream unless one is given.  Importing this
@@ -21,6 +22,10 @@ if not os.path.exists(LIB_PATH):
         "(nvcc, sm_100a). There is no fallback path.")
 
 _lib = ctypes.CDLL(LIB_PATH)
+
+from . import _xkv  # noqa: E402  (native module beside libxkv.so)
+
+_xkv.torch_hooks(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
 
 XKV_OK = 0
 XKV_ERR_INVALID_ARG = -1
@@ -171,7 +176,7 @@ def xkv_debug_set_fault_injection(grp, mask: int) -> None:
 
 def _stream(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -235,8 +240,7 @@ def xkv_group_destroy(grp: Group) -> None:
 
 
 def xkv_sr_select(grp: Group, layer_begin: int, layer_end: int, q, k: int, sel_idx, sel_cnt, stream=None) -> None:
-    st = _lib.xkv_sr_select(grp.handle, layer_begin, layer_end, _ptr(q), k, _ptr(sel_idx), _ptr(sel_cnt),
-                            _stream(stream))
+    st = _xkv.sr_select(grp.handle, layer_begin, layer_end, q, k, sel_idx, sel_cnt, stream)
     if st != XKV_OK:
         raise XKVError(st, "xkv_sr_select")
 
@@ -245,20 +249,15 @@ def xkv_sr_select_static(*, G, batch, T, H_kv, H_q, d_h, landmarks, layer_begin,
                          chunk=8, stream=None) -> None:
     """Selection without a handle and without any device allocation (fixed scratch inside the library, see
     include/xkv.h).  Same outputs as xkv_sr_select.  Raises XKVError(XKV_ERR_TOO_LARGE) beyond the fixed size."""
-    cfg = xkv_select_static_config()
-    cfg.struct_size = ctypes.sizeof(xkv_select_static_config)
-    cfg.G, cfg.batch, cfg.T, cfg.H_kv, cfg.H_q, cfg.d_h, cfg.chunk = G, batch, T, H_kv, H_q, d_h, chunk
-    cfg.landmarks = _ptr(landmarks)
-    st = _lib.xkv_sr_select_static(ctypes.byref(cfg), layer_begin, layer_end, _ptr(q), k, _ptr(sel_idx), _ptr(sel_cnt),
-                                   _stream(stream))
+    st = _xkv.sr_select_static(G, batch, T, H_kv, H_q, d_h, chunk, landmarks, layer_begin, layer_end, q, k, sel_idx, sel_cnt,
+                               stream)
     if st != XKV_OK:
         raise XKVError(st, "xkv_sr_select_static")
 
 
 def xkv_sr_reconstruct_attend(grp: Group, layer_begin: int, layer_end: int, q, sel_idx, sel_cnt, k_cap: int,
                               out, lse=None, stream=None) -> None:
-    st = _lib.xkv_sr_reconstruct_attend(grp.handle, layer_begin, layer_end, _ptr(q), _ptr(sel_idx), _ptr(sel_cnt),
-                                        k_cap, _ptr(out), _ptr(lse), _stream(stream))
+    st = _xkv.sr_reconstruct_attend(grp.handle, layer_begin, layer_end, q, sel_idx, sel_cnt, k_cap, out, lse, stream)
     if st != XKV_OK:
         raise XKVError(st, "xkv_sr_reconstruct_attend")
 
@@ -293,10 +292,8 @@ def xkv_sr_reconstruct_attend_tail(grp: Group, layer_begin: int, layer_end: int,
                                    tail_k, tail_v, tail_len, tail_cap: int, workspace, out, lse=None,
                                    stream=None) -> None:
     """`workspace`: a device tensor of at least xkv_tail_workspace_bytes(grp, tail_cap) bytes."""
-    st = _lib.xkv_sr_reconstruct_attend_tail(grp.handle, layer_begin, layer_end, _ptr(q), _ptr(sel_idx), _ptr(sel_cnt),
-                                             k_cap, _ptr(tail_k), _ptr(tail_v), _ptr(tail_len), tail_cap,
-                                             _ptr(workspace), workspace.numel() * workspace.element_size(),
-                                             _ptr(out), _ptr(lse), _stream(stream))
+    st = _xkv.sr_reconstruct_attend_tail(grp.handle, layer_begin, layer_end, q, sel_idx, sel_cnt, k_cap, tail_k, tail_v,
+                                         tail_len, tail_cap, workspace, workspace.nbytes, out, lse, stream)
     if st != XKV_OK:
         raise XKVError(st, "xkv_sr_reconstruct_attend_tail")
 
@@ -304,12 +301,12 @@ def xkv_sr_reconstruct_attend_tail(grp: Group, layer_begin: int, layer_end: int,
 def xkv_quantize_rtn(x, bits: int = 4, stream=None):
     """RTN-quantise a bf16 device tensor [..., cols] along its last axis in groups of 32 (include/xkv.h).
     Returns (codes uint8 [..., cols/2], meta int32 [..., cols/32] or None for 3 bits) device tensors."""
-    cols = x.shape[-1]
+    *lead, cols = x.shape
     rows = x.numel() // cols
-    codes = torch.empty(x.shape[:-1] + (cols // 2,), dtype=torch.uint8, device=x.device)
+    codes = x.new_empty((*lead, cols // 2), dtype=torch.uint8)
     # 4 bits: one scale/offset word per group beside the codes; 3 bits: the 16-byte records hold them (meta is None)
-    meta = torch.empty(x.shape[:-1] + (cols // 32,), dtype=torch.int32, device=x.device) if bits == 4 else None
-    st = _lib.xkv_quantize_rtn(_ptr(x), rows, cols, bits, _ptr(codes), _ptr(meta), _stream(stream))
+    meta = x.new_empty((*lead, cols // 32), dtype=torch.int32) if bits == 4 else None
+    st = _xkv.quantize_rtn(x, rows, cols, bits, codes, meta, stream)
     if st != XKV_OK:
         raise XKVError(st, "xkv_quantize_rtn")
     return codes, meta
@@ -317,10 +314,10 @@ def xkv_quantize_rtn(x, bits: int = 4, stream=None):
 
 def xkv_dequantize_rtn(codes, meta, bits: int = 4, stream=None):
     """bf16 tensor [..., cols] of the dequantised values x_hat."""
-    cols = codes.shape[-1] * 2
-    rows = codes.numel() // (cols // 2)
-    x = torch.empty(codes.shape[:-1] + (cols,), dtype=torch.bfloat16, device=codes.device)
-    st = _lib.xkv_dequantize_rtn(_ptr(codes), _ptr(meta), rows, cols, bits, _ptr(x), _stream(stream))
+    *lead, half = codes.shape
+    cols, rows = half * 2, codes.numel() // half
+    x = codes.new_empty((*lead, cols), dtype=torch.bfloat16)
+    st = _xkv.dequantize_rtn(codes, meta, rows, cols, bits, x, stream)
     if st != XKV_OK:
         raise XKVError(st, "xkv_dequantize_rtn")
     return x
@@ -405,9 +402,8 @@ def xkv_dense_workspace_bytes(grp: Group, cap: int) -> int:
 def xkv_dense_attend(grp: Group, layer_begin: int, layer_end: int, q, K, V, length, cap: int, workspace, out, lse=None,
                      stream=None) -> None:
     """Plain decode attention over an uncompressed cache K, V [G][batch][H_kv][cap][d_h] (the dense baseline)."""
-    st = _lib.xkv_dense_attend(grp.handle, layer_begin, layer_end, _ptr(q), _ptr(K), _ptr(V), _ptr(length), cap,
-                               _ptr(workspace), workspace.numel() * workspace.element_size(), _ptr(out), _ptr(lse),
-                               _stream(stream))
+    st = _xkv.dense_attend(grp.handle, layer_begin, layer_end, q, K, V, length, cap, workspace, workspace.nbytes, out, lse,
+                           stream)
     if st != XKV_OK:
         raise XKVError(st, "xkv_dense_attend")
 
