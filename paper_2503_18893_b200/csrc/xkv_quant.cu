@@ -16,156 +16,213 @@ namespace xkv {
 namespace {
 
 constexpr int kQuantThreads = 256;
+constexpr int kQuantPieces = 4;    // 16-byte pieces per thread, all requested before the first is used
 
-// One thread per group of 32 scalars.
+__device__ __forceinline__ uint32_t min_bf16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("min.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+
+// HBM bound: 2 bytes read and (bits + 1) / 8 written per scalar.  Four consecutive lanes share a group of 32 scalars, a
+// lane holds one 16-byte piece (8 scalars): loads and stores of a warp are contiguous, extrema are packed bf16 minima
+// folded by two shuffles.
+// The codes are rint(fl(f / scale)), f = x - zero.  The correctly rounded quotient comes from the correctly rounded
+// reciprocal y by q = f y, q + (f - q scale) y with fused multiply-adds (Markstein, IBM J. Res. Dev. 34(1), 1990); the
+// exact quotient of a 24-bit by an 8-bit number is never closer than 2^-33 to a rounding boundary and the value that is
+// rounded last is off by less than 2^-46, so every bit is that of the division.  Half-integers are common here
+// (differences of bf16 numbers over a bf16 scale): the quotient has to be exact, a test with a fallback diverged in most
+// warps (25 us for 65536 x 384 scalars, with an IEEE division per scalar and one thread per group 38 us; this form 12 us).
+// Rounding goes through 1.5 * 2^23, whose sum with the quotient holds the integer in its low bits.
+constexpr float kRintMagic = 12582912.0f;
+
+template <int BITS>
+__device__ __forceinline__ uint32_t rtn_code_exact(float f, float scale) {
+  constexpr float kTop = (float)((1 << BITS) - 1);
+  float q = 0.0f;
+  if (scale > 0.0f) q = rintf(__fdiv_rn(f, scale));          // ties to even
+  return (uint32_t)fminf(fmaxf(q, 0.0f), kTop);
+}
+
+template <int BITS>
 __global__ void __launch_bounds__(kQuantThreads)
-quantize_rtn4_kernel(const __nv_bfloat16* __restrict__ x, long long n_groups, uint4* __restrict__ codes,
-                     uint32_t* __restrict__ meta) {
-  const long long gidx = (long long)blockIdx.x * kQuantThreads + threadIdx.x;
-  if (gidx >= n_groups) return;
-  const uint4* src = reinterpret_cast<const uint4*>(x + gidx * 32);
-  float v[32];
+quantize_rtn_kernel(const uint4* __restrict__ x, long long n_pieces, uint32_t* __restrict__ codes, uint32_t* __restrict__ meta) {
+  constexpr float kTop = (float)((1 << BITS) - 1);
+  const int p = threadIdx.x & 3;                           // piece of the group; n_pieces is a multiple of 4
+  const long long first = (long long)blockIdx.x * (kQuantThreads * kQuantPieces) + threadIdx.x;
+  ptx::grid_dependency_wait();
+  ptx::grid_dependency_launch();
+  uint4 v[kQuantPieces];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint4 u = src[i];
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) { v[8 * i + 2 * e] = __uint_as_float(w[e] << 16); v[8 * i + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u); }
+  for (int u = 0; u < kQuantPieces; ++u) {
+    const long long i = first + u * kQuantThreads;
+    v[u] = i < n_pieces ? __ldcs(x + i) : make_uint4(0u, 0u, 0u, 0u);
   }
-  float lo = v[0], hi = v[0];
 #pragma unroll
-  for (int i = 1; i < 32; ++i) { lo = fminf(lo, v[i]); hi = fmaxf(hi, v[i]); }
-  const __nv_bfloat16 zb = __float2bfloat16_rn(lo);
-  const __nv_bfloat16 sb = __float2bfloat16_rn(__fdiv_rn(__fsub_rn(hi, lo), 15.0f));
-  const float zero = __bfloat162float(zb), scale = __bfloat162float(sb);
-  uint32_t word[4];
+  for (int u = 0; u < kQuantPieces; ++u) {
+    const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+    uint32_t lo2 = min_bf16x2(min_bf16x2(w[0], w[1]), min_bf16x2(w[2], w[3]));
+    uint32_t hi2 = max_bf16x2(max_bf16x2(w[0], w[1]), max_bf16x2(w[2], w[3]));
 #pragma unroll
-  for (int wi = 0; wi < 4; ++wi) {
-    uint32_t w = 0;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      float q = 0.0f;
-      if (scale > 0.0f) q = rintf(__fdiv_rn(__fsub_rn(v[8 * wi + e], zero), scale));     // ties to even
-      q = fminf(fmaxf(q, 0.0f), 15.0f);
-      const uint32_t c = (uint32_t)q;
-      w |= c << (4 * (e >> 1) + 16 * (e & 1));
+    for (int o = 1; o < 4; o <<= 1) {
+      lo2 = min_bf16x2(lo2, __shfl_xor_sync(0xffffffffu, lo2, o));
+      hi2 = max_bf16x2(hi2, __shfl_xor_sync(0xffffffffu, hi2, o));
     }
-    word[wi] = w;
-  }
-  codes[gidx] = make_uint4(word[0], word[1], word[2], word[3]);
-  meta[gidx] = (uint32_t)__bfloat16_as_ushort(sb) | ((uint32_t)__bfloat16_as_ushort(zb) << 16);
-}
-
-// x_hat of one group per thread: bf16(code * scale + zero) with a single rounding (the packed bf16 fused
-// multiply-add rounds the exact value once; small integers are exact in bf16).
-__global__ void __launch_bounds__(kQuantThreads)
-dequantize_rtn4_kernel(const uint4* __restrict__ codes, const uint32_t* __restrict__ meta, long long n_groups,
-                       uint4* __restrict__ x) {
-  const long long gidx = (long long)blockIdx.x * kQuantThreads + threadIdx.x;
-  if (gidx >= n_groups) return;
-  const uint4 cw = codes[gidx];
-  const uint32_t m = meta[gidx];
-  const uint32_t w[4] = {cw.x, cw.y, cw.z, cw.w};
-  uint32_t o[16];
+    const float lo = fminf(__uint_as_float(lo2 << 16), __uint_as_float(lo2 & 0xffff0000u));
+    const float hi = fmaxf(__uint_as_float(hi2 << 16), __uint_as_float(hi2 & 0xffff0000u));
+    const __nv_bfloat16 zb = __float2bfloat16_rn(lo);
+    const __nv_bfloat16 sb = __float2bfloat16_rn(__fdiv_rn(__fsub_rn(hi, lo), kTop));
+    const float zero = __bfloat162float(zb), scale = __bfloat162float(sb);
+    float f[8], m[8];                                      // m: rint(quotient) + kRintMagic
 #pragma unroll
-  for (int wi = 0; wi < 4; ++wi) ptx::dequant_word(w[wi], m, &o[4 * wi]);
-  uint4* dst = x + gidx * 4;
+    for (int e = 0; e < 4; ++e) {
+      f[2 * e] = __fsub_rn(__uint_as_float(w[e] << 16), zero);
+      f[2 * e + 1] = __fsub_rn(__uint_as_float(w[e] & 0xffff0000u), zero);
+    }
+    // constant groups, scales with an imprecise or overflowing reciprocal, infinities: the division for every scalar
+    if (!(scale >= 1e-30f && scale <= 1e30f)) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) dst[i] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
-}
-
-// The 3-bit variant: 16-byte records {meta, w0, w1, w2} per group (layout beside dequant_group3).
-__global__ void __launch_bounds__(kQuantThreads)
-quantize_rtn3_kernel(const __nv_bfloat16* __restrict__ x, long long n_groups, uint4* __restrict__ rec) {
-  const long long gidx = (long long)blockIdx.x * kQuantThreads + threadIdx.x;
-  if (gidx >= n_groups) return;
-  const uint4* src = reinterpret_cast<const uint4*>(x + gidx * 32);
-  float v[32];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint4 u = src[i];
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) { v[8 * i + 2 * e] = __uint_as_float(w[e] << 16); v[8 * i + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u); }
-  }
-  float lo = v[0], hi = v[0];
-#pragma unroll
-  for (int i = 1; i < 32; ++i) { lo = fminf(lo, v[i]); hi = fmaxf(hi, v[i]); }
-  const __nv_bfloat16 zb = __float2bfloat16_rn(lo);
-  const __nv_bfloat16 sb = __float2bfloat16_rn(__fdiv_rn(__fsub_rn(hi, lo), 7.0f));
-  const float zero = __bfloat162float(zb), scale = __bfloat162float(sb);
-  uint32_t word[3] = {0u, 0u, 0u};
-#pragma unroll
-  for (int e = 0; e < 32; ++e) {
-    float q = 0.0f;
-    if (scale > 0.0f) q = rintf(__fdiv_rn(__fsub_rn(v[e], zero), scale));       // ties to even
-    q = fminf(fmaxf(q, 0.0f), 7.0f);
-    const uint32_t c = (uint32_t)q;
-    if (e < 30) {
-      const int j = e / 10, k = (e % 10) >> 1;
-      word[j] |= c << (3 * k + 16 * (e & 1));
+      for (int e = 0; e < 8; ++e) m[e] = (float)rtn_code_exact<BITS>(f[e], scale) + kRintMagic;
     } else {
-      const int sh = e == 30 ? 15 : 31;
-      word[0] |= (c & 1u) << sh; word[1] |= ((c >> 1) & 1u) << sh; word[2] |= ((c >> 2) & 1u) << sh;
+      const float y = __frcp_rn(scale);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float t = __fmul_rn(f[e], y);
+        m[e] = __fadd_rn(__fmaf_rn(__fmaf_rn(-t, scale, f[e]), y, t), kRintMagic);
+      }
+    }
+    uint32_t c[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) c[e] = __float_as_uint(m[e]) & ((1u << BITS) - 1u);
+    const uint32_t mw = (uint32_t)__bfloat16_as_ushort(sb) | ((uint32_t)__bfloat16_as_ushort(zb) << 16);
+    uint32_t word = 0;
+    if constexpr (BITS == 4) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) word |= c[e] << (4 * (e >> 1) + 16 * (e & 1));
+    } else {
+      // the quad's 32 codes as four words of nibbles; lane 0 keeps the scale/offset word, lane j + 1 builds w_j
+#pragma unroll
+      for (int e = 0; e < 8; ++e) word |= c[e] << (4 * e);
+      uint32_t n[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) n[i] = __shfl_sync(0xffffffffu, word, i, 4);
+      const uint32_t a = p == 1 ? n[0] : p == 2 ? __funnelshift_r(n[1], n[2], 8) : __funnelshift_r(n[2], n[3], 16);
+      const uint32_t b = p == 1 ? n[1] : p == 2 ? n[2] >> 8 : n[3] >> 16;
+      word = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) word |= ((a >> (8 * k)) & 7u) << (3 * k) | ((a >> (8 * k + 4)) & 7u) << (3 * k + 16);
+      word |= (b & 7u) << 12 | ((b >> 4) & 7u) << 28;
+      word |= ((n[3] >> (24 + p - 1)) & 1u) << 15 | ((n[3] >> (28 + p - 1)) & 1u) << 31;
+      if (p == 0) word = mw;
+    }
+    const long long i = first + u * kQuantThreads;
+    if (i < n_pieces) {
+      __stcs(codes + i, word);
+      if (BITS == 4 && p == 0) __stcs(meta + (i >> 2), mw);
     }
   }
-  rec[gidx] = make_uint4((uint32_t)__bfloat16_as_ushort(sb) | ((uint32_t)__bfloat16_as_ushort(zb) << 16), word[0], word[1], word[2]);
 }
 
+// x_hat: bf16(code * scale + zero) with a single rounding (the packed bf16 fused multiply-add rounds the exact value
+// once; small integers are exact in bf16).  One thread per 8 scalars, so that the 16-byte stores of a warp are contiguous.
+__global__ void __launch_bounds__(kQuantThreads)
+dequantize_rtn4_kernel(const uint32_t* __restrict__ codes, const uint32_t* __restrict__ meta, long long n_pieces,
+                       uint4* __restrict__ x) {
+  const long long first = (long long)blockIdx.x * (kQuantThreads * kQuantPieces) + threadIdx.x;
+  ptx::grid_dependency_wait();
+  ptx::grid_dependency_launch();
+  uint32_t w[kQuantPieces], m[kQuantPieces];
+#pragma unroll
+  for (int u = 0; u < kQuantPieces; ++u) {
+    const long long i = first + u * kQuantThreads;
+    w[u] = i < n_pieces ? __ldg(codes + i) : 0u;
+    m[u] = i < n_pieces ? __ldg(meta + (i >> 2)) : 0u;
+  }
+#pragma unroll
+  for (int u = 0; u < kQuantPieces; ++u) {
+    const long long i = first + u * kQuantThreads;
+    uint32_t o[4];
+    ptx::dequant_word(w[u], m[u], o);
+    if (i < n_pieces) x[i] = make_uint4(o[0], o[1], o[2], o[3]);
+  }
+}
+
+// The 3-bit variant, one thread per 16-byte record; the 64 bytes of a group go through shared memory so that the
+// stores of a warp are contiguous (unit u of group g sits at g * 4 + (u ^ (g / 2 % 4)): no bank conflicts either way).
 __global__ void __launch_bounds__(kQuantThreads)
 dequantize_rtn3_kernel(const uint4* __restrict__ rec, long long n_groups, uint4* __restrict__ x) {
-  const long long gidx = (long long)blockIdx.x * kQuantThreads + threadIdx.x;
-  if (gidx >= n_groups) return;
-  const uint4 r = rec[gidx];
-  uint32_t o[16];
-  ptx::dequant_group3(r.x, r.y, r.z, r.w, o);
-  uint4* dst = x + gidx * 4;
+  __shared__ uint4 stage[kQuantThreads * 4];
+  const int tid = threadIdx.x;
+  const long long g0 = (long long)blockIdx.x * kQuantThreads;
+  ptx::grid_dependency_wait();
+  ptx::grid_dependency_launch();
+  if (g0 + tid < n_groups) {
+    const uint4 r = rec[g0 + tid];
+    uint32_t o[16];
+    ptx::dequant_group3(r.x, r.y, r.z, r.w, o);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) dst[i] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+    for (int i = 0; i < 4; ++i) stage[tid * 4 + (i ^ ((tid >> 1) & 3))] = make_uint4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int e = tid + i * kQuantThreads, g = e >> 2;
+    if (g0 + g < n_groups) x[g0 * 4 + e] = stage[g * 4 + ((e & 3) ^ ((g >> 1) & 3))];
+  }
+}
+
+// Blocks for n items, `per` to a block; false if there are too many for a grid.
+bool blocks_for(long long n, int per, unsigned* blocks) {
+  const long long b = (n + per - 1) / per;
+  *blocks = (unsigned)b;
+  return b <= 0x7fffffffLL;
 }
 
 }  // namespace
 
 cudaError_t launch_quantize_rtn3(const __nv_bfloat16* x, long long rows, int cols, void* rec, cudaStream_t s) {
-  const long long n_groups = rows * (cols / 32);
-  if (n_groups == 0) return cudaSuccess;
-  const long long blocks = (n_groups + kQuantThreads - 1) / kQuantThreads;
-  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  quantize_rtn3_kernel<<<(unsigned)blocks, kQuantThreads, 0, s>>>(x, n_groups, (uint4*)rec);
+  const long long n_pieces = rows * (cols / 8);
+  if (n_pieces == 0) return cudaSuccess;
+  unsigned blocks;
+  if (!blocks_for(n_pieces, kQuantThreads * kQuantPieces, &blocks)) return cudaErrorInvalidValue;
   count_launch(kFamPrep);
-  return cudaGetLastError();
+  return launch_pdl(quantize_rtn_kernel<3>, dim3(blocks), dim3(kQuantThreads), 0, s, (const uint4*)x, n_pieces, (uint32_t*)rec,
+                    (uint32_t*)nullptr);
 }
 
 cudaError_t launch_dequantize_rtn3(const void* rec, long long rows, int cols, __nv_bfloat16* x, cudaStream_t s) {
   const long long n_groups = rows * (cols / 32);
   if (n_groups == 0) return cudaSuccess;
-  const long long blocks = (n_groups + kQuantThreads - 1) / kQuantThreads;
-  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  dequantize_rtn3_kernel<<<(unsigned)blocks, kQuantThreads, 0, s>>>((const uint4*)rec, n_groups, (uint4*)x);
+  unsigned blocks;
+  if (!blocks_for(n_groups, kQuantThreads, &blocks)) return cudaErrorInvalidValue;
   count_launch(kFamPrep);
-  return cudaGetLastError();
+  return launch_pdl(dequantize_rtn3_kernel, dim3(blocks), dim3(kQuantThreads), 0, s, (const uint4*)rec, n_groups, (uint4*)x);
 }
 
 cudaError_t launch_quantize_rtn4(const __nv_bfloat16* x, long long rows, int cols, void* codes, void* meta, cudaStream_t s) {
-  const long long n_groups = rows * (cols / 32);
-  if (n_groups == 0) return cudaSuccess;
-  const long long blocks = (n_groups + kQuantThreads - 1) / kQuantThreads;
-  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  quantize_rtn4_kernel<<<(unsigned)blocks, kQuantThreads, 0, s>>>(x, n_groups, (uint4*)codes, (uint32_t*)meta);
+  const long long n_pieces = rows * (cols / 8);
+  if (n_pieces == 0) return cudaSuccess;
+  unsigned blocks;
+  if (!blocks_for(n_pieces, kQuantThreads * kQuantPieces, &blocks)) return cudaErrorInvalidValue;
   count_launch(kFamPrep);
-  return cudaGetLastError();
+  return launch_pdl(quantize_rtn_kernel<4>, dim3(blocks), dim3(kQuantThreads), 0, s, (const uint4*)x, n_pieces, (uint32_t*)codes,
+                    (uint32_t*)meta);
 }
 
 cudaError_t launch_dequantize_rtn4(const void* codes, const void* meta, long long rows, int cols, __nv_bfloat16* x,
                                    cudaStream_t s) {
-  const long long n_groups = rows * (cols / 32);
-  if (n_groups == 0) return cudaSuccess;
-  const long long blocks = (n_groups + kQuantThreads - 1) / kQuantThreads;
-  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  dequantize_rtn4_kernel<<<(unsigned)blocks, kQuantThreads, 0, s>>>((const uint4*)codes, (const uint32_t*)meta, n_groups,
-                                                                     (uint4*)x);
+  const long long n_pieces = rows * (cols / 8);
+  if (n_pieces == 0) return cudaSuccess;
+  unsigned blocks;
+  if (!blocks_for(n_pieces, kQuantThreads * kQuantPieces, &blocks)) return cudaErrorInvalidValue;
   count_launch(kFamPrep);
-  return cudaGetLastError();
+  return launch_pdl(dequantize_rtn4_kernel, dim3(blocks), dim3(kQuantThreads), 0, s, (const uint32_t*)codes, (const uint32_t*)meta,
+                    n_pieces, (uint4*)x);
 }
 
 }  // namespace xkv
