@@ -225,6 +225,255 @@ landmark_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restric
   }
 }
 
+using u64 = unsigned long long;    // two fp32 values, for the packed fp32 instructions
+__device__ __forceinline__ u64 pack2(float a, float b) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(u64 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+  u64 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
+  u64 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ u64 add2(u64 a, u64 b) {
+  u64 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// The default chunk of 8 rows (c == 8): HBM bound, persistent CTAs that walk a contiguous range of row blocks for every
+// (sequence, layer).
+// A chunk's rows are rotated by R^(8j + f), R the rotation by theta, so the mean is R^8j mu with mu = sum_f R^f x_f / 8,
+// a Horner recurrence in R alone; the cosines need no more than R either (<R^(8j+f) x_f, R^8j mu> = <x_f, R^-f mu>).
+// Only the one rotation by 8j per chunk comes from a table (fp64 recurrence from block to block, pow and sincos once
+// per CTA).  (With one table row per key row, built per CTA and layer, the fp64 work and the table loads took as long as
+// everything else: 677 us for 131072 rows of four layers of eight heads with cosines; 363 us with the table shared by
+// the layers and the rows kept in registers; this form 304 us, the issue slots 57 % busy.)
+// A thread holds the 8 rows of its 8 rotary pairs in registers (64 registers), so the cosine pass reads nothing again,
+// while its next chunk is on the way into 256 bytes of shared memory of its own (no barrier: nobody else reads them).
+// The arithmetic is packed fp32 (two pairs per instruction).  The sums of the cosine pass over the threads of a head are
+// folded by halving (a lane ends with one row: 14 shuffles for the 16 sums of a chunk instead of 6 per row).
+constexpr int kLm8MaxChunks = 8;    // chunks of a row block
+template <int DH, bool ROPE>
+__global__ void __launch_bounds__(kLmThreads, 2)
+landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restrict__ landmarks, float* __restrict__ min_cos,
+                 int G, int batch, int T, int H_kv, int n_c, int n_blocks, double rope_base) {
+  constexpr int HALF = DH / 2, APH = HALF / 8;
+  constexpr int EPT = ROPE ? kLm8MaxChunks * HALF / kLmThreads : 1;   // table entries per thread
+  extern __shared__ __align__(16) uint4 slots_s[];       // [16][kLmThreads] pieces of the chunk on its way
+  __shared__ __align__(16) float4 tab_s[ROPE ? kLm8MaxChunks * HALF / 2 : 1];   // [chunk][4][APH] {cos, cos, sin, sin} of two pairs
+  __shared__ double2 rot_s[ROPE ? EPT + 1 : 1][ROPE ? kLmThreads : 1];          // a thread's entries; the step to the next block
+  const int tid = threadIdx.x;
+  const int TPR = H_kv * APH, RG = kLmThreads / TPR;     // threads per row of all heads, chunks side by side
+  const int CPB = min(RG, kLm8MaxChunks);                // chunks of a row block; the other row groups take other layers
+  const int LG = RG / CPB;
+  const int rg = tid / TPR, tr = tid % TPR;
+  const int g = tr / APH, a = tr % APH;
+  const int jc = rg % CPB, lg = rg / CPB;
+  const int d = H_kv * DH, n_lb = G * batch;
+  const int b_begin = (int)((long long)blockIdx.x * n_blocks / gridDim.x), b_end = (int)((long long)(blockIdx.x + 1) * n_blocks / gridDim.x);
+
+  // table entries tid, tid + kLmThreads, ...: pair ii of chunk tid / HALF + i * (kLmThreads / HALF)
+  const int ii = tid % HALF;
+  float* const tab_f = reinterpret_cast<float*>(tab_s) + ((((ii & 7) >> 1) * APH + (ii >> 3)) * 4 + (ii & 1));
+  u64 c1[4], s1[4], n1[4];                               // R of this thread's pairs: cos, sin, -sin
+  if (ROPE) {
+    const double th = pow(rope_base, -(double)ii / (double)HALF) / 3.14159265358979323846;
+    double2 v;
+    sincospi(th, &v.y, &v.x);                            // R of pair ii for everybody, by way of the table
+    if (tid < HALF) { tab_f[0] = (float)v.x; tab_f[2] = (float)v.y; }
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) {
+      sincospi((double)(8 * (b_begin * CPB + tid / HALF + i * (kLmThreads / HALF))) * th, &v.y, &v.x);
+      rot_s[i][tid] = v;
+    }
+    sincospi((double)(8 * CPB) * th, &v.y, &v.x);
+    rot_s[EPT][tid] = v;
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float4 t = tab_s[e * APH + a];
+      c1[e] = pack2(t.x, t.y); s1[e] = pack2(t.z, t.w); n1[e] = pack2(-t.z, -t.w);
+    }
+  }
+
+  uint4 u1[8], u2[8];
+  uint4* const slot = slots_s + tid;
+  const uint32_t slot_addr = ptx::smem_u32(slot);
+  auto request_chunk = [&](int blk, int lb) {             // lb = sequence * G + layer
+    const int j = blk * CPB + jc;
+    if (j >= n_c) return;
+    const int row0 = j * 8, last = min(8, T - row0) - 1;
+    const __nv_bfloat16* kr = keys + ((size_t)lb * T + row0) * d + (size_t)g * DH + a * 8;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const __nv_bfloat16* p = kr + (size_t)min(r, last) * d;
+      ptx::cp_async16(slot_addr + (uint32_t)(2 * r) * (kLmThreads * 16), p, 16u);
+      ptx::cp_async16(slot_addr + (uint32_t)(2 * r + 1) * (kLmThreads * 16), p + HALF, 16u);
+    }
+  };
+  // (only the lanes of one head take part: the row groups of a warp may be in different chunks)
+  const uint32_t hmask = ((1u << APH) - 1u) << ((tid & 31) & ~(APH - 1));
+  // the four couples of pairs of one half of row r, widened to fp32
+  auto widen = [](const uint4& v, u64 (&x)[4]) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) x[e] = pack2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u));
+  };
+
+  if (b_begin < b_end && lg < n_lb) request_chunk(b_begin, lg);
+  for (int blk = b_begin; blk < b_end; ++blk) {
+    if (ROPE) {
+      __syncthreads();                                    // everybody is done with the table of the previous block
+      const double2 step = rot_s[EPT][tid];
+#pragma unroll
+      for (int i = 0; i < EPT; ++i) {
+        const int jj = tid / HALF + i * (kLmThreads / HALF);
+        if (jj < CPB) {
+          const double2 at = rot_s[i][tid];
+          tab_f[(size_t)jj * HALF * 2] = (float)at.x;
+          tab_f[(size_t)jj * HALF * 2 + 2] = (float)at.y;
+          rot_s[i][tid] = make_double2(at.x * step.x - at.y * step.y, at.y * step.x + at.x * step.y);
+        }
+      }
+      __syncthreads();
+    }
+    const int j = blk * CPB + jc;
+    for (int lb = lg; lb < n_lb; lb += LG) {
+      // this thread's own copies have landed; into registers, and the next chunk on its way
+      asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+      for (int r = 0; r < 8; ++r) { u1[r] = slot[(2 * r) * kLmThreads]; u2[r] = slot[(2 * r + 1) * kLmThreads]; }
+      if (lb + LG < n_lb) request_chunk(blk, lb + LG);
+      else if (blk + 1 < b_end) request_chunk(blk + 1, lg);
+      if (j >= n_c) continue;
+      const int rows = min(8, T - j * 8);
+      u64 m1[4], m2[4];                                   // mu = sum_f R^f x_f / rows
+#pragma unroll
+      for (int e = 0; e < 4; ++e) m1[e] = m2[e] = 0ull;
+#pragma unroll
+      for (int r = 7; r >= 0; --r) {
+        if (r < rows) {
+          u64 x1[4], x2[4];
+          widen(u1[r], x1); widen(u2[r], x2);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            if (ROPE) {
+              const u64 t = fma2(m1[e], c1[e], fma2(m2[e], n1[e], x1[e]));
+              m2[e] = fma2(m2[e], c1[e], fma2(m1[e], s1[e], x2[e]));
+              m1[e] = t;
+            } else {
+              m1[e] = add2(m1[e], x1[e]);
+              m2[e] = add2(m2[e], x2[e]);
+            }
+          }
+        }
+      }
+      const float inv = 1.0f / (float)rows;
+      const u64 inv2 = pack2(inv, inv);
+      float o1[8], o2[8];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        m1[e] = mul2(m1[e], inv2);
+        m2[e] = mul2(m2[e], inv2);
+        const float2 p = unpack2(m1[e]), q = unpack2(m2[e]);
+        if (ROPE) {
+          const float4 t = tab_s[(jc * 4 + e) * APH + a];
+          o1[2 * e] = p.x * t.x - q.x * t.z; o1[2 * e + 1] = p.y * t.y - q.y * t.w;
+          o2[2 * e] = q.x * t.x + p.x * t.z; o2[2 * e + 1] = q.y * t.y + p.y * t.w;
+        } else {
+          o1[2 * e] = p.x; o1[2 * e + 1] = p.y; o2[2 * e] = q.x; o2[2 * e + 1] = q.y;
+        }
+      }
+      __nv_bfloat16* L = landmarks + (((size_t)lb * H_kv + g) * n_c + j) * DH + a * 8;
+      *reinterpret_cast<uint4*>(L) = pack8(o1);
+      *reinterpret_cast<uint4*>(L + HALF) = pack8(o2);
+      if (min_cos) {
+        float v[16];                                      // per row: dot product with the mean, squared norm
+        u64 w = 0ull;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) w = fma2(m1[e], m1[e], fma2(m2[e], m2[e], w));
+        const float2 wf = unpack2(w);
+        float mn2 = wf.x + wf.y;
+#pragma unroll
+        for (int o = 1; o < APH; o <<= 1) mn2 += __shfl_xor_sync(hmask, mn2, o);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          u64 x1[4], x2[4], dot = 0ull, nn = 0ull;
+          widen(u1[r], x1); widen(u2[r], x2);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            nn = fma2(x1[e], x1[e], nn);
+            nn = fma2(x2[e], x2[e], nn);
+            dot = fma2(x1[e], m1[e], dot);
+            dot = fma2(x2[e], m2[e], dot);
+            if (ROPE && r < rows - 1) {                   // R^-1 for the next row (a repeated last row changes no minimum)
+              const u64 t = fma2(m1[e], c1[e], mul2(m2[e], s1[e]));
+              m2[e] = fma2(m2[e], c1[e], mul2(m1[e], n1[e]));
+              m1[e] = t;
+            }
+          }
+          const float2 d2 = unpack2(dot), n2 = unpack2(nn);
+          v[2 * r] = d2.x + d2.y; v[2 * r + 1] = n2.x + n2.y;
+        }
+        // fold by halving: after the step with distance o a lane keeps the half of the rows its bit selects
+#pragma unroll
+        for (int o = APH / 2, n = 8; o > 0; o >>= 1, n >>= 1) {
+          const bool up = (a & o) != 0;
+#pragma unroll
+          for (int i = 0; i < n; ++i) {
+            const float mine = up ? v[n + i] : v[i], other = up ? v[i] : v[n + i];
+            v[i] = mine + __shfl_xor_sync(hmask, other, o);
+          }
+        }
+        float best = INFINITY;
+#pragma unroll
+        for (int i = 0; i < 16 / APH; i += 2) {
+          const float den = sqrtf(v[i + 1]) * sqrtf(mn2);
+          best = fminf(best, den > 0.0f ? v[i] / den : 0.0f);
+        }
+#pragma unroll
+        for (int o = 1; o < APH; o <<= 1) best = fminf(best, __shfl_xor_sync(hmask, best, o));
+        const int b = lb / G, l = lb - b * G;
+        if (a == 0) min_cos[(((size_t)l * batch + b) * H_kv + g) * n_c + j] = best;
+      }
+    }
+  }
+}
+
+template <int DH>
+cudaError_t launch_landmark8(const __nv_bfloat16* keys, __nv_bfloat16* landmarks, float* min_cos, int G, int batch, int T,
+                             int H_kv, float rope_base, cudaStream_t s) {
+  const int n_c = (T + 7) / 8, tpr = H_kv * DH / 16;
+  const int cpb = kLmThreads / tpr < kLm8MaxChunks ? kLmThreads / tpr : kLm8MaxChunks;
+  const int n_blocks = (n_c + cpb - 1) / cpb;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int grid = n_blocks < 2 * sms ? n_blocks : 2 * sms;           // two CTAs per SM, one wave
+  const size_t smem = (size_t)kLmThreads * 256;
+  const bool rope = rope_base > 0.0f;
+  e = rope ? ensure_dyn_smem<landmark8_kernel<DH, true>>(smem, dev) : ensure_dyn_smem<landmark8_kernel<DH, false>>(smem, dev);
+  if (e != cudaSuccess) return e;
+  if (rope)
+    landmark8_kernel<DH, true><<<grid, kLmThreads, smem, s>>>(keys, landmarks, min_cos, G, batch, T, H_kv, n_c, n_blocks, (double)rope_base);
+  else
+    landmark8_kernel<DH, false><<<grid, kLmThreads, smem, s>>>(keys, landmarks, min_cos, G, batch, T, H_kv, n_c, n_blocks, 1.0);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_landmarks(const __nv_bfloat16* keys, __nv_bfloat16* landmarks, float* min_cos, int G, int batch, int T,
@@ -232,6 +481,12 @@ cudaError_t launch_landmarks(const __nv_bfloat16* keys, __nv_bfloat16* landmarks
   const int n_c = (T + c - 1) / c;
   const int tpr = H_kv * d_h / 16;                        // threads per key row
   if (tpr > kLmThreads || kLmThreads % tpr != 0) return cudaErrorInvalidValue;
+  if (c == 8) {                                           // the default chunk has a kernel of its own
+    const cudaError_t e = d_h == 128 ? launch_landmark8<128>(keys, landmarks, min_cos, G, batch, T, H_kv, rope_base, s)
+                                     : launch_landmark8<64>(keys, landmarks, min_cos, G, batch, T, H_kv, rope_base, s);
+    count_launch(kFamLandmarks);
+    return e;
+  }
   const int cpc = c >= kLmRows ? 1 : kLmRows / c;
   const dim3 grid((n_c + cpc - 1) / cpc, G, batch);
   const int use_rope = rope_base > 0.0f ? 1 : 0;
