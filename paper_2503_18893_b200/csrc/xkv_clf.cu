@@ -550,63 +550,61 @@ trsolve_mma_kernel(const float* __restrict__ U, const double* __restrict__ L, co
 
 namespace {
 
-// Eigen-decomposition of the symmetric l x l matrix M by cyclic Jacobi rotations in the round-robin (tournament)
-// order: every round rotates l/2 disjoint index pairs at once.  A check per sweep ends the sweeps once the
-// off-diagonal weight is below kJacobiTol.  On return the eigenvalues are on the diagonal of M, the
-// eigenvectors the columns of P.
-constexpr int kJacobiMaxPairs = 1024;
-constexpr int kJacobiSweeps = 12;
+// Eigen-decomposition of the symmetric l x l matrix M by block Jacobi in one cooperative kernel.  Blocks of 32 indices
+// meet in round-robin (tournament) order: l/32 - 1 rounds per sweep, l/64 disjoint block pairs in a round.  A round:
+//   A  one CTA per pair takes the pair's 64 x 64 submatrix through 32 rounds of 32 disjoint rotations between the two
+//      blocks (in the first round of a sweep also once through the pairs inside each block) and publishes their product
+//      Q; meanwhile the other CTAs bring the eigenvectors up to date with the Q of the round before;
+//   B  the grid applies M <- Q^T M Q, 64 x 32 pieces, from one buffer to the other.
+// Two grid barriers per 32 rounds of rotations.  (Applying every round of l/2 rotations to the whole matrix takes a
+// barrier per round: 575 per sweep of a 576 x 576 matrix, 4.9 us each, 8.5 ms for three sweeps; taking the 64 x 64
+// problems to convergence before they are applied was slower still.  This form takes less than 1 ms for the same three
+// sweeps; the factorisation of a 131072 x 4096 cache went from 26.2 to 17.2 ms.)  A check per sweep ends the sweeps once the off-diagonal weight is below kJacobiTol.  On return the eigenvalues are on the diagonal of M
+// (buffer 0), the eigenvectors the rows of Pt.
+constexpr int kJacobiMaxPairs = 1024;              // l <= 2048
+constexpr int kJacobiSweeps = 16;
 // The sweeps end when the off-diagonal weight (sum of squares) is below this fraction of the total.  The
 // eigenvectors are stored as bf16 (relative rounding 2^-9); an off-diagonal residue of 1e-4 in relative norm is
-// twenty times below that, and the convergence is quadratic (measured per sweep on a 576 x 576 Rayleigh-Ritz matrix:
-// 9e-4, 2e-5, 1e-6, 7e-9, 9e-12, 2e-14), so the value reached is well under the bound.
+// twenty times below that, and the convergence is quadratic.
 constexpr float kJacobiTol = 1e-8f;
-
-// The sweeps are one cooperative kernel.  All CTAs are resident at once, so a round needs no kernel boundary (as
-// three launches per round the ~7000 rounds of a 576 x 576 matrix were launch bound: 63 ms against 13 ms): every round reads the
-// matrices of the previous round (M, P in buffer `cur`) and writes the other buffer, and one grid-wide barrier
-// separates the rounds.  A round: every CTA works out the l/2 rotations of the round from M (cheap, and saves a
-// second barrier), then the grid updates M block by block -- the 2 x 2 block (rows p_a, q_a; columns p_b, q_b)
-// takes the column rotation of pair b and then the row rotation of pair a --
-// and rotates the column pairs of P.  Reads bypass L1 (other SMs wrote the data), the barrier is an arrival
-// counter that only grows plus a generation word; its wait is bounded like every wait of the library: a CTA that
-// gives up raises XKV_FLAG_TIMEOUT and the abort word, and every other CTA leaves at its next wait.
-constexpr int kJacobiCoopThreads = 512;
+constexpr int kJacobiThreads = 1024;
+constexpr int kJb = 32, kJp = 2 * kJb;             // indices of a block, of a pair
+constexpr int kJacobiSmem = 4 * (kJp * kJp * 3 + 8 * kJp * kJb + kJp * (kJb + 1));   // bytes, see the carve-up
 constexpr unsigned kJacobiSpinLimit = 1u << 18;   // polls of a barrier that normally opens within microseconds
-
-struct JacobiSync {          // words of the workspace's flag block
-  unsigned int* flags;       // status word
-  unsigned int* count;       // arrivals so far (monotonic)
-  unsigned int* gen;         // barriers completed
-  unsigned int* abort;       // a CTA gave up
-  unsigned int spin_limit;   // polls of one barrier wait
-  unsigned int skip_first;   // fault injection (tests of the give-up path): CTA 0 passes the first barrier without arriving
-};
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned int* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void st_release_u32(unsigned int* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ void red_release_u32(unsigned int* p, unsigned v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// A grid-wide barrier of cooperative kernels: an arrival counter that only grows, polled by everybody (an arrival and
+// one poll are the only trips to L2).  The wait is bounded like every wait of the library: a CTA that gives up raises
+// XKV_FLAG_TIMEOUT and the abort word, and every other CTA leaves at its next wait.  Data that crosses it is read past
+// L1 (other SMs wrote it).
+struct GridSync {            // words of the workspace's flag block
+  unsigned int* flags;       // status word
+  unsigned int* count;       // arrivals so far (monotonic)
+  unsigned int* abort;       // a CTA gave up
+  unsigned int spin_limit;   // polls of one barrier wait
+  unsigned int no_arrival;   // fault injection (tests of the give-up path): CTA 0 arrives at no barrier, and passes the first
+};
 // Returns false when the barrier was abandoned (by this CTA or another one).  `my_gen` counts this CTA's barriers.
-__device__ __forceinline__ bool jacobi_grid_barrier(const JacobiSync& sy, unsigned& my_gen, int* ok_s) {
+__device__ __forceinline__ bool grid_barrier(const GridSync& sy, unsigned& my_gen, int* ok_s) {
   __syncthreads();
+  ++my_gen;
   if (threadIdx.x == 0) {
-    ++my_gen;
-    __threadfence();
+    const bool silent = sy.no_arrival != 0u && blockIdx.x == 0;
     bool ok = true;
-    if (sy.skip_first && blockIdx.x == 0 && my_gen == 1u) {
-      // injected fault: the others never see this arrival, run into their limit and raise the abort word
-    } else if (atomicAdd(sy.count, 1u) == gridDim.x * my_gen - 1u) {
-      st_release_u32(sy.gen, my_gen);                      // last to arrive: open the barrier
-    } else {
-      unsigned i = 0;
-      while (ld_acquire_u32(sy.gen) < my_gen) {
-        if (++i >= sy.spin_limit || ld_acquire_u32(sy.abort) != 0u) { ok = false; break; }
+    __threadfence();
+    if (!silent) red_release_u32(sy.count, 1u);
+    if (!silent || my_gen > 1u) {
+      const unsigned want = gridDim.x * my_gen;
+      for (unsigned i = 0; ld_acquire_u32(sy.count) < want;) {
+        if (++i >= sy.spin_limit || ((i & 15u) == 0u && ld_acquire_u32(sy.abort) != 0u)) { ok = false; break; }
       }
     }
     if (!ok) { atomicOr(sy.flags, XKV_FLAG_TIMEOUT); atomicExch(sy.abort, 1u); }
@@ -617,21 +615,211 @@ __device__ __forceinline__ bool jacobi_grid_barrier(const JacobiSync& sy, unsign
   return *ok_s != 0;
 }
 
-__global__ void __launch_bounds__(kJacobiCoopThreads, 1)
-jacobi_coop_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __restrict__ P0, float* __restrict__ P1, int l,
-                   float2* __restrict__ partial, JacobiSync sy) {
-  __shared__ float2 cs_s[kJacobiMaxPairs];
-  __shared__ int2 pq_s[kJacobiMaxPairs];
-  __shared__ int ok_s;
-  __shared__ float2 red_s[kJacobiCoopThreads / 32];
-  __shared__ int done_s;
-  const int tid = threadIdx.x, nb = gridDim.x;
-  const int np = l / 2;                                   // l is even (a multiple of 64)
-  const long long gtid = (long long)blockIdx.x * kJacobiCoopThreads + tid, gstride = (long long)nb * kJacobiCoopThreads;
+// Pair k of round t of the round-robin tournament of n (even) players, the smaller first.
+__device__ __forceinline__ int2 tournament_pair(int k, int t, int n) {
+  int p, q;
+  if (k == 0) { p = n - 1; q = t; }
+  else {
+    p = t + k; if (p >= n - 1) p -= n - 1;
+    q = t - k; if (q < 0) q += n - 1;
+  }
+  return p < q ? make_int2(p, q) : make_int2(q, p);
+}
+
+// The rotation (c, s) that annihilates a_pq: columns (p, q) become (c p - s q, s p + c q).
+__device__ __forceinline__ float2 jacobi_rotation(float app, float aqq, float apq) {
+  float g, h;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(g) : "f"(fabsf(app * aqq)));
+  if (!(fabsf(apq) > 1e-30f && fabsf(apq) > 1e-9f * g)) return make_float2(1.0f, 0.0f);
+  const float tau = __fdividef(aqq - app, 2.0f * apq);
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(h) : "f"(fmaf(tau, tau, 1.0f)));
+  const float t = __fdividef(tau >= 0.0f ? 1.0f : -1.0f, fabsf(tau) + h);
+  const float c = rsqrtf(fmaf(t, t, 1.0f));
+  return make_float2(c, t * c);
+}
+
+// out[r][c] = sum_k A[k][r] B[k][c] for A [64][64], B [64][ldb] in shared memory, 64 x 32 outputs, by 1024 threads:
+// eight groups of eight k, 4 x 4 outputs per thread, partial sums through `red` [8][64][32].  The caller reads the sums
+// with piece_sum after the barrier that ends this function.
+__device__ __forceinline__ void piece_product(const float* __restrict__ A, const float* __restrict__ B, int ldb, float* __restrict__ red) {
+  const int tid = threadIdx.x, grp = tid >> 7, e = tid & 127;
+  const int r0 = (e >> 3) * 4, c0 = (e & 7) * 4;
+  float acc[4][4] = {};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int k = grp * 8 + i;
+    const float4 av = *reinterpret_cast<const float4*>(A + k * kJp + r0), bv = *reinterpret_cast<const float4*>(B + k * ldb + c0);
+    const float a[4] = {av.x, av.y, av.z, av.w}, b[4] = {bv.x, bv.y, bv.z, bv.w};
+#pragma unroll
+    for (int y = 0; y < 4; ++y)
+#pragma unroll
+      for (int x = 0; x < 4; ++x) acc[y][x] = fmaf(a[y], b[x], acc[y][x]);
+  }
+#pragma unroll
+  for (int y = 0; y < 4; ++y)
+    *reinterpret_cast<float4*>(red + grp * (kJp * kJb) + (r0 + y) * kJb + c0) = make_float4(acc[y][0], acc[y][1], acc[y][2], acc[y][3]);
+  __syncthreads();
+}
+__device__ __forceinline__ float piece_sum(const float* __restrict__ red, int o) {
+  float v = 0.0f;
+#pragma unroll
+  for (int g = 0; g < 8; ++g) v += red[g * (kJp * kJb) + o];
+  return v;
+}
+
+__global__ void __launch_bounds__(kJacobiThreads, 1)
+jacobi_block_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __restrict__ Pt, float* __restrict__ Qg, int l,
+                    float2* __restrict__ partial, GridSync sy) {
+  extern __shared__ __align__(16) float js[];
+  __shared__ int ok_s, done_s;
+  __shared__ float2 red_s[kJacobiThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = gridDim.x, bid = blockIdx.x;
+  const int nblk = l / kJb, npair = l / kJp;                 // l is a multiple of 64
+  const long long gtid = (long long)bid * kJacobiThreads + tid, gstride = (long long)nb * kJacobiThreads;
   unsigned my_gen = 0;
-  for (long long e = gtid; e < (long long)l * l; e += gstride) P0[e] = (e / l == e % l) ? 1.0f : 0.0f;
-  int cur = 0;
-  bool alive = jacobi_grid_barrier(sy, my_gen, &ok_s);
+  for (long long e = gtid; e < (long long)l * l; e += gstride) Pt[e] = (e / l == e % l) ? 1.0f : 0.0f;
+  float* const S0 = js;                                      // [64][64] each; phase A: the submatrix and its other buffer
+  float* const S1 = S0 + kJp * kJp;
+  float* const S2 = S1 + kJp * kJp;                          // phase A: the product of the rotations, Q
+  float* const R = S2 + kJp * kJp;                           // [8][64][32] partial products; phase A: rotations of all rounds
+  float* const T = R + 8 * kJp * kJb;                        // [64][33]
+  float2* const cs_s = reinterpret_cast<float2*>(R);         // [63][32]
+  // position i of pair pq (0..63) in the whole matrix
+  auto at = [&](int2 pq, int i) { return (i < kJb ? pq.x : pq.y) * kJb + (i & (kJb - 1)); };
+
+  // ---- A: rotations of one pair
+  auto solve_pair = [&](const float* M, int2 pq, bool inside, float* Qout) {
+    for (int e = tid; e < kJp * kJp; e += kJacobiThreads) {
+      S0[e] = __ldcg(M + (size_t)at(pq, e >> 6) * l + at(pq, e & 63));
+      S2[e] = (e >> 6) == (e & 63) ? 1.0f : 0.0f;
+    }
+    __syncthreads();
+    float* X = S0;
+    float* Xn = S1;
+    // one round of 32 disjoint rotations: lane b of every warp works out rotation b (index pair (i, j)); warps 0-15
+    // update the 2 x 2 blocks (a, b) of the submatrix for two a each
+    auto round = [&](int i, int j, int slot) {
+      const float2 cs = jacobi_rotation(X[i * kJp + i], X[j * kJp + j], X[i * kJp + j]);
+      if (warp == 0) cs_s[slot * 32 + lane] = cs;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int a = warp * 2 + k;
+        const int ia = __shfl_sync(0xffffffffu, i, a), ja = __shfl_sync(0xffffffffu, j, a);
+        const float ca = __shfl_sync(0xffffffffu, cs.x, a), sa = __shfl_sync(0xffffffffu, cs.y, a);
+        const float x00 = X[ia * kJp + i], x01 = X[ia * kJp + j], x10 = X[ja * kJp + i], x11 = X[ja * kJp + j];
+        const float u00 = cs.x * x00 - cs.y * x01, u01 = cs.y * x00 + cs.x * x01;
+        const float u10 = cs.x * x10 - cs.y * x11, u11 = cs.y * x10 + cs.x * x11;
+        Xn[ia * kJp + i] = ca * u00 - sa * u10; Xn[ia * kJp + j] = ca * u01 - sa * u11;
+        Xn[ja * kJp + i] = sa * u00 + ca * u10; Xn[ja * kJp + j] = sa * u01 + ca * u11;
+      }
+    };
+    if (inside) {
+      // the pairs inside the two blocks: 31 rounds, lanes 0-15 in the first block, lanes 16-31 in the second
+      for (int t = 0; t < kJb - 1; ++t) {
+        const int2 ij = tournament_pair(lane & 15, t, kJb);
+        const int off = (lane >> 4) * kJb;
+        if (warp < 16) round(ij.x + off, ij.y + off, t);
+        __syncthreads();
+        float* x = X; X = Xn; Xn = x;
+        if (warp >= 16) {                                    // (nobody writes this slot of cs_s again before the next barrier)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            float* row = S2 + ((warp - 16) * 4 + k) * kJp + off;
+            const float2 cs = cs_s[t * 32 + lane];
+            const float u = row[ij.x], v = row[ij.y];
+            row[ij.x] = cs.x * u - cs.y * v;
+            row[ij.y] = cs.y * u + cs.x * v;
+          }
+        }
+      }
+    }
+    __syncthreads();
+    // the pairs (i, 32 + (i + t) mod 32): warps 16-31 follow one round behind with Q in registers, lane = column i and,
+    // shifted by one lane per round, column 32 + (i + t) mod 32
+    float qu[4], qv[4];
+    if (warp >= 16) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float* row = S2 + ((warp - 16) * 4 + k) * kJp;
+        qu[k] = row[lane];
+        qv[k] = row[kJb + lane];
+      }
+    }
+    for (int t = 0; t <= kJb; ++t) {
+      if (warp < 16) {
+        if (t < kJb) round(lane, kJb + ((lane + t) & (kJb - 1)), t & 1);
+      } else if (t > 0) {
+        const float2 cs = cs_s[((t - 1) & 1) * 32 + lane];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float u = qu[k], v = qv[k];
+          qu[k] = cs.x * u - cs.y * v;
+          qv[k] = __shfl_sync(0xffffffffu, cs.y * u + cs.x * v, (lane + 1) & 31);
+        }
+      }
+      __syncthreads();
+      float* x = X; X = Xn; Xn = x;
+    }
+    if (warp >= 16) {                                        // after 32 shifts the columns are back where they began
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        float* row = Qout + ((warp - 16) * 4 + k) * kJp;
+        row[lane] = qu[k];
+        row[kJb + lane] = qv[k];
+      }
+    }
+  };
+  // ---- eigenvectors: rows of pair pq, columns c0 .. c0 + 63 of Pt  <-  Q^T times them
+  auto rotate_vectors = [&](int2 pq, int c0, const float* Q) {
+    __syncthreads();
+    for (int e = tid; e < kJp * kJp; e += kJacobiThreads) {
+      S0[e] = __ldcg(Pt + (size_t)at(pq, e >> 6) * l + c0 + (e & 63));      // [k][column of Pt]
+      S1[e] = __ldcg(Q + e);                                               // [k][new row]
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      piece_product(S0, S1 + h * kJb, kJp, R);               // [column][new row of block h]
+      for (int o = tid; o < kJp * kJb; o += kJacobiThreads) T[(o >> 5) * (kJb + 1) + (o & 31)] = piece_sum(R, o);
+      __syncthreads();
+      for (int o = tid; o < kJp * kJb; o += kJacobiThreads)
+        Pt[(size_t)at(pq, h * kJb + (o >> 6)) * l + c0 + (o & 63)] = T[(o & 63) * (kJb + 1) + (o >> 6)];
+      __syncthreads();
+    }
+  };
+  // ---- B: one 64 x 32 piece of Q_a^T M Q_b (block h of pair b), and its mirror image
+  auto rotate_matrix = [&](const float* M, float* Mn, int a, int b, int h, int t, const float* Q) {
+    const int2 pa = tournament_pair(a, t, nblk), pb = tournament_pair(b, t, nblk);
+    __syncthreads();
+    for (int e = tid; e < kJp * kJp; e += kJacobiThreads) {
+      S0[e] = __ldcg(M + (size_t)at(pb, e >> 6) * l + at(pa, e & 63));      // M is symmetric: [k in b][row in a]
+      S1[e] = __ldcg(Q + (size_t)b * kJp * kJp + e);                       // [k in b][column]
+      S2[e] = __ldcg(Q + (size_t)a * kJp * kJp + e);                       // [k in a][row]
+    }
+    __syncthreads();
+    piece_product(S0, S1 + h * kJb, kJp, R);
+    float v[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) v[i] = piece_sum(R, tid + i * kJacobiThreads);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 2; ++i) S0[tid + i * kJacobiThreads] = v[i];        // [k in a][column]
+    __syncthreads();
+    piece_product(S2, S0, kJb, R);
+    for (int o = tid; o < kJp * kJb; o += kJacobiThreads) {
+      const float y = piece_sum(R, o);
+      Mn[(size_t)at(pa, o >> 5) * l + at(pb, h * kJb + (o & 31))] = y;
+      T[(o >> 5) * (kJb + 1) + (o & 31)] = y;
+    }
+    if (a != b) {
+      __syncthreads();
+      for (int o = tid; o < kJp * kJb; o += kJacobiThreads)
+        Mn[(size_t)at(pb, h * kJb + (o >> 6)) * l + at(pa, o & 63)] = T[(o & 63) * (kJb + 1) + (o >> 6)];
+    }
+  };
+
+  int cur = 0, qb = 0;
+  bool alive = grid_barrier(sy, my_gen, &ok_s);
   int sweeps_done = 0;
   for (int sweep = 0; alive && sweep < kJacobiSweeps; ++sweep) {
     // ---- off-diagonal weight of M: per-CTA partial sums, then every CTA adds them up in the same order
@@ -643,140 +831,69 @@ jacobi_coop_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __rest
         all += v * v;
         if (e / l != e % l) off += v * v;
       }
+      auto total = [&]() {                                   // of (off, all) over the CTA, in a fixed order; in thread 0
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) { off += __shfl_xor_sync(0xffffffffu, off, o); all += __shfl_xor_sync(0xffffffffu, all, o); }
-      if ((tid & 31) == 0) red_s[tid >> 5] = make_float2(off, all);
-      __syncthreads();
-      if (tid == 0) {
-        float o2 = 0.0f, a2 = 0.0f;
-        for (int w = 0; w < kJacobiCoopThreads / 32; ++w) { o2 += red_s[w].x; a2 += red_s[w].y; }
-        partial[(sweep & 1) * nb + blockIdx.x] = make_float2(o2, a2);
-      }
-      alive = jacobi_grid_barrier(sy, my_gen, &ok_s);
+        for (int o = 16; o > 0; o >>= 1) { off += __shfl_xor_sync(0xffffffffu, off, o); all += __shfl_xor_sync(0xffffffffu, all, o); }
+        if (lane == 0) red_s[warp] = make_float2(off, all);
+        __syncthreads();
+        if (warp == 0) {
+          off = red_s[lane].x; all = red_s[lane].y;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) { off += __shfl_xor_sync(0xffffffffu, off, o); all += __shfl_xor_sync(0xffffffffu, all, o); }
+        }
+        __syncthreads();
+      };
+      total();
+      if (tid == 0) partial[(sweep & 1) * nb + bid] = make_float2(off, all);
+      alive = grid_barrier(sy, my_gen, &ok_s);
       if (!alive) break;
-      if (tid == 0) {
-        float o2 = 0.0f, a2 = 0.0f;
-        for (int b = 0; b < nb; ++b) { const float2 v = __ldcg(partial + (sweep & 1) * nb + b); o2 += v.x; a2 += v.y; }
-        done_s = (o2 <= kJacobiTol * a2) ? 1 : 0;
-      }
+      off = all = 0.0f;
+      for (int b = tid; b < nb; b += kJacobiThreads) { const float2 v = __ldcg(partial + (sweep & 1) * nb + b); off += v.x; all += v.y; }
+      total();
+      if (tid == 0) done_s = (off <= kJacobiTol * all) ? 1 : 0;
       __syncthreads();
-      if (done_s) break;                                  // the same decision in every CTA
+      if (done_s) break;                                     // the same decision in every CTA
     }
     ++sweeps_done;
-    for (int t = 0; alive && t < l - 1; ++t) {
+    const int items = npair * npair;                         // (pair, 64 columns of Pt)
+    for (int t = 0; alive && t < nblk - 1; ++t) {
       const float* M = cur ? M1 : M0;
-      const float* P = cur ? P1 : P0;
       float* Mn = cur ? M0 : M1;
-      float* Pn = cur ? P0 : P1;
-      // pair k of round t (round-robin order), smaller index first
-      auto pair_of = [&](int k) -> int2 {
-        int p, q;
-        if (k == 0) { p = l - 1; q = t; }
-        else { p = (t + k) % (l - 1); q = (t - k + l - 1) % (l - 1); }
-        return p < q ? make_int2(p, q) : make_int2(q, p);
-      };
-      // M: 2 x 2 blocks (pair a of rows, pair b of columns); P: column pairs, every row; kBatch items of each per
-      // pass.  The loads of the first pass are issued before the rotations are worked out -- their addresses
-      // depend on the round only -- so that a round of a 576 x 576 matrix is one trip to L2, not three.
-      constexpr int kBatch = 4;
-      const long long nM = (long long)np * np, nP = (long long)l * np;
-      float x0[kBatch], y0[kBatch], x1[kBatch], y1[kBatch], pu[kBatch], pv[kBatch];
-      int ka[kBatch], kb[kBatch], pi[kBatch], pk[kBatch];
-      auto load_m = [&](long long base) {
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const long long it = base + u * gstride;
-          ka[u] = -1;
-          if (it < nM) {
-            ka[u] = (int)(it / np); kb[u] = (int)(it - (long long)ka[u] * np);
-            const int2 ra = pair_of(ka[u]), cb = pair_of(kb[u]);
-            const float* r0 = M + (size_t)ra.x * l;
-            const float* r1 = M + (size_t)ra.y * l;
-            x0[u] = __ldcg(r0 + cb.x); y0[u] = __ldcg(r0 + cb.y); x1[u] = __ldcg(r1 + cb.x); y1[u] = __ldcg(r1 + cb.y);
-          }
-        }
-      };
-      auto load_p = [&](long long base) {
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const long long it = base + u * gstride;
-          pi[u] = -1;
-          if (it < nP) {
-            pi[u] = (int)(it / np); pk[u] = (int)(it - (long long)pi[u] * np);
-            const int2 ix = pair_of(pk[u]);
-            pu[u] = __ldcg(P + (size_t)pi[u] * l + ix.x); pv[u] = __ldcg(P + (size_t)pi[u] * l + ix.y);
-          }
-        }
-      };
-      auto finish_m = [&]() {
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          if (ka[u] < 0) continue;
-          const int2 ra = pq_s[ka[u]], cb = pq_s[kb[u]];
-          const float2 ja = cs_s[ka[u]], jb = cs_s[kb[u]];
-          float a0 = x0[u], b0 = y0[u], a1 = x1[u], b1 = y1[u];
-          if (jb.y != 0.0f) {                             // columns p_b, q_b
-            const float u0 = jb.x * a0 - jb.y * b0, v0 = jb.y * a0 + jb.x * b0;
-            const float u1 = jb.x * a1 - jb.y * b1, v1 = jb.y * a1 + jb.x * b1;
-            a0 = u0; b0 = v0; a1 = u1; b1 = v1;
-          }
-          if (ja.y != 0.0f) {                             // rows p_a, q_a
-            const float u0 = ja.x * a0 - ja.y * a1, u1 = ja.y * a0 + ja.x * a1;
-            const float v0 = ja.x * b0 - ja.y * b1, v1 = ja.y * b0 + ja.x * b1;
-            a0 = u0; a1 = u1; b0 = v0; b1 = v1;
-          }
-          float* w0 = Mn + (size_t)ra.x * l;
-          float* w1 = Mn + (size_t)ra.y * l;
-          w0[cb.x] = a0; w0[cb.y] = b0; w1[cb.x] = a1; w1[cb.y] = b1;
-        }
-      };
-      auto finish_p = [&]() {
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          if (pi[u] < 0) continue;
-          const int2 ix = pq_s[pk[u]];
-          const float2 j = cs_s[pk[u]];
-          float nu = pu[u], nv = pv[u];
-          if (j.y != 0.0f) { nu = j.x * pu[u] - j.y * pv[u]; nv = j.y * pu[u] + j.x * pv[u]; }
-          Pn[(size_t)pi[u] * l + ix.x] = nu;
-          Pn[(size_t)pi[u] * l + ix.y] = nv;
-        }
-      };
-      load_m(gtid);
-      load_p(gtid);
-      for (int k = tid; k < np; k += kJacobiCoopThreads) {
-        const int2 ix = pair_of(k);
-        const int p = ix.x, q = ix.y;
-        float c = 1.0f, sn = 0.0f;
-        const float app = __ldcg(M + (size_t)p * l + p), aqq = __ldcg(M + (size_t)q * l + q), apq = __ldcg(M + (size_t)p * l + q);
-        if (fabsf(apq) > 1e-30f && fabsf(apq) > 1e-9f * sqrtf(fabsf(app * aqq))) {
-          const float tau = (aqq - app) / (2.0f * apq);
-          const float tt = (tau >= 0.0f ? 1.0f : -1.0f) / (fabsf(tau) + sqrtf(1.0f + tau * tau));
-          c = rsqrtf(1.0f + tt * tt);
-          sn = tt * c;
-        }
-        cs_s[k] = make_float2(c, sn);
-        pq_s[k] = ix;
+      float* Q = Qg + (size_t)qb * npair * kJp * kJp;
+      const float* Qprev = Qg + (size_t)(qb ^ 1) * npair * kJp * kJp;
+      if (bid < npair) {
+        for (int k = bid; k < npair; k += nb) solve_pair(M, tournament_pair(k, t, nblk), t == 0, Q + (size_t)k * kJp * kJp);
+      } else if (t > 0) {
+        for (int it = bid - npair; it < items; it += nb - npair)
+          rotate_vectors(tournament_pair(it / npair, t - 1, nblk), (it % npair) * kJp, Qprev + (size_t)(it / npair) * kJp * kJp);
       }
-      __syncthreads();
-      finish_m();
-      finish_p();
-      for (long long base = gtid + kBatch * gstride; base < nM; base += kBatch * gstride) { load_m(base); finish_m(); }
-      for (long long base = gtid + kBatch * gstride; base < nP; base += kBatch * gstride) { load_p(base); finish_p(); }
-      alive = jacobi_grid_barrier(sy, my_gen, &ok_s);
+      alive = grid_barrier(sy, my_gen, &ok_s);
+      if (!alive) break;
+      for (int it = bid; it < npair * (npair + 1); it += nb) {   // pieces (a <= b, h)
+        const int h = it & 1;
+        int a = 0, rest = it >> 1;
+        while (rest >= npair - a) { rest -= npair - a; ++a; }
+        rotate_matrix(M, Mn, a, a + rest, h, t, Q);
+      }
+      alive = grid_barrier(sy, my_gen, &ok_s);
       cur ^= 1;
+      qb ^= 1;
     }
+    if (!alive) break;
+    for (int it = bid; it < items; it += nb)
+      rotate_vectors(tournament_pair(it / npair, nblk - 2, nblk), (it % npair) * kJp,
+                     Qg + ((size_t)(qb ^ 1) * npair + it / npair) * kJp * kJp);
   }
-  if (blockIdx.x == 0 && tid == 0) sy.abort[1] = (unsigned)sweeps_done;   // diagnostic: sweeps that ran
-  if (alive && cur == 1) {                                // the callers read buffer 0
-    for (long long e = gtid; e < (long long)l * l; e += gstride) { M0[e] = __ldcg(M1 + e); P0[e] = __ldcg(P1 + e); }
+  if (bid == 0 && tid == 0) sy.abort[1] = (unsigned)sweeps_done;   // diagnostic: sweeps that ran
+  if (alive && cur == 1) {                                   // the callers read buffer 0
+    for (long long e = gtid; e < (long long)l * l; e += gstride) M0[e] = __ldcg(M1 + e);
   }
 }
 
 // The r largest eigenvalues (ties to the lower index) and their eigenvectors as the columns of Psel (l x r);
 // sigma = sqrt(lambda).
 __global__ void __launch_bounds__(1024)
-eig_select_kernel(const float* __restrict__ M, const float* __restrict__ P, int l, int r, float* __restrict__ Psel,
+eig_select_kernel(const float* __restrict__ M, const float* __restrict__ Pt, int l, int r, float* __restrict__ Psel,
                   float* __restrict__ sigma) {
   extern __shared__ int rank_s[];                      // [l]
   const int tid = threadIdx.x;
@@ -794,7 +911,7 @@ eig_select_kernel(const float* __restrict__ M, const float* __restrict__ P, int 
   for (int e = tid; e < l * l; e += 1024) {
     const int row = e / l, i = e % l;
     const int rk = rank_s[i];
-    if (rk < r) Psel[(size_t)row * r + rk] = P[e];
+    if (rk < r) Psel[(size_t)row * r + rk] = Pt[(size_t)i * l + row];
   }
 }
 
@@ -829,7 +946,7 @@ __global__ void symmetrize_kernel(float* __restrict__ M, int l) {
 
 struct ClfPlan {
   int T, Tp, N, r, l, q;
-  size_t off_flags, off_zb, off_yt, off_u, off_z, off_g, off_m, off_p, off_ps, off_v, off_vb, off_cs, off_m2, off_p2, off_xinv, total;
+  size_t off_flags, off_zb, off_yt, off_u, off_z, off_g, off_m, off_p, off_ps, off_v, off_vb, off_cs, off_m2, off_q, off_xinv, total;
 };
 
 size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -854,7 +971,7 @@ bool make_plan(const xkv_clf_config* c, ClfPlan* p) {
   p->off_vb = o; o = align_up(o + (size_t)p->N * p->r * 2);
   p->off_cs = o; o = align_up(o + (size_t)2 * 1024 * 8);            // per-CTA partial sums of the Jacobi convergence check
   p->off_m2 = o; o = align_up(o + (size_t)p->l * p->l * 4);      // second buffers of the one-kernel Jacobi sweeps
-  p->off_p2 = o; o = align_up(o + (size_t)p->l * p->l * 4);
+  p->off_q = o; o = align_up(o + (size_t)2 * p->l * kJp * 4);    // rotation products of the block pairs, two rounds
   p->off_xinv = o; o = align_up(o + (size_t)p->l * kTriBlock * 8);   // inverses of the diagonal blocks of a Cholesky factor
   p->total = o;
   return true;
@@ -1013,19 +1130,20 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
     symmetrize_kernel<<<(l * l + 255) / 256, 256, 0, s>>>(Mm, l);
     {
       int per_sm = 0, sms = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_coop_kernel, kJacobiCoopThreads, 0);
+      e = ensure_dyn_smem<jacobi_block_kernel>(kJacobiSmem, device);
+      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_block_kernel, kJacobiThreads, kJacobiSmem);
       if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
       if (e == cudaSuccess && per_sm < 1) e = cudaErrorLaunchOutOfResources;
       if (e == cudaSuccess) {
         float* M2 = (float*)(w + p.off_m2);
-        float* P2 = (float*)(w + p.off_p2);
+        float* Qm = (float*)(w + p.off_q);
         float2* partial = (float2*)(w + p.off_cs);
         const bool inject = (g_clf_inject.load(std::memory_order_relaxed) & XKV_INJECT_CLF_BARRIER) != 0u;
-        JacobiSync sy{flags, flags + 8, flags + 9, flags + 10,            // zeroed with the flag block above
-                      inject ? 1024u : kJacobiSpinLimit, inject ? 1u : 0u};
+        GridSync sy{flags, flags + 8, flags + 10,                         // zeroed with the flag block above
+                    inject ? 1024u : kJacobiSpinLimit, inject ? 1u : 0u};
         int l_arg = l;
-        void* args[] = {&Mm, &M2, &Pm, &P2, &l_arg, &partial, &sy};
-        e = cudaLaunchCooperativeKernel((const void*)jacobi_coop_kernel, dim3(sms), dim3(kJacobiCoopThreads), args, 0, s);
+        void* args[] = {&Mm, &M2, &Pm, &Qm, &l_arg, &partial, &sy};
+        e = cudaLaunchCooperativeKernel((const void*)jacobi_block_kernel, dim3(sms), dim3(kJacobiThreads), args, kJacobiSmem, s);
         count_launch(kFamClf, 1);
       }
     }
