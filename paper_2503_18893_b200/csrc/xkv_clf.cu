@@ -5,14 +5,14 @@
 //   Z (N x l) <- the random test matrix
 //   repeat q + 1 times:   Y^T = Z^T X^T   (l x T, bf16)          tensor core
 //                         U   = X^T Y     (N x l, fp32)          tensor core
-//                         Z   = U R^-1,  R^T R = U^T U + shift I (shifted Cholesky QR in fp64: two passes inside the
-//                               iteration, five for the last iterate, which has to be orthonormal)
-//   Rayleigh-Ritz:        W^T = Z^T X^T,  U' = X^T W,  M = Z^T U' (= Z^T X^T X Z, l x l),  M = P Lambda P^T (Jacobi)
+//                         Z   = U R^-1,  R^T R = U^T U + shift I (shifted Cholesky QR in fp64: one pass inside the
+//                               iteration, three for the last iterate, which has to be orthonormal)
+//   Rayleigh-Ritz:        W^T = Z^T X^T,  M = W^T W (= Z^T X^T X Z, l x l),  M = P Lambda P^T (Jacobi)
 //   V = Z P_r (N x r);    B_l = rows of V^T (bf16);   A = X V_bf16 (T x r, tensor core);   sigma = sqrt(Lambda).
 // A = U Sigma and B = V^T of the truncated SVD of X, up to the accuracy of the subspace (checked against the exact
 // optimum sum_{i>r} sigma_i^2, never factor by factor: signs and degenerate subspaces are not unique).
 //
-// One tensor-core kernel serves the three tall products.  It computes C (M x N) = A B^T for A given as [K][M]
+// One tensor-core kernel serves the tall products.  It computes C (M x N) = A B^T for A given as [K][M]
 // row-major (an MN-major operand: the M index is contiguous) and B as [N][K] row-major (K-major), the two operand
 // forms the fused decode kernel already uses, so no matrix is ever transposed in memory:
 //   Y^T = Z-as-A (K = N_x)  x  X-as-B;     U = X-as-A (K = T)  x  Y^T-as-B;     A^T = V-as-A  x  X-as-B (stored transposed).
@@ -45,12 +45,13 @@ __device__ __forceinline__ bool gemm_wait(uint32_t bar, uint32_t parity) {
   return false;
 }
 
-// C[m][n] = sum_k A[k][m] B[n][k].  grid = (ceil(N/BN), ceil(M/128)).  TRANS: store C^T (out[n][m]).
+// C[m][n] = sum_k A[k][m] B[n][k].  grid = (ceil(N/BN), ceil(M/128), K ranges).  TRANS: store C^T (out[n][m]).
+// AROW: A is given as [m][k] instead (K-major, like B).  K range z covers k_per columns and writes Cf + z * M * ldc.
 // Out-of-range rows and columns of the operands are zero-filled by the copy engine; stores are guarded.
-template <bool TRANS, int BN>
+template <bool TRANS, bool AROW, int BN>
 __global__ void __launch_bounds__(kGemmThreads)
 clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M, int N, int K,
-                float* __restrict__ Cf, __nv_bfloat16* __restrict__ Cb, long long ldc, unsigned int* __restrict__ flags) {
+                int k_per, float* __restrict__ Cf, __nv_bfloat16* __restrict__ Cb, long long ldc, unsigned int* __restrict__ flags) {
   extern __shared__ uint8_t gemm_smem[];
   constexpr int kGemmStages = gemm_stages<BN>(), kGemmStageBytes = gemm_stage_bytes<BN>();
   constexpr uint32_t kCols = BN <= 128 ? 128u : 256u;      // tensor-memory columns (a power of two)
@@ -60,7 +61,8 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   const uint32_t base = (smem_u32(gemm_smem) + 1023u) & ~1023u;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n0 = blockIdx.x * BN, m0 = blockIdx.y * 128;
-  const int KB = (K + 63) / 64;
+  const int k_first = blockIdx.z * k_per, KB = (min(K - k_first, k_per) + 63) / 64;
+  if (Cf) Cf += (size_t)blockIdx.z * M * ldc;
   const uint32_t bar0 = smem_u32(bars);
   auto FULL = [&](int s) { return bar0 + 8u * (uint32_t)s; };
   auto EMPTY = [&](int s) { return bar0 + 8u * (uint32_t)(kGemmStages + s); };
@@ -87,26 +89,34 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         if (kb >= kGemmStages && !gemm_wait(EMPTY(s), (uint32_t)((kb / kGemmStages - 1) & 1))) { ok = false; break; }
         const uint32_t st = base + (uint32_t)s * kGemmStageBytes;
         mbar_expect_tx(FULL(s), kGemmStageBytes);
-        tma_load_2d(st, &map_a, m0, kb * 64, FULL(s));                 // A: columns m0..m0+63, rows (k) kb*64..+63
-        tma_load_2d(st + 8192, &map_a, m0 + 64, kb * 64, FULL(s));     //    columns m0+64..m0+127
-        tma_load_2d(st + 16384, &map_b, kb * 64, n0, FULL(s));         // B: columns (k) kb*64..+63, rows n0..n0+BN-1
+        const int k = k_first + kb * 64;
+        if (AROW) {
+          tma_load_2d(st, &map_a, k, m0, FULL(s));                     // A: columns (k) k..k+63, rows m0..m0+127
+        } else {
+          tma_load_2d(st, &map_a, m0, k, FULL(s));                     // A: columns m0..m0+63, rows (k) k..k+63
+          tma_load_2d(st + 8192, &map_a, m0 + 64, k, FULL(s));         //    columns m0+64..m0+127
+        }
+        tma_load_2d(st + 16384, &map_b, k, n0, FULL(s));               // B: columns (k) k..k+63, rows n0..n0+BN-1
       }
     }
   } else if (warp == 5) {
     if (lane == 0) {
       const uint64_t desc_hi = smem_desc_sw128(0, 0) & 0xFFFFFFFF00000000ull;
-      constexpr uint32_t idesc = idesc_bf16_f32(128, BN) | (1u << 15);    // A is read along its rows (MN-major)
+      constexpr uint32_t idesc = idesc_bf16_f32(128, BN) | (AROW ? 0u : 1u << 15);    // not AROW: A is read along its rows (MN-major)
       for (int kb = 0; kb < KB; ++kb) {
         const int s = kb % kGemmStages;
         if (!gemm_wait(FULL(s), (uint32_t)((kb / kGemmStages) & 1))) { ok = false; break; }
         tc_fence_after();
         const uint32_t st = base + (uint32_t)s * kGemmStageBytes;
         // A: two 64-column slabs 8192 bytes apart, 8-row groups (along k) 1024 bytes apart; 16 k-rows per step
-        const uint32_t a_lo = ((uint32_t)((st & 0x3FFFFu) >> 4)) | ((uint32_t)(8192 >> 4) << 16);
+        // (AROW: one slab of 128 rows, 32 bytes per step, like B)
+        const uint32_t a_lo = AROW ? (uint32_t)(smem_desc_sw128(st, 0) & 0xFFFFFFFFull)
+                                   : ((uint32_t)((st & 0x3FFFFu) >> 4)) | ((uint32_t)(8192 >> 4) << 16);
+        constexpr uint32_t a_step = AROW ? 2u : (2048u >> 4);
         const uint32_t b_lo = (uint32_t)(smem_desc_sw128(st + 16384, 0) & 0xFFFFFFFFull);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          tc_mma_bf16(tmem, desc_hi | (a_lo + (uint32_t)kk * (2048u >> 4)), desc_hi | (b_lo + 2u * (uint32_t)kk), idesc,
+          tc_mma_bf16(tmem, desc_hi | (a_lo + (uint32_t)kk * a_step), desc_hi | (b_lo + 2u * (uint32_t)kk), idesc,
                       (kb | kk) ? 1u : 0u);
         tc_commit(EMPTY(s));
       }
@@ -179,67 +189,30 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
-// The small matrices (l x l, N x l) in fp32 on the ordinary cores.
+// The small matrices (l x l, N x l).
 namespace {
 
-// C (m x n, ldc) = op(A) B with B (k x n, ldb) row-major and op(A) = A^T for A (k x m, lda) if TA, else A (m x k, lda).
-// 64 x 64 tiles, 256 threads, 4 x 4 outputs per thread.
-// TO = double accumulates in double.
-template <bool TA, typename TO>
-__global__ void __launch_bounds__(256)
-sgemm_small_kernel(const float* __restrict__ A, const float* __restrict__ B, TO* __restrict__ C, int m, int n, int k,
-                   int lda, int ldb, int ldc) {
-  __shared__ float As[16][64 + 4], Bs[16][64 + 4];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  TO acc[4][4] = {};
-  for (int k0 = 0; k0 < k; k0 += 16) {
-    for (int i = tid; i < 16 * 64; i += 256) {
-      const int kk = TA ? i / 64 : i % 16, mm = TA ? i % 64 : i / 16;
-      const int gk = k0 + kk, gm = m0 + mm;
-      As[kk][mm] = (gk < k && gm < m) ? (TA ? A[(size_t)gk * lda + gm] : A[(size_t)gm * lda + gk]) : 0.0f;
-      const int bk = i / 64, bn = i % 64;
-      Bs[bk][bn] = (k0 + bk < k && n0 + bn < n) ? B[(size_t)(k0 + bk) * ldb + n0 + bn] : 0.0f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = As[kk][ty * 4 + i]; b[i] = Bs[kk][tx * 4 + i]; }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += (TO)a[i] * (TO)b[j];
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gm = m0 + ty * 4 + i, gn = n0 + tx * 4 + j;
-      if (gm < m && gn < n) C[(size_t)gm * ldc + gn] = acc[i][j];
-    }
-}
-
-// C (m x n, fp64 or rounded to fp32) = A^T B for fp32 A (k x m) and B (k x n) on the fp64 tensor-core path (mma.sync m8n8k4): the Gram
-// matrices of the Cholesky QR, accumulated in fp64 because their condition number is the square of the iterate's.
-// (A scalar fp64 kernel with 4 x 4 outputs per thread spent 0.79 ms on a 576 x 576 x 4096 product, this one 0.33 ms.)  64 x 64 tiles, 8 warps of 16 x 32, chunks of 32 rows
-// widened to fp64 on their way into shared memory; m, n multiples of 64, k a multiple of 32.
-constexpr int kDgemmLd = 68;                         // doubles per staged row: 4 mod 16, so fragment loads are conflict free
+// ---- fp64 pieces of the Cholesky QR, on the fp64 tensor-core path (mma.sync m8n8k4) ----
+constexpr int kDgemmLd = 68;                         // doubles per staged row of 64: 4 mod 16, so fragment loads are conflict free
 __device__ __forceinline__ void dmma_8x8x4(double (&d)[2], double a, double b) {
   asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
                : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
 }
-template <typename TO>
+
+// Gram matrix U^T U of the fp32 iterate U (n x l), accumulated in fp64 because its condition number is the square of
+// the iterate's: part[z][l][l] for the rows [z * rows_per, (z + 1) * rows_per), 64 x 64 tiles of the lower triangle.
+// The rows are split so that the tiles fill the SMs about twice (81 full tiles of a 576 x 576 matrix, one CTA per SM
+// and all 4096 rows each, took 193 us; half the tiles over six row ranges 61 us); the partial sums are added in a fixed
+// order by the factorisation.  8 warps of 16 x 32, chunks of 32 rows widened to fp64 on their way into shared memory.
 __global__ void __launch_bounds__(256)
-dgemm_tn_mma_kernel(const float* __restrict__ A, const float* __restrict__ B, TO* __restrict__ C, int k, int lda,
-                    int ldb, int ldc) {
+gram_kernel(const float* __restrict__ U, double* __restrict__ part, int n, int l, int rows_per) {
   __shared__ double As[32][kDgemmLd], Bs[32][kDgemmLd];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int wm = (warp & 3) * 16, wn = (warp >> 2) * 32;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+  int ti = 0, tj = blockIdx.x;                        // tile (ti, tj), tj <= ti
+  while (tj > ti) { ++ti; tj -= ti; }
+  const int m0 = ti * 64, n0 = tj * 64;
+  const int k_begin = blockIdx.y * rows_per, k_end = min(n, k_begin + rows_per);
   const int lr = tid >> 4, lc = (tid & 15) * 4;       // this thread's piece of a staged chunk: rows lr, lr + 16; 4 columns
   double acc[2][4][2];
 #pragma unroll
@@ -250,12 +223,14 @@ dgemm_tn_mma_kernel(const float* __restrict__ A, const float* __restrict__ B, TO
   auto fetch = [&](int k0) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      pa[h] = *reinterpret_cast<const float4*>(A + (size_t)(k0 + lr + 16 * h) * lda + m0 + lc);
-      pb[h] = *reinterpret_cast<const float4*>(B + (size_t)(k0 + lr + 16 * h) * ldb + n0 + lc);
+      const int k = k0 + lr + 16 * h;
+      const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      pa[h] = k < k_end ? *reinterpret_cast<const float4*>(U + (size_t)k * l + m0 + lc) : z;
+      pb[h] = k < k_end ? *reinterpret_cast<const float4*>(U + (size_t)k * l + n0 + lc) : z;
     }
   };
-  fetch(0);
-  for (int k0 = 0; k0 < k; k0 += 32) {
+  fetch(k_begin);
+  for (int k0 = k_begin; k0 < k_end; k0 += 32) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       double* da = &As[lr + 16 * h][lc];
@@ -264,7 +239,7 @@ dgemm_tn_mma_kernel(const float* __restrict__ A, const float* __restrict__ B, TO
       db[0] = (double)pb[h].x; db[1] = (double)pb[h].y; db[2] = (double)pb[h].z; db[3] = (double)pb[h].w;
     }
     __syncthreads();
-    if (k0 + 32 < k) fetch(k0 + 32);                  // the next chunk travels while this one is multiplied
+    if (k0 + 32 < k_end) fetch(k0 + 32);              // the next chunk travels while this one is multiplied
 #pragma unroll
     for (int kk = 0; kk < 32; kk += 4) {
       double a[2], b[4];
@@ -279,271 +254,342 @@ dgemm_tn_mma_kernel(const float* __restrict__ A, const float* __restrict__ B, TO
     }
     __syncthreads();
   }
+  double* C = part + (size_t)blockIdx.y * l * l;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      *reinterpret_cast<double2*>(C + (size_t)(m0 + wm + 8 * i + (lane >> 2)) * l + n0 + wn + 8 * j + 2 * (lane & 3)) =
+          make_double2(acc[i][j][0], acc[i][j][1]);
+}
+
+// A grid-wide barrier of cooperative kernels: an arrival counter that only grows, polled by everybody (an arrival and
+// one poll are the only trips to L2).  The wait is bounded like every wait of the library: a CTA that gives up raises
+// XKV_FLAG_TIMEOUT and the abort word, and every other CTA leaves at its next wait.  Data that crosses it is read past
+// L1 (other SMs wrote it).
+constexpr unsigned kGridSpinLimit = 1u << 18;   // polls of a barrier that normally opens within microseconds
+struct GridSync {            // words of the workspace's flag block
+  unsigned int* flags;       // status word
+  unsigned int* count;       // arrivals so far (monotonic)
+  unsigned int* abort;       // a CTA gave up
+  unsigned int spin_limit;   // polls of one barrier wait
+  unsigned int no_arrival;   // fault injection (tests of the give-up path): CTA 0 arrives at no barrier, and passes the first
+};
+__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned int* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void red_release_u32(unsigned int* p, unsigned v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// Returns false when the barrier was abandoned (by this CTA or another one).  `arrived` counts the arrivals expected so
+// far: it starts at the counter's value before the kernel, the same in every CTA.
+__device__ __forceinline__ bool grid_barrier(const GridSync& sy, unsigned& arrived, int* ok_s) {
+  __syncthreads();
+  const bool first = arrived == 0u;
+  arrived += gridDim.x;
+  if (threadIdx.x == 0) {
+    const bool silent = sy.no_arrival != 0u && blockIdx.x == 0;
+    bool ok = true;
+    __threadfence();
+    if (!silent) red_release_u32(sy.count, 1u);
+    if (!silent || !first) {
+      for (unsigned i = 0; ld_acquire_u32(sy.count) < arrived;) {
+        if (++i >= sy.spin_limit || ((i & 15u) == 0u && ld_acquire_u32(sy.abort) != 0u)) { ok = false; break; }
+      }
+    }
+    if (!ok) { atomicOr(sy.flags, XKV_FLAG_TIMEOUT); atomicExch(sy.abort, 1u); }
+    __threadfence();
+    *ok_s = ok ? 1 : 0;
+  }
+  __syncthreads();
+  return *ok_s != 0;
+}
+
+// 1/sqrt(d) for d > 0 by Newton's iteration from the fp32 value (two steps: relative error 2^-22 -> 2^-43 -> rounding).
+// The argument is scaled into [1, 4) by an even power of two first.
+__device__ __forceinline__ double newton_rsqrt(double d) {
+  const int hi = __double2hiint(d);
+  const int e = ((hi >> 20) - 1023) & ~1;                      // even exponent
+  const double m = __hiloint2double(hi - (e << 20), __double2loint(d));
+  double y = (double)rsqrtf((float)m);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) y = fma(0.5 * y, fma(-m * y, y, 1.0), y);
+  return __hiloint2double(__double2hiint(y) - ((e >> 1) << 20), __double2loint(y));
+}
+
+// Cholesky factorisation in fp64 of G + shift_rel * max_diag(G) * I and the inverse W = L^-1 of its factor, one
+// cooperative kernel.  Blocks of 32.  A step p of the factorisation: every lower tile (i, k), k > p, forms the two
+// blocks of the panel it needs, L_ip = A_ip inv(L_pp)^T and L_kp, by itself (they cost less than handing them over would)
+// and takes L_ip L_kp^T out; the CTA of tile (p+1, p+1) then factors it at once, so that one grid barrier per step
+// suffices.  (As three launches per panel the factorisation of a 576 x 576 matrix was 52 launches of 7 to 16 us.)
+// W by columns of eight: W_ik = -inv(L_ii) sum_{k <= j < i} L_ij W_jk.  With W at hand the solve is a product.
+// Buffers: part [n_part][l][l] partial Gram matrices (lower tiles of 64), Gm [l][l] the working matrix, Lf [l][l] the
+// factor's blocks below the diagonal blocks, Iv [l/32][32][32] inverses of the diagonal blocks, W [l][l] lower.
+constexpr int kCholNb = 32, kCholThreads = 256, kCholLd = 36;   // 36 doubles per staged row: 4 mod 16, conflict free fragments
+
+// One 8-row, 32-deep fragment product: acc (8 x 8 per tile) += A rows [m8..m8+7] of a staged block times B rows^T.
+__device__ __forceinline__ void dmma_block(double (&acc)[2], const double* A, const double* B, int lane, double sign) {
+#pragma unroll
+  for (int kk = 0; kk < kCholNb; kk += 4)
+    dmma_8x8x4(acc, sign * A[(lane >> 2) * kCholLd + kk + (lane & 3)], B[(lane >> 2) * kCholLd + kk + (lane & 3)]);
+}
+
+__global__ void __launch_bounds__(kCholThreads, 1)
+chol_inverse_kernel(const double* __restrict__ part, int n_part, double* __restrict__ Gm, double* __restrict__ Lf,
+                    double* __restrict__ Iv, double* __restrict__ W, int l, double shift_rel, unsigned arrived, GridSync sy) {
+  extern __shared__ __align__(16) double cs_d[];               // [l][9] columns of W (second half of the kernel)
+  __shared__ double A_s[kCholNb * kCholLd], B_s[kCholNb * kCholLd], V_s[kCholNb * kCholLd], Li_s[kCholNb * kCholLd], Lk_s[kCholNb * kCholLd];
+  __shared__ __align__(16) double col_s[2][kCholNb];
+  __shared__ double piv_s[2];
+  __shared__ double red_s[kCholThreads / 32];
+  __shared__ int ok_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = gridDim.x, bid = blockIdx.x;
+  const int nbk = l / kCholNb;
+  // ---- the Gram matrix: partial sums added in order, every CTA a share of the elements of the lower 64 x 64 tiles
+  for (long long e2 = (long long)bid * kCholThreads + tid; e2 < (long long)l * l / 2; e2 += (long long)nb * kCholThreads) {
+    const int row = (int)(e2 / (l / 2)), c = (int)(e2 % (l / 2)) * 2;
+    if (c / 64 > row / 64) continue;
+    double2 v = make_double2(0.0, 0.0);
+    for (int z = 0; z < n_part; ++z) {
+      const double2 u = *reinterpret_cast<const double2*>(part + ((size_t)z * l + row) * l + c);
+      v.x += u.x; v.y += u.y;
+    }
+    *reinterpret_cast<double2*>(Gm + (size_t)row * l + c) = v;
+  }
+  if (!grid_barrier(sy, arrived, &ok_s)) return;
+  double shift;
+  {
+    double mx = 0.0;
+    for (int i = tid; i < l; i += kCholThreads) mx = fmax(mx, __ldcg(Gm + (size_t)i * l + i));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) red_s[warp] = mx;
+    __syncthreads();
+    mx = red_s[lane & (kCholThreads / 32 - 1)];
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    shift = shift_rel * mx;
+  }
+  auto stage = [&](double* dst, const double* src, int ld) {   // a 32 x 32 block
+    for (int e = tid; e < kCholNb * kCholNb / 2; e += kCholThreads) {
+      const int r = e >> 4, c = (e & 15) * 2;
+      const double2 v = __ldcg(reinterpret_cast<const double2*>(src + (size_t)r * ld + c));
+      dst[r * kCholLd + c] = v.x; dst[r * kCholLd + c + 1] = v.y;
+    }
+  };
+  const int t_m = warp & 3, t_n = (warp >> 2) * 2;             // this warp's 8 x 8 tiles of a 32 x 32 block: (t_m, t_n), (t_m, t_n + 1)
+  auto put = [&](double* dst, int ld, const double (&acc)[2][2]) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      double* d = dst + (size_t)(t_m * 8 + (lane >> 2)) * ld + (t_n + j) * 8 + 2 * (lane & 3);
+      d[0] = acc[j][0]; d[1] = acc[j][1];
+    }
+  };
+  // ---- factor the diagonal block in A_s and invert the factor.  Warp 0: lane i holds row i; warp 1: lane k holds column k
+  // of the inverse and follows from column to column.  A pivot that is not positive (breakdown) is replaced by a tiny
+  // one and reported.
+  auto factor = [&](int p) {
+    __syncthreads();
+    if (warp < 2) {
+      double a[kCholNb];
+#pragma unroll
+      for (int j = 0; j < kCholNb; ++j) a[j] = warp == 0 ? A_s[lane * kCholLd + j] : (j == lane ? 1.0 : 0.0);
+#pragma unroll
+      for (int c = 0; c < kCholNb; ++c) {
+        if (warp == 0) {
+          double d = __shfl_sync(0xffffffffu, a[c], c);
+          if (!(d > 0.0)) { if (lane == 0) atomicOr(sy.flags, XKV_FLAG_CLF_BREAKDOWN); d = 1e-300; }
+          const double y = newton_rsqrt(d);
+          a[c] = lane == c ? d * y : a[c] * y;
+          col_s[c & 1][lane] = a[c];
+          if (lane == 0) piv_s[c & 1] = y;
+        }
+        named_bar_sync(1, 64);
+        if (warp == 0) {
+#pragma unroll
+          for (int j = c + 1; j < kCholNb; ++j) a[j] = fma(-a[c], col_s[c & 1][j], a[j]);   // entries above the diagonal: unused
+        } else {
+          a[c] *= piv_s[c & 1];
+#pragma unroll
+          for (int j = c + 1; j < kCholNb; ++j) a[j] = fma(-a[c], col_s[c & 1][j], a[j]);
+        }
+      }
+      if (warp == 1) {
+#pragma unroll
+        for (int j = 0; j < kCholNb; ++j) Iv[((size_t)p * kCholNb + j) * kCholNb + lane] = j >= lane ? a[j] : 0.0;
+      }
+    }
+  };
+  const int n_tiles = nbk * (nbk + 1) / 2;
+  auto tile_of = [&](int t, int& i, int& k) { i = 0; k = t; while (k > i) { ++i; k -= i; } };
+  if (bid == 0) {                                              // tile 0 is (0, 0)
+    stage(A_s, Gm, l);
+    __syncthreads();
+    if (tid < kCholNb) A_s[tid * kCholLd + tid] += shift;
+    factor(0);
+  }
+  if (!grid_barrier(sy, arrived, &ok_s)) return;
+  for (int p = 0; p + 1 < nbk; ++p) {
+    // (the tile whose factor everybody waits for comes first in its CTA: its index is the smallest of those with k > p)
+    for (int t = bid; t < n_tiles; t += nb) {
+      int i, k;
+      tile_of(t, i, k);
+      if (k <= p) continue;
+      __syncthreads();
+      stage(V_s, Iv + (size_t)p * kCholNb * kCholNb, kCholNb);
+      stage(A_s, Gm + (size_t)i * kCholNb * l + p * kCholNb, l);
+      if (i != k) stage(B_s, Gm + (size_t)k * kCholNb * l + p * kCholNb, l);
+      double acc[2][2];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const double2 v = __ldcg(reinterpret_cast<const double2*>(Gm + (size_t)(i * kCholNb + t_m * 8 + (lane >> 2)) * l + k * kCholNb + (t_n + j) * 8 + 2 * (lane & 3)));
+        acc[j][0] = v.x; acc[j][1] = v.y;
+      }
+      __syncthreads();
+      double li[2][2] = {{0.0, 0.0}, {0.0, 0.0}}, lk[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        dmma_block(li[j], A_s + t_m * 8 * kCholLd, V_s + (t_n + j) * 8 * kCholLd, lane, 1.0);
+        if (i != k) dmma_block(lk[j], B_s + t_m * 8 * kCholLd, V_s + (t_n + j) * 8 * kCholLd, lane, 1.0);
+      }
+      put(Li_s, kCholLd, li);
+      if (i != k) put(Lk_s, kCholLd, lk);
+      else put(Lf + (size_t)i * kCholNb * l + p * kCholNb, l, li);
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        if (i == k && p == 0) {                                // first touch of a diagonal tile
+#pragma unroll
+          for (int x = 0; x < 2; ++x) if (t_m * 8 + (lane >> 2) == (t_n + j) * 8 + 2 * (lane & 3) + x) acc[j][x] += shift;
+        }
+        dmma_block(acc[j], Li_s + t_m * 8 * kCholLd, (i != k ? Lk_s : Li_s) + (t_n + j) * 8 * kCholLd, lane, -1.0);
+      }
+      if (i == k && k == p + 1) {
+        put(A_s, kCholLd, acc);
+        factor(p + 1);
+      } else {
+        put(Gm + (size_t)i * kCholNb * l + k * kCholNb, l, acc);
+      }
+    }
+    if (!grid_barrier(sy, arrived, &ok_s)) return;
+  }
+  // ---- W: columns c0 .. c0 + 7 of block column k, rows downwards; warps: 8-row tile t_m, half (warp >> 2) of the terms
+  const int ldw = 9;
+  double* const Wc = cs_d;                                     // [l][9]
+  double* const H_s = A_s;                                     // [2][32][9] partial sums of the two halves
+  for (int st = bid; st < nbk * 4; st += nb) {
+    const int k = st >> 2, c0 = (st & 3) * 8;
+    __syncthreads();
+    for (int e = tid; e < kCholNb * 8; e += kCholThreads) {
+      const double v = __ldcg(Iv + ((size_t)k * kCholNb + (e >> 3)) * kCholNb + c0 + (e & 7));
+      Wc[(size_t)(k * kCholNb + (e >> 3)) * ldw + (e & 7)] = v;
+      W[(size_t)(k * kCholNb + (e >> 3)) * l + k * kCholNb + c0 + (e & 7)] = v;
+    }
+    for (int i = k + 1; i < nbk; ++i) {
+      stage(V_s, Iv + (size_t)i * kCholNb * kCholNb, kCholNb);
+      __syncthreads();
+      double acc[2] = {0.0, 0.0};
+      const double* Lrow = Lf + (size_t)(i * kCholNb + t_m * 8 + (lane >> 2)) * l + (lane & 3);
+#pragma unroll 2
+      for (int j = k + (warp >> 2); j < i; j += 2) {
+        double a[8];
+#pragma unroll
+        for (int s8 = 0; s8 < 8; ++s8) a[s8] = __ldcg(Lrow + j * kCholNb + s8 * 4);
+#pragma unroll
+        for (int s8 = 0; s8 < 8; ++s8)
+          dmma_8x8x4(acc, a[s8], Wc[(size_t)(j * kCholNb + s8 * 4 + (lane & 3)) * ldw + (lane >> 2)]);
+      }
+      double* h = H_s + (size_t)((warp >> 2) * kCholNb + t_m * 8 + (lane >> 2)) * ldw + 2 * (lane & 3);
+      h[0] = acc[0]; h[1] = acc[1];
+      __syncthreads();
+      if (warp < 4) {
+        double w[2] = {0.0, 0.0};
+#pragma unroll
+        for (int kk = 0; kk < kCholNb; kk += 4) {
+          const int r = kk + (lane & 3), c = lane >> 2;
+          dmma_8x8x4(w, -V_s[(t_m * 8 + (lane >> 2)) * kCholLd + r], H_s[(size_t)r * ldw + c] + H_s[(size_t)(kCholNb + r) * ldw + c]);
+        }
+        const int row = i * kCholNb + t_m * 8 + (lane >> 2), c = 2 * (lane & 3);
+        Wc[(size_t)row * ldw + c] = w[0]; Wc[(size_t)row * ldw + c + 1] = w[1];
+        *reinterpret_cast<double2*>(W + (size_t)row * l + k * kCholNb + c0 + c) = make_double2(w[0], w[1]);
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// Z (n x l) = U W^T for the lower-triangular W = L^-1 (fp64): 64 x 64 tiles, tile column J takes the first J + 1 blocks of
+// 64.  Longest tiles first.  Also writes the bf16 copy the tensor-core products read.  (The blocked triangular solve that
+// kept 32 rows of Z in shared memory took 161 us and 69 us for the inverses of its diagonal blocks at 4096 x 576; this
+// product 59 us.)
+__global__ void __launch_bounds__(256)
+tri_product_kernel(const float* __restrict__ U, const double* __restrict__ W, float* __restrict__ Z,
+                   __nv_bfloat16* __restrict__ Zb, int n, int l) {
+  __shared__ double As[64][kCholLd], Bs[64][kCholLd];          // 32 k of 64 rows of U, of 64 rows of W
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int wm = (warp & 3) * 16, wn = (warp >> 2) * 32;
+  const int J = l / 64 - 1 - blockIdx.y, row0 = blockIdx.x * 64, n0 = J * 64;
+  const int k_end = (J + 1) * 64;
+  double acc[2][4][2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { acc[i][j][0] = 0.0; acc[i][j][1] = 0.0; }
+  float4 pa[2];
+  double2 pb[4];
+  const int ar = tid >> 3, ac = (tid & 7) * 4;                 // U: rows ar, ar + 32; 4 columns
+  const int br = tid >> 4, bc = (tid & 15) * 2;                // W: rows br + 16 h; 2 columns
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = row0 + ar + 32 * h;
+      pa[h] = r < n ? *reinterpret_cast<const float4*>(U + (size_t)r * l + k0 + ac) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int j = n0 + br + 16 * h, k = k0 + bc;             // above the diagonal W is not stored
+      pb[h] = make_double2(0.0, 0.0);
+      if (k / kCholNb <= j / kCholNb) pb[h] = *reinterpret_cast<const double2*>(W + (size_t)j * l + k);
+    }
+  };
+  fetch(0);
+  for (int k0 = 0; k0 < k_end; k0 += 32) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      double* d = &As[ar + 32 * h][ac];
+      d[0] = (double)pa[h].x; d[1] = (double)pa[h].y; d[2] = (double)pa[h].z; d[3] = (double)pa[h].w;
+    }
+#pragma unroll
+    for (int h = 0; h < 4; ++h) { Bs[br + 16 * h][bc] = pb[h].x; Bs[br + 16 * h][bc + 1] = pb[h].y; }
+    __syncthreads();
+    if (k0 + 32 < k_end) fetch(k0 + 32);
+#pragma unroll
+    for (int kk = 0; kk < 32; kk += 4) {
+      double a[2], b[4];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) a[i] = As[wm + 8 * i + (lane >> 2)][kk + (lane & 3)];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = Bs[wn + 8 * j + (lane >> 2)][kk + (lane & 3)];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dmma_8x8x4(acc[i][j], a[i], b[j]);
+    }
+    __syncthreads();
+  }
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      TO* dst = C + (size_t)(m0 + wm + 8 * i + (lane >> 2)) * ldc + n0 + wn + 8 * j + 2 * (lane & 3);
-      dst[0] = (TO)acc[i][j][0];
-      dst[1] = (TO)acc[i][j][1];
-    }
-}
-
-// Blocked Cholesky factorisation (fp64) of the symmetric l x l matrix G + shift_rel * max_diag(G) * I, lower factor in
-// place, in panels of 32 columns: factor the diagonal block, solve the panel below it, update the trailing matrix.
-constexpr int kCholNb = 32;
-
-__global__ void __launch_bounds__(1024)
-chol_shift_kernel(double* __restrict__ G, int l, double shift_rel) {
-  __shared__ double red[32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  double mx = 0.0;
-  for (int i = tid; i < l; i += 1024) mx = fmax(mx, G[(size_t)i * l + i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) red[warp] = mx;
-  __syncthreads();
-  mx = red[lane];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  for (int i = tid; i < l; i += 1024) G[(size_t)i * l + i] += shift_rel * mx;
-}
-
-// Diagonal block [kb, kb+nb): unblocked factorisation by one warp.  A pivot that is not positive (breakdown) is
-// replaced by a tiny one and reported in flags.
-__global__ void __launch_bounds__(kCholNb)
-chol_diag_kernel(double* __restrict__ G, int l, int kb, int nb, unsigned int* __restrict__ flags) {
-  // One warp, lane i holds row i of the block in registers.  Step c: lane c takes the root of its diagonal entry, every
-  // lane below scales its entry of column c, the column goes through shared memory, and every lane takes it out of
-  // the rest of its row (independent multiply-adds).  Roots and quotients go through rsqrt: a step is a chain of
-  // dependent fp64 latencies, and sqrt and division are the longest of them.
-  __shared__ double col[kCholNb];
-  __shared__ double piv;
-  const int i = threadIdx.x;
-  double a[kCholNb];
-#pragma unroll
-  for (int j = 0; j < kCholNb; ++j) a[j] = (i < nb && j < nb && j <= i) ? G[(size_t)(kb + i) * l + kb + j] : (i == j ? 1.0 : 0.0);
-#pragma unroll
-  for (int c = 0; c < kCholNb; ++c) {
-    if (i == c) {
-      double d = a[c];
-      if (!(d > 0.0)) { atomicOr(flags, XKV_FLAG_CLF_BREAKDOWN); d = 1e-300; }
-      const double y = rsqrt(d);
-      a[c] = d * y;                                   // sqrt(d)
-      piv = y;
-    }
-    __syncwarp();
-    const double y = piv;
-    if (i > c) a[c] *= y;
-    col[i] = a[c];
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < kCholNb; ++j) {
-      if (j > c && j <= i) a[j] -= a[c] * col[j];
-    }
-    __syncwarp();
-  }
-#pragma unroll
-  for (int j = 0; j < kCholNb; ++j) if (i < nb && j < nb && j <= i) G[(size_t)(kb + i) * l + kb + j] = a[j];
-}
-
-constexpr int kCholPanelThreads = 128;             // (one warp per CTA, to spread the rows over more SMs: 24 us instead of 16)
-// Panel below the diagonal block: row i of L21 solves x L11^T = A21[i] (one thread per row).
-__global__ void __launch_bounds__(kCholPanelThreads)
-chol_panel_kernel(double* __restrict__ G, int l, int kb, int nb) {
-  __shared__ double L11[kCholNb][kCholNb + 1];
-  __shared__ double dinv[kCholNb];
-  for (int e = threadIdx.x; e < kCholNb * kCholNb; e += kCholPanelThreads) {
-    const int r = e / kCholNb, c = e % kCholNb;
-    const double v = (r < nb && c <= r) ? G[(size_t)(kb + r) * l + kb + c] : 0.0;
-    L11[r][c] = v;
-    if (r == c) dinv[r] = r < nb ? 1.0 / v : 0.0;
-  }
-  __syncthreads();
-  const int i = kb + nb + blockIdx.x * kCholPanelThreads + threadIdx.x;
-  if (i >= l) return;
-  // column sweep: once x_c is known it is taken out of every later entry, so the multiply-adds of a step are
-  // independent of one another (a dot product per entry is one long dependent chain on the fp64 pipe)
-  double x[kCholNb];
-  double* row = G + (size_t)i * l + kb;
-#pragma unroll
-  for (int c = 0; c < kCholNb; ++c) x[c] = c < nb ? row[c] : 0.0;
-#pragma unroll
-  for (int c = 0; c < kCholNb; ++c) {
-    if (c < nb) {
-      x[c] *= dinv[c];
-#pragma unroll
-      for (int t = 0; t < kCholNb; ++t) if (t > c) x[t] -= x[c] * L11[t][c];
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < kCholNb; ++c) if (c < nb) row[c] = x[c];
-}
-
-// Trailing update of the lower triangle: G[i][k] -= sum_t L21[i][t] L21[k][t]; one 32 x 32 tile per CTA.
-__global__ void __launch_bounds__(1024)
-chol_update_kernel(double* __restrict__ G, int l, int kb, int nb) {
-  if (blockIdx.x > blockIdx.y) return;                                 // upper triangle: not needed
-  __shared__ double Li[kCholNb][kCholNb + 1], Lk[kCholNb][kCholNb + 1];
-  const int t0 = kb + nb;
-  const int i = t0 + blockIdx.y * kCholNb + threadIdx.y, k = t0 + blockIdx.x * kCholNb + threadIdx.x;
-  const int ii = t0 + blockIdx.y * kCholNb + threadIdx.x;              // the row this thread loads for the tiles
-  const int kk = t0 + blockIdx.x * kCholNb + threadIdx.x;
-  // thread (y, x) loads element (row x of the tile, column y of the panel)
-  Li[threadIdx.x][threadIdx.y] = (ii < l && threadIdx.y < nb) ? G[(size_t)ii * l + kb + threadIdx.y] : 0.0;
-  Lk[threadIdx.x][threadIdx.y] = (kk < l && threadIdx.y < nb) ? G[(size_t)kk * l + kb + threadIdx.y] : 0.0;
-  __syncthreads();
-  if (i < l && k <= i) {
-    double acc = 0.0;
-#pragma unroll
-    for (int t = 0; t < kCholNb; ++t) acc += Li[threadIdx.y][t] * Lk[threadIdx.x][t];
-    G[(size_t)i * l + k] -= acc;
-  }
-}
-
-// Z (n x l) = U L^-T for the lower factor L: row by row, z_j = (u_j - sum_{i<j} z_i L[j][i]) / L[j][j] (fp64).  One warp
-// per row; the row lives in shared memory.  Also writes the bf16 copy the tensor-core products read.
-constexpr int kSolveWarps = 4;
-__global__ void __launch_bounds__(kSolveWarps * 32)
-trsolve_rows_kernel(const float* __restrict__ U, const double* __restrict__ L, float* __restrict__ Z,
-                    __nv_bfloat16* __restrict__ Zb, int n, int l) {
-  extern __shared__ double zrow[];                   // [kSolveWarps][l]
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int row = blockIdx.x * kSolveWarps + warp;
-  if (row >= n) return;
-  double* z = zrow + (size_t)warp * l;
-  for (int j = lane; j < l; j += 32) z[j] = (double)U[(size_t)row * l + j];
-  __syncwarp();
-  for (int j = 0; j < l; ++j) {
-    const double* Lj = L + (size_t)j * l;
-    double s = 0.0;
-    for (int i = lane; i < j; i += 32) s += z[i] * Lj[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) z[j] = (z[j] - s) / Lj[j];
-    __syncwarp();
-  }
-  for (int j = lane; j < l; j += 32) {
-    Z[(size_t)row * l + j] = (float)z[j];
-    if (Zb) Zb[(size_t)row * l + j] = __float2bfloat16((float)z[j]);
-  }
-}
-
-// ---- the triangular solve Z = U L^-T in 64-column blocks on the fp64 tensor-core path ----
-// Z[:, J] = (U[:, J] - sum_{I<J} Z[:, I] L[J, I]^T) inv(L[J, J])^T.  The inverses of the 64 x 64 diagonal blocks come
-// from a small kernel (one thread per column of the inverse, forward substitution); the solve keeps 32 rows of Z in
-// fp64 in shared memory per CTA and streams the blocks of L through a 64 x 64 staging tile.
-constexpr int kTriBlock = 64;
-__global__ void __launch_bounds__(kTriBlock)
-tri_inv_diag_kernel(const double* __restrict__ L, int l, double* __restrict__ Xinv) {
-  __shared__ double Xs[kTriBlock][kTriBlock + 1];
-  const int c = threadIdx.x, jb = blockIdx.x * kTriBlock;
-  const double* Lb = L + (size_t)jb * l + jb;
-  for (int j = 0; j < kTriBlock; ++j) {
-    double x = 0.0;
-    if (j >= c) {
-      double s0 = (j == c) ? 1.0 : 0.0, s1 = 0.0;
-      const double* Lj = Lb + (size_t)j * l;
-      int i = c;
-      for (; i + 1 < j; i += 2) { s0 -= Lj[i] * Xs[i][c]; s1 -= Lj[i + 1] * Xs[i + 1][c]; }
-      if (i < j) s0 -= Lj[i] * Xs[i][c];
-      x = (s0 + s1) / Lj[j];
-    }
-    Xs[j][c] = x;                                    // a thread only ever reads its own column
-  }
-  __syncthreads();
-  double* out = Xinv + (size_t)blockIdx.x * kTriBlock * kTriBlock;
-  for (int e = c; e < kTriBlock * kTriBlock; e += kTriBlock) out[e] = Xs[e / kTriBlock][e % kTriBlock];
-}
-
-constexpr int kTriRows = 32;                         // rows of Z per CTA
-__global__ void __launch_bounds__(256)
-trsolve_mma_kernel(const float* __restrict__ U, const double* __restrict__ L, const double* __restrict__ Xinv,
-                   float* __restrict__ Z, __nv_bfloat16* __restrict__ Zb, int n, int l) {
-  extern __shared__ double tri_s[];
-  const int ldz = l + 4;                             // 4 mod 16 doubles: fragment loads are conflict free
-  double* Zs = tri_s;                                // [kTriRows][ldz]
-  double* Ls = tri_s + (size_t)kTriRows * ldz;       // [64][kDgemmLd]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int wm = (warp & 1) * 16, wn = (warp >> 1) * 16;
-  const int row0 = blockIdx.x * kTriRows;
-  const int fr = lane >> 2, fc = lane & 3;
-  auto stage = [&](const double* src, int ld) {      // 64 x 64 block, row-major
-    for (int e = tid; e < kTriBlock * kTriBlock; e += 256) Ls[(e >> 6) * kDgemmLd + (e & 63)] = src[(size_t)(e >> 6) * ld + (e & 63)];
-  };
-  const int nb = l / kTriBlock;
-  for (int J = 0; J < nb; ++J) {
-    double acc[2][2][2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int r = row0 + wm + 8 * i + fr;
-        const float2 u = r < n ? *reinterpret_cast<const float2*>(U + (size_t)r * l + J * kTriBlock + wn + 8 * j + 2 * fc)
-                               : make_float2(0.0f, 0.0f);
-        acc[i][j][0] = (double)u.x;
-        acc[i][j][1] = (double)u.y;
-      }
-    for (int I = 0; I < J; ++I) {
-      __syncthreads();                               // the staging tile and the last block of Z are free / written
-      stage(L + (size_t)J * kTriBlock * l + (size_t)I * kTriBlock, l);
-      __syncthreads();
-#pragma unroll 4
-      for (int kk = 0; kk < kTriBlock; kk += 4) {
-        double a[2], b[2];
-#pragma unroll
-        for (int i = 0; i < 2; ++i) a[i] = -Zs[(size_t)(wm + 8 * i + fr) * ldz + I * kTriBlock + kk + fc];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) b[j] = Ls[(wn + 8 * j + fr) * kDgemmLd + kk + fc];
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-          for (int j = 0; j < 2; ++j) dmma_8x8x4(acc[i][j], a[i], b[j]);
+      const int r = row0 + wm + 8 * i + (lane >> 2), c = n0 + wn + 8 * j + 2 * (lane & 3);
+      if (r < n) {
+        const float z0 = (float)acc[i][j][0], z1 = (float)acc[i][j][1];
+        *reinterpret_cast<float2*>(Z + (size_t)r * l + c) = make_float2(z0, z1);
+        *reinterpret_cast<__nv_bfloat162*>(Zb + (size_t)r * l + c) = __floats2bfloat162_rn(z0, z1);
       }
     }
-    __syncthreads();
-    // the right-hand side of the diagonal step goes through the block's own columns of Zs
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        double* d = Zs + (size_t)(wm + 8 * i + fr) * ldz + J * kTriBlock + wn + 8 * j + 2 * fc;
-        d[0] = acc[i][j][0];
-        d[1] = acc[i][j][1];
-        acc[i][j][0] = 0.0;
-        acc[i][j][1] = 0.0;
-      }
-    stage(Xinv + (size_t)J * kTriBlock * kTriBlock, kTriBlock);
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < kTriBlock; kk += 4) {
-      double a[2], b[2];
-#pragma unroll
-      for (int i = 0; i < 2; ++i) a[i] = Zs[(size_t)(wm + 8 * i + fr) * ldz + J * kTriBlock + kk + fc];
-#pragma unroll
-      for (int j = 0; j < 2; ++j) b[j] = Ls[(wn + 8 * j + fr) * kDgemmLd + kk + fc];
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) dmma_8x8x4(acc[i][j], a[i], b[j]);
-    }
-    __syncthreads();                                 // every warp has read the right-hand side
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int rl = wm + 8 * i + fr, col = J * kTriBlock + wn + 8 * j + 2 * fc;
-        double* d = Zs + (size_t)rl * ldz + col;
-        d[0] = acc[i][j][0];
-        d[1] = acc[i][j][1];
-        const int r = row0 + rl;
-        if (r < n) {
-          const float z0 = (float)acc[i][j][0], z1 = (float)acc[i][j][1];
-          *reinterpret_cast<float2*>(Z + (size_t)r * l + col) = make_float2(z0, z1);
-          if (Zb) *reinterpret_cast<__nv_bfloat162*>(Zb + (size_t)r * l + col) = __floats2bfloat162_rn(z0, z1);
-        }
-      }
-  }
 }
 
 }  // namespace
@@ -570,51 +616,6 @@ constexpr float kJacobiTol = 1e-8f;
 constexpr int kJacobiThreads = 1024;
 constexpr int kJb = 32, kJp = 2 * kJb;             // indices of a block, of a pair
 constexpr int kJacobiSmem = 4 * (kJp * kJp * 3 + 8 * kJp * kJb + kJp * (kJb + 1));   // bytes, see the carve-up
-constexpr unsigned kJacobiSpinLimit = 1u << 18;   // polls of a barrier that normally opens within microseconds
-
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned int* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void red_release_u32(unsigned int* p, unsigned v) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// A grid-wide barrier of cooperative kernels: an arrival counter that only grows, polled by everybody (an arrival and
-// one poll are the only trips to L2).  The wait is bounded like every wait of the library: a CTA that gives up raises
-// XKV_FLAG_TIMEOUT and the abort word, and every other CTA leaves at its next wait.  Data that crosses it is read past
-// L1 (other SMs wrote it).
-struct GridSync {            // words of the workspace's flag block
-  unsigned int* flags;       // status word
-  unsigned int* count;       // arrivals so far (monotonic)
-  unsigned int* abort;       // a CTA gave up
-  unsigned int spin_limit;   // polls of one barrier wait
-  unsigned int no_arrival;   // fault injection (tests of the give-up path): CTA 0 arrives at no barrier, and passes the first
-};
-// Returns false when the barrier was abandoned (by this CTA or another one).  `my_gen` counts this CTA's barriers.
-__device__ __forceinline__ bool grid_barrier(const GridSync& sy, unsigned& my_gen, int* ok_s) {
-  __syncthreads();
-  ++my_gen;
-  if (threadIdx.x == 0) {
-    const bool silent = sy.no_arrival != 0u && blockIdx.x == 0;
-    bool ok = true;
-    __threadfence();
-    if (!silent) red_release_u32(sy.count, 1u);
-    if (!silent || my_gen > 1u) {
-      const unsigned want = gridDim.x * my_gen;
-      for (unsigned i = 0; ld_acquire_u32(sy.count) < want;) {
-        if (++i >= sy.spin_limit || ((i & 15u) == 0u && ld_acquire_u32(sy.abort) != 0u)) { ok = false; break; }
-      }
-    }
-    if (!ok) { atomicOr(sy.flags, XKV_FLAG_TIMEOUT); atomicExch(sy.abort, 1u); }
-    __threadfence();
-    *ok_s = ok ? 1 : 0;
-  }
-  __syncthreads();
-  return *ok_s != 0;
-}
-
 // Pair k of round t of the round-robin tournament of n (even) players, the smaller first.
 __device__ __forceinline__ int2 tournament_pair(int k, int t, int n) {
   int p, q;
@@ -669,14 +670,13 @@ __device__ __forceinline__ float piece_sum(const float* __restrict__ red, int o)
 
 __global__ void __launch_bounds__(kJacobiThreads, 1)
 jacobi_block_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __restrict__ Pt, float* __restrict__ Qg, int l,
-                    float2* __restrict__ partial, GridSync sy) {
+                    float2* __restrict__ partial, unsigned arrived, GridSync sy) {
   extern __shared__ __align__(16) float js[];
   __shared__ int ok_s, done_s;
   __shared__ float2 red_s[kJacobiThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = gridDim.x, bid = blockIdx.x;
   const int nblk = l / kJb, npair = l / kJp;                 // l is a multiple of 64
   const long long gtid = (long long)bid * kJacobiThreads + tid, gstride = (long long)nb * kJacobiThreads;
-  unsigned my_gen = 0;
   for (long long e = gtid; e < (long long)l * l; e += gstride) Pt[e] = (e / l == e % l) ? 1.0f : 0.0f;
   float* const S0 = js;                                      // [64][64] each; phase A: the submatrix and its other buffer
   float* const S1 = S0 + kJp * kJp;
@@ -819,7 +819,7 @@ jacobi_block_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __res
   };
 
   int cur = 0, qb = 0;
-  bool alive = grid_barrier(sy, my_gen, &ok_s);
+  bool alive = grid_barrier(sy, arrived, &ok_s);
   int sweeps_done = 0;
   for (int sweep = 0; alive && sweep < kJacobiSweeps; ++sweep) {
     // ---- off-diagonal weight of M: per-CTA partial sums, then every CTA adds them up in the same order
@@ -845,7 +845,7 @@ jacobi_block_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __res
       };
       total();
       if (tid == 0) partial[(sweep & 1) * nb + bid] = make_float2(off, all);
-      alive = grid_barrier(sy, my_gen, &ok_s);
+      alive = grid_barrier(sy, arrived, &ok_s);
       if (!alive) break;
       off = all = 0.0f;
       for (int b = tid; b < nb; b += kJacobiThreads) { const float2 v = __ldcg(partial + (sweep & 1) * nb + b); off += v.x; all += v.y; }
@@ -867,7 +867,7 @@ jacobi_block_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __res
         for (int it = bid - npair; it < items; it += nb - npair)
           rotate_vectors(tournament_pair(it / npair, t - 1, nblk), (it % npair) * kJp, Qprev + (size_t)(it / npair) * kJp * kJp);
       }
-      alive = grid_barrier(sy, my_gen, &ok_s);
+      alive = grid_barrier(sy, arrived, &ok_s);
       if (!alive) break;
       for (int it = bid; it < npair * (npair + 1); it += nb) {   // pieces (a <= b, h)
         const int h = it & 1;
@@ -875,7 +875,7 @@ jacobi_block_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __res
         while (rest >= npair - a) { rest -= npair - a; ++a; }
         rotate_matrix(M, Mn, a, a + rest, h, t, Q);
       }
-      alive = grid_barrier(sy, my_gen, &ok_s);
+      alive = grid_barrier(sy, arrived, &ok_s);
       cur ^= 1;
       qb ^= 1;
     }
@@ -890,63 +890,103 @@ jacobi_block_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __res
   }
 }
 
-// The r largest eigenvalues (ties to the lower index) and their eigenvectors as the columns of Psel (l x r);
-// sigma = sqrt(lambda).
-__global__ void __launch_bounds__(1024)
-eig_select_kernel(const float* __restrict__ M, const float* __restrict__ Pt, int l, int r, float* __restrict__ Psel,
+// The r largest eigenvalues (ties to the lower index) and their eigenvectors as the rows of Ps (r x l); sigma =
+// sqrt(lambda).  One warp per eigenvalue.
+constexpr int kSelectWarps = 8;
+__global__ void __launch_bounds__(kSelectWarps * 32)
+eig_select_kernel(const float* __restrict__ M, const float* __restrict__ Pt, int l, int r, float* __restrict__ Ps,
                   float* __restrict__ sigma) {
-  extern __shared__ int rank_s[];                      // [l]
-  const int tid = threadIdx.x;
-  for (int i = tid; i < l; i += 1024) {
-    const float li = M[(size_t)i * l + i];
-    int rk = 0;
-    for (int j = 0; j < l; ++j) {
-      const float lj = M[(size_t)j * l + j];
-      rk += (lj > li || (lj == li && j < i)) ? 1 : 0;
-    }
-    rank_s[i] = rk;
-    if (rk < r && sigma) sigma[rk] = sqrtf(fmaxf(li, 0.0f));
+  const int lane = threadIdx.x & 31, i = blockIdx.x * kSelectWarps + (threadIdx.x >> 5);
+  if (i >= l) return;
+  const float li = M[(size_t)i * l + i];
+  int rk = 0;
+  for (int j = lane; j < l; j += 32) {
+    const float lj = M[(size_t)j * l + j];
+    rk += (lj > li || (lj == li && j < i)) ? 1 : 0;
   }
-  __syncthreads();
-  for (int e = tid; e < l * l; e += 1024) {
-    const int row = e / l, i = e % l;
-    const int rk = rank_s[i];
-    if (rk < r) Psel[(size_t)row * r + rk] = Pt[(size_t)i * l + row];
-  }
+  rk = __reduce_add_sync(0xffffffffu, rk);
+  if (rk >= r) return;
+  if (lane == 0 && sigma) sigma[rk] = sqrtf(fmaxf(li, 0.0f));
+  for (int j = lane; j < l; j += 32) Ps[(size_t)rk * l + j] = Pt[(size_t)i * l + j];
 }
 
-// V (N x r, fp32) -> its bf16 copy and the per-layer matrices B [G][r][d], B[g][m][j] = V[g d + j][m].
-__global__ void clf_finish_kernel(const float* __restrict__ V, int G, int d, int r, __nv_bfloat16* __restrict__ Vb,
-                                  __nv_bfloat16* __restrict__ B) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long total = (long long)G * d * r;
-  if (idx >= total) return;
-  const int m = (int)(idx % r);
-  const long long row = idx / r;                       // g d + j
-  const int g = (int)(row / d), j = (int)(row % d);
-  const __nv_bfloat16 v = __float2bfloat16(V[idx]);
-  Vb[idx] = v;
-  B[((size_t)g * r + m) * d + j] = v;
+// V = Z Ps^T (N x r, fp32), rounded to bf16: row-major, and as the per-layer matrices B [G][r][d], B[g][m][j] = V[g d + j][m].
+// 64 x 64 tiles, 256 threads, 4 x 4 outputs per thread, chunks of 32 k.
+__global__ void __launch_bounds__(256)
+ritz_vectors_kernel(const float* __restrict__ Z, const float* __restrict__ Ps, int l, int r, int d, __nv_bfloat16* __restrict__ Vb,
+                    __nv_bfloat16* __restrict__ B) {
+  __shared__ __align__(16) float As[32][68], Bs[32][68];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int n0 = blockIdx.y * 64, m0 = blockIdx.x * 64;
+  const int fr = tid >> 3, fc = (tid & 7) * 4;         // staged rows fr, fr + 32; 4 k
+  float4 pa[2], pb[2];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      pa[h] = *reinterpret_cast<const float4*>(Z + (size_t)(n0 + fr + 32 * h) * l + k0 + fc);
+      const int m = m0 + fr + 32 * h;
+      pb[h] = m < r ? *reinterpret_cast<const float4*>(Ps + (size_t)m * l + k0 + fc) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+  };
+  float acc[4][4] = {};
+  fetch(0);
+  for (int k0 = 0; k0 < l; k0 += 32) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int row = fr + 32 * h;
+      As[fc][row] = pa[h].x; As[fc + 1][row] = pa[h].y; As[fc + 2][row] = pa[h].z; As[fc + 3][row] = pa[h].w;
+      Bs[fc][row] = pb[h].x; Bs[fc + 1][row] = pb[h].y; Bs[fc + 2][row] = pb[h].z; Bs[fc + 3][row] = pb[h].w;
+    }
+    __syncthreads();
+    if (k0 + 32 < l) fetch(k0 + 32);
+#pragma unroll
+    for (int kk = 0; kk < 32; ++kk) {
+      const float4 av = *reinterpret_cast<const float4*>(&As[kk][ty * 4]), bv = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
+      const float a[4] = {av.x, av.y, av.z, av.w}, b[4] = {bv.x, bv.y, bv.z, bv.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int n = n0 + ty * 4 + i, g = n / d, j = n - g * d;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const int m = m0 + tx * 4 + x;
+      if (m < r) {
+        const __nv_bfloat16 v = __float2bfloat16(acc[i][x]);
+        Vb[(size_t)n * r + m] = v;
+        B[((size_t)g * r + m) * d + j] = v;
+      }
+    }
+  }
 }
 
 }  // namespace
 
 namespace {
 
-__global__ void symmetrize_kernel(float* __restrict__ M, int l) {
+// M = (S + S^T) / 2 for the sum S of the partial products part [n_part][l][l], in a fixed order.
+__global__ void symmetrize_kernel(const float* __restrict__ part, int n_part, float* __restrict__ M, int l) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= l * l) return;
   const int i = e / l, j = e % l;
-  if (i < j) {
-    const float v = 0.5f * (M[(size_t)i * l + j] + M[(size_t)j * l + i]);
-    M[(size_t)i * l + j] = v;
-    M[(size_t)j * l + i] = v;
-  }
+  if (i > j) return;
+  float a = 0.0f, b = 0.0f;
+  for (int z = 0; z < n_part; ++z) { a += part[((size_t)z * l + i) * l + j]; b += part[((size_t)z * l + j) * l + i]; }
+  const float v = 0.5f * (a + b);
+  M[(size_t)i * l + j] = v;
+  M[(size_t)j * l + i] = v;
 }
 
 struct ClfPlan {
   int T, Tp, N, r, l, q;
-  size_t off_flags, off_zb, off_yt, off_u, off_z, off_g, off_m, off_p, off_ps, off_v, off_vb, off_cs, off_m2, off_q, off_xinv, total;
+  int gram_split, gram_rows, ritz_split;                     // row ranges of a Gram matrix and rows of each; K ranges of the Ritz matrix
+  size_t off_flags, off_zb, off_yt, off_u, off_z, off_part, off_g, off_lf, off_w, off_iv, off_m, off_p, off_ps, off_vb, off_cs, off_m2,
+      off_q, total;
 };
 
 size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -963,16 +1003,28 @@ bool make_plan(const xkv_clf_config* c, ClfPlan* p) {
   p->off_yt = o; o = align_up(o + (size_t)p->l * p->Tp * 2);
   p->off_u = o; o = align_up(o + (size_t)p->N * p->l * 4);
   p->off_z = o; o = align_up(o + (size_t)p->N * p->l * 4);
-  p->off_g = o; o = align_up(o + (size_t)p->l * p->l * 8);      // the Gram matrix / Cholesky factor, fp64
+  // row ranges so that the lower 64 x 64 tiles of the Gram matrix fill the SMs about twice; the K ranges of the
+  // Rayleigh-Ritz matrix fill them once (both for 148 SMs; fewer only queue)
+  const int tiles = (p->l / 64) * (p->l / 64 + 1) / 2, ritz_tiles = ((p->l + 127) / 128) * ((p->l + 191) / 192);
+  p->gram_split = 296 / tiles < 1 ? 1 : (296 / tiles > 8 ? 8 : 296 / tiles);
+  p->gram_rows = ((p->N + p->gram_split - 1) / p->gram_split + 31) & ~31;
+  p->gram_split = (p->N + p->gram_rows - 1) / p->gram_rows;
+  p->ritz_split = 148 / ritz_tiles < 1 ? 1 : (148 / ritz_tiles > 16 ? 16 : 148 / ritz_tiles);
+  const int ritz_cols = ((p->T + p->ritz_split - 1) / p->ritz_split + 63) & ~63;
+  p->ritz_split = (p->T + ritz_cols - 1) / ritz_cols;            // none of the ranges is empty
+  const size_t part_words = p->gram_split * 2 > p->ritz_split ? p->gram_split * 2 : p->ritz_split;
+  p->off_part = o; o = align_up(o + part_words * p->l * p->l * 4);   // partial Gram matrices (fp64) / Ritz matrices (fp32)
+  p->off_g = o; o = align_up(o + (size_t)p->l * p->l * 8);      // the Gram matrix, factorised in place of its tiles, fp64
+  p->off_lf = o; o = align_up(o + (size_t)p->l * p->l * 8);     // its factor below the diagonal blocks
+  p->off_w = o; o = align_up(o + (size_t)p->l * p->l * 8);      // the factor's inverse
+  p->off_iv = o; o = align_up(o + (size_t)p->l * kCholNb * 8);  // inverses of its diagonal blocks
   p->off_m = o; o = align_up(o + (size_t)p->l * p->l * 4);
   p->off_p = o; o = align_up(o + (size_t)p->l * p->l * 4);
   p->off_ps = o; o = align_up(o + (size_t)p->l * p->r * 4);
-  p->off_v = o; o = align_up(o + (size_t)p->N * p->r * 4);
   p->off_vb = o; o = align_up(o + (size_t)p->N * p->r * 2);
   p->off_cs = o; o = align_up(o + (size_t)2 * 1024 * 8);            // per-CTA partial sums of the Jacobi convergence check
   p->off_m2 = o; o = align_up(o + (size_t)p->l * p->l * 4);      // second buffers of the one-kernel Jacobi sweeps
   p->off_q = o; o = align_up(o + (size_t)2 * p->l * kJp * 4);    // rotation products of the block pairs, two rounds
-  p->off_xinv = o; o = align_up(o + (size_t)p->l * kTriBlock * 8);   // inverses of the diagonal blocks of a Cholesky factor
   p->total = o;
   return true;
 }
@@ -987,36 +1039,49 @@ int check_clf_config(const xkv_clf_config* c) {
   return XKV_OK;
 }
 
-template <bool TRANS, int BN>
-cudaError_t launch_gemm_bn(const void* a, int a_rows_k, int a_cols_m, int a_pitch, const void* b, int b_rows_n, int b_cols_k,
-                           int b_pitch, float* Cf, __nv_bfloat16* Cb, long long ldc, unsigned int* flags, int device,
-                           cudaStream_t s) {
+// A operand of a product: a matrix [rows][cols] with a row pitch (elements); rows are k unless AROW.
+struct GemmOperand {
+  const void* p;
+  int rows, cols, pitch;
+};
+
+template <bool TRANS, bool AROW, int BN>
+cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, int splits, float* Cf, __nv_bfloat16* Cb, long long ldc,
+                           unsigned int* flags, int device, cudaStream_t s) {
+  const int M = AROW ? a.rows : a.cols, N = b.rows, K = b.cols;
   CUtensorMap ma, mb;
-  if (!encode_bf16_map(&ma, a, (uint64_t)a_rows_k, (uint64_t)a_cols_m, (uint64_t)a_pitch, 64) ||
-      !encode_bf16_map(&mb, b, (uint64_t)b_rows_n, (uint64_t)b_cols_k, (uint64_t)b_pitch, BN))
+  if (!encode_bf16_map(&ma, a.p, (uint64_t)a.rows, (uint64_t)a.cols, (uint64_t)a.pitch, AROW ? 128 : 64) ||
+      !encode_bf16_map(&mb, b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BN))
     return cudaErrorInvalidValue;
   const size_t smem = 1024 + (size_t)gemm_stages<BN>() * gemm_stage_bytes<BN>();
-  cudaError_t e = ensure_dyn_smem<clf_gemm_kernel<TRANS, BN>>(smem, device);
+  cudaError_t e = ensure_dyn_smem<clf_gemm_kernel<TRANS, AROW, BN>>(smem, device);
   if (e != cudaSuccess) return e;
-  const dim3 grid((b_rows_n + BN - 1) / BN, (a_cols_m + 127) / 128);
-  clf_gemm_kernel<TRANS, BN><<<grid, kGemmThreads, smem, s>>>(ma, mb, a_cols_m, b_rows_n, a_rows_k, Cf, Cb, ldc, flags);
+  const int k_per = ((K + splits - 1) / splits + 63) & ~63;
+  const dim3 grid((N + BN - 1) / BN, (M + 127) / 128, splits);
+  clf_gemm_kernel<TRANS, AROW, BN><<<grid, kGemmThreads, smem, s>>>(ma, mb, M, N, K, k_per, Cf, Cb, ldc, flags);
   count_launch(kFamClf);
   return cudaGetLastError();
 }
 
 // The tile width that pads N least (the widest on a tie): 576 columns are three tiles of 192, a tall N is tiles of 256.
-template <bool TRANS>
-cudaError_t launch_gemm(const void* a, int a_rows_k, int a_cols_m, int a_pitch, const void* b, int b_rows_n, int b_cols_k,
-                        int b_pitch, float* Cf, __nv_bfloat16* Cb, long long ldc, unsigned int* flags, int device,
-                        cudaStream_t s) {
-  const int N = b_rows_n;
-  auto padded = [&](int bn) { return (long long)((N + bn - 1) / bn) * bn; };
+template <bool TRANS, bool AROW>
+cudaError_t launch_gemm(GemmOperand a, GemmOperand b, int splits, float* Cf, __nv_bfloat16* Cb, long long ldc,
+                        unsigned int* flags, int device, cudaStream_t s) {
+  auto padded = [&](int bn) { return (long long)((b.rows + bn - 1) / bn) * bn; };
   int bn = 256;
   if (padded(192) < padded(bn)) bn = 192;
   if (padded(128) < padded(bn)) bn = 128;
-  if (bn == 256) return launch_gemm_bn<TRANS, 256>(a, a_rows_k, a_cols_m, a_pitch, b, b_rows_n, b_cols_k, b_pitch, Cf, Cb, ldc, flags, device, s);
-  if (bn == 192) return launch_gemm_bn<TRANS, 192>(a, a_rows_k, a_cols_m, a_pitch, b, b_rows_n, b_cols_k, b_pitch, Cf, Cb, ldc, flags, device, s);
-  return launch_gemm_bn<TRANS, 128>(a, a_rows_k, a_cols_m, a_pitch, b, b_rows_n, b_cols_k, b_pitch, Cf, Cb, ldc, flags, device, s);
+  if (bn == 256) return launch_gemm_bn<TRANS, AROW, 256>(a, b, splits, Cf, Cb, ldc, flags, device, s);
+  if (bn == 192) return launch_gemm_bn<TRANS, AROW, 192>(a, b, splits, Cf, Cb, ldc, flags, device, s);
+  return launch_gemm_bn<TRANS, AROW, 128>(a, b, splits, Cf, Cb, ldc, flags, device, s);
+}
+
+template <auto Kernel>
+cudaError_t launch_cooperative(int grid, int threads, size_t smem, void** args, int device, cudaStream_t s) {
+  cudaError_t e = ensure_dyn_smem<Kernel>(smem, device);
+  if (e != cudaSuccess) return e;
+  count_launch(kFamClf);
+  return cudaLaunchCooperativeKernel((const void*)Kernel, dim3(grid), dim3(threads), args, smem, s);
 }
 
 }  // namespace
@@ -1041,7 +1106,7 @@ int clf_workspace_bytes(const xkv_clf_config* c, uint64_t* bytes) {
 
 // Debug/test entry of the tensor-core product alone: C (M x N, fp32) = A B^T, A bf16 [K][M], B bf16 [N][K].
 cudaError_t clf_gemm(const void* a, const void* b, int M, int N, int K, float* C, unsigned int* flags, int device, cudaStream_t s) {
-  return launch_gemm<false>(a, K, M, M, b, N, K, K, C, nullptr, N, flags, device, s);
+  return launch_gemm<false, false>({a, K, M, M}, {b, N, K, K}, 1, C, nullptr, N, flags, device, s);
 }
 
 static std::atomic<unsigned> g_clf_inject{0};
@@ -1060,104 +1125,80 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
   __nv_bfloat16* Yt = (__nv_bfloat16*)(w + p.off_yt);
   float* U = (float*)(w + p.off_u);
   float* Z = (float*)(w + p.off_z);
+  double* part = (double*)(w + p.off_part);
   double* Gm = (double*)(w + p.off_g);
+  double* Lf = (double*)(w + p.off_lf);
+  double* W = (double*)(w + p.off_w);
+  double* Iv = (double*)(w + p.off_iv);
   float* Mm = (float*)(w + p.off_m);
   float* Pm = (float*)(w + p.off_p);
   float* Ps = (float*)(w + p.off_ps);
-  float* V = (float*)(w + p.off_v);
   __nv_bfloat16* Vb = (__nv_bfloat16*)(w + p.off_vb);
-  const int N = p.N, l = p.l, r = p.r, T = p.T;
-  cudaError_t e = cudaMemsetAsync(flags, 0, 256, s);
+  const int N = p.N, r = p.r, T = p.T;
+  int l = p.l, sms = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+  if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 256, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(Zb, omega, (size_t)N * l * 2, cudaMemcpyDeviceToDevice, s);
-  const dim3 g_ll((l + 63) / 64, (l + 63) / 64);
-  // Y^T = Z^T X^T  then  U = X^T Y
-  auto two_products = [&]() -> cudaError_t {
-    cudaError_t e2 = launch_gemm<false>(Zb, N, l, l, X, T, N, N, nullptr, Yt, p.Tp, flags, device, s);
-    if (e2 != cudaSuccess) return e2;
-    return launch_gemm<false>(X, T, N, N, Yt, l, T, p.Tp, U, nullptr, l, flags, device, s);
-  };
-  // Z = orth(src) by three passes of shifted Cholesky QR.  The Gram matrix is accumulated, factorised and solved
-  // in fp64: its condition number is the square of the iterate's, which after a multiplication by X^T X spans the
-  // whole range between the largest singular value and the noise floor.
-  const size_t solve_smem = (size_t)kSolveWarps * l * sizeof(double);
-  e = e == cudaSuccess ? ensure_dyn_smem<trsolve_rows_kernel>(solve_smem, device) : e;
-  const size_t tri_smem = ((size_t)kTriRows * (l + 4) + (size_t)kTriBlock * kDgemmLd) * sizeof(double);
-  // the blocked solve keeps 32 rows of Z in shared memory: sketches wider than about 700 columns take the row-wise kernel
-  const bool mma_solve = tri_smem <= 227u * 1024u;
-  if (mma_solve) e = e == cudaSuccess ? ensure_dyn_smem<trsolve_mma_kernel>(tri_smem, device) : e;
-  double* Xinv = (double*)(w + p.off_xinv);
-  // Every pass divides the condition number by about shift^-1/2; the iterate of a power iteration only has to stay
-  // well conditioned (two passes), the last one has to be orthonormal (five passes with decreasing shifts: the
-  // columns of U that lie in the noise floor are 10^8 times smaller than the leading ones).
-  static const double kShifts[5] = {1e-4, 1e-5, 1e-6, 1e-8, 1e-10};
-  auto cholqr = [&](const float* src, int passes) -> cudaError_t {
+  // Y^T = Z^T X^T  and  U = X^T Y
+  auto product_y = [&]() { return launch_gemm<false, false>({Zb, N, l, l}, {X, T, N, N}, 1, nullptr, Yt, p.Tp, flags, device, s); };
+  auto product_u = [&]() { return launch_gemm<false, false>({X, T, N, N}, {Yt, l, T, p.Tp}, 1, U, nullptr, l, flags, device, s); };
+  // Z = orth(U) by shifted Cholesky QR, the Gram matrix accumulated, factorised and inverted in fp64: its condition
+  // number is the square of the iterate's, which after a multiplication by X^T X spans the whole range between the
+  // largest singular value and the noise floor.  A pass divides the condition number by up to shift^-1/2; U is stored
+  // in fp32, so its own is below 1e9 and the fp64 Gram matrix carries a shift of 1e-11 safely (its rounding errors are
+  // below 1e-13).  One pass leaves an iterate well conditioned, which is all that the next multiplication needs; the last
+  // iterate takes three and is orthonormal to fp32 rounding.  (Shifts that start at 1e-4 need two and five passes for a
+  // worse subspace: residual 1.088 instead of 1.081 of the optimum.)
+  constexpr double kShift = 1e-11;
+  const int nbk = l / kCholNb, n_tiles = nbk * (nbk + 1) / 2;
+  const int chol_grid = sms < (n_tiles > 32 ? n_tiles : 32) ? sms : (n_tiles > 32 ? n_tiles : 32);
+  const size_t chol_smem = (size_t)l * 9 * sizeof(double);
+  unsigned chol_arrived = 0;
+  auto cholqr = [&](int passes) -> cudaError_t {                       // an odd number of passes ends in Z
+    float* in = U;
+    float* out = Z;
     for (int pass = 0; pass < passes; ++pass) {
-      const float* in = pass == 0 ? src : Z;
-      dgemm_tn_mma_kernel<double><<<g_ll, 256, 0, s>>>(in, in, Gm, N, l, l, l);
-      const double shift_rel = kShifts[pass];
-      chol_shift_kernel<<<1, 1024, 0, s>>>(Gm, l, shift_rel);
-      int launches = 2;
-      for (int kb = 0; kb < l; kb += kCholNb) {
-        const int nb = l - kb < kCholNb ? l - kb : kCholNb;
-        chol_diag_kernel<<<1, kCholNb, 0, s>>>(Gm, l, kb, nb, flags);
-        const int rem = l - kb - nb;
-        ++launches;
-        if (rem > 0) {
-          chol_panel_kernel<<<(rem + kCholPanelThreads - 1) / kCholPanelThreads, kCholPanelThreads, 0, s>>>(Gm, l, kb, nb);
-          const int tiles = (rem + kCholNb - 1) / kCholNb;
-          chol_update_kernel<<<dim3(tiles, tiles), dim3(kCholNb, kCholNb), 0, s>>>(Gm, l, kb, nb);
-          launches += 2;
-        }
-      }
-      if (!mma_solve) {
-        trsolve_rows_kernel<<<(N + kSolveWarps - 1) / kSolveWarps, kSolveWarps * 32, solve_smem, s>>>(in, Gm, Z, Zb, N, l);
-      } else {
-        tri_inv_diag_kernel<<<l / kTriBlock, kTriBlock, 0, s>>>(Gm, l, Xinv);
-        trsolve_mma_kernel<<<(N + kTriRows - 1) / kTriRows, 256, tri_smem, s>>>(in, Gm, Xinv, Z, Zb, N, l);
-        ++launches;
-      }
-      count_launch(kFamClf, launches + 1);
+      gram_kernel<<<dim3((l / 64) * (l / 64 + 1) / 2, p.gram_split), 256, 0, s>>>(in, part, N, l, p.gram_rows);
+      double shift = kShift;
+      int n_part = p.gram_split;
+      GridSync sy{flags, flags + 12, flags + 10, kGridSpinLimit, 0u};
+      void* args[] = {&part, &n_part, &Gm, &Lf, &Iv, &W, &l, &shift, &chol_arrived, &sy};
+      cudaError_t e2 = launch_cooperative<chol_inverse_kernel>(chol_grid, kCholThreads, chol_smem, args, device, s);
+      if (e2 != cudaSuccess) return e2;
+      chol_arrived += (unsigned)chol_grid * (unsigned)(nbk + 1);       // barriers of one factorisation
+      tri_product_kernel<<<dim3((N + 63) / 64, l / 64), 256, 0, s>>>(in, W, out, Zb, N, l);
+      count_launch(kFamClf, 2);
+      float* t = in; in = out; out = t;
     }
     return cudaGetLastError();
   };
   for (int it = 0; it <= p.q && e == cudaSuccess; ++it) {
-    e = two_products();
-    if (e == cudaSuccess) e = cholqr(U, it == p.q ? 5 : 2);
+    e = product_y();
+    if (e == cudaSuccess) e = product_u();
+    if (e == cudaSuccess) e = cholqr(it == p.q ? 3 : 1);
   }
-  if (e == cudaSuccess) e = two_products();              // W = X Z and U' = X^T W for the Rayleigh-Ritz step
+  // Rayleigh-Ritz: W = X Z, M = W^T W (= Z^T X^T X Z), its eigenvectors by Jacobi
+  if (e == cudaSuccess) e = product_y();
+  if (e == cudaSuccess) e = launch_gemm<false, true>({Yt, l, T, p.Tp}, {Yt, l, T, p.Tp}, p.ritz_split, (float*)part, nullptr, l, flags, device, s);
   if (e == cudaSuccess) {
-    dgemm_tn_mma_kernel<float><<<g_ll, 256, 0, s>>>(Z, U, Mm, N, l, l, l);     // M = Z^T U', accumulated in fp64
-    symmetrize_kernel<<<(l * l + 255) / 256, 256, 0, s>>>(Mm, l);
-    {
-      int per_sm = 0, sms = 0;
-      e = ensure_dyn_smem<jacobi_block_kernel>(kJacobiSmem, device);
-      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_block_kernel, kJacobiThreads, kJacobiSmem);
-      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-      if (e == cudaSuccess && per_sm < 1) e = cudaErrorLaunchOutOfResources;
-      if (e == cudaSuccess) {
-        float* M2 = (float*)(w + p.off_m2);
-        float* Qm = (float*)(w + p.off_q);
-        float2* partial = (float2*)(w + p.off_cs);
-        const bool inject = (g_clf_inject.load(std::memory_order_relaxed) & XKV_INJECT_CLF_BARRIER) != 0u;
-        GridSync sy{flags, flags + 8, flags + 10,                         // zeroed with the flag block above
-                    inject ? 1024u : kJacobiSpinLimit, inject ? 1u : 0u};
-        int l_arg = l;
-        void* args[] = {&Mm, &M2, &Pm, &Qm, &l_arg, &partial, &sy};
-        e = cudaLaunchCooperativeKernel((const void*)jacobi_block_kernel, dim3(sms), dim3(kJacobiThreads), args, kJacobiSmem, s);
-        count_launch(kFamClf, 1);
-      }
-    }
-    if (e == cudaSuccess) {
-      eig_select_kernel<<<1, 1024, (size_t)l * sizeof(int), s>>>(Mm, Pm, l, r, Ps, sigma);
-      sgemm_small_kernel<false, float><<<dim3((r + 63) / 64, (N + 63) / 64), 256, 0, s>>>(Z, Ps, V, N, r, l, l, r, r);
-      const long long tot = (long long)N * r;
-      clf_finish_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(V, c->G, c->d, r, Vb, (__nv_bfloat16*)B_out);
-      count_launch(kFamClf, 5);
-      e = cudaGetLastError();
-    }
+    symmetrize_kernel<<<(l * l + 255) / 256, 256, 0, s>>>((const float*)part, p.ritz_split, Mm, l);
+    float* M2 = (float*)(w + p.off_m2);
+    float* Qm = (float*)(w + p.off_q);
+    float2* partial = (float2*)(w + p.off_cs);
+    const bool inject = (g_clf_inject.load(std::memory_order_relaxed) & XKV_INJECT_CLF_BARRIER) != 0u;
+    GridSync sy{flags, flags + 8, flags + 10, inject ? 1024u : kGridSpinLimit, inject ? 1u : 0u};   // zeroed with the flag block above
+    unsigned arrived = 0;
+    void* args[] = {&Mm, &M2, &Pm, &Qm, &l, &partial, &arrived, &sy};
+    e = launch_cooperative<jacobi_block_kernel>(sms, kJacobiThreads, kJacobiSmem, args, device, s);
+  }
+  if (e == cudaSuccess) {
+    eig_select_kernel<<<(l + kSelectWarps - 1) / kSelectWarps, kSelectWarps * 32, 0, s>>>(Mm, Pm, l, r, Ps, sigma);
+    ritz_vectors_kernel<<<dim3((r + 63) / 64, N / 64), 256, 0, s>>>(Z, Ps, l, r, c->d, Vb, (__nv_bfloat16*)B_out);
+    count_launch(kFamClf, 3);
+    e = cudaGetLastError();
   }
   // A = X V_bf16, stored [T][r]
-  if (e == cudaSuccess) e = launch_gemm<true>(Vb, N, r, r, X, T, N, N, nullptr, (__nv_bfloat16*)A_out, r, flags, device, s);
+  if (e == cudaSuccess) e = launch_gemm<true, false>({Vb, N, r, r}, {X, T, N, N}, 1, nullptr, (__nv_bfloat16*)A_out, r, flags, device, s);
   if (e != cudaSuccess) { set_cuda_error(e); (void)cudaGetLastError(); return XKV_ERR_CUDA; }
   return XKV_OK;
 }
