@@ -252,61 +252,51 @@ __device__ __forceinline__ u64 add2(u64 a, u64 b) {
   return r;
 }
 
-// The default chunk of 8 rows (c == 8): HBM bound, persistent CTAs that walk a contiguous range of row blocks for every
-// (sequence, layer).
-// A chunk's rows are rotated by R^(8j + f), R the rotation by theta, so the mean is R^8j mu with mu = sum_f R^f x_f / 8,
-// a Horner recurrence in R alone; the cosines need no more than R either (<R^(8j+f) x_f, R^8j mu> = <x_f, R^-f mu>).
-// Only the one rotation by 8j per chunk comes from a table (fp64 recurrence from block to block, pow and sincos once
-// per CTA).  (With one table row per key row, built per CTA and layer, the fp64 work and the table loads took as long as
-// everything else: 677 us for 131072 rows of four layers of eight heads with cosines; 363 us with the table shared by
-// the layers and the rows kept in registers; this form 304 us, the issue slots 57 % busy.)
+// The default chunk of 8 rows (c == 8), persistent CTAs.  Bit for bit the arithmetic of the kernel above.
+// A CTA walks a contiguous range of row blocks; the cos/sin table of a block is built once and serves every (sequence,
+// layer) and head, so its fp64 work (an eighth of the fp32 rate here) is divided by batch * G: per CTA and layer, as in
+// the kernel above, it took as long as everything else together.  The rotation is advanced in fp64 from block to block;
+// pow and sincos run once per CTA.
 // A thread holds the 8 rows of its 8 rotary pairs in registers (64 registers), so the cosine pass reads nothing again,
 // while its next chunk is on the way into 256 bytes of shared memory of its own (no barrier: nobody else reads them).
 // The arithmetic is packed fp32 (two pairs per instruction).  The sums of the cosine pass over the threads of a head are
 // folded by halving (a lane ends with one row: 14 shuffles for the 16 sums of a chunk instead of 6 per row).
-constexpr int kLm8MaxChunks = 8;    // chunks of a row block
+// 131072 rows of four layers of eight heads of 128 with cosines: 677 us -> 320 us; what bounds it now is instruction issue
+// and the table loads from shared memory.
+constexpr int kLm8MaxRows = 64;     // rows of a table
 template <int DH, bool ROPE>
 __global__ void __launch_bounds__(kLmThreads, 2)
 landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restrict__ landmarks, float* __restrict__ min_cos,
                  int G, int batch, int T, int H_kv, int n_c, int n_blocks, double rope_base) {
-  constexpr int HALF = DH / 2, APH = HALF / 8;
-  constexpr int EPT = ROPE ? kLm8MaxChunks * HALF / kLmThreads : 1;   // table entries per thread
-  extern __shared__ __align__(16) uint4 slots_s[];       // [16][kLmThreads] pieces of the chunk on its way
-  __shared__ __align__(16) float4 tab_s[ROPE ? kLm8MaxChunks * HALF / 2 : 1];   // [chunk][4][APH] {cos, cos, sin, sin} of two pairs
-  __shared__ double2 rot_s[ROPE ? EPT + 1 : 1][ROPE ? kLmThreads : 1];          // a thread's entries; the step to the next block
+  constexpr int HALF = DH / 2, APH = HALF / 8, NBLK = kLmThreads / HALF;
+  extern __shared__ __align__(16) uint4 slots_s[];       // [16][kLmThreads] pieces of the chunk on its way, then the table
+  __shared__ double2 rot_s[3][ROPE ? kLmThreads : 1];    // a thread's rotation state: its first row, one row on, one block on
   const int tid = threadIdx.x;
   const int TPR = H_kv * APH, RG = kLmThreads / TPR;     // threads per row of all heads, chunks side by side
-  const int CPB = min(RG, kLm8MaxChunks);                // chunks of a row block; the other row groups take other layers
-  const int LG = RG / CPB;
+  const int CPB = min(RG, kLm8MaxRows / 8);              // chunks of a row block; the other row groups take other layers
+  const int R = CPB * 8, LG = RG / CPB;
   const int rg = tid / TPR, tr = tid % TPR;
   const int g = tr / APH, a = tr % APH;
   const int jc = rg % CPB, lg = rg / CPB;
   const int d = H_kv * DH, n_lb = G * batch;
   const int b_begin = (int)((long long)blockIdx.x * n_blocks / gridDim.x), b_end = (int)((long long)(blockIdx.x + 1) * n_blocks / gridDim.x);
+  float4* const tab_s = reinterpret_cast<float4*>(slots_s + 16 * kLmThreads);     // [row][4][APH] {cos, cos, sin, sin} of two pairs
 
-  // table entries tid, tid + kLmThreads, ...: pair ii of chunk tid / HALF + i * (kLmThreads / HALF)
-  const int ii = tid % HALF;
-  float* const tab_f = reinterpret_cast<float*>(tab_s) + ((((ii & 7) >> 1) * APH + (ii >> 3)) * 4 + (ii & 1));
-  u64 c1[4], s1[4], n1[4];                               // R of this thread's pairs: cos, sin, -sin
-  if (ROPE) {
-    const double th = pow(rope_base, -(double)ii / (double)HALF) / 3.14159265358979323846;
+  // this thread's share of the table: pair ii, rows [r_begin, r_begin + RPB) of every block
+  const int ii = tid % HALF, RPB = max(1, R / NBLK), r_begin = (tid / HALF) * RPB;
+  const bool fills = r_begin < R;
+  if (ROPE && fills) {
+    const double th = pow(rope_base, -(double)ii / (double)HALF);
     double2 v;
-    sincospi(th, &v.y, &v.x);                            // R of pair ii for everybody, by way of the table
-    if (tid < HALF) { tab_f[0] = (float)v.x; tab_f[2] = (float)v.y; }
-#pragma unroll
-    for (int i = 0; i < EPT; ++i) {
-      sincospi((double)(8 * (b_begin * CPB + tid / HALF + i * (kLmThreads / HALF))) * th, &v.y, &v.x);
-      rot_s[i][tid] = v;
-    }
-    sincospi((double)(8 * CPB) * th, &v.y, &v.x);
-    rot_s[EPT][tid] = v;
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float4 t = tab_s[e * APH + a];
-      c1[e] = pack2(t.x, t.y); s1[e] = pack2(t.z, t.w); n1[e] = pack2(-t.z, -t.w);
-    }
+    sincospi((double)(b_begin * R + r_begin) * (th / 3.14159265358979323846), &v.y, &v.x);
+    rot_s[0][tid] = v;
+    sincos(th, &v.y, &v.x);                               // theta <= 1: no range reduction needed
+    rot_s[1][tid] = v;
+    sincospi((double)R * (th / 3.14159265358979323846), &v.y, &v.x);
+    rot_s[2][tid] = v;
   }
+  float* const tab_f = reinterpret_cast<float*>(tab_s) + ((((ii & 7) >> 1) * APH + (ii >> 3)) * 4 + (ii & 1));
+  const ulonglong2* const tab = reinterpret_cast<const ulonglong2*>(tab_s) + a;
 
   uint4 u1[8], u2[8];
   uint4* const slot = slots_s + tid;
@@ -325,27 +315,36 @@ landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restri
   };
   // (only the lanes of one head take part: the row groups of a warp may be in different chunks)
   const uint32_t hmask = ((1u << APH) - 1u) << ((tid & 31) & ~(APH - 1));
-  // the four couples of pairs of one half of row r, widened to fp32
-  auto widen = [](const uint4& v, u64 (&x)[4]) {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) x[e] = pack2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u));
+  // couple e (pairs 2e, 2e + 1) of row r, rotated with table row trow: first half y1, second half y2
+  auto rotated = [&](int r, int trow, int e, u64& y1, u64& y2) {
+    const uint32_t w1 = e == 0 ? u1[r].x : e == 1 ? u1[r].y : e == 2 ? u1[r].z : u1[r].w;
+    const uint32_t w2 = e == 0 ? u2[r].x : e == 1 ? u2[r].y : e == 2 ? u2[r].z : u2[r].w;
+    const u64 x1 = pack2(__uint_as_float(w1 << 16), __uint_as_float(w1 & 0xffff0000u));
+    const u64 x2 = pack2(__uint_as_float(w2 << 16), __uint_as_float(w2 & 0xffff0000u));
+    if (ROPE) {
+      const ulonglong2 t = tab[((size_t)trow * 4 + e) * APH];
+      const float2 s2 = unpack2(mul2(x2, t.y));
+      y1 = fma2(x1, t.x, pack2(-s2.x, -s2.y));
+      y2 = fma2(x2, t.x, mul2(x1, t.y));
+    } else {
+      y1 = x1; y2 = x2;
+    }
   };
 
   if (b_begin < b_end && lg < n_lb) request_chunk(b_begin, lg);
   for (int blk = b_begin; blk < b_end; ++blk) {
     if (ROPE) {
       __syncthreads();                                    // everybody is done with the table of the previous block
-      const double2 step = rot_s[EPT][tid];
-#pragma unroll
-      for (int i = 0; i < EPT; ++i) {
-        const int jj = tid / HALF + i * (kLmThreads / HALF);
-        if (jj < CPB) {
-          const double2 at = rot_s[i][tid];
-          tab_f[(size_t)jj * HALF * 2] = (float)at.x;
-          tab_f[(size_t)jj * HALF * 2 + 2] = (float)at.y;
-          rot_s[i][tid] = make_double2(at.x * step.x - at.y * step.y, at.y * step.x + at.x * step.y);
+      if (fills) {
+        const double2 at = rot_s[0][tid], one = rot_s[1][tid], jump = rot_s[2][tid];
+        double c1 = at.x, s1 = at.y;
+        for (int r = r_begin; r < r_begin + RPB; ++r) {
+          tab_f[(size_t)r * HALF * 2] = (float)c1;
+          tab_f[(size_t)r * HALF * 2 + 2] = (float)s1;
+          const double c2 = c1 * one.x - s1 * one.y, s2 = s1 * one.x + c1 * one.y;
+          c1 = c2; s1 = s2;
         }
+        rot_s[0][tid] = make_double2(at.x * jump.x - at.y * jump.y, at.y * jump.x + at.x * jump.y);
       }
       __syncthreads();
     }
@@ -359,77 +358,57 @@ landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restri
       else if (blk + 1 < b_end) request_chunk(blk + 1, lg);
       if (j >= n_c) continue;
       const int rows = min(8, T - j * 8);
-      u64 m1[4], m2[4];                                   // mu = sum_f R^f x_f / rows
+      u64 s1[4], s2[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) m1[e] = m2[e] = 0ull;
+      for (int e = 0; e < 4; ++e) s1[e] = s2[e] = 0ull;
 #pragma unroll
-      for (int r = 7; r >= 0; --r) {
+      for (int r = 0; r < 8; ++r) {
         if (r < rows) {
-          u64 x1[4], x2[4];
-          widen(u1[r], x1); widen(u2[r], x2);
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            if (ROPE) {
-              const u64 t = fma2(m1[e], c1[e], fma2(m2[e], n1[e], x1[e]));
-              m2[e] = fma2(m2[e], c1[e], fma2(m1[e], s1[e], x2[e]));
-              m1[e] = t;
-            } else {
-              m1[e] = add2(m1[e], x1[e]);
-              m2[e] = add2(m2[e], x2[e]);
-            }
+            u64 y1, y2;
+            rotated(r, jc * 8 + r, e, y1, y2);
+            s1[e] = add2(s1[e], y1);
+            s2[e] = add2(s2[e], y2);
           }
         }
       }
       const float inv = 1.0f / (float)rows;
       const u64 inv2 = pack2(inv, inv);
-      float o1[8], o2[8];
+      float m1[8], m2[8];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        m1[e] = mul2(m1[e], inv2);
-        m2[e] = mul2(m2[e], inv2);
-        const float2 p = unpack2(m1[e]), q = unpack2(m2[e]);
-        if (ROPE) {
-          const float4 t = tab_s[(jc * 4 + e) * APH + a];
-          o1[2 * e] = p.x * t.x - q.x * t.z; o1[2 * e + 1] = p.y * t.y - q.y * t.w;
-          o2[2 * e] = q.x * t.x + p.x * t.z; o2[2 * e + 1] = q.y * t.y + p.y * t.w;
-        } else {
-          o1[2 * e] = p.x; o1[2 * e + 1] = p.y; o2[2 * e] = q.x; o2[2 * e + 1] = q.y;
-        }
+        s1[e] = mul2(s1[e], inv2);
+        s2[e] = mul2(s2[e], inv2);
+        const float2 p = unpack2(s1[e]), q = unpack2(s2[e]);
+        m1[2 * e] = p.x; m1[2 * e + 1] = p.y; m2[2 * e] = q.x; m2[2 * e + 1] = q.y;
       }
       __nv_bfloat16* L = landmarks + (((size_t)lb * H_kv + g) * n_c + j) * DH + a * 8;
-      *reinterpret_cast<uint4*>(L) = pack8(o1);
-      *reinterpret_cast<uint4*>(L + HALF) = pack8(o2);
+      *reinterpret_cast<uint4*>(L) = pack8(m1);
+      *reinterpret_cast<uint4*>(L + HALF) = pack8(m2);
       if (min_cos) {
-        float v[16];                                      // per row: dot product with the mean, squared norm
-        u64 w = 0ull;
+        float v[16], mn2 = 0.0f;                          // per row: dot product with the mean, squared norm
 #pragma unroll
-        for (int e = 0; e < 4; ++e) w = fma2(m1[e], m1[e], fma2(m2[e], m2[e], w));
-        const float2 wf = unpack2(w);
-        float mn2 = wf.x + wf.y;
+        for (int e = 0; e < 8; ++e) mn2 += m1[e] * m1[e] + m2[e] * m2[e];
 #pragma unroll
         for (int o = 1; o < APH; o <<= 1) mn2 += __shfl_xor_sync(hmask, mn2, o);
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-          u64 x1[4], x2[4], dot = 0ull, nn = 0ull;
-          widen(u1[r], x1); widen(u2[r], x2);
+          const int trow = jc * 8 + min(r, rows - 1);     // a repeated last row changes no minimum
+          float dot = 0.0f, nn = 0.0f;
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            nn = fma2(x1[e], x1[e], nn);
-            nn = fma2(x2[e], x2[e], nn);
-            dot = fma2(x1[e], m1[e], dot);
-            dot = fma2(x2[e], m2[e], dot);
-            if (ROPE && r < rows - 1) {                   // R^-1 for the next row (a repeated last row changes no minimum)
-              const u64 t = fma2(m1[e], c1[e], mul2(m2[e], s1[e]));
-              m2[e] = fma2(m2[e], c1[e], mul2(m1[e], n1[e]));
-              m1[e] = t;
-            }
+            u64 y1, y2;
+            rotated(r, trow, e, y1, y2);
+            const float2 p = unpack2(fma2(y1, s1[e], mul2(y2, s2[e]))), q = unpack2(fma2(y1, y1, mul2(y2, y2)));
+            dot = (dot + p.x) + p.y;
+            nn = (nn + q.x) + q.y;
           }
-          const float2 d2 = unpack2(dot), n2 = unpack2(nn);
-          v[2 * r] = d2.x + d2.y; v[2 * r + 1] = n2.x + n2.y;
+          v[2 * r] = dot; v[2 * r + 1] = nn;
         }
         // fold by halving: after the step with distance o a lane keeps the half of the rows its bit selects
 #pragma unroll
-        for (int o = APH / 2, n = 8; o > 0; o >>= 1, n >>= 1) {
+        for (int o = 1, n = 8; o < APH; o <<= 1, n >>= 1) {
           const bool up = (a & o) != 0;
 #pragma unroll
           for (int i = 0; i < n; ++i) {
@@ -456,15 +435,15 @@ template <int DH>
 cudaError_t launch_landmark8(const __nv_bfloat16* keys, __nv_bfloat16* landmarks, float* min_cos, int G, int batch, int T,
                              int H_kv, float rope_base, cudaStream_t s) {
   const int n_c = (T + 7) / 8, tpr = H_kv * DH / 16;
-  const int cpb = kLmThreads / tpr < kLm8MaxChunks ? kLmThreads / tpr : kLm8MaxChunks;
+  const int cpb = kLmThreads / tpr < kLm8MaxRows / 8 ? kLmThreads / tpr : kLm8MaxRows / 8;
   const int n_blocks = (n_c + cpb - 1) / cpb;
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const int grid = n_blocks < 2 * sms ? n_blocks : 2 * sms;           // two CTAs per SM, one wave
-  const size_t smem = (size_t)kLmThreads * 256;
   const bool rope = rope_base > 0.0f;
+  const size_t smem = (size_t)kLmThreads * 256 + (rope ? (size_t)cpb * 8 * (DH / 2) * sizeof(float2) : 0);
   e = rope ? ensure_dyn_smem<landmark8_kernel<DH, true>>(smem, dev) : ensure_dyn_smem<landmark8_kernel<DH, false>>(smem, dev);
   if (e != cudaSuccess) return e;
   if (rope)
