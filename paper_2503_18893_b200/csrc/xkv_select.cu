@@ -580,19 +580,29 @@ topk_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __restrict
 
 
 // ---------------------------------------------------------------------------------------------
-// The same selection for n_c <= 16384 chunks (one super-block), organised so that almost all of the work is done
-// on a short list instead of on every key.  Each thread holds 16 consecutive keys, split into GPT groups; the
-// k_ch-th largest of the group maxima is a lower bound P of the k_ch-th largest key (at least k_ch keys -- those
-// maxima -- are >= it), and with k_ch a few percent of n_c only a few percent of the keys pass it.  The keys >= P
-// go to a list in shared memory (key, chunk index); the exact k_ch-th largest key is then found on the list by
-// the radix select of topk_kernel; membership goes to a bitmap over the chunks (united with the head's outlier
-// chunks), whose prefix popcounts give the ascending output positions.  GPT = 0 disables the filter (P = the
-// smallest key): chosen by the host when there are fewer groups than k_ch.  ITEMS = 16 keys per thread serve
-// n_c <= 16384 chunks, ITEMS = 32 (keys read twice instead of held in registers) n_c <= 32768.  The result is
-// identical to topk_kernel's for every input; only the amount of work differs.
-// Bin (counted from the top) that holds the `need`-th largest of the keys counted in hist[0..kTopkBins), by a
-// suffix sum over the bins; thread t of the TH owns the kTopkBins / TH bins from t * (kTopkBins / TH).  Results in
-// sh[0] = bin, sh[1] = rank wanted inside the bin, sh[2] = keys in the bin.  Contains barriers: call it from all threads.
+// The same selection for n_c <= 32768 chunks, organised so that almost all of the work is done on a short list instead
+// of on every key.  Latency bound: one CTA per problem on an otherwise idle chip, a chain of barriers; what counts is
+// their number (eleven) and what lies between them.
+//   1  every thread's keys (16-byte loads side by side), the maximum of each of its GPT groups
+//   2  the k_ch-th largest group maximum, by one histogram, is a lower bound P of the k_ch-th largest key (at least k_ch
+//      keys -- those maxima -- are >= it), and with k_ch a few percent of n_c only a few percent of the keys pass it
+//   3  the keys >= P go to a list in shared memory (key, chunk index)
+//   4  a histogram over the list finds the bin of the k_ch-th largest key; keys of higher bins are taken
+//   5  the few keys of that bin are ranked against one another by (key, chunk index), which also settles ties: a warp
+//      per candidate, its lanes holding the candidates in registers
+//   6  membership is a bitmap over the chunks (united with the head's outlier chunks); its prefix popcounts give the
+//      ascending output positions
+// Bins of more than kTopkCand keys are subdivided; if all their keys are equal, the lowest chunk indices are taken from a
+// second bitmap.  GPT = 0 disables the filter (P = the smallest key): chosen by the host when there are fewer groups than
+// k_ch.  ITEMS = 16 keys per thread serve n_c <= 16384 chunks, ITEMS = 32 (keys read twice instead of held in registers)
+// n_c <= 32768.  The result is identical to topk_kernel's for every input.
+// (With consecutive keys per thread, extrema by shuffles, a thread per candidate and separate scans for ties and
+// positions, about 25 barriers: 32768 rows decoded layer by layer 129.4 us, 122.4 us with this form; 121873 rows 212.6 ->
+// 193.6; 2048 rows 19.3 -> 17.6.)
+
+// Bin (counted from the top) that holds the `need`-th largest of the keys counted in hist[0..kTopkBins), by a suffix sum
+// over the bins; thread t of the TH owns the kTopkBins / TH bins from t * (kTopkBins / TH).  Results in sh[0] = bin,
+// sh[1] = rank wanted inside the bin, sh[2] = keys in the bin.  Contains barriers: call it from all threads.
 template <int TH>
 __device__ __forceinline__ void find_bin(const uint32_t* hist, uint32_t need, uint32_t* warp_tot, uint32_t* sh, int tid) {
   constexpr int BPT = kTopkBins / TH, NWARP = TH / 32;
@@ -602,32 +612,26 @@ __device__ __forceinline__ void find_bin(const uint32_t* hist, uint32_t need, ui
   uint32_t mine = 0;
 #pragma unroll
   for (int i = 0; i < BPT; ++i) { h[i] = hist[BPT * tid + i]; mine += h[i]; }
-  uint32_t suf = mine;                                     // inclusive over higher lanes of the warp
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t v = __shfl_down_sync(0xffffffffu, suf, o);
-    if (lane + o < 32) suf += v;
-  }
-  if (lane == 0) warp_tot[warp] = suf;
+  const uint32_t wsum = __reduce_add_sync(0xffffffffu, mine);
+  if (lane == 0) warp_tot[warp] = wsum;
   __syncthreads();
-  if (warp == 0) {
-    const uint32_t t = lane < NWARP ? warp_tot[lane] : 0u;
-    uint32_t ws = t;                                       // inclusive over higher warps
+  // every warp works out which warp owns the bin; that warp goes on
+  const uint32_t t = lane < NWARP ? warp_tot[lane] : 0u;
+  const uint32_t higher = __reduce_add_sync(0xffffffffu, lane > warp ? t : 0u);     // keys in bins of higher warps
+  if (higher < need && higher + wsum >= need) {
+    uint32_t suf = mine;                                   // inclusive over higher lanes of the warp
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t v = __shfl_down_sync(0xffffffffu, ws, o);
-      if (lane + o < 32) ws += v;
+      const uint32_t v = __shfl_down_sync(0xffffffffu, suf, o);
+      if (lane + o < 32) suf += v;
     }
-    if (lane < NWARP) warp_tot[lane] = ws - t;             // keys in bins of higher warps
-  }
-  __syncthreads();
-  const uint32_t above = warp_tot[warp] + (suf - mine);    // keys in bins above this thread's
-  if (above < need && above + mine >= need) {              // exactly one thread
-    uint32_t acc = above;
+    uint32_t acc = higher + suf - mine;                    // keys in bins above this thread's
+    if (acc < need && acc + mine >= need) {                // exactly one thread
 #pragma unroll
-    for (int i = BPT - 1; i >= 0; --i) {
-      if (acc < need && acc + h[i] >= need) { sh[0] = (uint32_t)(BPT * tid + i); sh[1] = need - acc; sh[2] = h[i]; }
-      acc += h[i];
+      for (int i = BPT - 1; i >= 0; --i) {
+        if (acc < need && acc + h[i] >= need) { sh[0] = (uint32_t)(BPT * tid + i); sh[1] = need - acc; sh[2] = h[i]; }
+        acc += h[i];
+      }
     }
   }
   __syncthreads();
@@ -639,180 +643,179 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
                   int32_t* __restrict__ sel_idx, int32_t* __restrict__ sel_cnt) {
   extern __shared__ __align__(16) uint8_t pivot_smem[];
   constexpr int kPivotListMax = TH * ITEMS;                              // every key may pass (all keys equal)
-  static_assert(kPivotListMax <= 65536 && kPivotListMax / 32 <= TH, "16-bit chunk index, one bitmap word per thread");
+  constexpr int NW = kPivotListMax / 32;                                 // words of a bitmap
+  static_assert(kPivotListMax <= 65536 && NW <= TH, "16-bit chunk index, one bitmap word per thread");
   uint32_t* list_key = reinterpret_cast<uint32_t*>(pivot_smem);                    // [kPivotListMax]; later the chunk list
   uint16_t* list_idx = reinterpret_cast<uint16_t*>(list_key + kPivotListMax);      // [kPivotListMax]
-  __shared__ __align__(16) uint32_t hist[kTopkBins];
-  __shared__ uint32_t take_w[kPivotListMax / 32], eq_w[kPivotListMax / 32];        // bitmaps over the chunks
-  __shared__ uint32_t warp_tot[TH / 32];
+  __shared__ __align__(16) uint32_t hist0[kTopkBins], hist1[kTopkBins];
+  __shared__ uint32_t take_w[NW], eq_w[NW];                                        // bitmaps over the chunks
+  __shared__ uint32_t warp_tot[TH / 32], warp_eq[TH / 32];
   __shared__ uint32_t warp_min[TH / 32], warp_max[TH / 32];
-  __shared__ uint32_t sh[4];
-  __shared__ uint32_t sh_n;
+  __shared__ unsigned long long cand_s[kTopkCand];                                 // (key, ~chunk index): larger = earlier
+  __shared__ uint32_t sh[3];
+  __shared__ uint32_t sh_n, sh_cand;
 
   constexpr int NWARP = TH / 32;
-  constexpr int kCand = kTopkCand < TH ? kTopkCand : TH;      // every candidate is ranked by a thread of its own
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int per_layer = dev.batch * dev.H_kv;
   const long long prob = (long long)l0 * per_layer + blockIdx.x;     // [G][batch][H_kv] order
   const float* __restrict__ S = dev.pooled + prob * dev.n_c;
   int32_t* __restrict__ out = sel_idx + prob * k_cap;
   const int n_c = dev.n_c, c = dev.c, T = dev.T;
-  constexpr int NW = kPivotListMax / 32;                               // words of a bitmap
   constexpr int NG = GPT == 0 ? 1 : GPT;                               // group maxima kept per thread
-  constexpr int GS = ITEMS / NG;                                       // keys per group
+  const bool all = (k_ch >= n_c);
+  // chunk of this thread's key i: runs of four side by side where a row of scores starts on 16 bytes, else single ones
+  const bool vec = (n_c & 3) == 0;
+  auto chunk_of = [&](int i) { return vec ? (i >> 2) * (TH * 4) + tid * 4 + (i & 3) : i * TH + tid; };
 
+  for (int i = tid; i < kTopkBins; i += TH) { hist0[i] = 0; hist1[i] = 0; }
+  for (int w = tid; w < NW; w += TH) {
+    const int first = w * 32;
+    take_w[w] = !all ? 0u : first + 32 <= n_c ? 0xffffffffu : (first < n_c ? ((1u << (n_c - first)) - 1u) : 0u);
+    eq_w[w] = 0u;
+  }
+  if (tid == 0) { sh_n = 0; sh_cand = 0; sh[0] = sh[1] = sh[2] = 0; }
   grid_dependency_wait();                      // the pooled scores come from the kernel launched before
   grid_dependency_launch();
-  const int j0 = tid * ITEMS;
-  const bool all = (k_ch >= n_c);
-  uint32_t thr = 0, need_eq = 0;
-  for (int w = tid; w < NW; w += TH) { take_w[w] = 0u; eq_w[w] = 0u; }
-  if (tid == 0) sh_n = 0;
+  bool ties = false;                           // the bin of the k_ch-th largest key holds equal keys only, and many of them
+  uint32_t need = (uint32_t)k_ch;
   if (!all) {
     uint32_t key[ITEMS];
-    load_keys(S, j0, n_c, sign, key);
-    // ---- extrema of this thread's keys and of its groups
-    uint32_t kmin = 0xffffffffu, kmax = 0u;
-    uint32_t gmax[NG];
+    // sign == 0: the array already holds keys (the landmark scan writes them); else the key is that of sign * value
+    auto load = [&]() {
+      if (vec) {
 #pragma unroll
-    for (int g = 0; g < NG; ++g) gmax[g] = 0u;
-#pragma unroll
-    for (int i = 0; i < ITEMS; ++i) {
-      if (j0 + i < n_c) {
-        kmin = min(kmin, key[i]); kmax = max(kmax, key[i]);
-        if (GPT != 0) gmax[i / GS] = max(gmax[i / GS], key[i]);
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
-      kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
-    }
-    if (lane == 0) { warp_min[warp] = kmin; warp_max[warp] = kmax; }
-    for (int i = tid; i < kTopkBins; i += TH) hist[i] = 0;
-    __syncthreads();
-    kmin = lane < NWARP ? warp_min[lane] : 0xffffffffu; kmax = lane < NWARP ? warp_max[lane] : 0u;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
-      kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
-    }
-    // ---- pivot: lower edge of the bin that holds the k_ch-th largest group maximum
-    uint32_t P = kmin;
-    if (GPT != 0) {
-      const uint32_t span1 = kmax - kmin;
-      const int bits1 = 32 - __clz(span1);
-      const int sh1 = bits1 > 11 ? bits1 - 11 : 0;
-#pragma unroll
-      for (int g = 0; g < NG; ++g) {
-        if (j0 + g * GS < n_c) atomicAdd(&hist[(gmax[g] - kmin) >> sh1], 1u);    // the group has at least one key
-      }
-      __syncthreads();
-      find_bin<TH>(hist, (uint32_t)k_ch, warp_tot, sh, tid);
-      P = kmin + (sh[0] << sh1);
-      __syncthreads();
-    }
-    // ---- the keys >= P, with their chunk index, to the list (one shared-memory atomic per warp)
-    {
-      if (ITEMS > 16) load_keys(S, j0, n_c, sign, key);   // 32 keys are not held across the barriers above: read them again
-      uint32_t cm = 0;
-#pragma unroll
-      for (int i = 0; i < ITEMS; ++i) {
-        if (j0 + i < n_c && key[i] >= P) cm |= 1u << i;
-      }
-      const uint32_t mine_c = (uint32_t)__popc(cm);
-      if (__any_sync(0xffffffffu, cm != 0u)) {
-        uint32_t inc = mine_c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
-          if (lane >= o) inc += v;
+        for (int u = 0; u < ITEMS / 4; ++u) {
+          const int j = u * (TH * 4) + tid * 4;
+          const uint4 v = j < n_c ? __ldcg(reinterpret_cast<const uint4*>(S + j)) : make_uint4(0u, 0u, 0u, 0u);
+          key[4 * u] = v.x; key[4 * u + 1] = v.y; key[4 * u + 2] = v.z; key[4 * u + 3] = v.w;
         }
-        uint32_t wbase = 0;
-        if (lane == 31) wbase = atomicAdd(&sh_n, inc);
-        wbase = __shfl_sync(0xffffffffu, wbase, 31);
-        uint32_t at = wbase + inc - mine_c;
+      } else {
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
-          if ((cm >> i) & 1u) { list_key[at] = key[i]; list_idx[at] = (uint16_t)(j0 + i); ++at; }
+          const int j = i * TH + tid;
+          key[i] = j < n_c ? __float_as_uint(__ldcg(S + j)) : 0u;
+        }
+      }
+      if (sign != 0.0f) {
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) key[i] = chunk_of(i) < n_c ? score_key(__uint_as_float(key[i]) * sign) : 0u;
+      }
+    };
+    load();
+    // ---- 1: maxima of the groups that hold a chunk, and their range (keys beyond the last chunk are 0)
+    uint32_t gmax[NG], kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+      uint32_t m = 0u;
+#pragma unroll
+      for (int i = g * (ITEMS / NG); i < (g + 1) * (ITEMS / NG); ++i) m = max(m, key[i]);
+      gmax[g] = m;
+      kmax = max(kmax, m);
+      if (GPT != 0 && chunk_of(g * (ITEMS / NG)) < n_c) kmin = min(kmin, m);
+    }
+    if (GPT == 0) {
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) if (chunk_of(i) < n_c) kmin = min(kmin, key[i]);
+    }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) { warp_min[warp] = kmin; warp_max[warp] = kmax; }
+    __syncthreads();
+    kmin = __reduce_min_sync(0xffffffffu, lane < NWARP ? warp_min[lane] : 0xffffffffu);
+    kmax = __reduce_max_sync(0xffffffffu, lane < NWARP ? warp_max[lane] : 0u);
+    // ---- 2: pivot: lower edge of the bin that holds the k_ch-th largest group maximum
+    uint32_t P = kmin;
+    if (GPT != 0) {
+      const int bits1 = 32 - __clz(kmax - kmin);
+      const int sh1 = bits1 > 11 ? bits1 - 11 : 0;
+#pragma unroll
+      for (int g = 0; g < NG; ++g) if (chunk_of(g * (ITEMS / NG)) < n_c) atomicAdd(&hist0[(gmax[g] - kmin) >> sh1], 1u);
+      __syncthreads();
+      find_bin<TH>(hist0, (uint32_t)k_ch, warp_tot, sh, tid);
+      P = kmin + (sh[0] << sh1);
+    }
+    // ---- 3: the keys >= P, with their chunk index, to the list (one shared-memory atomic per warp)
+    {
+      if (ITEMS > 16) load();                              // 32 keys are not held across the barriers above: read them again
+      uint32_t cm = 0;
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) if (key[i] >= P && chunk_of(i) < n_c) cm |= 1u << i;
+      const uint32_t mine_c = (uint32_t)__popc(cm);
+      uint32_t inc = mine_c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+      }
+      uint32_t wbase = 0;
+      if (lane == 31 && inc != 0u) wbase = atomicAdd(&sh_n, inc);
+      uint32_t at = __shfl_sync(0xffffffffu, wbase, 31) + inc - mine_c;
+      if (cm != 0u) {
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+          if ((cm >> i) & 1u) { list_key[at] = key[i]; list_idx[at] = (uint16_t)chunk_of(i); ++at; }
         }
       }
     }
     __syncthreads();
     const int n_list = (int)sh_n;                                      // >= k_ch
-    // ---- radix select of the k_ch-th largest key on the list: bins subdivide the window [lo, lo + span]
-    uint32_t lo = P, span = kmax - P, need = (uint32_t)k_ch;
-    for (;;) {
+    // ---- 4: bins subdivide the window [lo, lo + span] that holds the k_ch-th largest key
+    uint32_t lo = P, span = kmax - P, in_bin;
+    for (bool again = false;; again = true) {
       const int bits = 32 - __clz(span);                               // span < 2^bits
       const int shb = bits > 11 ? bits - 11 : 0;
-      for (int i = tid; i < kTopkBins; i += TH) hist[i] = 0;
-      __syncthreads();
+      if (again) {
+        for (int i = tid; i < kTopkBins; i += TH) hist1[i] = 0;
+        __syncthreads();
+      }
       for (int e = tid; e < n_list; e += TH) {
         const uint32_t rel = list_key[e] - lo;                         // keys below lo wrap to huge values
-        if (rel <= span) atomicAdd(&hist[rel >> shb], 1u);
+        if (rel <= span) atomicAdd(&hist1[rel >> shb], 1u);
       }
       __syncthreads();
-      find_bin<TH>(hist, need, warp_tot, sh, tid);
-      const uint32_t bsel = sh[0], in_bin = sh[2];
+      find_bin<TH>(hist1, need, warp_tot, sh, tid);
+      const uint32_t bsel = sh[0];
       need = sh[1];
+      in_bin = sh[2];
       lo += bsel << shb;
       span = min(span - (bsel << shb), (shb ? (1u << shb) : 1u) - 1u);
-      __syncthreads();
-      if (shb == 0) { thr = lo; need_eq = need; break; }
-      if (in_bin <= (uint32_t)kCand) {
-        // few keys are left in the window: collect them and rank them against one another
-        uint32_t* cand = hist;
-        if (tid == 0) sh[3] = 0;
-        __syncthreads();
-        for (int e = tid; e < n_list; e += TH) {
-          const uint32_t kk = list_key[e];
-          if (kk - lo <= span) cand[atomicAdd(&sh[3], 1u)] = kk;
+      if (shb == 0 || in_bin <= (uint32_t)kTopkCand) break;
+      __syncthreads();                                                 // sh is read before the next pass writes it
+    }
+    ties = in_bin > (uint32_t)kTopkCand;
+    // ---- 5: keys above the bin are taken; the keys of the bin become candidates (or, all equal and many, a bitmap)
+    for (int e = tid; e < n_list; e += TH) {
+      const uint32_t kk = list_key[e], j = list_idx[e];
+      if (kk >= lo) {
+        if (kk - lo > span) atomicOr(&take_w[j >> 5], 1u << (j & 31u));
+        else if (ties) atomicOr(&eq_w[j >> 5], 1u << (j & 31u));
+        else {
+          const uint32_t at = atomicAdd(&sh_cand, 1u);
+          if (at < (uint32_t)kTopkCand) cand_s[at] = ((unsigned long long)kk << 32) | (0xffffffffu - j);
         }
-        __syncthreads();
-        const uint32_t n_cand = sh[3];                                 // == in_bin
-        __syncthreads();
-        if ((uint32_t)tid < n_cand) {
-          const uint32_t mykey = cand[tid];
-          uint32_t gt = 0, eq = 0;
-          const uint32_t n4 = n_cand & ~3u;
-          const uint4* c4 = reinterpret_cast<const uint4*>(cand);
-#pragma unroll 4
-          for (uint32_t i = 0; i < n4; i += 4) {
-            const uint4 v = c4[i >> 2];
-            gt += (v.x > mykey ? 1u : 0u) + (v.y > mykey ? 1u : 0u) + (v.z > mykey ? 1u : 0u) + (v.w > mykey ? 1u : 0u);
-            eq += (v.x == mykey ? 1u : 0u) + (v.y == mykey ? 1u : 0u) + (v.z == mykey ? 1u : 0u) + (v.w == mykey ? 1u : 0u);
-          }
-          for (uint32_t i = n4; i < n_cand; ++i) {
-            const uint32_t c2 = cand[i];
-            gt += c2 > mykey ? 1u : 0u;
-            eq += c2 == mykey ? 1u : 0u;
-          }
-          if (gt < need && need <= gt + eq) { sh[0] = mykey; sh[1] = need - gt; }   // equal keys write the same pair
-        }
-        __syncthreads();
-        thr = sh[0];
-        need_eq = sh[1];
-        __syncthreads();
-        break;
       }
     }
-    // ---- membership: keys above the threshold, and (separately) keys equal to it
-    for (int e = tid; e < n_list; e += TH) {
-      const uint32_t kk = list_key[e];
-      const uint32_t j = list_idx[e];
-      if (kk > thr) atomicOr(&take_w[j >> 5], 1u << (j & 31u));
-      else if (kk == thr) atomicOr(&eq_w[j >> 5], 1u << (j & 31u));
-    }
-  } else {
-    __syncthreads();                                                   // the bitmaps are zeroed
-    for (int w = tid; w < NW; w += TH) {
-      const int first = w * 32;
-      take_w[w] = first + 32 <= n_c ? 0xffffffffu : (first < n_c ? ((1u << (n_c - first)) - 1u) : 0u);
+    __syncthreads();
+    if (!ties && (uint32_t)warp < in_bin) {
+      constexpr int CL = kTopkCand / 32;
+      unsigned long long held[CL];                         // this lane's share of the candidates
+#pragma unroll
+      for (int i = 0; i < CL; ++i) held[i] = (uint32_t)(lane + 32 * i) < in_bin ? cand_s[lane + 32 * i] : 0ull;
+#pragma unroll 2
+      for (uint32_t e = (uint32_t)warp; e < in_bin; e += NWARP) {
+        const unsigned long long mine = cand_s[e];
+        uint32_t before = 0;
+#pragma unroll
+        for (int i = 0; i < CL; ++i) before += held[i] > mine ? 1u : 0u;
+        before = __reduce_add_sync(0xffffffffu, before);
+        const uint32_t j = 0xffffffffu - (uint32_t)mine;
+        if (lane == 0 && before < need) atomicOr(&take_w[j >> 5], 1u << (j & 31u));
+      }
     }
   }
   // Algorithm 2 line 5: the head's static outlier chunks join the set
   if (n_out > 0) {
-    __syncthreads();
     const int32_t* outl = outliers + (size_t)prob * (size_t)n_out;     // [G][batch][H_kv][n_out], like sel_idx
     for (int o = tid; o < n_out; o += TH) {
       const int jo = outl[o];
@@ -820,51 +823,35 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
     }
   }
   __syncthreads();
-  // ---- exclusive prefix over the CTA in thread order; the total goes to sh[3]
-  auto block_scan = [&](uint32_t mine) -> uint32_t {
+  // ---- 6: exclusive prefix over the CTA in thread order (thread w owns word w), and the total
+  auto block_scan = [&](uint32_t mine, uint32_t* tot, uint32_t& total) -> uint32_t {
     uint32_t inc = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
       if (lane >= o) inc += v;
     }
-    if (lane == 31) warp_tot[warp] = inc;
+    if (lane == 31) tot[warp] = inc;
     __syncthreads();
-    if (warp == 0) {
-      const uint32_t t = lane < NWARP ? warp_tot[lane] : 0u;
-      uint32_t ti = t;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, ti, o);
-        if (lane >= o) ti += v;
-      }
-      if (lane < NWARP) warp_tot[lane] = ti - t;
-      if (lane == 31) sh[3] = ti;
-    }
-    __syncthreads();
-    return inc - mine + warp_tot[warp];
+    const uint32_t t = lane < NWARP ? tot[lane] : 0u;
+    total = __reduce_add_sync(0xffffffffu, t);
+    return inc - mine + __reduce_add_sync(0xffffffffu, lane < warp ? t : 0u);
   };
-  // keys equal to the threshold: the need_eq with the lowest chunk index are taken (thread w owns word w)
-  static_assert(NW <= TH, "one bitmap word per thread");
   uint32_t fw = tid < NW ? take_w[tid] : 0u;
-  {
+  if (ties) {                                              // of the equal keys, the `need` with the lowest chunk index
     const uint32_t ew = tid < NW ? eq_w[tid] : 0u;
-    const uint32_t eq_before = block_scan((uint32_t)__popc(ew));
-    uint32_t room = need_eq > eq_before ? need_eq - eq_before : 0u;
+    uint32_t total;
+    const uint32_t eq_before = block_scan((uint32_t)__popc(ew), warp_eq, total);
+    uint32_t room = need > eq_before ? need - eq_before : 0u;
     uint32_t rest = ew;
     while (rest && room) { fw |= rest & (0u - rest); rest &= rest - 1u; --room; }   // lowest set bits first
-    __syncthreads();                                                   // sh[3] and warp_tot are reused below
   }
-  // ---- positions over the union, chunk ids to the chunk list (ascending), rows written by the whole CTA
-  const uint32_t before = block_scan((uint32_t)__popc(fw));
-  const uint32_t taken = sh[3];
-  {
-    uint32_t pos = before, rest = fw;
-    while (rest) {
-      list_key[pos++] = (uint32_t)(tid * 32 + __ffs(rest) - 1);
-      rest &= rest - 1u;
-    }
-  }
+  uint32_t taken;
+  uint32_t pos = block_scan((uint32_t)__popc(fw), warp_tot, taken);
+  // whole chunks unless the ragged last chunk was taken (it is then the last one)
+  if (tid == (n_c - 1) >> 5) sh[0] = (fw >> ((n_c - 1) & 31)) & 1u;
+  // chunk ids to the chunk list (ascending), rows written by the whole CTA
+  for (uint32_t rest = fw; rest; rest &= rest - 1u) list_key[pos++] = (uint32_t)(tid * 32 + __ffs(rest) - 1);
   __syncthreads();
   if (c == 8) {
     for (uint32_t w = (uint32_t)tid; w < taken * 8u; w += TH) {
@@ -878,9 +865,8 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
       if (row < T) out[w] = row;
     }
   }
-  // whole chunks unless the ragged last chunk was taken (it is then the last one)
   int cnt = (int)taken * c;
-  if (taken > 0 && list_key[taken - 1] == (uint32_t)(n_c - 1)) cnt -= (n_c * c - T);
+  if (sh[0]) cnt -= (n_c * c - T);
   for (int i = cnt + tid; i < k_cap; i += TH) out[i] = -1;
   if (tid == 0 && sel_cnt) sel_cnt[prob] = cnt;
 }
