@@ -12,10 +12,10 @@
 // so the rebuilt value rows are consumed in factored form and never materialised.  Rebuilt key rows live in
 // TMEM only.  Every gathered byte is written to shared memory once and read by the tensor core once.
 //
-// Warp roles: 0-3 key epilogue, 4-7 value epilogue, 8-9 gather producers of the key stream, 10-11 of the value
-// stream (cp.async of the selected rows of A_k / A_v into two rings of 16 KB slabs, one per stream), 12 MMA issue
-// for the key phases, 13 TMA loader of the B_k slabs (a short ring: they come from L2), 14 MMA issue for the value
-// phases.  The two streams are coupled only through the data: a value phase needs the weights that the key
+// Warp roles: 0-3 key epilogue, 4-7 value epilogue, then gather producers, half of them for the key stream and half for
+// the value stream (cp.async of the selected rows of A_k / A_v into two rings of 16 KB slabs, one per stream), then one
+// warp of MMA issue for the key phases, one TMA loader of the B_k slabs (a short ring: they come from L2) and one warp of
+// MMA issue for the value phases.  The two streams are coupled only through the data: a value phase needs the weights that the key
 // epilogue derives from the same tile's key phase.  Slots are released in pairs by tcgen05.commit; every barrier
 // has one producer side and waiters that see each of its phases in order, so that one parity bit per waiter is
 // enough.  Every wait is bounded; a wait that runs out raises XKV_FLAG_TIMEOUT and the CTA winds down.
@@ -41,7 +41,10 @@ using namespace ptx;
 constexpr int kTile = 128;                       // selected rows per tile
 constexpr int kSlabBytes = kTile * 128;          // 128 rows x 64 bf16 (one 128-byte swizzle row each)
 constexpr int kNB = 4;                           // slots of the B-slab ring
-constexpr int kThreads = 15 * 32;
+// Gather producers: four warps (two per stream) issue asynchronous copies; eight where the rows are dequantised on the way,
+// which is instruction work of the producers (4-bit bases at T = 131072, k = 4096: step 111.8 us with four, 93.7 with eight).
+constexpr int prod_warps(int quant) { return quant ? 8 : 4; }
+constexpr int fused_threads(int quant) { return (11 + prod_warps(quant)) * 32; }
 constexpr int kSmemLimit = 227 * 1024;
 constexpr int kRopeStride = 66;                  // float2 per staged rotary row (64 + pad against bank conflicts)
 constexpr int kPBytes = 2 * 16 * 128;            // softmax weights of a tile as a bf16 MMA operand: [2][16 heads][64 rows]
@@ -237,11 +240,13 @@ __host__ __device__ constexpr int ring_slots() {
 // QUANT = 4 or 3: the token bases are gathered from 4-bit or 3-bit codes (xkv_group_set_quantized_bases) and
 // dequantised by the producer warps on their way into the rings; 0: bf16 bases.
 template <int DH, int NR, int WB, bool PROF, int QUANT>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(fused_threads(QUANT), 1)
 sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched sc, const __nv_bfloat16* __restrict__ q,
                 const int32_t* __restrict__ sel_idx, const int32_t* __restrict__ sel_cnt) {
   extern __shared__ uint8_t smem_raw[];
   constexpr int HALF = DH / 2;
+  constexpr int kThreads = fused_threads(QUANT), PW = prod_warps(QUANT), SPT = PW * 16;   // SPT: producer threads per stream
+  constexpr int kWarpK = 8 + PW, kWarpB = kWarpK + 1, kWarpV = kWarpK + 2;                // key MMA, B loader, value MMA
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - smem_u32(smem_raw));
@@ -279,7 +284,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   const int nst_k = (nks_k + 1) & ~1, nst_v = (nks_v + 1) & ~1;
 
   if (tid == 0) {
-    for (int s = 0; s < S; ++s) { mbar_init(BAR(bl.full + s), 64); mbar_init(BAR(bl.fullv + s), 64); }   // 64 threads per stream
+    for (int s = 0; s < S; ++s) { mbar_init(BAR(bl.full + s), SPT); mbar_init(BAR(bl.fullv + s), SPT); }
     for (int s = 0; s < S / 2; ++s) { mbar_init(BAR(bl.emptyk + s), 1); mbar_init(BAR(bl.emptyv + s), 1); }
     for (int s = 0; s < kNB; ++s) mbar_init(BAR(bl.bfull + s), 1);
     for (int b = 0; b < 2; ++b) {
@@ -288,7 +293,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       mbar_init(BAR(bl.pfull + b), 128);
       mbar_init(BAR(bl.rfree + b), 128);
     }
-    for (int b = 0; b < 4; ++b) { mbar_init(BAR(bl.posfull + b), 64); mbar_init(BAR(bl.vfree + b), 64); }
+    for (int b = 0; b < 4; ++b) { mbar_init(BAR(bl.posfull + b), SPT); mbar_init(BAR(bl.vfree + b), SPT); }
     mbar_init(BAR(bl.grp), 128);
     mbar_init(BAR(bl.drain), 1); mbar_init(BAR(bl.drain + 1), 1);
     abort_flag[0] = 0;
@@ -301,7 +306,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   // weights of heads that do not exist stay zero for the whole kernel
   for (int i = tid; i < 2 * kPBytes / 4; i += kThreads) reinterpret_cast<uint32_t*>(P_gen)[i] = 0u;
   fence_proxy_async();
-  if (warp == 12) {
+  if (warp == kWarpK) {
     tmem_alloc(smem_u32(tmem_slot), 512);
     tmem_relinquish();
   }
@@ -363,7 +368,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     return dev.part + ((size_t)prob * sc.n_slots + seg) * (size_t)n_rep * (dev.r_v + 2);
   };
 
-  if (warp >= 8 && warp < 12) {
+  if (warp >= 8 && warp < kWarpK) {
     // =============================== producers: gather rows of A ===============================
     // Two independent streams with a ring of their own each: warps 8-9 gather the rows of A_k of every tile into
     // the key ring, warps 10-11 the same rows of A_v into the value ring.  A stream waits only for releases of its
@@ -372,12 +377,12 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     // last value slab of tile i, which itself waited for the last key MMA of tile i+1).
     // Eight consecutive lanes copy the eight 16-byte pieces of one 128-byte row slab, so that every request of a
     // warp covers whole 128-byte lines; thread t of a stream serves rows (t>>3) + 8*i, i = 0..15.
-    const bool kstream = warp < 10;
-    const int t64 = (tid - 256) & 63, pw = (warp - 8) & 1;
-    const uint32_t c8 = (uint32_t)(t64 & 7), r8 = (uint32_t)(t64 >> 3);
+    const bool kstream = warp < 8 + PW / 2;
+    const int ts = (tid - 256) & (SPT - 1), pw = (warp - 8) & (PW / 2 - 1);
+    const uint32_t c8 = (uint32_t)(ts & 7), r8 = (uint32_t)(ts >> 3);
     // rows r8 + 8*i share the swizzle phase r8; slab-relative destination of the i = 0 piece
     const uint32_t dst0 = r8 * 128u + ((c8 ^ r8) << 4);
-    const int ps = (warp == 8) ? 0 : (warp == 10 ? 48 : -1000);
+    const int ps = (warp == 8) ? 0 : (warp == 8 + PW / 2 ? 48 : -1000);
     const long long role_t0 = clock64();
     int slot = 0;                     // position in this stream's ring
     uint32_t used = 0, rel_par = 0;   // per slot pair: filled before; parity of the release to wait for next
@@ -423,24 +428,25 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     // The same phase from 4-bit codes.  Four consecutive lanes share a tile row: lane q4 fetches the 16 bytes of
     // codes and the scale/offset word of one 32-column group of the slot pair (64 contiguous bytes per row and
     // request), turns them into 32 bf16 values (packed arithmetic, one rounding) and stores them as four 16-byte
-    // units of the swizzled slab; a stream's 64 threads cover 16 rows per pass, 8 passes per pair.  The loads of a
+    // units of the swizzled slab; a stream's 128 threads cover 32 rows per pass, 4 passes per pair.  The loads of a
     // pair are issued before the wait for the pair's release, so their latency overlaps it.
-    const uint32_t q4 = (uint32_t)(t64 & 3), rq = (uint32_t)(t64 >> 2);
-    auto issue_phase_q = [&](const uint32_t (&rw)[8], int b) {
+    const uint32_t q4 = (uint32_t)(ts & 3), rq = (uint32_t)(ts >> 2);
+    constexpr int QP = 4;                                  // passes per slot pair
+    auto issue_phase_q = [&](const uint32_t (&rw)[QP], int b) {
       const uint8_t* Cb = (kstream ? dev.Aq_k : dev.Aq_v) + (size_t)b * dev.T * (size_t)(r >> 1);
       const uint32_t* Mb = (kstream ? dev.Am_k : dev.Am_v) + (size_t)b * dev.T * (size_t)(r >> 5);
       const uint32_t ring_q = base + (kstream ? 0u : (uint32_t)SK * kSlabBytes);
-      auto fetch = [&](int ks, uint4 (&cw)[8], uint32_t (&mw)[8]) {
+      auto fetch = [&](int ks, uint4 (&cw)[QP], uint32_t (&mw)[QP]) {
         const int col0 = ks * 64 + (int)q4 * 32;           // first column of this lane's group
         const bool in = col0 < r;                          // false in a padding slab: zeros are stored
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < QP; ++i) {
           // 4 bits: 16 bytes of codes and a separate scale/offset word; 3 bits: one 16-byte record {meta, w0, w1, w2}
           cw[i] = in ? __ldg(reinterpret_cast<const uint4*>(Cb + (size_t)rw[i] * (size_t)(r >> 1) + (col0 >> 1))) : make_uint4(0, 0, 0, 0);
           if (QUANT == 4) mw[i] = in ? __ldg(Mb + (size_t)rw[i] * (size_t)(r >> 5) + (col0 >> 5)) : 0u;
         }
       };
-      auto store = [&](const uint4 (&cw)[8], const uint32_t (&mw)[8]) -> bool {
+      auto store = [&](const uint4 (&cw)[QP], const uint32_t (&mw)[QP]) -> bool {
         const int pr = slot >> 1;
         const uint32_t bit = 1u << pr;
         if (used & bit) {             // wait for the release of the pair's previous occupant
@@ -452,8 +458,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
         const uint32_t st = ring_q + (uint32_t)(slot + (int)(q4 >> 1)) * kSlabBytes;
         const uint32_t u0 = (q4 & 1u) * 4u;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const uint32_t j = rq + 16u * (uint32_t)i;       // tile row
+        for (int i = 0; i < QP; ++i) {
+          const uint32_t j = rq + 32u * (uint32_t)i;       // tile row
           const uint32_t w[4] = {cw[i].x, cw[i].y, cw[i].z, cw[i].w};
           uint32_t o[16];
           if (QUANT == 4) {
@@ -470,26 +476,26 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
         }
         asm volatile("cp.async.wait_all;" ::: "memory");   // the staged rotary rows of this tile (key stream) have landed too
         fence_proxy_async();                               // the tensor core reads these stores
-        mbar_arrive(BAR(bar_full + slot));                 // both slabs of the pair are complete when all 64 threads are done
+        mbar_arrive(BAR(bar_full + slot));                 // both slabs of the pair are complete when all threads of the stream are done
         mbar_arrive(BAR(bar_full + slot + 1));
         slot += 2;
         if (slot == RS) slot = 0;
         return true;
       };
-      // (a second register set, so that the next pair's loads are in flight while this pair is converted, was
-      // measured and lost: 103 us against 85 us per call at the headline size)
-      uint4 ca[8];
-      uint32_t ma[8];
+      // (a second register set, so that the next pair's loads are in flight while this pair is converted, loses: step 98.2
+      // against 94.3 us at the headline size)
+      uint4 ca[QP];
+      uint32_t ma[QP];
 #pragma unroll 1
       for (int ks = 0; ks < nst; ks += 2) {
         fetch(ks, ca, ma);
         if (!store(ca, ma)) return;
       }
     };
-    auto load_rows_q = [&](uint32_t (&rw)[8]) {
+    auto load_rows_q = [&](uint32_t (&rw)[QP]) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int p = pos_s[pb * kTile + (int)rq + 16 * i];
+      for (int i = 0; i < QP; ++i) {
+        const int p = pos_s[pb * kTile + (int)rq + 32 * i];
         rw[i] = p < 0 ? 0u : (uint32_t)p;
       }
     };
@@ -501,7 +507,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       }
     };
     // One loop for both streams (one copy of the issue code).  The key stream also publishes the row positions and
-    // the coarse rotary rows of every tile: thread t loads the positions of tile rows t and t + 64, one tile ahead;
+    // the coarse rotary rows of every tile: thread t loads the positions of tile rows t, t + SPT, ..., one tile ahead;
     // the range check is made when the value is used, so that nobody waits for the load here.
     TileIter cur, nxt;
     iter_begin(nxt);
@@ -513,28 +519,34 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       if (x.ti * kTile + row < x.cnt && (p < 0 || p >= dev.T)) { atomicOr(dev.flags, XKV_FLAG_INDEX_RANGE); p = -1; }
       return p;
     };
-    int pn0 = -1, pn1 = -1;
-    if (kstream && have) { pn0 = load_pos(nxt, t64); pn1 = load_pos(nxt, t64 + 64); }
+    constexpr int PP = kTile / SPT;                        // positions per thread
+    int pn[PP];
+#pragma unroll
+    for (int i = 0; i < PP; ++i) pn[i] = kstream && have ? load_pos(nxt, ts + SPT * i) : -1;
     while (ok && have) {
       cur = nxt;
-      int pq[2] = {-1, -1};
-      if (kstream) { pq[0] = checked(cur, t64, pn0); pq[1] = checked(cur, t64 + 64, pn1); }
+      int pq[PP];
+#pragma unroll
+      for (int i = 0; i < PP; ++i) pq[i] = kstream ? checked(cur, ts + SPT * i, pn[i]) : -1;
       have = iter_next(nxt, no_op, no_op);
       if (kstream) {
-        if (have) { pn0 = load_pos(nxt, t64); pn1 = load_pos(nxt, t64 + 64); }
+        if (have) {
+#pragma unroll
+          for (int i = 0; i < PP; ++i) pn[i] = load_pos(nxt, ts + SPT * i);
+        }
         const int buf = it & 1;
         // the key epilogue must be done with this buffer's rotary rows (tile it-2), and the value stream with
         // the positions of tile it-4
         if (!wait_bar(ctx, BAR(bl.rfree + buf), (uint32_t)(((it >> 1) & 1) ^ 1), ps + 1)) { ok = false; break; }
         if (it >= 4 && !wait_bar(ctx, BAR(bl.vfree + pb), (uint32_t)(((it >> 2) & 1) ^ 1), ps + 1)) { ok = false; break; }
-        pos_s[pb * kTile + t64] = pq[0];
-        pos_s[pb * kTile + t64 + 64] = pq[1];
+#pragma unroll
+        for (int i = 0; i < PP; ++i) pos_s[pb * kTile + ts + SPT * i] = pq[i];
         if (rope_smem) {
           // rows 8a..8a+7 of the tile usually share one coarse rotary row (a landmark chunk): stage it once.
-          // Warp pw handles the 32-row blocks pw and pw + 2 (lane = row inside the block).
+          // Warp pw handles the 32-row blocks pw, pw + PW / 2, ... (lane = row inside the block).
 #pragma unroll
-          for (int hb = 0; hb < 2; ++hb) {
-            const int blk = pw + 2 * hb, p = pq[hb];
+          for (int hb = 0; hb < PP; ++hb) {
+            const int blk = pw + (PW / 2) * hb, p = pq[hb];
             const int hidx = p < 0 ? -1 : (p >> 3);
             int gmax = hidx;
             gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, 1));
@@ -559,7 +571,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       }
       if (!wait_bar(ctx, BAR(bl.posfull + pb), (uint32_t)((it >> 2) & 1), ps + 2)) { ok = false; break; }
       if constexpr (QUANT != 0) {
-        uint32_t rw[8];
+        uint32_t rw[QP];
         load_rows_q(rw);
         if (!kstream) mbar_arrive(BAR(bl.vfree + pb));     // this thread is done with the position buffer
         issue_phase_q(rw, cur.b);
@@ -573,15 +585,15 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       if (++pb == 4) pb = 0;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    if (ctx.prof && (warp == 8 || warp == 10) && lane == 0) {
+    if (ctx.prof && (warp == 8 || warp == 8 + PW / 2) && lane == 0) {
       ctx.prof[ps] = (unsigned long long)(clock64() - role_t0);
       if (warp == 8) ctx.prof[4] = (unsigned long long)it;
     }
-  } else if (warp == 12 || warp == 14) {
-    // =============================== MMA issue: warp 12 the key phases, warp 14 the value phases ===============
+  } else if (warp == kWarpK || warp == kWarpV) {
+    // =============================== MMA issue: one warp the key phases, one the value phases ===============
     // Two issuing threads, each walking its own ring (one thread spends 70-130 cycles per tcgen05.mma and about
     // 235 per tcgen05.commit).
-    const bool kside = warp == 12;
+    const bool kside = warp == kWarpK;
     // the whole warp walks the loop (all values are warp-uniform); one lane issues the tensor-core instructions
     constexpr uint32_t idesc_k = idesc_bf16_f32(128, 128);                     // keys: both operands K-major
     constexpr uint32_t idesc_v = idesc_bf16_f32(128, 16) | (1u << 15);         // values: A is read along its rows (MN-major)
@@ -693,7 +705,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       for (uint32_t i = 0; i < (1u << 22); ++i) if (mbar_try_wait(db, 0)) break;
     }
     __syncwarp();
-  } else if (warp == 13) {
+  } else if (warp == kWarpB) {
     // =============================== B_k slab loader (TMA) ===============================
     // B slab n goes to slot n % kNB, which held slab n - kNB.  That slab's MMAs are known to be complete
     //   - if it belongs to an earlier tile: when the previous tile's key accumulator was committed (kfull);
@@ -954,7 +966,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   asm volatile("cp.async.wait_all;" ::: "memory");
   tc_fence_before();
   __syncthreads();
-  if (warp == 12) {
+  if (warp == kWarpK) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
@@ -1307,19 +1319,19 @@ cudaError_t launch_fused_t(const xkv_group* grp, int l0, int l1, const __nv_bflo
     if (dev.Aq_k) return cudaErrorNotSupported;        // no diagnostic variant of the quantised gather
     e = ensure_dyn_smem<sr_fused_kernel<DH, NR, WB, true, 0>>(smem, grp->device);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(sr_fused_kernel<DH, NR, WB, true, 0>, dim3(sc.n_ctas), dim3(kThreads), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
+    e = launch_pdl(sr_fused_kernel<DH, NR, WB, true, 0>, dim3(sc.n_ctas), dim3(fused_threads(0)), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
   } else if (dev.Aq_k && dev.quant_bits == 3) {
     e = ensure_dyn_smem<sr_fused_kernel<DH, NR, WB, false, 3>>(smem, grp->device);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(sr_fused_kernel<DH, NR, WB, false, 3>, dim3(sc.n_ctas), dim3(kThreads), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
+    e = launch_pdl(sr_fused_kernel<DH, NR, WB, false, 3>, dim3(sc.n_ctas), dim3(fused_threads(3)), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
   } else if (dev.Aq_k) {
     e = ensure_dyn_smem<sr_fused_kernel<DH, NR, WB, false, 4>>(smem, grp->device);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(sr_fused_kernel<DH, NR, WB, false, 4>, dim3(sc.n_ctas), dim3(kThreads), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
+    e = launch_pdl(sr_fused_kernel<DH, NR, WB, false, 4>, dim3(sc.n_ctas), dim3(fused_threads(4)), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
   } else {
     e = ensure_dyn_smem<sr_fused_kernel<DH, NR, WB, false, 0>>(smem, grp->device);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(sr_fused_kernel<DH, NR, WB, false, 0>, dim3(sc.n_ctas), dim3(kThreads), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
+    e = launch_pdl(sr_fused_kernel<DH, NR, WB, false, 0>, dim3(sc.n_ctas), dim3(fused_threads(0)), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
   }
   count_launch(kFamFused);
   if (e != cudaSuccess) return e;
