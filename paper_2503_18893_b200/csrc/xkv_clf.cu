@@ -12,10 +12,11 @@
 // A = U Sigma and B = V^T of the truncated SVD of X, up to the accuracy of the subspace (checked against the exact
 // optimum sum_{i>r} sigma_i^2, never factor by factor: signs and degenerate subspaces are not unique).
 //
-// One tensor-core kernel serves the tall products.  It computes C (M x N) = A B^T for A given as [K][M]
-// row-major (an MN-major operand: the M index is contiguous) and B as [N][K] row-major (K-major), the two operand
-// forms the fused decode kernel already uses, so no matrix is ever transposed in memory:
-//   Y^T = Z-as-A (K = N_x)  x  X-as-B;     U = X-as-A (K = T)  x  Y^T-as-B;     A^T = V-as-A  x  X-as-B (stored transposed).
+// One tensor-core kernel serves the tall products.  It computes C (M x N) = A B with either operand K-major (its rows run
+// along k) or MN-major (its rows run along m or n), which the shared-memory descriptors cover, so no matrix is ever
+// transposed in memory:
+//   Y = X Z (X K-major, Z MN-major), stored transposed as Y^T;    U = X^T Y (X MN-major, Y^T K-major);
+//   M = W^T W (W^T K-major twice);                                 A = X V (X K-major, V MN-major).
 #include <cuda.h>
 #include <math.h>
 
@@ -28,13 +29,15 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kGemmThreads = 192;                 // warps 0-3 epilogue, 4 TMA producer, 5 MMA issue
-// One stage of the operand ring: A, two slabs of [64 k][64 m] (8 KB each), and B, [BN n][64 k] (BN * 128 bytes).
-// Tiles are 128 x BN with BN = 256, 192 or 128: an N = 128 step reads 8 KB of operands per 64 cycles, all the shared-
-// memory pipe gives, an N = 256 step 12 KB per 128 cycles.  Four stages for the wide tiles (one CTA per SM), three
-// for BN = 128 (two CTAs per SM, so that one's epilogue hides behind the other's products).
-template <int BN> constexpr int gemm_stage_bytes() { return 16384 + BN * 128; }
-template <int BN> constexpr int gemm_stages() { return BN == 128 ? 3 : 4; }
+// Tiles are (128 MB) x BN, MB accumulators of 128 rows in tensor memory sharing the B operand; one stage of the operand
+// ring holds 64 k.  What bounds the products is the rate at which L2 feeds the SMs (about 53 bytes per cycle and SM when
+// all of them ask): a 128 x 256 tile wants 96, a 256 x 192 tile 73 and a 256 x 256 tile 64 at the full rate of the tensor
+// core.  X Z at 131072 x 4096 x 576: 0.87 ms with 128 x 256 tiles, 0.50 with 256 x 192;
+// X^T Y 0.65 ms with 96 tiles of 128 x 192, 0.40 with 48 of 256 x 192 over three K ranges.
+constexpr int kGemmEpiWarps = 4;                  // per 128 rows; then one TMA producer warp, one MMA issue warp
+template <int MB> constexpr int gemm_threads() { return (MB * kGemmEpiWarps + 2) * 32; }
+template <int MB, int BN> constexpr int gemm_stage_bytes() { return MB * 16384 + BN * 128; }
+template <int MB, int BN> constexpr int gemm_stages() { return MB == 2 && BN == 256 ? 3 : MB == 1 && BN == 128 ? 3 : 4; }
 constexpr int kGemmMaxStages = 4;
 constexpr uint32_t kGemmWaitLimit = 1u << 24;
 
@@ -45,22 +48,23 @@ __device__ __forceinline__ bool gemm_wait(uint32_t bar, uint32_t parity) {
   return false;
 }
 
-// C[m][n] = sum_k A[k][m] B[n][k].  grid = (ceil(N/BN), ceil(M/128), K ranges).  TRANS: store C^T (out[n][m]).
-// AROW: A is given as [m][k] instead (K-major, like B).  K range z covers k_per columns and writes Cf + z * M * ldc.
-// Out-of-range rows and columns of the operands are zero-filled by the copy engine; stores are guarded.
-template <bool TRANS, bool AROW, int BN>
-__global__ void __launch_bounds__(kGemmThreads)
+// C[m][n] = sum_k A(k, m) B(k, n).  grid = (ceil(N/BN), ceil(M/(128 MB)), K ranges).  TRANS: store C^T (out[n][m]).
+// AK: A is given as [m][k] (K-major), else as [k][m]; BK likewise for B.  K range z covers k_per columns and writes
+// Cf + z * M * ldc.  Out-of-range rows and columns of the operands are zero-filled by the copy engine; stores are guarded.
+template <bool TRANS, bool AK, bool BK, int MB, int BN>
+__global__ void __launch_bounds__(gemm_threads<MB>(), 1)
 clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M, int N, int K,
                 int k_per, float* __restrict__ Cf, __nv_bfloat16* __restrict__ Cb, long long ldc, unsigned int* __restrict__ flags) {
   extern __shared__ uint8_t gemm_smem[];
-  constexpr int kGemmStages = gemm_stages<BN>(), kGemmStageBytes = gemm_stage_bytes<BN>();
-  constexpr uint32_t kCols = BN <= 128 ? 128u : 256u;      // tensor-memory columns (a power of two)
+  constexpr int kGemmStages = gemm_stages<MB, BN>(), kGemmStageBytes = gemm_stage_bytes<MB, BN>();
+  constexpr uint32_t kAccCols = BN <= 128 ? 128u : 256u, kCols = MB * kAccCols;      // tensor-memory columns
+  constexpr int kWarpLoad = MB * kGemmEpiWarps, kWarpMma = kWarpLoad + 1;
   __shared__ __align__(8) uint64_t bars[2 * kGemmMaxStages + 1];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_s;
   const uint32_t base = (smem_u32(gemm_smem) + 1023u) & ~1023u;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * 128;
+  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * (128 * MB);
   const int k_first = blockIdx.z * k_per, KB = (min(K - k_first, k_per) + 63) / 64;
   if (Cf) Cf += (size_t)blockIdx.z * M * ldc;
   const uint32_t bar0 = smem_u32(bars);
@@ -73,7 +77,7 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     abort_s = 0;
     fence_mbar_init();
   }
-  if (warp == 5) {
+  if (warp == kWarpMma) {
     tmem_alloc(smem_u32(&tmem_slot), kCols);
     tmem_relinquish();
   }
@@ -82,7 +86,8 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
   bool ok = true;
-  if (warp == 4) {
+  constexpr uint32_t kOffB = MB * 16384u;
+  if (warp == kWarpLoad) {
     if (lane == 0) {
       for (int kb = 0; kb < KB; ++kb) {
         const int s = kb % kGemmStages;
@@ -90,40 +95,50 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         const uint32_t st = base + (uint32_t)s * kGemmStageBytes;
         mbar_expect_tx(FULL(s), kGemmStageBytes);
         const int k = k_first + kb * 64;
-        if (AROW) {
-          tma_load_2d(st, &map_a, k, m0, FULL(s));                     // A: columns (k) k..k+63, rows m0..m0+127
+        // K-major: one box of 64 k by all rows; MN-major: slabs of 64 columns by 64 k, 8 KB each
+        if (AK) {
+          tma_load_2d(st, &map_a, k, m0, FULL(s));
         } else {
-          tma_load_2d(st, &map_a, m0, k, FULL(s));                     // A: columns m0..m0+63, rows (k) k..k+63
-          tma_load_2d(st + 8192, &map_a, m0 + 64, k, FULL(s));         //    columns m0+64..m0+127
+#pragma unroll
+          for (int i = 0; i < 2 * MB; ++i) tma_load_2d(st + i * 8192, &map_a, m0 + i * 64, k, FULL(s));
         }
-        tma_load_2d(st + 16384, &map_b, k, n0, FULL(s));               // B: columns (k) k..k+63, rows n0..n0+BN-1
+        if (BK) {
+          tma_load_2d(st + kOffB, &map_b, k, n0, FULL(s));
+        } else {
+#pragma unroll
+          for (int i = 0; i < BN / 64; ++i) tma_load_2d(st + kOffB + i * 8192, &map_b, n0 + i * 64, k, FULL(s));
+        }
       }
     }
-  } else if (warp == 5) {
+  } else if (warp == kWarpMma) {
     if (lane == 0) {
       const uint64_t desc_hi = smem_desc_sw128(0, 0) & 0xFFFFFFFF00000000ull;
-      constexpr uint32_t idesc = idesc_bf16_f32(128, BN) | (AROW ? 0u : 1u << 15);    // not AROW: A is read along its rows (MN-major)
+      constexpr uint32_t idesc = idesc_bf16_f32(128, BN) | (AK ? 0u : 1u << 15) | (BK ? 0u : 1u << 16);   // bits: MN-major
+      // MN-major: 64-column slabs 8192 bytes apart, 8-row groups (along k) 1024 bytes apart; 16 k are 2048 bytes.
+      // K-major: 16 k are 32 bytes along the rows.
+      constexpr uint32_t kSlab = (uint32_t)(8192 >> 4) << 16;
+      constexpr uint32_t a_step = AK ? 2u : (2048u >> 4), b_step = BK ? 2u : (2048u >> 4);
+      auto lo = [&](uint32_t at, bool kmajor) {
+        return kmajor ? (uint32_t)(smem_desc_sw128(at, 0) & 0xFFFFFFFFull) : ((at & 0x3FFFFu) >> 4) | kSlab;
+      };
       for (int kb = 0; kb < KB; ++kb) {
         const int s = kb % kGemmStages;
         if (!gemm_wait(FULL(s), (uint32_t)((kb / kGemmStages) & 1))) { ok = false; break; }
         tc_fence_after();
         const uint32_t st = base + (uint32_t)s * kGemmStageBytes;
-        // A: two 64-column slabs 8192 bytes apart, 8-row groups (along k) 1024 bytes apart; 16 k-rows per step
-        // (AROW: one slab of 128 rows, 32 bytes per step, like B)
-        const uint32_t a_lo = AROW ? (uint32_t)(smem_desc_sw128(st, 0) & 0xFFFFFFFFull)
-                                   : ((uint32_t)((st & 0x3FFFFu) >> 4)) | ((uint32_t)(8192 >> 4) << 16);
-        constexpr uint32_t a_step = AROW ? 2u : (2048u >> 4);
-        const uint32_t b_lo = (uint32_t)(smem_desc_sw128(st + 16384, 0) & 0xFFFFFFFFull);
+        const uint32_t b_lo = lo(st + kOffB, BK);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          tc_mma_bf16(tmem, desc_hi | (a_lo + (uint32_t)kk * a_step), desc_hi | (b_lo + 2u * (uint32_t)kk), idesc,
-                      (kb | kk) ? 1u : 0u);
+#pragma unroll
+          for (int mb = 0; mb < MB; ++mb)
+            tc_mma_bf16(tmem + (uint32_t)mb * kAccCols, desc_hi | (lo(st + mb * 16384u, AK) + (uint32_t)kk * a_step),
+                        desc_hi | (b_lo + (uint32_t)kk * b_step), idesc, (kb | kk) ? 1u : 0u);
         tc_commit(EMPTY(s));
       }
       tc_commit(ACC);
     }
   }
-  if (warp >= 4) {                  // a producer or issuer that gave up tells the epilogue not to wait for ever
+  if (warp >= kWarpLoad) {          // a producer or issuer that gave up tells the epilogue not to wait for ever
     if (!ok && lane == 0) { abort_s = 1; atomicOr(flags, XKV_FLAG_TIMEOUT); }
   } else {
     // ---- epilogue: thread = accumulator lane = row m0 + tid
@@ -135,7 +150,7 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     if (done) {
       tc_fence_after();
       const int m = m0 + tid;
-      const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+      const uint32_t lane_base = ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * kAccCols;
 #pragma unroll 1
       for (int cb = 0; cb < BN / 32; ++cb) {
         float v[32];
@@ -180,7 +195,7 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 5) {
+  if (warp == kWarpMma) {
     tc_fence_after();
     tmem_dealloc(tmem, kCols);
   }
@@ -969,6 +984,19 @@ ritz_vectors_kernel(const float* __restrict__ Z, const float* __restrict__ Ps, i
 
 namespace {
 
+// out = the sum of n_part arrays of n4 float4, in a fixed order.
+__global__ void __launch_bounds__(256)
+sum_parts_kernel(const float4* __restrict__ part, int n_part, long long n4, float4* __restrict__ out) {
+  const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (i >= n4) return;
+  float4 v = part[i];
+  for (int z = 1; z < n_part; ++z) {
+    const float4 u = part[(long long)z * n4 + i];
+    v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+  }
+  out[i] = v;
+}
+
 // M = (S + S^T) / 2 for the sum S of the partial products part [n_part][l][l], in a fixed order.
 __global__ void symmetrize_kernel(const float* __restrict__ part, int n_part, float* __restrict__ M, int l) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -982,10 +1010,13 @@ __global__ void symmetrize_kernel(const float* __restrict__ part, int n_part, fl
   M[(size_t)j * l + i] = v;
 }
 
+int gemm_splits(int M, int N, int K, int most);
+
 struct ClfPlan {
   int T, Tp, N, r, l, q;
-  int gram_split, gram_rows, ritz_split;                     // row ranges of a Gram matrix and rows of each; K ranges of the Ritz matrix
-  size_t off_flags, off_zb, off_yt, off_u, off_z, off_part, off_g, off_lf, off_w, off_iv, off_m, off_p, off_ps, off_vb, off_cs, off_m2,
+  int gram_split, gram_rows;                                 // row ranges of a Gram matrix and rows of each
+  int u_split, ritz_split;                                   // K ranges of U = X^T Y and of the Ritz matrix
+  size_t off_flags, off_zb, off_yt, off_up, off_u, off_z, off_part, off_g, off_lf, off_w, off_iv, off_m, off_p, off_ps, off_vb, off_cs, off_m2,
       off_q, total;
 };
 
@@ -1001,17 +1032,16 @@ bool make_plan(const xkv_clf_config* c, ClfPlan* p) {
   p->off_flags = o; o = align_up(o + 256);
   p->off_zb = o; o = align_up(o + (size_t)p->N * p->l * 2);
   p->off_yt = o; o = align_up(o + (size_t)p->l * p->Tp * 2);
+  p->u_split = gemm_splits(p->N, p->l, p->T, 8);
+  p->off_up = o; if (p->u_split > 1) o = align_up(o + (size_t)p->u_split * p->N * p->l * 4);   // partial sums of U
   p->off_u = o; o = align_up(o + (size_t)p->N * p->l * 4);
   p->off_z = o; o = align_up(o + (size_t)p->N * p->l * 4);
-  // row ranges so that the lower 64 x 64 tiles of the Gram matrix fill the SMs about twice; the K ranges of the
-  // Rayleigh-Ritz matrix fill them once (both for 148 SMs; fewer only queue)
-  const int tiles = (p->l / 64) * (p->l / 64 + 1) / 2, ritz_tiles = ((p->l + 127) / 128) * ((p->l + 191) / 192);
+  // row ranges so that the lower 64 x 64 tiles of the Gram matrix fill the SMs about twice (148 SMs; fewer only queue)
+  const int tiles = (p->l / 64) * (p->l / 64 + 1) / 2;
   p->gram_split = 296 / tiles < 1 ? 1 : (296 / tiles > 8 ? 8 : 296 / tiles);
   p->gram_rows = ((p->N + p->gram_split - 1) / p->gram_split + 31) & ~31;
   p->gram_split = (p->N + p->gram_rows - 1) / p->gram_rows;
-  p->ritz_split = 148 / ritz_tiles < 1 ? 1 : (148 / ritz_tiles > 16 ? 16 : 148 / ritz_tiles);
-  const int ritz_cols = ((p->T + p->ritz_split - 1) / p->ritz_split + 63) & ~63;
-  p->ritz_split = (p->T + ritz_cols - 1) / ritz_cols;            // none of the ranges is empty
+  p->ritz_split = gemm_splits(p->l, p->l, p->T, 16);
   const size_t part_words = p->gram_split * 2 > p->ritz_split ? p->gram_split * 2 : p->ritz_split;
   p->off_part = o; o = align_up(o + part_words * p->l * p->l * 4);   // partial Gram matrices (fp64) / Ritz matrices (fp32)
   p->off_g = o; o = align_up(o + (size_t)p->l * p->l * 8);      // the Gram matrix, factorised in place of its tiles, fp64
@@ -1039,41 +1069,69 @@ int check_clf_config(const xkv_clf_config* c) {
   return XKV_OK;
 }
 
-// A operand of a product: a matrix [rows][cols] with a row pitch (elements); rows are k unless AROW.
+// An operand of a product: a matrix [rows][cols] with a row pitch (elements); its columns are k if it is K-major, else its
+// rows are.
 struct GemmOperand {
   const void* p;
   int rows, cols, pitch;
 };
+struct GemmOut {
+  float* f;                 // either may be null
+  __nv_bfloat16* b;
+  long long ld;
+};
 
-template <bool TRANS, bool AROW, int BN>
-cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, int splits, float* Cf, __nv_bfloat16* Cb, long long ldc,
-                           unsigned int* flags, int device, cudaStream_t s) {
-  const int M = AROW ? a.rows : a.cols, N = b.rows, K = b.cols;
+template <bool TRANS, bool AK, bool BK, int MB, int BN>
+cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, int splits, GemmOut c, unsigned int* flags, int device, cudaStream_t s) {
+  const int M = AK ? a.rows : a.cols, N = BK ? b.rows : b.cols, K = AK ? a.cols : a.rows;
   CUtensorMap ma, mb;
-  if (!encode_bf16_map(&ma, a.p, (uint64_t)a.rows, (uint64_t)a.cols, (uint64_t)a.pitch, AROW ? 128 : 64) ||
-      !encode_bf16_map(&mb, b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BN))
+  if (!encode_bf16_map(&ma, a.p, (uint64_t)a.rows, (uint64_t)a.cols, (uint64_t)a.pitch, AK ? 128 * MB : 64) ||
+      !encode_bf16_map(&mb, b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BK ? BN : 64))
     return cudaErrorInvalidValue;
-  const size_t smem = 1024 + (size_t)gemm_stages<BN>() * gemm_stage_bytes<BN>();
-  cudaError_t e = ensure_dyn_smem<clf_gemm_kernel<TRANS, AROW, BN>>(smem, device);
+  const size_t smem = 1024 + (size_t)gemm_stages<MB, BN>() * gemm_stage_bytes<MB, BN>();
+  cudaError_t e = ensure_dyn_smem<clf_gemm_kernel<TRANS, AK, BK, MB, BN>>(smem, device);
   if (e != cudaSuccess) return e;
   const int k_per = ((K + splits - 1) / splits + 63) & ~63;
-  const dim3 grid((N + BN - 1) / BN, (M + 127) / 128, splits);
-  clf_gemm_kernel<TRANS, AROW, BN><<<grid, kGemmThreads, smem, s>>>(ma, mb, M, N, K, k_per, Cf, Cb, ldc, flags);
+  const dim3 grid((N + BN - 1) / BN, (M + 128 * MB - 1) / (128 * MB), splits);
+  clf_gemm_kernel<TRANS, AK, BK, MB, BN><<<grid, gemm_threads<MB>(), smem, s>>>(ma, mb, M, N, K, k_per, c.f, c.b, c.ld, flags);
   count_launch(kFamClf);
   return cudaGetLastError();
 }
 
-// The tile width that pads N least (the widest on a tie): 576 columns are three tiles of 192, a tall N is tiles of 256.
-template <bool TRANS, bool AROW>
-cudaError_t launch_gemm(GemmOperand a, GemmOperand b, int splits, float* Cf, __nv_bfloat16* Cb, long long ldc,
-                        unsigned int* flags, int device, cudaStream_t s) {
-  auto padded = [&](int bn) { return (long long)((b.rows + bn - 1) / bn) * bn; };
+// Tile width: the one that pads N least (the widest on a tie): 576 columns are three tiles of 192, 512 are two of 256.
+int gemm_bn(int N) {
+  auto padded = [&](int bn) { return (long long)((N + bn - 1) / bn) * bn; };
   int bn = 256;
   if (padded(192) < padded(bn)) bn = 192;
   if (padded(128) < padded(bn)) bn = 128;
-  if (bn == 256) return launch_gemm_bn<TRANS, AROW, 256>(a, b, splits, Cf, Cb, ldc, flags, device, s);
-  if (bn == 192) return launch_gemm_bn<TRANS, AROW, 192>(a, b, splits, Cf, Cb, ldc, flags, device, s);
-  return launch_gemm_bn<TRANS, AROW, 128>(a, b, splits, Cf, Cb, ldc, flags, device, s);
+  return bn;
+}
+// Two accumulators unless that pads M by more than an eighth.
+int gemm_mb(int M) { return ((M + 255) & ~255) * 8LL <= ((M + 127) & ~127) * 9LL ? 2 : 1; }
+
+template <bool TRANS, bool AK, bool BK>
+cudaError_t launch_gemm(GemmOperand a, GemmOperand b, int splits, GemmOut c, unsigned int* flags, int device, cudaStream_t s) {
+  const int bn = gemm_bn(BK ? b.rows : b.cols);
+  if (gemm_mb(AK ? a.rows : a.cols) == 2) {
+    if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, 2, 256>(a, b, splits, c, flags, device, s);
+    if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, 2, 192>(a, b, splits, c, flags, device, s);
+    return launch_gemm_bn<TRANS, AK, BK, 2, 128>(a, b, splits, c, flags, device, s);
+  }
+  if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, 1, 256>(a, b, splits, c, flags, device, s);
+  if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, 1, 192>(a, b, splits, c, flags, device, s);
+  return launch_gemm_bn<TRANS, AK, BK, 1, 128>(a, b, splits, c, flags, device, s);
+}
+
+// K ranges that bring a product's tiles to about one per SM (148), none of them empty or shorter than 1024.
+int gemm_splits(int M, int N, int K, int most) {
+  const int mb = gemm_mb(M) * 128, bn = gemm_bn(N);
+  const long long tiles = (long long)((M + mb - 1) / mb) * ((N + bn - 1) / bn);
+  long long sp = 148 / tiles;
+  if (sp > most) sp = most;
+  if (sp > K / 1024) sp = K / 1024;
+  if (sp < 1) sp = 1;
+  const int k_per = (int)(((K + sp - 1) / sp + 63) & ~63);
+  return (K + k_per - 1) / k_per;
 }
 
 template <auto Kernel>
@@ -1106,7 +1164,7 @@ int clf_workspace_bytes(const xkv_clf_config* c, uint64_t* bytes) {
 
 // Debug/test entry of the tensor-core product alone: C (M x N, fp32) = A B^T, A bf16 [K][M], B bf16 [N][K].
 cudaError_t clf_gemm(const void* a, const void* b, int M, int N, int K, float* C, unsigned int* flags, int device, cudaStream_t s) {
-  return launch_gemm<false, false>({a, K, M, M}, {b, N, K, K}, 1, C, nullptr, N, flags, device, s);
+  return launch_gemm<false, false, true>({a, K, M, M}, {b, N, K, K}, 1, {C, nullptr, N}, flags, device, s);
 }
 
 static std::atomic<unsigned> g_clf_inject{0};
@@ -1139,9 +1197,17 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
   cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 256, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(Zb, omega, (size_t)N * l * 2, cudaMemcpyDeviceToDevice, s);
-  // Y^T = Z^T X^T  and  U = X^T Y
-  auto product_y = [&]() { return launch_gemm<false, false>({Zb, N, l, l}, {X, T, N, N}, 1, nullptr, Yt, p.Tp, flags, device, s); };
-  auto product_u = [&]() { return launch_gemm<false, false>({X, T, N, N}, {Yt, l, T, p.Tp}, 1, U, nullptr, l, flags, device, s); };
+  // Y = X Z (stored as Y^T)  and  U = X^T Y
+  auto product_y = [&]() { return launch_gemm<true, true, false>({X, T, N, N}, {Zb, N, l, l}, 1, {nullptr, Yt, p.Tp}, flags, device, s); };
+  auto product_u = [&]() -> cudaError_t {
+    float* out = p.u_split > 1 ? (float*)(w + p.off_up) : U;
+    cudaError_t e2 = launch_gemm<false, false, true>({X, T, N, N}, {Yt, l, T, p.Tp}, p.u_split, {out, nullptr, l}, flags, device, s);
+    if (e2 != cudaSuccess || p.u_split == 1) return e2;
+    const long long n4 = (long long)N * l / 4;
+    sum_parts_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, s>>>((const float4*)out, p.u_split, n4, (float4*)U);
+    count_launch(kFamClf);
+    return cudaGetLastError();
+  };
   // Z = orth(U) by shifted Cholesky QR, the Gram matrix accumulated, factorised and inverted in fp64: its condition
   // number is the square of the iterate's, which after a multiplication by X^T X spans the whole range between the
   // largest singular value and the noise floor.  A pass divides the condition number by up to shift^-1/2; U is stored
@@ -1179,7 +1245,7 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
   }
   // Rayleigh-Ritz: W = X Z, M = W^T W (= Z^T X^T X Z), its eigenvectors by Jacobi
   if (e == cudaSuccess) e = product_y();
-  if (e == cudaSuccess) e = launch_gemm<false, true>({Yt, l, T, p.Tp}, {Yt, l, T, p.Tp}, p.ritz_split, (float*)part, nullptr, l, flags, device, s);
+  if (e == cudaSuccess) e = launch_gemm<false, true, true>({Yt, l, T, p.Tp}, {Yt, l, T, p.Tp}, p.ritz_split, {(float*)part, nullptr, l}, flags, device, s);
   if (e == cudaSuccess) {
     symmetrize_kernel<<<(l * l + 255) / 256, 256, 0, s>>>((const float*)part, p.ritz_split, Mm, l);
     float* M2 = (float*)(w + p.off_m2);
@@ -1198,7 +1264,7 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
     e = cudaGetLastError();
   }
   // A = X V_bf16, stored [T][r]
-  if (e == cudaSuccess) e = launch_gemm<true, false>({Vb, N, r, r}, {X, T, N, N}, 1, nullptr, (__nv_bfloat16*)A_out, r, flags, device, s);
+  if (e == cudaSuccess) e = launch_gemm<false, true, false>({X, T, N, N}, {Vb, N, r, r}, 1, {nullptr, (__nv_bfloat16*)A_out, r}, flags, device, s);
   if (e != cudaSuccess) { set_cuda_error(e); (void)cudaGetLastError(); return XKV_ERR_CUDA; }
   return XKV_OK;
 }
