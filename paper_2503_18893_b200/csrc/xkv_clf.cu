@@ -335,13 +335,17 @@ __device__ __forceinline__ double newton_rsqrt(double d) {
 }
 
 // Cholesky factorisation in fp64 of G + shift_rel * max_diag(G) * I and the inverse W = L^-1 of its factor, one
-// cooperative kernel.  Blocks of 32.  A step p of the factorisation: every lower tile (i, k), k > p, forms the two
-// blocks of the panel it needs, L_ip = A_ip inv(L_pp)^T and L_kp, by itself (they cost less than handing them over would)
-// and takes L_ip L_kp^T out; the CTA of tile (p+1, p+1) then factors it at once, so that one grid barrier per step
-// suffices.  (As three launches per panel the factorisation of a 576 x 576 matrix was 52 launches of 7 to 16 us.)
-// W by columns of eight: W_ik = -inv(L_ii) sum_{k <= j < i} L_ij W_jk.  With W at hand the solve is a product.
-// Buffers: part [n_part][l][l] partial Gram matrices (lower tiles of 64), Gm [l][l] the working matrix, Lf [l][l] the
-// factor's blocks below the diagonal blocks, Iv [l/32][32][32] inverses of the diagonal blocks, W [l][l] lower.
+// cooperative kernel.  Blocks of 32.  At step p every lower tile (i, k), i >= p, is one item:
+//   i > p, k > p    A_ik -= L_ip L_kp^T; the two blocks of the panel, L_ip = A_ip inv(L_pp)^T and L_kp, are formed by the item
+//                   itself (they cost less than handing them over would); tile (p+1, p+1) is then factored at once, so that
+//                   one grid barrier per step suffices
+//   i > p, k <= p   the same elimination on the identity, R_ik -= L_ip W_pk (R starts as I), with W_pk = inv(L_pp) R_pk
+//   i == p          W_pk is written
+// A latency chain: 576 columns one after the other in the diagonal blocks, 19 barriers.  (As three launches per panel the
+// factorisation of a 576 x 576 matrix was 52 launches of 7 to 16 us; with the inverse formed after it, column by column, the
+// kernel took 321 us, with the inverse carried along 235.)  With W at hand the solve is a product.
+// Buffers: part [n_part][l][l] partial Gram matrices (lower tiles of 64), Gm [l][l] the working matrix, Rt [l][l] the tiles
+// of R below the diagonal, each transposed, Iv [l/32][32][32] inverses of the diagonal blocks, W [l][l] lower.
 constexpr int kCholNb = 32, kCholThreads = 256, kCholLd = 36;   // 36 doubles per staged row: 4 mod 16, conflict free fragments
 
 // One 8-row, 32-deep fragment product: acc (8 x 8 per tile) += A rows [m8..m8+7] of a staged block times B rows^T.
@@ -352,9 +356,8 @@ __device__ __forceinline__ void dmma_block(double (&acc)[2], const double* A, co
 }
 
 __global__ void __launch_bounds__(kCholThreads, 1)
-chol_inverse_kernel(const double* __restrict__ part, int n_part, double* __restrict__ Gm, double* __restrict__ Lf,
+chol_inverse_kernel(const double* __restrict__ part, int n_part, double* __restrict__ Gm, double* __restrict__ Rt,
                     double* __restrict__ Iv, double* __restrict__ W, int l, double shift_rel, unsigned arrived, GridSync sy) {
-  extern __shared__ __align__(16) double cs_d[];               // [l][9] columns of W (second half of the kernel)
   __shared__ double A_s[kCholNb * kCholLd], B_s[kCholNb * kCholLd], V_s[kCholNb * kCholLd], Li_s[kCholNb * kCholLd], Lk_s[kCholNb * kCholLd];
   __shared__ __align__(16) double col_s[2][kCholNb];
   __shared__ double piv_s[2];
@@ -437,101 +440,79 @@ chol_inverse_kernel(const double* __restrict__ part, int n_part, double* __restr
       }
     }
   };
-  const int n_tiles = nbk * (nbk + 1) / 2;
+  auto first_of = [&](int i) { return i * (i + 1) / 2; };      // tiles of the lower triangle, row by row
   auto tile_of = [&](int t, int& i, int& k) { i = 0; k = t; while (k > i) { ++i; k -= i; } };
-  if (bid == 0) {                                              // tile 0 is (0, 0)
+  if (bid == 0) {
     stage(A_s, Gm, l);
     __syncthreads();
     if (tid < kCholNb) A_s[tid * kCholLd + tid] += shift;
     factor(0);
   }
   if (!grid_barrier(sy, arrived, &ok_s)) return;
-  for (int p = 0; p + 1 < nbk; ++p) {
-    // (the tile whose factor everybody waits for comes first in its CTA: its index is the smallest of those with k > p)
-    for (int t = bid; t < n_tiles; t += nb) {
+  const int fr = t_m * 8 + (lane >> 2), fc = 2 * (lane & 3);   // this thread's fragment: row fr, columns (t_n + j) * 8 + fc, + 1
+  for (int p = 0; p < nbk; ++p) {
+    // CTA 0 takes the tile whose factor everybody waits for, the others share the rest
+    const int critical = p + 1 < nbk ? first_of(p + 1) + p + 1 : -1, items = first_of(nbk) - first_of(p) - (critical >= 0 ? 1 : 0);
+    for (int e = bid == 0 ? items : bid - 1;; e += nb - 1) {
+      const bool crit = bid == 0 && critical >= 0;
+      if (!crit && e >= items) break;
+      int t = crit ? critical : first_of(p) + e;
+      if (!crit && critical >= 0 && t >= critical) ++t;
       int i, k;
       tile_of(t, i, k);
-      if (k <= p) continue;
+      const bool trail = k > p;
       __syncthreads();
       stage(V_s, Iv + (size_t)p * kCholNb * kCholNb, kCholNb);
-      stage(A_s, Gm + (size_t)i * kCholNb * l + p * kCholNb, l);
-      if (i != k) stage(B_s, Gm + (size_t)k * kCholNb * l + p * kCholNb, l);
-      double acc[2][2];
+      if (i > p) stage(A_s, Gm + (size_t)i * kCholNb * l + p * kCholNb, l);
+      if (trail ? i != k : k < p) stage(B_s, (trail ? Gm + (size_t)k * kCholNb * l + p * kCholNb : Rt + (size_t)p * kCholNb * l + k * kCholNb), l);
+      double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+      double* const own = (trail ? Gm : Rt) + (size_t)i * kCholNb * l + k * kCholNb;
+      if (i > p && (trail || k < p)) {
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const double2 v = __ldcg(reinterpret_cast<const double2*>(Gm + (size_t)(i * kCholNb + t_m * 8 + (lane >> 2)) * l + k * kCholNb + (t_n + j) * 8 + 2 * (lane & 3)));
-        acc[j][0] = v.x; acc[j][1] = v.y;
+        for (int j = 0; j < 2; ++j) {
+          const double2 v = __ldcg(reinterpret_cast<const double2*>(own + (size_t)fr * l + (t_n + j) * 8 + fc));
+          acc[j][0] = v.x; acc[j][1] = v.y;
+        }
       }
       __syncthreads();
       double li[2][2] = {{0.0, 0.0}, {0.0, 0.0}}, lk[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        dmma_block(li[j], A_s + t_m * 8 * kCholLd, V_s + (t_n + j) * 8 * kCholLd, lane, 1.0);
-        if (i != k) dmma_block(lk[j], B_s + t_m * 8 * kCholLd, V_s + (t_n + j) * 8 * kCholLd, lane, 1.0);
+        if (i > p) dmma_block(li[j], A_s + t_m * 8 * kCholLd, V_s + (t_n + j) * 8 * kCholLd, lane, 1.0);
+        // L_kp, or W_pk^T = R_pk^T inv(L_pp)^T
+        if (trail ? i != k : k < p) dmma_block(lk[j], B_s + t_m * 8 * kCholLd, V_s + (t_n + j) * 8 * kCholLd, lane, 1.0);
+        else if (!trail) { lk[j][0] = V_s[((t_n + j) * 8 + fc) * kCholLd + fr]; lk[j][1] = V_s[((t_n + j) * 8 + fc + 1) * kCholLd + fr]; }
+      }
+      if (i == p) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+          for (int x = 0; x < 2; ++x) W[(size_t)(p * kCholNb + (t_n + j) * 8 + fc + x) * l + k * kCholNb + fr] = lk[j][x];
+        continue;
       }
       put(Li_s, kCholLd, li);
       if (i != k) put(Lk_s, kCholLd, lk);
-      else put(Lf + (size_t)i * kCholNb * l + p * kCholNb, l, li);
       __syncthreads();
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        if (i == k && p == 0) {                                // first touch of a diagonal tile
+        if (trail) {
+          if (i == k && p == 0) {                              // first touch of a diagonal tile
 #pragma unroll
-          for (int x = 0; x < 2; ++x) if (t_m * 8 + (lane >> 2) == (t_n + j) * 8 + 2 * (lane & 3) + x) acc[j][x] += shift;
+            for (int x = 0; x < 2; ++x) if (fr == (t_n + j) * 8 + fc + x) acc[j][x] += shift;
+          }
+          dmma_block(acc[j], Li_s + t_m * 8 * kCholLd, (i != k ? Lk_s : Li_s) + (t_n + j) * 8 * kCholLd, lane, -1.0);
+        } else {
+          dmma_block(acc[j], Lk_s + t_m * 8 * kCholLd, Li_s + (t_n + j) * 8 * kCholLd, lane, -1.0);
         }
-        dmma_block(acc[j], Li_s + t_m * 8 * kCholLd, (i != k ? Lk_s : Li_s) + (t_n + j) * 8 * kCholLd, lane, -1.0);
       }
-      if (i == k && k == p + 1) {
+      if (crit) {
         put(A_s, kCholLd, acc);
         factor(p + 1);
-      } else {
-        put(Gm + (size_t)i * kCholNb * l + k * kCholNb, l, acc);
+        break;
       }
+      put(own, l, acc);
     }
-    if (!grid_barrier(sy, arrived, &ok_s)) return;
-  }
-  // ---- W: columns c0 .. c0 + 7 of block column k, rows downwards; warps: 8-row tile t_m, half (warp >> 2) of the terms
-  const int ldw = 9;
-  double* const Wc = cs_d;                                     // [l][9]
-  double* const H_s = A_s;                                     // [2][32][9] partial sums of the two halves
-  for (int st = bid; st < nbk * 4; st += nb) {
-    const int k = st >> 2, c0 = (st & 3) * 8;
-    __syncthreads();
-    for (int e = tid; e < kCholNb * 8; e += kCholThreads) {
-      const double v = __ldcg(Iv + ((size_t)k * kCholNb + (e >> 3)) * kCholNb + c0 + (e & 7));
-      Wc[(size_t)(k * kCholNb + (e >> 3)) * ldw + (e & 7)] = v;
-      W[(size_t)(k * kCholNb + (e >> 3)) * l + k * kCholNb + c0 + (e & 7)] = v;
-    }
-    for (int i = k + 1; i < nbk; ++i) {
-      stage(V_s, Iv + (size_t)i * kCholNb * kCholNb, kCholNb);
-      __syncthreads();
-      double acc[2] = {0.0, 0.0};
-      const double* Lrow = Lf + (size_t)(i * kCholNb + t_m * 8 + (lane >> 2)) * l + (lane & 3);
-#pragma unroll 2
-      for (int j = k + (warp >> 2); j < i; j += 2) {
-        double a[8];
-#pragma unroll
-        for (int s8 = 0; s8 < 8; ++s8) a[s8] = __ldcg(Lrow + j * kCholNb + s8 * 4);
-#pragma unroll
-        for (int s8 = 0; s8 < 8; ++s8)
-          dmma_8x8x4(acc, a[s8], Wc[(size_t)(j * kCholNb + s8 * 4 + (lane & 3)) * ldw + (lane >> 2)]);
-      }
-      double* h = H_s + (size_t)((warp >> 2) * kCholNb + t_m * 8 + (lane >> 2)) * ldw + 2 * (lane & 3);
-      h[0] = acc[0]; h[1] = acc[1];
-      __syncthreads();
-      if (warp < 4) {
-        double w[2] = {0.0, 0.0};
-#pragma unroll
-        for (int kk = 0; kk < kCholNb; kk += 4) {
-          const int r = kk + (lane & 3), c = lane >> 2;
-          dmma_8x8x4(w, -V_s[(t_m * 8 + (lane >> 2)) * kCholLd + r], H_s[(size_t)r * ldw + c] + H_s[(size_t)(kCholNb + r) * ldw + c]);
-        }
-        const int row = i * kCholNb + t_m * 8 + (lane >> 2), c = 2 * (lane & 3);
-        Wc[(size_t)row * ldw + c] = w[0]; Wc[(size_t)row * ldw + c + 1] = w[1];
-        *reinterpret_cast<double2*>(W + (size_t)row * l + k * kCholNb + c0 + c) = make_double2(w[0], w[1]);
-      }
-      __syncthreads();
-    }
+    if (p + 1 < nbk && !grid_barrier(sy, arrived, &ok_s)) return;
   }
 }
 
@@ -1016,7 +997,7 @@ struct ClfPlan {
   int T, Tp, N, r, l, q;
   int gram_split, gram_rows;                                 // row ranges of a Gram matrix and rows of each
   int u_split, ritz_split;                                   // K ranges of U = X^T Y and of the Ritz matrix
-  size_t off_flags, off_zb, off_yt, off_up, off_u, off_z, off_part, off_g, off_lf, off_w, off_iv, off_m, off_p, off_ps, off_vb, off_cs, off_m2,
+  size_t off_flags, off_zb, off_yt, off_up, off_u, off_z, off_part, off_g, off_rt, off_w, off_iv, off_m, off_p, off_ps, off_vb, off_cs, off_m2,
       off_q, total;
 };
 
@@ -1045,7 +1026,7 @@ bool make_plan(const xkv_clf_config* c, ClfPlan* p) {
   const size_t part_words = p->gram_split * 2 > p->ritz_split ? p->gram_split * 2 : p->ritz_split;
   p->off_part = o; o = align_up(o + part_words * p->l * p->l * 4);   // partial Gram matrices (fp64) / Ritz matrices (fp32)
   p->off_g = o; o = align_up(o + (size_t)p->l * p->l * 8);      // the Gram matrix, factorised in place of its tiles, fp64
-  p->off_lf = o; o = align_up(o + (size_t)p->l * p->l * 8);     // its factor below the diagonal blocks
+  p->off_rt = o; o = align_up(o + (size_t)p->l * p->l * 8);     // the identity under elimination, tiles transposed
   p->off_w = o; o = align_up(o + (size_t)p->l * p->l * 8);      // the factor's inverse
   p->off_iv = o; o = align_up(o + (size_t)p->l * kCholNb * 8);  // inverses of its diagonal blocks
   p->off_m = o; o = align_up(o + (size_t)p->l * p->l * 4);
@@ -1185,7 +1166,7 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
   float* Z = (float*)(w + p.off_z);
   double* part = (double*)(w + p.off_part);
   double* Gm = (double*)(w + p.off_g);
-  double* Lf = (double*)(w + p.off_lf);
+  double* Rt = (double*)(w + p.off_rt);
   double* W = (double*)(w + p.off_w);
   double* Iv = (double*)(w + p.off_iv);
   float* Mm = (float*)(w + p.off_m);
@@ -1218,7 +1199,6 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
   constexpr double kShift = 1e-11;
   const int nbk = l / kCholNb, n_tiles = nbk * (nbk + 1) / 2;
   const int chol_grid = sms < (n_tiles > 32 ? n_tiles : 32) ? sms : (n_tiles > 32 ? n_tiles : 32);
-  const size_t chol_smem = (size_t)l * 9 * sizeof(double);
   unsigned chol_arrived = 0;
   auto cholqr = [&](int passes) -> cudaError_t {                       // an odd number of passes ends in Z
     float* in = U;
@@ -1228,8 +1208,8 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
       double shift = kShift;
       int n_part = p.gram_split;
       GridSync sy{flags, flags + 12, flags + 10, kGridSpinLimit, 0u};
-      void* args[] = {&part, &n_part, &Gm, &Lf, &Iv, &W, &l, &shift, &chol_arrived, &sy};
-      cudaError_t e2 = launch_cooperative<chol_inverse_kernel>(chol_grid, kCholThreads, chol_smem, args, device, s);
+      void* args[] = {&part, &n_part, &Gm, &Rt, &Iv, &W, &l, &shift, &chol_arrived, &sy};
+      cudaError_t e2 = launch_cooperative<chol_inverse_kernel>(chol_grid, kCholThreads, 0, args, device, s);
       if (e2 != cudaSuccess) return e2;
       chol_arrived += (unsigned)chol_grid * (unsigned)(nbk + 1);       // barriers of one factorisation
       tri_product_kernel<<<dim3((N + 63) / 64, l / 64), 256, 0, s>>>(in, W, out, Zb, N, l);
