@@ -426,11 +426,10 @@ int xkv_sr_reconstruct_attend_tail(xkv_group* g, int layer_begin, int layer_end,
     return XKV_ERR_INVALID_ARG;
   if (g->attend_impl || !fused_supported(g)) return XKV_ERR_UNSUPPORTED;
   cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = launch_tail_partials(g, layer_begin, layer_end, (const __nv_bfloat16*)q, (const __nv_bfloat16*)tail_k,
-                                       (const __nv_bfloat16*)tail_v, tail_len, tail_cap, (float*)workspace, s);
-  if (e == cudaSuccess)
-    e = launch_fused(g, layer_begin, layer_end, (const __nv_bfloat16*)q, sel_idx, sel_cnt, k_cap, (__nv_bfloat16*)out,
-                     lse, s, TailParts{(const float*)workspace, tail_splits(tail_cap)});
+  const cudaError_t e = launch_fused(g, layer_begin, layer_end, (const __nv_bfloat16*)q, sel_idx, sel_cnt, k_cap,
+                                     (__nv_bfloat16*)out, lse, s,
+                                     TailCall{(const __nv_bfloat16*)tail_k, (const __nv_bfloat16*)tail_v, tail_len, tail_cap,
+                                              (float*)workspace});
   if (e != cudaSuccess) { set_cuda_error(e); (void)cudaGetLastError(); return XKV_ERR_CUDA; }
   return XKV_OK;
 }
@@ -567,7 +566,7 @@ int xkv_dense_attend(xkv_group* g, int layer_begin, int layer_end, const void* q
     return XKV_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = launch_tail_partials(g, layer_begin, layer_end, (const __nv_bfloat16*)q, (const __nv_bfloat16*)K,
-                                       (const __nv_bfloat16*)V, len, cap, (float*)workspace, s);
+                                       (const __nv_bfloat16*)V, len, cap, (float*)workspace, false, s);
   if (e == cudaSuccess)
     e = launch_dense_merge(g, layer_begin, layer_end, (const float*)workspace, cap, (__nv_bfloat16*)out, lse, s);
   if (e != cudaSuccess) { set_cuda_error(e); (void)cudaGetLastError(); return XKV_ERR_CUDA; }

@@ -1320,7 +1320,7 @@ constexpr size_t fused_smem_bytes() {
 
 template <int DH, int NR, int WB>
 cudaError_t launch_fused_t(const xkv_group* grp, int l0, int l1, const __nv_bfloat16* q, const int32_t* sel_idx,
-                           const int32_t* sel_cnt, int k_cap, __nv_bfloat16* out, float* lse, cudaStream_t s, TailParts tail) {
+                           const int32_t* sel_cnt, int k_cap, __nv_bfloat16* out, float* lse, cudaStream_t s, const TailCall& tc) {
   const GroupDev& dev = grp->dev;
   const int problems = (l1 - l0) * dev.batch * dev.H_kv;
   Sched sc;
@@ -1358,6 +1358,12 @@ cudaError_t launch_fused_t(const xkv_group* grp, int l0, int l1, const __nv_bflo
   }
   count_launch(kFamFused);
   if (e != cudaSuccess) return e;
+  TailParts tail{nullptr, 0};
+  if (tc.k) {
+    e = launch_tail_partials(grp, l0, l1, q, tc.k, tc.v, tc.len, tc.cap, tc.part, true, s);
+    if (e != cudaSuccess) return e;
+    tail = TailParts{tc.part, tail_splits(tc.cap)};
+  }
   // one CTA per query head while those CTAs fit the SMs about twice over; beyond that one CTA per group of heads
   constexpr int HG = NR <= 4 ? 4 : 8;
   bool multi = false;
@@ -1401,7 +1407,7 @@ bool fused_supported(const xkv_group* grp) {
 }
 
 cudaError_t launch_fused(const xkv_group* grp, int l0, int l1, const __nv_bfloat16* q, const int32_t* sel_idx,
-                         const int32_t* sel_cnt, int k_cap, __nv_bfloat16* out, float* lse, cudaStream_t s, TailParts tail) {
+                         const int32_t* sel_cnt, int k_cap, __nv_bfloat16* out, float* lse, cudaStream_t s, const TailCall& tail) {
   const int n_rep = grp->dev.n_rep, blocks = (grp->dev.r_v + 127) / 128;   // WB: the smallest variant that holds r_v
 #define XKV_DISPATCH(DH)                                                                                 \
   if (n_rep <= 4 && blocks <= 4) return launch_fused_t<DH, 4, 4>(grp, l0, l1, q, sel_idx, sel_cnt, k_cap, out, lse, s, tail);  \

@@ -167,8 +167,16 @@ cudaError_t launch_dense_merge(const xkv_group* grp, int l0, int l1, const float
                                float* lse, cudaStream_t s);
 size_t tail_part_floats(const xkv_group* grp, int tail_cap);
 cudaError_t launch_tail_partials(const xkv_group* grp, int l0, int l1, const __nv_bfloat16* q, const __nv_bfloat16* tail_k,
-                                 const __nv_bfloat16* tail_v, const int32_t* tail_len, int tail_cap, float* part,
+                                 const __nv_bfloat16* tail_v, const int32_t* tail_len, int tail_cap, float* part, bool behind,
                                  cudaStream_t s);
+// What launch_fused has to know to launch the partials of a tail between its two kernels.
+struct TailCall {
+  const __nv_bfloat16* k;   // nullptr: no tail
+  const __nv_bfloat16* v;
+  const int32_t* len;
+  int cap;
+  float* part;
+};
 
 // xkv_quant.cu
 cudaError_t launch_quantize_rtn4(const __nv_bfloat16* x, long long rows, int cols, void* codes, void* meta, cudaStream_t s);
@@ -193,6 +201,6 @@ bool fused_supported(const xkv_group* grp);
 bool fused_sm_count_ok(int sm_count);
 cudaError_t launch_fused(const xkv_group* grp, int l0, int l1, const __nv_bfloat16* q, const int32_t* sel_idx,
                          const int32_t* sel_cnt, int k_cap, __nv_bfloat16* out, float* lse, cudaStream_t s,
-                         TailParts tail = TailParts{nullptr, 0});
+                         const TailCall& tail = TailCall{});
 
 }  // namespace xkv
