@@ -73,9 +73,11 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
     if r.returncode != 0:
         sys.stderr.write(r.stdout + r.stderr)
         raise RuntimeError("link failed")
+    from torch.utils import cpp_extension      # (its libraries are loaded by `import torch` before the module is)
     cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I", os.path.join(ROOT, "include"),
-           "-I", sysconfig.get_paths()["include"], os.path.join(CSRC, "xkv_py.cpp"), "-o", PYMOD, "-L", HERE, "-lxkv",
-           "-Wl,-rpath,$ORIGIN"]
+           "-I", sysconfig.get_paths()["include"], *("-isystem" + p for p in cpp_extension.include_paths()),
+           os.path.join(CSRC, "xkv_py.cpp"), "-o", PYMOD, "-L", HERE, "-lxkv", "-Wl,-rpath,$ORIGIN",
+           *("-L" + p for p in cpp_extension.library_paths()), "-ltorch_python", "-ltorch_cpu", "-lc10"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         sys.stderr.write(r.stdout + r.stderr)

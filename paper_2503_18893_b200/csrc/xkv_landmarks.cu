@@ -225,32 +225,7 @@ landmark_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restric
   }
 }
 
-using u64 = unsigned long long;    // two fp32 values, for the packed fp32 instructions
-__device__ __forceinline__ u64 pack2(float a, float b) {
-  u64 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float2 unpack2(u64 v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
-  u64 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
-  u64 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ u64 add2(u64 a, u64 b) {
-  u64 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
+using namespace ptx;                // packed fp32
 
 // The default chunk of 8 rows (c == 8), persistent CTAs.  Bit for bit the arithmetic of the kernel above.
 // A CTA walks a contiguous range of row blocks; the cos/sin table of a block is built once and serves every (sequence,

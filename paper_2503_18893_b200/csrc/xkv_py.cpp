@@ -1,12 +1,17 @@
 // CPython module over the C ABI for the calls of a decode step and the other per-prompt calls (argument marshalling
 // only).  A decode step is a handful of kernels of a few microseconds each, so what a call costs on the host is part
 // of its latency: through ctypes and torch.cuda.current_stream() a call spent 4.5 us before its first launch, here
-// 0.7 us.  Tensor arguments are anything with a data_ptr() method (or None, or an integer address); a stream is None
+// 0.7 us.  The quantiser's calls, whose kernels take as long as their launches, allocate their results here too (10.5 us of
+// host time for a pair of torch.empty and a launch through Python, 5 us here).  Tensor arguments are anything with a data_ptr() method (or None, or an integer address); a stream is None
 // (torch's current one), an integer, or an object with a cuda_stream attribute.  Every function returns the status.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
 #include <stdint.h>
+
+#include <ATen/core/Tensor.h>
+#include <ATen/ops/empty.h>
+#include <torch/csrc/autograd/python_variable.h>
 
 #include "xkv.h"
 
@@ -157,23 +162,62 @@ XKV_PY(dense_attend, 13)
   void* s = a.stream();
 XKV_PY_END(xkv_dense_attend(g, l0, l1, q, K, V, len, cap, ws, ws_bytes, out, lse, s))
 
-XKV_PY(quantize_rtn, 7)
-  void* x = a.ptr();
-  const int64_t rows = a.i64();
-  const int cols = a.i32(), bits = a.i32();
-  void* codes = a.ptr();
-  void* meta = a.ptr();
-  void* s = a.stream();
-XKV_PY_END(xkv_quantize_rtn(x, rows, cols, bits, codes, meta, s))
+// An uninitialised tensor of x's device with x's leading sizes and `last` columns.
+at::Tensor like(const at::Tensor& x, int64_t last, at::ScalarType type) {
+  c10::DimVector sizes(x.sizes().begin(), x.sizes().end());
+  sizes.back() = last;
+  return at::empty(sizes, x.options().dtype(type));
+}
+const at::Tensor* tensor(PyObject* o) {
+  if (!THPVariable_Check(o) || THPVariable_Unpack(o).dim() < 1) {
+    PyErr_SetString(PyExc_TypeError, "expected a tensor of at least one dimension");
+    return nullptr;
+  }
+  return &THPVariable_Unpack(o);
+}
 
-XKV_PY(dequantize_rtn, 7)
-  void* codes = a.ptr();
-  void* meta = a.ptr();
-  const int64_t rows = a.i64();
-  const int cols = a.i32(), bits = a.i32();
-  void* x = a.ptr();
+// quantize_rtn(x, bits, stream) -> (status, codes, meta or None)
+PyObject* quantize_rtn(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
+  Args a(args, nargs, 3);
+  const at::Tensor* x = a.bad ? nullptr : tensor(a.next());
+  if (!x) return nullptr;
+  const int bits = a.i32();
   void* s = a.stream();
-XKV_PY_END(xkv_dequantize_rtn(codes, meta, rows, cols, bits, x, s))
+  if (a.bad) return nullptr;
+  try {
+    const int64_t cols = x->size(-1), rows = cols ? x->numel() / cols : 0;
+    at::Tensor codes = like(*x, cols / 2, at::kByte), meta;
+    // 4 bits: one scale/offset word per group beside the codes; 3 bits: the 16-byte records hold them
+    if (bits == 4) meta = like(*x, cols / 32, at::kInt);
+    const int st = xkv_quantize_rtn(x->const_data_ptr(), rows, cols > INT32_MAX ? 0 : (int)cols, bits, codes.mutable_data_ptr(),
+                                    bits == 4 ? meta.mutable_data_ptr() : nullptr, s);
+    return Py_BuildValue("iNN", st, THPVariable_Wrap(codes), bits == 4 ? THPVariable_Wrap(meta) : Py_NewRef(Py_None));
+  } catch (const std::exception& e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+}
+
+// dequantize_rtn(codes, meta, bits, stream) -> (status, x)
+PyObject* dequantize_rtn(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
+  Args a(args, nargs, 4);
+  const at::Tensor* codes = a.bad ? nullptr : tensor(a.next());
+  if (!codes) return nullptr;
+  void* meta = a.ptr();
+  const int bits = a.i32();
+  void* s = a.stream();
+  if (a.bad) return nullptr;
+  try {
+    const int64_t half = codes->size(-1), rows = half ? codes->numel() / half : 0;
+    at::Tensor x = like(*codes, half * 2, at::kBFloat16);
+    const int st = xkv_dequantize_rtn(codes->const_data_ptr(), meta, rows, half > INT32_MAX / 2 ? 0 : (int)(half * 2), bits,
+                                      x.mutable_data_ptr(), s);
+    return Py_BuildValue("iN", st, THPVariable_Wrap(x));
+  } catch (const std::exception& e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+}
 
 // torch_hooks(get_device, get_current_raw_stream): how "the current stream" is found.
 PyObject* torch_hooks(PyObject*, PyObject* const* args, Py_ssize_t nargs) {

@@ -37,7 +37,8 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
 // exact quotient of a 24-bit by an 8-bit number is never closer than 2^-33 to a rounding boundary and the value that is
 // rounded last is off by less than 2^-46, so every bit is that of the division.  Half-integers are common here
 // (differences of bf16 numbers over a bf16 scale): the quotient has to be exact, a test with a fallback diverged in most
-// warps (25 us for 65536 x 384 scalars, with an IEEE division per scalar and one thread per group 38 us; this form 12 us).
+// warps (25 us for 65536 x 384 scalars, with an IEEE division per scalar and one thread per group 38 us; this form 19.5, and 17 with
+// two scalars per packed instruction).
 // Rounding goes through 1.5 * 2^23, whose sum with the quotient holds the integer in its low bits.
 constexpr float kRintMagic = 12582912.0f;
 
@@ -78,36 +79,43 @@ quantize_rtn_kernel(const uint4* __restrict__ x, long long n_pieces, uint32_t* _
     const __nv_bfloat16 zb = __float2bfloat16_rn(lo);
     const __nv_bfloat16 sb = __float2bfloat16_rn(__fdiv_rn(__fsub_rn(hi, lo), kTop));
     const float zero = __bfloat162float(zb), scale = __bfloat162float(sb);
-    float f[8], m[8];                                      // m: rint(quotient) + kRintMagic
+    // two scalars per packed instruction; m: rint(quotient) + kRintMagic of the pairs (2e, 2e + 1)
+    ptx::u64 f[4], m[4];
+    const ptx::u64 nz2 = ptx::pack2(-zero, -zero);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      f[2 * e] = __fsub_rn(__uint_as_float(w[e] << 16), zero);
-      f[2 * e + 1] = __fsub_rn(__uint_as_float(w[e] & 0xffff0000u), zero);
-    }
+    for (int e = 0; e < 4; ++e) f[e] = ptx::add2(ptx::pack2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u)), nz2);
     // constant groups, scales with an imprecise or overflowing reciprocal, infinities: the division for every scalar
     if (!(scale >= 1e-30f && scale <= 1e30f)) {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) m[e] = (float)rtn_code_exact<BITS>(f[e], scale) + kRintMagic;
+      for (int e = 0; e < 4; ++e) {
+        const float2 x2 = ptx::unpack2(f[e]);
+        m[e] = ptx::pack2((float)rtn_code_exact<BITS>(x2.x, scale) + kRintMagic, (float)rtn_code_exact<BITS>(x2.y, scale) + kRintMagic);
+      }
     } else {
       const float y = __frcp_rn(scale);
+      const ptx::u64 y2 = ptx::pack2(y, y), ns2 = ptx::pack2(-scale, -scale), magic2 = ptx::pack2(kRintMagic, kRintMagic);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const float t = __fmul_rn(f[e], y);
-        m[e] = __fadd_rn(__fmaf_rn(__fmaf_rn(-t, scale, f[e]), y, t), kRintMagic);
+      for (int e = 0; e < 4; ++e) {
+        const ptx::u64 t = ptx::mul2(f[e], y2);
+        m[e] = ptx::add2(ptx::fma2(ptx::fma2(t, ns2, f[e]), y2, t), magic2);
       }
     }
-    uint32_t c[8];
+    // a pair of codes as the low and the high half of a word
+    uint32_t c[4];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) c[e] = __float_as_uint(m[e]) & ((1u << BITS) - 1u);
+    for (int e = 0; e < 4; ++e) {
+      const float2 x2 = ptx::unpack2(m[e]);
+      c[e] = __byte_perm(__float_as_uint(x2.x), __float_as_uint(x2.y), 0x5410) & (((1u << BITS) - 1u) * 0x00010001u);
+    }
     const uint32_t mw = (uint32_t)__bfloat16_as_ushort(sb) | ((uint32_t)__bfloat16_as_ushort(zb) << 16);
     uint32_t word = 0;
     if constexpr (BITS == 4) {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) word |= c[e] << (4 * (e >> 1) + 16 * (e & 1));
+      for (int e = 0; e < 4; ++e) word |= c[e] << (4 * e);
     } else {
       // the quad's 32 codes as four words of nibbles; lane 0 keeps the scale/offset word, lane j + 1 builds w_j
 #pragma unroll
-      for (int e = 0; e < 8; ++e) word |= c[e] << (4 * e);
+      for (int e = 0; e < 4; ++e) word |= ((c[e] & 0xffffu) | (c[e] >> 12)) << (8 * e);
       uint32_t n[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) n[i] = __shfl_sync(0xffffffffu, word, i, 4);

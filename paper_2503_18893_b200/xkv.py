@@ -301,12 +301,7 @@ def xkv_sr_reconstruct_attend_tail(grp: Group, layer_begin: int, layer_end: int,
 def xkv_quantize_rtn(x, bits: int = 4, stream=None):
     """RTN-quantise a bf16 device tensor [..., cols] along its last axis in groups of 32 (include/xkv.h).
     Returns (codes uint8 [..., cols/2], meta int32 [..., cols/32] or None for 3 bits) device tensors."""
-    *lead, cols = x.shape
-    rows = x.numel() // cols
-    codes = x.new_empty((*lead, cols // 2), dtype=torch.uint8)
-    # 4 bits: one scale/offset word per group beside the codes; 3 bits: the 16-byte records hold them (meta is None)
-    meta = x.new_empty((*lead, cols // 32), dtype=torch.int32) if bits == 4 else None
-    st = _xkv.quantize_rtn(x, rows, cols, bits, codes, meta, stream)
+    st, codes, meta = _xkv.quantize_rtn(x, bits, stream)
     if st != XKV_OK:
         raise XKVError(st, "xkv_quantize_rtn")
     return codes, meta
@@ -314,10 +309,7 @@ def xkv_quantize_rtn(x, bits: int = 4, stream=None):
 
 def xkv_dequantize_rtn(codes, meta, bits: int = 4, stream=None):
     """bf16 tensor [..., cols] of the dequantised values x_hat."""
-    *lead, half = codes.shape
-    cols, rows = half * 2, codes.numel() // half
-    x = codes.new_empty((*lead, cols), dtype=torch.bfloat16)
-    st = _xkv.dequantize_rtn(codes, meta, rows, cols, bits, x, stream)
+    st, x = _xkv.dequantize_rtn(codes, meta, bits, stream)
     if st != XKV_OK:
         raise XKVError(st, "xkv_dequantize_rtn")
     return x
