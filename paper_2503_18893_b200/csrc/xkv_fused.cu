@@ -718,7 +718,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   } else if (warp == kWarpB) {
     // =============================== B_k slab loader (TMA) ===============================
     // B slab n goes to slot n % kNB, which held slab n - kNB.  That slab's MMAs are known to be complete
-    //   - if it belongs to an earlier tile: when the previous tile's key accumulator was committed (kfull);
+    //   - if it belongs to an earlier tile: when the previous tile's key accumulator was committed (kfull); with at most two
+    //     slabs per tile, when that of the tile before it was;
     //   - if it belongs to this tile: when the key-ring pair of its stage was released.
     // In both cases the barrier's previous phase is already known to be complete and its next phase cannot
     // complete before the slab being loaded is consumed, so the parity test is unambiguous.
@@ -750,6 +751,11 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
         if (ks >= kNB || (by_pair && it > 0)) {
           const uint32_t e = (fifo >> (4 * bslot)) & 15u;
           if (!wait_bar(ctx, BAR(bl.emptyk + (int)(e & 7u)), e >> 3, 17)) { ok = false; break; }
+        } else if (2 * nks_k <= kNB) {
+          // the ring holds two tiles: slab n - kNB or a later one ends tile it-2.  Waited for at every tile, so that no phase
+          // of the barrier is skipped (a test of a phase too early passes: with one slab per tile and a first wait at the
+          // fifth tile the loader overwrote slabs in use)
+          if (it >= 2 && ks == 0 && !wait_bar(ctx, BAR(bl.kfull + (it & 1)), (uint32_t)(((it - 2) >> 1) & 1), 18)) { ok = false; break; }
         } else if (it > 0 && it * nks_k + ks >= kNB) {
           if (!wait_bar(ctx, BAR(bl.kfull + ((it - 1) & 1)), (uint32_t)(((it - 1) >> 1) & 1), 18)) { ok = false; break; }
         }
