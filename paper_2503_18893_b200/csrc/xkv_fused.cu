@@ -399,16 +399,6 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     // pairs, one tcgen05.commit per two slabs); ro: the tile rows of this thread
     auto issue_phase = [&](const uint32_t (&ro)[16], int b) {
       const char* Ab = reinterpret_cast<const char*>(Abase + (long long)b * dev.T * r) + c8 * 16u;
-      // A CTA's first tile: what its ring cannot hold yet is requested into L2 meanwhile, one 128-byte line per lane
-      if (it == 0 && RS < nst) {
-        const char* A0 = Ab - c8 * 16u;
-        for (int ks = RS + (int)c8; ks < nst; ks += 8) {
-          if (ks * 64 < r) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) prefetch_l2(A0 + (size_t)ro[i] * row_bytes + ks * 128);
-          }
-        }
-      }
 #pragma unroll 1
       for (int ks = 0; ks < nst; ks += 2) {
         const int pr = slot >> 1;
@@ -718,8 +708,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   } else if (warp == kWarpB) {
     // =============================== B_k slab loader (TMA) ===============================
     // B slab n goes to slot n % kNB, which held slab n - kNB.  That slab's MMAs are known to be complete
-    //   - if it belongs to an earlier tile: when the previous tile's key accumulator was committed (kfull); with at most two
-    //     slabs per tile, when that of the tile before it was;
+    //   - if it belongs to an earlier tile: when the previous tile's key accumulator was committed (kfull); with one slab
+    //     per tile, when that of the tile before it was;
     //   - if it belongs to this tile: when the key-ring pair of its stage was released.
     // In both cases the barrier's previous phase is already known to be complete and its next phase cannot
     // complete before the slab being loaded is consumed, so the parity test is unambiguous.
@@ -751,11 +741,11 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
         if (ks >= kNB || (by_pair && it > 0)) {
           const uint32_t e = (fifo >> (4 * bslot)) & 15u;
           if (!wait_bar(ctx, BAR(bl.emptyk + (int)(e & 7u)), e >> 3, 17)) { ok = false; break; }
-        } else if (2 * nks_k <= kNB) {
-          // the ring holds two tiles: slab n - kNB or a later one ends tile it-2.  Waited for at every tile, so that no phase
-          // of the barrier is skipped (a test of a phase too early passes: with one slab per tile and a first wait at the
-          // fifth tile the loader overwrote slabs in use)
-          if (it >= 2 && ks == 0 && !wait_bar(ctx, BAR(bl.kfull + (it & 1)), (uint32_t)(((it - 2) >> 1) & 1), 18)) { ok = false; break; }
+        } else if (nks_k == 1) {
+          // slab n - kNB belongs to tile it-4.  Tile it-2 is waited for, and at every tile, so that no phase of the barrier
+          // is skipped (a test of a phase too early passes: with a first wait at the fifth tile the loader overwrote slabs in
+          // use)
+          if (it >= 2 && !wait_bar(ctx, BAR(bl.kfull + (it & 1)), (uint32_t)(((it - 2) >> 1) & 1), 18)) { ok = false; break; }
         } else if (it > 0 && it * nks_k + ks >= kNB) {
           if (!wait_bar(ctx, BAR(bl.kfull + ((it - 1) & 1)), (uint32_t)(((it - 1) >> 1) & 1), 18)) { ok = false; break; }
         }

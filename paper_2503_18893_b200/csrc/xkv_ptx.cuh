@@ -241,9 +241,6 @@ __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepco
 // once every CTA of this grid has passed this point or exited.
 __device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Requests the 128-byte line at `p` into L2.
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-
 __device__ __forceinline__ void named_bar_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
