@@ -884,7 +884,9 @@ static cudaError_t launch_topk(const GroupDev& dev, int device, int problems, in
   // chunks (a short context needs fewer barriers' worth of warps, and several of its CTAs share an SM); groups per
   // thread: the fewest with at least k_ch groups in all (0 = no filter)
   const int items = dev.n_c <= kTopkThreads * 16 ? 16 : 32;
-  const int th = items == 32 ? 1024 : (dev.n_c <= 128 * 16 ? 128 : dev.n_c <= 256 * 16 ? 256 : dev.n_c <= 512 * 16 ? 512 : 1024);
+  auto groups = [&](int gpt) { return (dev.n_c + items / gpt - 1) / (items / gpt); };
+  int th = items == 32 ? 1024 : (dev.n_c <= 128 * 16 ? 128 : dev.n_c <= 256 * 16 ? 256 : dev.n_c <= 512 * 16 ? 512 : 1024);
+  if (groups(4) < k_ch && th < 512) th *= 2;       // no filter: every key is listed, more threads pay
   const size_t smem = (size_t)th * items * (sizeof(uint32_t) + sizeof(uint16_t));
   cudaError_t e;
 #define XKV_PIVOT(GPT, ITEMS, TH)                                                                                     \
@@ -901,7 +903,6 @@ static cudaError_t launch_topk(const GroupDev& dev, int device, int problems, in
     else if (groups(4) >= k_ch) XKV_PIVOT(4, ITEMS, TH);                                                              \
     else XKV_PIVOT(0, ITEMS, TH);                                                                                     \
   } while (0)
-  auto groups = [&](int gpt) { return (dev.n_c + items / gpt - 1) / (items / gpt); };
   if (items == 32) XKV_PIVOT_G(32, 1024);
   else if (th == 128) XKV_PIVOT_G(16, 128);
   else if (th == 256) XKV_PIVOT_G(16, 256);
