@@ -2,8 +2,9 @@
 // only).  A decode step is a handful of kernels of a few microseconds each, so what a call costs on the host is part
 // of its latency: through ctypes and torch.cuda.current_stream() a call spent 4.5 us before its first launch, here
 // 0.7 us.  The quantiser's calls, whose kernels take as long as their launches, allocate their results here too (10.5 us of
-// host time for a pair of torch.empty and a launch through Python, 5 us here).  Tensor arguments are anything with a data_ptr() method (or None, or an integer address); a stream is None
-// (torch's current one), an integer, or an object with a cuda_stream attribute.  Every function returns the status.
+// host time for a pair of torch.empty and a launch through Python, 5 us here).  Tensor arguments are anything with a
+// data_ptr() method (or None, or an integer address); a stream is None (torch's current one), an integer, or an object
+// with a cuda_stream attribute.  Every function returns the status.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
