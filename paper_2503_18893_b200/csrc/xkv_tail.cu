@@ -6,7 +6,7 @@
 // (thread = tail row for the logits, thread = output column for the weighted sum of value rows), used for
 // d_h = 64 and when the handle was created with XKV_TAIL_IMPL=c.
 //
-// `behind`: the kernel is launched behind the fused kernel, whose results it does not need.  It starts on the SMs that the
+// BEHIND: the kernel is launched behind the fused kernel, whose results it does not need.  It starts on the SMs that the
 // fused kernel leaves idle or leaves early, reads at once (its inputs come from before the fused kernel, which waits for
 // everything before it before it lets this one start) and waits for the fused kernel only before it ends, so that the
 // merge behind it finds both complete.  In front of the fused kernel it is one more link of the chain: a step of 121873
@@ -35,11 +35,11 @@ constexpr size_t tail_smem_bytes() {
   return (size_t)kTailThreads * tail_k_stride<DH>() + (size_t)kTailThreads * DH * 2 + sizeof(float) * (NR * DH + NR * kTailThreads);
 }
 
-template <int DH, int NR>
+template <int DH, int NR, bool BEHIND>
 __global__ void __launch_bounds__(kTailThreads)
 tail_partial_kernel(GroupDev dev, int l0, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ tail_k,
                     const __nv_bfloat16* __restrict__ tail_v, const int32_t* __restrict__ tail_len, int tail_cap,
-                    int n_split, float* __restrict__ part, int behind) {
+                    int n_split, float* __restrict__ part) {
   static_assert(kTailSplitRows == kTailThreads, "one tile per CTA");
   extern __shared__ __align__(16) uint8_t tail_smem[];
   constexpr int KS = tail_k_stride<DH>();
@@ -56,7 +56,7 @@ tail_partial_kernel(GroupDev dev, int l0, const __nv_bfloat16* __restrict__ q, c
   const int g = py % dev.H_kv, b = (py / dev.H_kv) % dev.batch, l = l0 + py / per_layer;
   const float scale2 = dev.att_scale * kLog2e;
 
-  if (!behind) ptx::grid_dependency_wait();            // q (and the tail rows) may come from the kernel before
+  if constexpr (!BEHIND) ptx::grid_dependency_wait();  // q (and the tail rows) may come from the kernel before
   ptx::grid_dependency_launch();
   int len = tail_len ? tail_len[b] : tail_cap;
   if (len < 0 || len > tail_cap) {
@@ -201,7 +201,7 @@ tail_partial_kernel(GroupDev dev, int l0, const __nv_bfloat16* __restrict__ q, c
       }
     }
   }
-  if (behind) ptx::grid_dependency_wait();
+  if constexpr (BEHIND) ptx::grid_dependency_wait();
 }
 
 
@@ -227,11 +227,11 @@ __device__ __forceinline__ bool tc_wait_bounded(uint32_t bar, uint32_t parity) {
   return false;
 }
 
-template <int NR>
+template <int NR, bool BEHIND>
 __global__ void __launch_bounds__(kTailThreads)
 tail_tc_kernel(GroupDev dev, int l0, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ tail_k,
                const __nv_bfloat16* __restrict__ tail_v, const int32_t* __restrict__ tail_len, int tail_cap,
-               int n_split, int tiles_per_split, float* __restrict__ part, int behind) {
+               int n_split, int tiles_per_split, float* __restrict__ part) {
   using namespace ptx;
   constexpr int DH = 128;
   extern __shared__ uint8_t tc_smem[];
@@ -268,7 +268,7 @@ tail_tc_kernel(GroupDev dev, int l0, const __nv_bfloat16* __restrict__ q, const 
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (!behind) grid_dependency_wait();                 // q (and the tail rows) may come from the kernel before
+  if constexpr (!BEHIND) grid_dependency_wait();       // q (and the tail rows) may come from the kernel before
   grid_dependency_launch();
   int len = tail_len ? tail_len[b] : tail_cap;
   if (len < 0 || len > tail_cap) {
@@ -445,7 +445,7 @@ tail_tc_kernel(GroupDev dev, int l0, const __nv_bfloat16* __restrict__ q, const 
     tc_fence_after();
     tmem_dealloc(tmem, 32);
   }
-  if (behind) grid_dependency_wait();
+  if constexpr (BEHIND) grid_dependency_wait();
 }
 
 // Merge of dense-attention partials (xkv_dense_attend): one CTA per (problem, query head); the splits are
@@ -531,20 +531,22 @@ cudaError_t launch_tail_partials(const xkv_group* grp, int l0, int l1, const __n
   const dim3 grid(problems, n_split), block(kTailThreads);
   // only the tensor-core kernel walks several tiles per CTA
   if (tps > 1 && !(dev.d_h == 128 && !grp->tail_impl)) return cudaErrorInvalidValue;
-#define XKV_TAIL(DH, NR)                                                                                            \
+#define XKV_TAIL_AT(DH, NR, BEHIND)                                                                                  \
   do {                                                                                                              \
-    e = ensure_dyn_smem<tail_partial_kernel<DH, NR>>(tail_smem_bytes<DH, NR>(), grp->device);                       \
+    e = ensure_dyn_smem<tail_partial_kernel<DH, NR, BEHIND>>(tail_smem_bytes<DH, NR>(), grp->device);                \
     if (e == cudaSuccess)                                                                                           \
-      e = launch_pdl(tail_partial_kernel<DH, NR>, grid, block, tail_smem_bytes<DH, NR>(), s, dev, l0, q, tail_k,     \
-                     tail_v, tail_len, tail_cap, n_split, part, behind ? 1 : 0);                                    \
+      e = launch_pdl(tail_partial_kernel<DH, NR, BEHIND>, grid, block, tail_smem_bytes<DH, NR>(), s, dev, l0, q,     \
+                     tail_k, tail_v, tail_len, tail_cap, n_split, part);                                            \
   } while (0)
-#define XKV_TAIL_TC(NR)                                                                                            \
+#define XKV_TAIL_TC_AT(NR, BEHIND)                                                                                   \
   do {                                                                                                              \
-    e = ensure_dyn_smem<tail_tc_kernel<NR>>(tail_tc_smem_bytes<NR>(), grp->device);                                 \
+    e = ensure_dyn_smem<tail_tc_kernel<NR, BEHIND>>(tail_tc_smem_bytes<NR>(), grp->device);                          \
     if (e == cudaSuccess)                                                                                           \
-      e = launch_pdl(tail_tc_kernel<NR>, grid, block, tail_tc_smem_bytes<NR>(), s, dev, l0, q, tail_k, tail_v,       \
-                     tail_len, tail_cap, n_split, tps, part, behind ? 1 : 0);                                       \
+      e = launch_pdl(tail_tc_kernel<NR, BEHIND>, grid, block, tail_tc_smem_bytes<NR>(), s, dev, l0, q, tail_k,       \
+                     tail_v, tail_len, tail_cap, n_split, tps, part);                                               \
   } while (0)
+#define XKV_TAIL(DH, NR) do { if (behind) XKV_TAIL_AT(DH, NR, true); else XKV_TAIL_AT(DH, NR, false); } while (0)
+#define XKV_TAIL_TC(NR) do { if (behind) XKV_TAIL_TC_AT(NR, true); else XKV_TAIL_TC_AT(NR, false); } while (0)
   if (dev.d_h == 128 && !grp->tail_impl) {
     if (dev.n_rep <= 4) XKV_TAIL_TC(4); else if (dev.n_rep <= 8) XKV_TAIL_TC(8); else XKV_TAIL_TC(16);
   } else if (dev.d_h == 128) {
@@ -554,6 +556,8 @@ cudaError_t launch_tail_partials(const xkv_group* grp, int l0, int l1, const __n
   }
 #undef XKV_TAIL
 #undef XKV_TAIL_TC
+#undef XKV_TAIL_AT
+#undef XKV_TAIL_TC_AT
   count_launch((dev.d_h == 128 && !grp->tail_impl) ? kFamTailTc : kFamTailCuda);
   return e;
 }
