@@ -7,7 +7,8 @@
 //                         U   = X^T Y     (N x l, fp32)          tensor core
 //                         Z   = U R^-1,  R^T R = U^T U + shift I (shifted Cholesky QR in fp64: one pass inside the
 //                               iteration, three for the last iterate, which has to be orthonormal)
-//   Rayleigh-Ritz:        W^T = Z^T X^T,  M = W^T W (= Z^T X^T X Z, l x l),  M = P Lambda P^T (Jacobi)
+//   Rayleigh-Ritz:        W^T = Z^T X^T,  M = W^T W (= Z^T X^T X Z, l x l),  M = P Lambda P^T (Jacobi); Z as the sum of two
+//                         bf16 matrices here
 //   V = Z P_r (N x r);    B_l = rows of V^T (bf16);   A = X V_bf16 (T x r, tensor core);   sigma = sqrt(Lambda).
 // A = U Sigma and B = V^T of the truncated SVD of X, up to the accuracy of the subspace (checked against the exact
 // optimum sum_{i>r} sigma_i^2, never factor by factor: signs and degenerate subspaces are not unique).
@@ -50,11 +51,12 @@ __device__ __forceinline__ bool gemm_wait(uint32_t bar, uint32_t parity) {
 
 // C[m][n] = sum_k A(k, m) B(k, n).  grid = (ceil(N/BN), ceil(M/(128 MB)), K ranges).  TRANS: store C^T (out[n][m]).
 // AK: A is given as [m][k] (K-major), else as [k][m]; BK likewise for B.  K range z covers k_per columns and writes
-// Cf + z * M * ldc.  Out-of-range rows and columns of the operands are zero-filled by the copy engine; stores are guarded.
+// Cf + z * M * ldc.  A may hold a_k < K of the k only (a multiple of 64, K = 2 a_k): it is then gone through twice, for a B
+// that is a sum of two matrices, one below the other.  Out-of-range rows and columns of the operands are zero-filled by the copy engine; stores are guarded.
 template <bool TRANS, bool AK, bool BK, int MB, int BN>
 __global__ void __launch_bounds__(gemm_threads<MB>(), 1)
 clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M, int N, int K,
-                int k_per, float* __restrict__ Cf, __nv_bfloat16* __restrict__ Cb, long long ldc, unsigned int* __restrict__ flags) {
+                int a_k, int k_per, float* __restrict__ Cf, __nv_bfloat16* __restrict__ Cb, long long ldc, unsigned int* __restrict__ flags) {
   extern __shared__ uint8_t gemm_smem[];
   constexpr int kGemmStages = gemm_stages<MB, BN>(), kGemmStageBytes = gemm_stage_bytes<MB, BN>();
   constexpr uint32_t kAccCols = BN <= 128 ? 128u : 256u, kCols = MB * kAccCols;      // tensor-memory columns
@@ -94,13 +96,13 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         if (kb >= kGemmStages && !gemm_wait(EMPTY(s), (uint32_t)((kb / kGemmStages - 1) & 1))) { ok = false; break; }
         const uint32_t st = base + (uint32_t)s * kGemmStageBytes;
         mbar_expect_tx(FULL(s), kGemmStageBytes);
-        const int k = k_first + kb * 64;
+        const int k = k_first + kb * 64, ka = k < a_k ? k : k - a_k;
         // K-major: one box of 64 k by all rows; MN-major: slabs of 64 columns by 64 k, 8 KB each
         if (AK) {
-          tma_load_2d(st, &map_a, k, m0, FULL(s));
+          tma_load_2d(st, &map_a, ka, m0, FULL(s));
         } else {
 #pragma unroll
-          for (int i = 0; i < 2 * MB; ++i) tma_load_2d(st + i * 8192, &map_a, m0 + i * 64, k, FULL(s));
+          for (int i = 0; i < 2 * MB; ++i) tma_load_2d(st + i * 8192, &map_a, m0 + i * 64, ka, FULL(s));
         }
         if (BK) {
           tma_load_2d(st + kOffB, &map_b, k, n0, FULL(s));
@@ -517,7 +519,8 @@ chol_inverse_kernel(const double* __restrict__ part, int n_part, double* __restr
 }
 
 // Z (n x l) = U W^T for the lower-triangular W = L^-1 (fp64): 64 x 64 tiles, tile column J takes the first J + 1 blocks of
-// 64.  Longest tiles first.  Also writes the bf16 copy the tensor-core products read.  (The blocked triangular solve that
+// 64.  Longest tiles first.  Also writes the bf16 copy the tensor-core products read, and behind it (n rows on) the bf16 of
+// what the copy leaves out.  (The blocked triangular solve that
 // kept 32 rows of Z in shared memory took 161 us and 69 us for the inverses of its diagonal blocks at 4096 x 576; this
 // product 59 us.)
 __global__ void __launch_bounds__(256)
@@ -583,7 +586,10 @@ tri_product_kernel(const float* __restrict__ U, const double* __restrict__ W, fl
       if (r < n) {
         const float z0 = (float)acc[i][j][0], z1 = (float)acc[i][j][1];
         *reinterpret_cast<float2*>(Z + (size_t)r * l + c) = make_float2(z0, z1);
-        *reinterpret_cast<__nv_bfloat162*>(Zb + (size_t)r * l + c) = __floats2bfloat162_rn(z0, z1);
+        const __nv_bfloat162 hi = __floats2bfloat162_rn(z0, z1);
+        const float2 h = __bfloat1622float2(hi);
+        *reinterpret_cast<__nv_bfloat162*>(Zb + (size_t)r * l + c) = hi;
+        *reinterpret_cast<__nv_bfloat162*>(Zb + (size_t)(n + r) * l + c) = __floats2bfloat162_rn(z0 - h.x, z1 - h.y);
       }
     }
 }
@@ -1019,7 +1025,7 @@ bool make_plan(const xkv_clf_config* c, ClfPlan* p) {
   if (p->l < c->r || p->l < 64 || p->l / 2 > kJacobiMaxPairs) return false;
   size_t o = 0;
   p->off_flags = o; o = align_up(o + 256);
-  p->off_zb = o; o = align_up(o + (size_t)p->N * p->l * 2);
+  p->off_zb = o; o = align_up(o + (size_t)2 * p->N * p->l * 2);  // Z as two bf16 matrices, one below the other
   p->off_yt = o; o = align_up(o + (size_t)p->l * p->Tp * 2);
   p->u_split = gemm_splits(p->N, p->l, p->T, 8);
   p->off_up = o; if (p->u_split > 1) o = align_up(o + (size_t)p->u_split * p->N * p->l * 4);   // partial sums of U
@@ -1072,7 +1078,7 @@ struct GemmOut {
 
 template <bool TRANS, bool AK, bool BK, int MB, int BN>
 cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, int splits, GemmOut c, unsigned int* flags, int device, cudaStream_t s) {
-  const int M = AK ? a.rows : a.cols, N = BK ? b.rows : b.cols, K = AK ? a.cols : a.rows;
+  const int M = AK ? a.rows : a.cols, N = BK ? b.rows : b.cols, K = BK ? b.cols : b.rows, a_k = AK ? a.cols : a.rows;
   CUtensorMap ma, mb;
   if (!encode_bf16_map(&ma, a.p, (uint64_t)a.rows, (uint64_t)a.cols, (uint64_t)a.pitch, AK ? 128 * MB : 64) ||
       !encode_bf16_map(&mb, b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BK ? BN : 64))
@@ -1082,7 +1088,7 @@ cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, int splits, GemmOut c, 
   if (e != cudaSuccess) return e;
   const int k_per = ((K + splits - 1) / splits + 63) & ~63;
   const dim3 grid((N + BN - 1) / BN, (M + 128 * MB - 1) / (128 * MB), splits);
-  clf_gemm_kernel<TRANS, AK, BK, MB, BN><<<grid, gemm_threads<MB>(), smem, s>>>(ma, mb, M, N, K, k_per, c.f, c.b, c.ld, flags);
+  clf_gemm_kernel<TRANS, AK, BK, MB, BN><<<grid, gemm_threads<MB>(), smem, s>>>(ma, mb, M, N, K, a_k, k_per, c.f, c.b, c.ld, flags);
   count_launch(kFamClf);
   return cudaGetLastError();
 }
@@ -1186,8 +1192,10 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
   cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 256, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(Zb, omega, (size_t)N * l * 2, cudaMemcpyDeviceToDevice, s);
-  // Y = X Z (stored as Y^T)  and  U = X^T Y
-  auto product_y = [&]() { return launch_gemm<true, true, false>({X, T, N, N}, {Zb, N, l, l}, 1, {nullptr, Yt, p.Tp}, flags, device, s); };
+  // Y = X Z (stored as Y^T), Z rounded to bf16 or as both of its parts,  and  U = X^T Y
+  auto product_y = [&](int parts) {
+    return launch_gemm<true, true, false>({X, T, N, N}, {Zb, parts * N, l, l}, 1, {nullptr, Yt, p.Tp}, flags, device, s);
+  };
   auto product_u = [&]() -> cudaError_t {
     float* out = p.u_split > 1 ? (float*)(w + p.off_up) : U;
     cudaError_t e2 = launch_gemm<false, false, true>({X, T, N, N}, {Yt, l, T, p.Tp}, p.u_split, {out, nullptr, l}, flags, device, s);
@@ -1227,12 +1235,15 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
     return cudaGetLastError();
   };
   for (int it = 0; it <= p.q && e == cudaSuccess; ++it) {
-    e = product_y();
+    e = product_y(1);
     if (e == cudaSuccess) e = product_u();
     if (e == cudaSuccess) e = cholqr(it == p.q ? 3 : 1);
   }
-  // Rayleigh-Ritz: W = X Z, M = W^T W (= Z^T X^T X Z), its eigenvectors by Jacobi
-  if (e == cudaSuccess) e = product_y();
+  // Rayleigh-Ritz: W = X Z, M = W^T W (= Z^T X^T X Z), its eigenvectors by Jacobi.  M is that of the fp32 Z whose
+  // combinations become V, so Z's rounding to bf16 must not enter: a column in the noise floor, rounded, holds a part of
+  // 2^-9 of the largest singular values (error of M_ij relative to sqrt(M_ii M_jj), rms: 1e-2 with the rounded Z on both
+  // sides, 3e-3 as Z^T X^T (X Z_bf16), 1e-5 to 4e-5 this way; the rounding of W itself averages out over the T rows).
+  if (e == cudaSuccess) e = product_y(2);
   if (e == cudaSuccess) e = launch_gemm<false, true, true>({Yt, l, T, p.Tp}, {Yt, l, T, p.Tp}, p.ritz_split, {(float*)part, nullptr, l}, flags, device, s);
   if (e == cudaSuccess) {
     symmetrize_kernel<<<(l * l + 255) / 256, 256, 0, s>>>((const float*)part, p.ritz_split, Mm, l);

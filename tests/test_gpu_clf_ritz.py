@@ -1,0 +1,34 @@
+"""The Rayleigh-Ritz step of the factorisation: the rows of B are the Ritz vectors of their own span, as good as bf16 can
+hold them.  The measure is the off-diagonal part of V^T X^T X V, relative to the diagonal; exact Ritz vectors rounded to bf16
+set the scale (a rounded noise direction holds 2^-9 of the largest singular values), and an error of the l x l matrix or of
+its eigenvectors adds to it."""
+import pytest
+import torch
+
+from tests.test_gpu_clf import _factorize_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def _off_diagonal(H, V):
+    M = V.T @ H @ V
+    d = M.diagonal().sqrt()
+    M = M / d[:, None] / d[None, :]
+    return float((M - torch.diag(M.diagonal())).pow(2).mean().sqrt())
+
+
+@pytest.mark.parametrize("T,G,d,r", [(4096, 4, 256, 128), (3001, 2, 320, 200), (20000, 4, 128, 64)])
+def test_rows_of_b_are_ritz_vectors_to_bf16(T, G, d, r):
+    g = torch.Generator(device="cuda").manual_seed(T)
+    N, rho = G * d, r // 2
+    s = 1.0 / torch.arange(1, rho + 1, device="cuda")
+    signal = (torch.randn(T, rho, generator=g, device="cuda") * s) @ torch.randn(rho, N, generator=g, device="cuda")
+    X = (signal / signal.std() + 0.01 * torch.randn(T, N, generator=g, device="cuda")).to(torch.bfloat16)
+    A, B, sig, _ = _factorize_gpu(X, G, d, r, 32, 2, seed=7)
+    Xd = X.double()
+    H = Xd.T @ Xd
+    V = torch.cat([B[i] for i in range(G)], dim=1).double().T                # (N, r)
+    Q = torch.linalg.qr(V)[0]
+    exact = Q @ torch.linalg.eigh(Q.T @ H @ Q)[1]
+    rounded = exact.to(torch.bfloat16).double()
+    assert _off_diagonal(H, V) <= 1.2 * _off_diagonal(H, rounded)
