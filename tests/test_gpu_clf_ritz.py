@@ -32,3 +32,27 @@ def test_rows_of_b_are_ritz_vectors_to_bf16(T, G, d, r):
     exact = Q @ torch.linalg.eigh(Q.T @ H @ Q)[1]
     rounded = exact.to(torch.bfloat16).double()
     assert _off_diagonal(H, V) <= 1.2 * _off_diagonal(H, rounded)
+
+
+@pytest.mark.parametrize("T,N,r", [(4096, 640, 608), (2500, 192, 136)])
+def test_rotations_keep_the_length(T, N, r):
+    """With l = N the sketch holds everything and a flat spectrum takes the most sweeps; the singular values are those of X
+    up to the drift of the eigenvectors' length.  A vector takes part in l - 1 rotations of a sweep; with c and s rounded to
+    nearest c^2 + s^2 is off by 2^-23 and the length by 2^-24 at most, with no preferred sign: a quarter of that is allowed
+    as a bias.  (The rounding of X Z to bf16 has none: 1e-6 in the mean.)"""
+    from paper_2503_18893_b200 import xkv
+    g = torch.Generator(device="cuda").manual_seed(N)
+    X = torch.randn(T, N, generator=g, device="cuda").to(torch.bfloat16)
+    cfg = xkv.make_clf_config(T=T, G=1, d=N, r=r, oversample=32, power_iters=1)
+    assert xkv.xkv_clf_rank_l(cfg) == N
+    omega = torch.randn(N, N, generator=g, device="cuda").to(torch.bfloat16)
+    ws = torch.empty(xkv.xkv_clf_workspace_bytes(cfg), dtype=torch.uint8, device="cuda")
+    A = torch.empty((T, r), dtype=torch.bfloat16, device="cuda")
+    B = torch.empty((1, r, N), dtype=torch.bfloat16, device="cuda")
+    sig = torch.empty(r, dtype=torch.float32, device="cuda")
+    xkv.xkv_clf_factorize(cfg, X, omega, ws, A, B, sig)
+    assert xkv.xkv_clf_status(ws) == (0, 0)
+    sweeps = int(ws[44:48].view(torch.int32))
+    sv = torch.linalg.svdvals(X.double())[:r]
+    drift = (sig.double() / sv - 1).mean().abs()
+    assert drift <= (N - 1) * sweeps * 2.0 ** -26 + 2e-6
