@@ -12,6 +12,7 @@
 
 #include <ATen/core/Tensor.h>
 #include <ATen/ops/empty.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "xkv.h"
@@ -185,18 +186,15 @@ PyObject* quantize_rtn(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
   const int bits = a.i32();
   void* s = a.stream();
   if (a.bad) return nullptr;
-  try {
-    const int64_t cols = x->size(-1), rows = cols ? x->numel() / cols : 0;
-    at::Tensor codes = like(*x, cols / 2, at::kByte), meta;
-    // 4 bits: one scale/offset word per group beside the codes; 3 bits: the 16-byte records hold them
-    if (bits == 4) meta = like(*x, cols / 32, at::kInt);
-    const int st = xkv_quantize_rtn(x->const_data_ptr(), rows, cols > INT32_MAX ? 0 : (int)cols, bits, codes.mutable_data_ptr(),
-                                    bits == 4 ? meta.mutable_data_ptr() : nullptr, s);
-    return Py_BuildValue("iNN", st, THPVariable_Wrap(codes), bits == 4 ? THPVariable_Wrap(meta) : Py_NewRef(Py_None));
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
-  }
+  HANDLE_TH_ERRORS
+  const int64_t cols = x->size(-1), rows = cols ? x->numel() / cols : 0;
+  at::Tensor codes = like(*x, cols / 2, at::kByte), meta;
+  // 4 bits: one scale/offset word per group beside the codes; 3 bits: the 16-byte records hold them
+  if (bits == 4) meta = like(*x, cols / 32, at::kInt);
+  const int st = xkv_quantize_rtn(x->const_data_ptr(), rows, cols > INT32_MAX ? 0 : (int)cols, bits, codes.mutable_data_ptr(),
+                                  bits == 4 ? meta.mutable_data_ptr() : nullptr, s);
+  return Py_BuildValue("iNN", st, THPVariable_Wrap(codes), bits == 4 ? THPVariable_Wrap(meta) : Py_NewRef(Py_None));
+  END_HANDLE_TH_ERRORS
 }
 
 // dequantize_rtn(codes, meta, bits, stream) -> (status, x)
@@ -208,16 +206,13 @@ PyObject* dequantize_rtn(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
   const int bits = a.i32();
   void* s = a.stream();
   if (a.bad) return nullptr;
-  try {
-    const int64_t half = codes->size(-1), rows = half ? codes->numel() / half : 0;
-    at::Tensor x = like(*codes, half * 2, at::kBFloat16);
-    const int st = xkv_dequantize_rtn(codes->const_data_ptr(), meta, rows, half > INT32_MAX / 2 ? 0 : (int)(half * 2), bits,
-                                      x.mutable_data_ptr(), s);
-    return Py_BuildValue("iN", st, THPVariable_Wrap(x));
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
-  }
+  HANDLE_TH_ERRORS
+  const int64_t half = codes->size(-1), rows = half ? codes->numel() / half : 0;
+  at::Tensor x = like(*codes, half * 2, at::kBFloat16);
+  const int st = xkv_dequantize_rtn(codes->const_data_ptr(), meta, rows, half > INT32_MAX / 2 ? 0 : (int)(half * 2), bits,
+                                    x.mutable_data_ptr(), s);
+  return Py_BuildValue("iN", st, THPVariable_Wrap(x));
+  END_HANDLE_TH_ERRORS
 }
 
 // torch_hooks(get_device, get_current_raw_stream): how "the current stream" is found.
