@@ -164,6 +164,16 @@ XKV_PY(dense_attend, 13)
   void* s = a.stream();
 XKV_PY_END(xkv_dense_attend(g, l0, l1, q, K, V, len, cap, ws, ws_bytes, out, lse, s))
 
+// The interpreter lock is given back for a scope: an allocation or a launch may wait for the device (a full launch queue),
+// and the device for another Python thread.
+struct WithoutGil {
+  PyThreadState* state = PyEval_SaveThread();
+  WithoutGil() = default;
+  WithoutGil(const WithoutGil&) = delete;
+  WithoutGil& operator=(const WithoutGil&) = delete;
+  ~WithoutGil() { PyEval_RestoreThread(state); }
+};
+
 // An uninitialised tensor of x's device with x's leading sizes and `last` columns.
 at::Tensor like(const at::Tensor& x, int64_t last, at::ScalarType type) {
   c10::DimVector sizes(x.sizes().begin(), x.sizes().end());
@@ -187,12 +197,17 @@ PyObject* quantize_rtn(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
   void* s = a.stream();
   if (a.bad) return nullptr;
   HANDLE_TH_ERRORS
-  const int64_t cols = x->size(-1), rows = cols ? x->numel() / cols : 0;
-  at::Tensor codes = like(*x, cols / 2, at::kByte), meta;
-  // 4 bits: one scale/offset word per group beside the codes; 3 bits: the 16-byte records hold them
-  if (bits == 4) meta = like(*x, cols / 32, at::kInt);
-  const int st = xkv_quantize_rtn(x->const_data_ptr(), rows, cols > INT32_MAX ? 0 : (int)cols, bits, codes.mutable_data_ptr(),
-                                  bits == 4 ? meta.mutable_data_ptr() : nullptr, s);
+  at::Tensor codes, meta;
+  int st;
+  {
+    const WithoutGil no_gil;
+    const int64_t cols = x->size(-1), rows = cols ? x->numel() / cols : 0;
+    codes = like(*x, cols / 2, at::kByte);
+    // 4 bits: one scale/offset word per group beside the codes; 3 bits: the 16-byte records hold them
+    if (bits == 4) meta = like(*x, cols / 32, at::kInt);
+    st = xkv_quantize_rtn(x->const_data_ptr(), rows, cols > INT32_MAX ? 0 : (int)cols, bits, codes.mutable_data_ptr(),
+                          bits == 4 ? meta.mutable_data_ptr() : nullptr, s);
+  }
   return Py_BuildValue("iNN", st, THPVariable_Wrap(codes), bits == 4 ? THPVariable_Wrap(meta) : Py_NewRef(Py_None));
   END_HANDLE_TH_ERRORS
 }
@@ -207,10 +222,15 @@ PyObject* dequantize_rtn(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
   void* s = a.stream();
   if (a.bad) return nullptr;
   HANDLE_TH_ERRORS
-  const int64_t half = codes->size(-1), rows = half ? codes->numel() / half : 0;
-  at::Tensor x = like(*codes, half * 2, at::kBFloat16);
-  const int st = xkv_dequantize_rtn(codes->const_data_ptr(), meta, rows, half > INT32_MAX / 2 ? 0 : (int)(half * 2), bits,
-                                    x.mutable_data_ptr(), s);
+  at::Tensor x;
+  int st;
+  {
+    const WithoutGil no_gil;
+    const int64_t half = codes->size(-1), rows = half ? codes->numel() / half : 0;
+    x = like(*codes, half * 2, at::kBFloat16);
+    st = xkv_dequantize_rtn(codes->const_data_ptr(), meta, rows, half > INT32_MAX / 2 ? 0 : (int)(half * 2), bits,
+                            x.mutable_data_ptr(), s);
+  }
   return Py_BuildValue("iN", st, THPVariable_Wrap(x));
   END_HANDLE_TH_ERRORS
 }
