@@ -3,8 +3,8 @@
 // of its latency: through ctypes and torch.cuda.current_stream() a call spent 4.5 us before its first launch, here
 // 0.7 us.  The quantiser's calls, whose kernels take as long as their launches, allocate their results here too (10.5 us of
 // host time for a pair of torch.empty and a launch through Python, 5 us here).  Tensor arguments are anything with a
-// data_ptr() method (or None, or an integer address); a stream is None (torch's current one), an integer, or an object
-// with a cuda_stream attribute.  Every function returns the status.
+// data_ptr() method (or None, or an integer address); a stream is None (torch's current one), an object with a
+// cuda_stream attribute, or something that int() takes.  Every function returns the status.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -76,6 +76,10 @@ struct Args {
       Py_DECREF(dev);
     } else {
       r = PyObject_GetAttr(o, s_cuda_stream);
+      if (!r && PyErr_ExceptionMatches(PyExc_AttributeError)) {      // anything int() takes, such as numpy's integers
+        PyErr_Clear();
+        r = PyNumber_Long(o);
+      }
     }
     if (!r) { bad = true; return nullptr; }
     void* p = address(r);

@@ -23,3 +23,15 @@ def test_an_error_of_the_allocation_keeps_its_type(error):
     for call in (lambda: xkv._xkv.quantize_rtn(x, 4, 0), lambda: xkv._xkv.dequantize_rtn(codes, meta, 4, 0)):
         with _Refuse(error), pytest.raises(type(error)):
             call()
+
+
+@pytest.mark.parametrize("stream", [0, np.int64(0), np.uint64(0), True])
+def test_streams_that_convert_to_an_integer(stream):
+    # no handle: the call is refused by the library, after its arguments have been converted
+    assert xkv._xkv.sr_select(0, 0, 1, None, 8, None, None, stream) == xkv.XKV_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("stream", ["0x10", object(), 1.5j])
+def test_streams_that_are_none(stream):
+    with pytest.raises((TypeError, ValueError)):
+        xkv._xkv.sr_select(0, 0, 1, None, 8, None, None, stream)
