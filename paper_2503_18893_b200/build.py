@@ -34,12 +34,21 @@ def sources():
     return sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cu"))
 
 
+def _module_command() -> list:
+    from torch.utils import cpp_extension      # (its libraries are loaded by `import torch` before the module is)
+    return ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I", os.path.join(ROOT, "include"),
+            "-I", sysconfig.get_paths()["include"], *("-isystem" + p for p in cpp_extension.include_paths()),
+            os.path.join(CSRC, "xkv_py.cpp"), "-o", PYMOD, "-L", HERE, "-lxkv", "-Wl,-rpath,$ORIGIN",
+            *("-L" + p for p in cpp_extension.library_paths()), "-ltorch_python", "-ltorch_cpu", "-lc10"]
+
+
 def _stamp() -> str:
+    import torch                               # the module is bound to torch's C++ interface
     h = hashlib.sha256()
     for f in sorted(os.listdir(CSRC)) + ["../../include/xkv.h"]:
         with open(os.path.join(CSRC, f), "rb") as fh:
             h.update(f.encode() + b"\0" + fh.read())
-    h.update(" ".join(NVCC_FLAGS + [sysconfig.get_paths()["include"]]).encode())
+    h.update(" ".join(NVCC_FLAGS + _module_command() + [torch.__version__]).encode())
     return h.hexdigest()
 
 
@@ -73,12 +82,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
     if r.returncode != 0:
         sys.stderr.write(r.stdout + r.stderr)
         raise RuntimeError("link failed")
-    from torch.utils import cpp_extension      # (its libraries are loaded by `import torch` before the module is)
-    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I", os.path.join(ROOT, "include"),
-           "-I", sysconfig.get_paths()["include"], *("-isystem" + p for p in cpp_extension.include_paths()),
-           os.path.join(CSRC, "xkv_py.cpp"), "-o", PYMOD, "-L", HERE, "-lxkv", "-Wl,-rpath,$ORIGIN",
-           *("-L" + p for p in cpp_extension.library_paths()), "-ltorch_python", "-ltorch_cpu", "-lc10"]
-    r = subprocess.run(cmd, capture_output=True, text=True)
+    r = subprocess.run(_module_command(), capture_output=True, text=True)
     if r.returncode != 0:
         sys.stderr.write(r.stdout + r.stderr)
         raise RuntimeError("building the Python module failed")
