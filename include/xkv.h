@@ -364,8 +364,11 @@ XKV_API int xkv_debug_set_fault_injection(xkv_group* grp, uint32_t mask);
  *                             that kernel's barriers is shortened to about a millisecond; the other CTAs give up,
  *                             the workspace's flag word gets XKV_FLAG_TIMEOUT (xkv_clf_status returns
  *                             XKV_ERR_TIMEOUT) and the factors of that call are unspecified.
+ *   XKV_INJECT_CLF_CHOLESKY   the same in the Cholesky kernels of the call: the first of them is abandoned at its first
+ *                             barrier, and every one behind it, whose arrivals are counted on, ends at once.
  */
 #define XKV_INJECT_CLF_BARRIER 4u
+#define XKV_INJECT_CLF_CHOLESKY 8u
 XKV_API int xkv_debug_set_clf_fault_injection(uint32_t mask);
 
 /*

@@ -472,7 +472,7 @@ int xkv_clf_factorize(const xkv_clf_config* cfg, const void* X, const void* omeg
 }
 
 int xkv_debug_set_clf_fault_injection(uint32_t mask) {
-  if (mask & ~XKV_INJECT_CLF_BARRIER) return XKV_ERR_INVALID_ARG;
+  if (mask & ~(XKV_INJECT_CLF_BARRIER | XKV_INJECT_CLF_CHOLESKY)) return XKV_ERR_INVALID_ARG;
   clf_set_fault_injection(mask);
   return XKV_OK;
 }

@@ -1219,6 +1219,11 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
   const int nbk = l / kCholNb, n_tiles = nbk * (nbk + 1) / 2;
   const int chol_grid = sms < (n_tiles > 32 ? n_tiles : 32) ? sms : (n_tiles > 32 ? n_tiles : 32);
   unsigned chol_arrived = 0;
+  const unsigned injected = g_clf_inject.load(std::memory_order_relaxed);
+  auto grid_sync = [&](int count, unsigned mask) {                     // the words were zeroed with the flag block above
+    const bool inject = (injected & mask) != 0u;
+    return GridSync{flags, flags + count, flags + 10, inject ? 1024u : kGridSpinLimit, inject ? 1u : 0u};
+  };
   auto cholqr = [&](int passes) -> cudaError_t {                       // an odd number of passes ends in Z
     float* in = U;
     float* out = Z;
@@ -1226,7 +1231,7 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
       gram_kernel<<<dim3((l / 64) * (l / 64 + 1) / 2, p.gram_split), 256, 0, s>>>(in, part, N, l, p.gram_rows);
       double shift = kShift;
       int n_part = p.gram_split;
-      GridSync sy{flags, flags + 12, flags + 10, kGridSpinLimit, 0u};
+      GridSync sy = grid_sync(12, XKV_INJECT_CLF_CHOLESKY);
       void* args[] = {&part, &n_part, &Gm, &Rt, &Iv, &W, &l, &shift, &chol_arrived, &sy};
       cudaError_t e2 = launch_cooperative<chol_inverse_kernel>(chol_grid, kCholThreads, 0, args, device, s);
       if (e2 != cudaSuccess) return e2;
@@ -1253,8 +1258,7 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
     float* M2 = (float*)(w + p.off_m2);
     float* Qm = (float*)(w + p.off_q);
     float2* partial = (float2*)(w + p.off_cs);
-    const bool inject = (g_clf_inject.load(std::memory_order_relaxed) & XKV_INJECT_CLF_BARRIER) != 0u;
-    GridSync sy{flags, flags + 8, flags + 10, inject ? 1024u : kGridSpinLimit, inject ? 1u : 0u};   // zeroed with the flag block above
+    GridSync sy = grid_sync(8, XKV_INJECT_CLF_BARRIER);
     unsigned arrived = 0;
     void* args[] = {&Mm, &M2, &Pm, &Qm, &l, &partial, &arrived, &sy};
     e = launch_cooperative<jacobi_block_kernel>(sms, kJacobiThreads, kJacobiSmem, args, device, s);
