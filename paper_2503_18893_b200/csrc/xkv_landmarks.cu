@@ -227,7 +227,12 @@ landmark_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restric
 
 using namespace ptx;                // packed fp32
 
-// The default chunk of 8 rows (c == 8), persistent CTAs.  Bit for bit the arithmetic of the kernel above.
+// The default chunk of 8 rows (c == 8), persistent CTAs.  The arithmetic of the kernel above, landmarks operation by
+// operation; two things may move a last bit.  The table entries come from an fp64 rotation carried from block to block
+// instead of a sincospi per 4 or 8 rows (apart by the rounding of an fp64 angle; as fp32 they differ so rarely that 7 of
+// 512 M landmark elements do at 1000003 rows of 32 heads, none at 131072 rows of four layers of 8), and the sums of a cosine over the lanes
+// of a head are folded in another order (1e-5 of the cosines, by 1.2e-7).  The error against fp64 is that of the kernel
+// above: cosines 2.4e-7 at most, 5.7e-8 rms; 261 of 8.4 M landmarks on the other side of a rounding boundary, for both.
 // A CTA walks a contiguous range of row blocks; the cos/sin table of a block is built once and serves every (sequence,
 // layer) and head, so its fp64 work (an eighth of the fp32 rate here) is divided by batch * G: per CTA and layer, as in
 // the kernel above, it took as long as everything else together.  The rotation is advanced in fp64 from block to block;
