@@ -227,8 +227,7 @@ __device__ __forceinline__ void load_keys(const float* __restrict__ S, int j0, i
 // One CTA per (layer, sequence, KV head).  grid.x = problems of the call.
 // Exact k_ch-th largest key by a radix select whose bins subdivide the range that still contains it
 // (first the [min, max] range of all keys, then the chosen bin, ...: at most three 11-bit passes), followed
-// by an ordered compaction.  CACHED: n_c fits one super-block and the keys stay in registers.
-template <bool CACHED>
+// by an ordered compaction.  The keys are read again in every pass (they come from L2).
 __global__ void __launch_bounds__(kTopkThreads)
 topk_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __restrict__ outliers, int n_out, float sign,
             int32_t* __restrict__ sel_idx, int32_t* __restrict__ sel_cnt) {
@@ -248,8 +247,6 @@ topk_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __restrict
 
   grid_dependency_wait();                      // the pooled scores come from the kernel launched before
   grid_dependency_launch();
-  uint32_t creg[kTopkItems];
-  if (CACHED) load_keys(S, tid * kTopkItems, n_c, sign, creg);
 
   uint32_t thr = 0, need_eq = 0;
   const bool all = (k_ch >= n_c);
@@ -259,12 +256,7 @@ topk_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __restrict
     for (int base = 0; base < n_c; base += super) {
       uint32_t key[kTopkItems];
       const int j0 = base + tid * kTopkItems;
-      if (CACHED) {
-#pragma unroll
-        for (int i = 0; i < kTopkItems; ++i) key[i] = creg[i];
-      } else {
-        load_keys(S, j0, n_c, sign, key);
-      }
+      load_keys(S, j0, n_c, sign, key);
 #pragma unroll
       for (int i = 0; i < kTopkItems; ++i) {
         if (j0 + i < n_c) { kmin = min(kmin, key[i]); kmax = max(kmax, key[i]); }
@@ -293,12 +285,7 @@ topk_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __restrict
       for (int base = 0; base < n_c; base += super) {
         uint32_t key[kTopkItems];
         const int j0 = base + tid * kTopkItems;
-        if (CACHED) {
-#pragma unroll
-          for (int i = 0; i < kTopkItems; ++i) key[i] = creg[i];
-        } else {
-          load_keys(S, j0, n_c, sign, key);
-        }
+        load_keys(S, j0, n_c, sign, key);
 #pragma unroll
         for (int i = 0; i < kTopkItems; ++i) {
           const uint32_t rel = key[i] - lo;
@@ -349,12 +336,7 @@ topk_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __restrict
         for (int base = 0; base < n_c; base += super) {
           uint32_t key[kTopkItems];
           const int j0 = base + tid * kTopkItems;
-          if (CACHED) {
-#pragma unroll
-            for (int i = 0; i < kTopkItems; ++i) key[i] = creg[i];
-          } else {
-            load_keys(S, j0, n_c, sign, key);
-          }
+          load_keys(S, j0, n_c, sign, key);
           // this thread's candidates as a bit mask; the warp reserves room for all of its candidates with one atomic
           uint32_t cm = 0;
 #pragma unroll
@@ -464,12 +446,7 @@ topk_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __restrict
       for (int i = 0; i < kTopkItems; ++i) if (j0 + i < n_c) gtm |= 1u << i;
     } else {
       uint32_t key[kTopkItems];
-      if (CACHED) {
-#pragma unroll
-        for (int i = 0; i < kTopkItems; ++i) key[i] = creg[i];
-      } else {
-        load_keys(S, j0, n_c, sign, key);
-      }
+      load_keys(S, j0, n_c, sign, key);
 #pragma unroll
       for (int i = 0; i < kTopkItems; ++i) {
         if (j0 + i < n_c) {
@@ -878,7 +855,7 @@ static cudaError_t launch_topk(const GroupDev& dev, int device, int problems, in
                                const int32_t* outliers, int n_out, float sign, int32_t* sel_idx, int32_t* sel_cnt,
                                cudaStream_t s) {
   if (dev.n_c > kTopkThreads * 32)
-    return launch_pdl(topk_kernel<false>, dim3(problems), dim3(kTopkThreads), 0, s, dev, l0, k_ch, k_cap, outliers, n_out,
+    return launch_pdl(topk_kernel, dim3(problems), dim3(kTopkThreads), 0, s, dev, l0, k_ch, k_cap, outliers, n_out,
                       sign, sel_idx, sel_cnt);
   // keys per thread: 16 up to 16384 chunks, 32 beyond; threads: the fewest of 128, 256, 512, 1024 that cover the
   // chunks (a short context needs fewer barriers' worth of warps, and several of its CTAs share an SM); groups per
