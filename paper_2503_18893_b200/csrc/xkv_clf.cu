@@ -1034,9 +1034,10 @@ bool make_plan(const xkv_clf_config* c, ClfPlan* p) {
   p->off_up = o; if (p->u_split > 1) o = align_up(o + (size_t)p->u_split * p->N * p->l * 4);   // partial sums of U
   p->off_u = o; o = align_up(o + (size_t)p->N * p->l * 4);
   p->off_z = o; o = align_up(o + (size_t)p->N * p->l * 4);
-  // row ranges so that the lower 64 x 64 tiles of the Gram matrix fill the SMs about twice (148 SMs; fewer only queue)
+  // row ranges so that the lower 64 x 64 tiles of the Gram matrix fill the SMs about twice
   const int tiles = (p->l / 64) * (p->l / 64 + 1) / 2;
-  p->gram_split = 296 / tiles < 1 ? 1 : (296 / tiles > 8 ? 8 : 296 / tiles);
+  const int fill = 2 * kPlanSms / tiles;
+  p->gram_split = fill < 1 ? 1 : fill > 8 ? 8 : fill;
   p->gram_rows = ((p->N + p->gram_split - 1) / p->gram_split + 31) & ~31;
   p->gram_split = (p->N + p->gram_rows - 1) / p->gram_rows;
   p->ritz_split = gemm_splits(p->l, p->l, p->T, 16);
@@ -1120,11 +1121,11 @@ cudaError_t launch_gemm(GemmOperand a, GemmOperand b, int splits, GemmOut c, uns
   return launch_gemm_bn<TRANS, AK, BK, 1, 128>(a, b, splits, c, flags, device, s);
 }
 
-// K ranges that bring a product's tiles to about one per SM (148), none of them empty or shorter than 1024.
+// K ranges that bring a product's tiles to about one per SM, none of them empty or shorter than 1024.
 int gemm_splits(int M, int N, int K, int most) {
   const int mb = gemm_mb(M) * 128, bn = gemm_bn(N);
   const long long tiles = (long long)((M + mb - 1) / mb) * ((N + bn - 1) / bn);
-  long long sp = 148 / tiles;
+  long long sp = kPlanSms / tiles;
   if (sp > most) sp = most;
   if (sp > K / 1024) sp = K / 1024;
   if (sp < 1) sp = 1;
@@ -1192,7 +1193,7 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
   __nv_bfloat16* Vb = (__nv_bfloat16*)(w + p.off_vb);
   const int N = p.N, r = p.r, T = p.T;
   int l = p.l, sms = 0;
-  cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+  cudaError_t e = device_sms(device, &sms);
   if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 256, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(Zb, omega, (size_t)N * l * 2, cudaMemcpyDeviceToDevice, s);
   // Y = X Z (stored as Y^T), Z rounded to bf16 or as both of its parts,  and  U = X^T Y

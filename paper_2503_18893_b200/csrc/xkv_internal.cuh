@@ -18,6 +18,7 @@ constexpr int kLandmarkBoxRows = 64;   // landmark rows per TMA box = chunks sco
 constexpr int kTailSplitRows = 128;     // tail rows per partial result
 constexpr int kTailMaxSplit = XKV_TAIL_MAX_ROWS / kTailSplitRows;
 constexpr int kMaxSplit = 64;     // most partial results per (layer, sequence, head) problem
+constexpr int kPlanSms = 148;     // SMs that a plan made without a device counts on (sizes of splits only; a B200 has 148)
 
 // Device-side description of one window; a copy lives in the handle and is passed by value.
 struct GroupDev {
@@ -121,6 +122,17 @@ inline cudaError_t ensure_dyn_smem(size_t bytes, int device) {
   if (bytes + (size_t)st <= 48 * 1024) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess) have[device].store(bytes, std::memory_order_release);
+  return e;
+}
+
+// SMs of a device, looked up once per device.
+inline cudaError_t device_sms(int device, int* sms) {
+  static std::atomic<int> have[kMaxDevices];
+  if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
+  *sms = have[device].load(std::memory_order_relaxed);
+  if (*sms > 0) return cudaSuccess;
+  const cudaError_t e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, device);
+  if (e == cudaSuccess) have[device].store(*sms, std::memory_order_relaxed);
   return e;
 }
 

@@ -419,7 +419,7 @@ cudaError_t launch_landmark8(const __nv_bfloat16* keys, __nv_bfloat16* landmarks
   const int n_blocks = (n_c + cpb - 1) / cpb;
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = device_sms(dev, &sms);
   if (e != cudaSuccess) return e;
   const int grid = n_blocks < 2 * sms ? n_blocks : 2 * sms;           // two CTAs per SM, one wave
   const bool rope = rope_base > 0.0f;

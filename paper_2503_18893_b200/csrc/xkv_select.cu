@@ -860,13 +860,20 @@ static cudaError_t launch_topk(const GroupDev& dev, int device, int problems, in
   // keys per thread: 16 up to 16384 chunks, 32 beyond; threads: the fewest of 128, 256, 512, 1024 that cover the
   // chunks (a short context needs fewer barriers' worth of warps, and several of its CTAs share an SM); groups per
   // thread: the fewest with at least k_ch groups in all (0 = no filter)
+  int sms = 0;
+  cudaError_t e = device_sms(device, &sms);
+  if (e != cudaSuccess) return e;
   const int items = dev.n_c <= kTopkThreads * 16 ? 16 : 32;
   auto groups = [&](int gpt) { return (dev.n_c + items / gpt - 1) / (items / gpt); };
   int th = items == 32 ? 1024 : (dev.n_c <= 128 * 16 ? 128 : dev.n_c <= 256 * 16 ? 256 : dev.n_c <= 512 * 16 ? 512 : 1024);
   if (groups(4) < k_ch && th < 512) th *= 2;       // no filter: every key is listed, more threads pay
-  if (problems <= 148 && th < 1024) th *= 2;       // a CTA per SM: nothing is gained by small ones (32K rows by layer 121.5 -> 118.8 us)
+  // Where a CTA has its SM to itself small ones leave room for nobody.  Selections of 4 to 128 problems, base threads
+  // against twice as many: 2048 rows 7.27 -> 7.05 us, 16384 rows and budget 2048 10.6 -> 9.4, 32768 rows 13.3 -> 12.1 (128
+  // problems 38.6 -> 38.2); with 256 problems 2048 rows lose (9.0 -> 10.0).  From 512 to 1024 threads the barriers cost
+  // more than the threads bring (65536 rows, 8 problems, budget 2048: 8.9 -> 9.7 us), unless the lists are long (4
+  // problems, budget 8192: 10.5 -> 10.1) or the problems many (window of 128: 158.2 -> 157.5 us).
+  if (problems <= sms && (th < 512 || (th == 512 && (problems > sms / 4 || groups(1) < k_ch)))) th *= 2;
   const size_t smem = (size_t)th * items * (sizeof(uint32_t) + sizeof(uint16_t));
-  cudaError_t e;
 #define XKV_PIVOT(GPT, ITEMS, TH)                                                                                     \
   do {                                                                                                                \
     e = ensure_dyn_smem<topk_pivot_kernel<GPT, ITEMS, TH>>(smem, device);                                             \
