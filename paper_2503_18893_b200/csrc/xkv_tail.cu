@@ -9,8 +9,11 @@
 // BEHIND: the kernel is launched behind the fused kernel, whose results it does not need.  It starts on the SMs that the
 // fused kernel leaves idle or leaves early, reads at once (its inputs come from before the fused kernel, which waits for
 // everything before it before it lets this one start) and waits for the fused kernel only before it ends, so that the
-// merge behind it finds both complete.  In front of the fused kernel it is one more link of the chain: a step of 121873
-// rows and a 1500-row tail, layer by layer, takes 188 us that way and 173.5 this way.
+// merge behind it finds both complete.  What it reads before that wait it reads past L1 (asynchronous copies, ld.cg): only
+// a wait of its own would promise that no line from an earlier call is left there.  (A dense call waits first and reads its
+// queries through L1: 360 us, 374 past it, 65536 and 64533 rows of four layers of eight heads.)  In front of the fused
+// kernel it is one more link of the chain: a step of 121873 rows and a 1500-row tail, layer by layer, takes 188 us that
+// way and 171 this way.
 #include <math.h>
 
 #include "xkv_internal.cuh"
@@ -33,6 +36,12 @@ constexpr int tail_k_stride() { return DH * 2 + 16; }   // bytes per staged key 
 template <int DH, int NR>
 constexpr size_t tail_smem_bytes() {
   return (size_t)kTailThreads * tail_k_stride<DH>() + (size_t)kTailThreads * DH * 2 + sizeof(float) * (NR * DH + NR * kTailThreads);
+}
+
+template <bool PAST_L1, typename T>
+__device__ __forceinline__ T early_load(const T* p) {
+  if constexpr (PAST_L1) return __ldcg(p);
+  else return *p;
 }
 
 template <int DH, int NR, bool BEHIND>
@@ -58,7 +67,7 @@ tail_partial_kernel(GroupDev dev, int l0, const __nv_bfloat16* __restrict__ q, c
 
   if constexpr (!BEHIND) ptx::grid_dependency_wait();  // q (and the tail rows) may come from the kernel before
   ptx::grid_dependency_launch();
-  int len = tail_len ? tail_len[b] : tail_cap;
+  int len = tail_len ? early_load<BEHIND>(tail_len + b) : tail_cap;
   if (len < 0 || len > tail_cap) {
     if (tid == 0 && split == 0) atomicOr(dev.flags, XKV_FLAG_INDEX_RANGE);
     len = len < 0 ? 0 : tail_cap;
@@ -87,7 +96,7 @@ tail_partial_kernel(GroupDev dev, int l0, const __nv_bfloat16* __restrict__ q, c
   // packed multiply-adds below
   for (int i = tid; i < NR * DH; i += kTailThreads) {
     const int h = i / DH, dd = i - h * DH;
-    q_s[dd * NR + h] = h < n_rep ? __bfloat162float(qg[i]) : 0.0f;
+    q_s[dd * NR + h] = h < n_rep ? __bfloat162float(early_load<BEHIND>(qg + i)) : 0.0f;
   }
   ptx::cp_async_wait<1>();                             // the keys of this thread's copies are in
   __syncthreads();
@@ -270,7 +279,7 @@ tail_tc_kernel(GroupDev dev, int l0, const __nv_bfloat16* __restrict__ q, const 
 
   if constexpr (!BEHIND) grid_dependency_wait();       // q (and the tail rows) may come from the kernel before
   grid_dependency_launch();
-  int len = tail_len ? tail_len[b] : tail_cap;
+  int len = tail_len ? early_load<BEHIND>(tail_len + b) : tail_cap;
   if (len < 0 || len > tail_cap) {
     if (tid == 0 && split == 0) atomicOr(dev.flags, XKV_FLAG_INDEX_RANGE);
     len = len < 0 ? 0 : tail_cap;
@@ -279,7 +288,7 @@ tail_tc_kernel(GroupDev dev, int l0, const __nv_bfloat16* __restrict__ q, const 
   const __nv_bfloat16* qg = q + (((long long)l * dev.batch + b) * dev.H_q + (long long)g * n_rep) * DH;
   for (int i = tid; i < n_rep * 16; i += kTailThreads) {
     const int h = i >> 4, c = i & 15;
-    const uint4 v = *reinterpret_cast<const uint4*>(qg + h * DH + c * 8);
+    const uint4 v = early_load<BEHIND>(reinterpret_cast<const uint4*>(qg + h * DH + c * 8));
     *reinterpret_cast<uint4*>(q_gen + (c >> 3) * 2048 + h * 128 + (((c & 7) ^ (h & 7)) << 4)) = v;
   }
   const uint64_t desc_hi = smem_desc_sw128(0, 0) & 0xFFFFFFFF00000000ull;
