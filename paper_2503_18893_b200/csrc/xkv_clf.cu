@@ -606,9 +606,10 @@ namespace {
 //   B  the grid applies M <- Q^T M Q, 64 x 32 pieces, from one buffer to the other.
 // Two grid barriers per 32 rounds of rotations.  (Applying every round of l/2 rotations to the whole matrix takes a
 // barrier per round: 575 per sweep of a 576 x 576 matrix, 4.9 us each, 8.5 ms for three sweeps; taking the 64 x 64
-// problems to convergence before they are applied was slower still.  This form takes less than 1 ms for the same three
-// sweeps; the factorisation of a 131072 x 4096 cache went from 26.2 to 17.2 ms.)  A check per sweep ends the sweeps once the off-diagonal weight is below kJacobiTol.  On return the eigenvalues are on the diagonal of M
-// (buffer 0), the eigenvectors the rows of Pt.
+// problems to convergence before they are applied was slower still.  This form takes 1.5 ms for the same three sweeps; the
+// factorisation of a 131072 x 4096 cache went from 26.2 to 17.2 ms.)  A check per sweep ends the sweeps once the
+// off-diagonal weight is below kJacobiTol.  On return the eigenvalues are on the diagonal of M (buffer 0), the
+// eigenvectors the rows of Pt.
 constexpr int kJacobiMaxPairs = 1024;              // l <= 2048
 constexpr int kJacobiSweeps = 16;
 // The sweeps end when the off-diagonal weight (sum of squares) is below this fraction of the total.  The

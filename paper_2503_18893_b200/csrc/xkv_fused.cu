@@ -370,9 +370,9 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
 
   if (warp >= 8 && warp < kWarpK) {
     // =============================== producers: gather rows of A ===============================
-    // Two independent streams with a ring of their own each: warps 8-9 gather the rows of A_k of every tile into
-    // the key ring, warps 10-11 the same rows of A_v into the value ring.  A stream waits only for releases of its
-    // own ring, so the key MMAs of consecutive tiles follow one another without waiting for the value phase that
+    // Two independent streams with a ring of their own each: the first half of the producer warps (8-9, with quantised
+    // bases 8-11) gather the rows of A_k of every tile into the key ring, the second half (10-11, 12-15) the same rows of
+    // A_v into the value ring.  A stream waits only for releases of its own ring, so the key MMAs of consecutive tiles follow one another without waiting for the value phase that
     // sits between them in time (with one shared ring the key slabs of tile i+2 could not be requested before the
     // last value slab of tile i, which itself waited for the last key MMA of tile i+1).
     // Eight consecutive lanes copy the eight 16-byte pieces of one 128-byte row slab, so that every request of a
