@@ -7,8 +7,8 @@
 //                         U   = X^T Y     (N x l, fp32)          tensor core
 //                         Z   = U R^-1,  R^T R = U^T U + shift I (shifted Cholesky QR in fp64: one pass inside the
 //                               iteration, three for the last iterate, which has to be orthonormal)
-//   Rayleigh-Ritz:        W^T = Z^T X^T,  M = W^T W (= Z^T X^T X Z, l x l),  M = P Lambda P^T (Jacobi); Z as the sum of two
-//                         bf16 matrices here
+//   Rayleigh-Ritz:        W^T = Z^T X^T,  M = W^T W (= Z^T X^T X Z, l x l),  M = P Lambda P^T (Jacobi); Z and W as sums of
+//                         two bf16 matrices here
 //   V = Z P_r (N x r);    B_l = rows of V^T (bf16);   A = X V_bf16 (T x r, tensor core);   sigma = sqrt(Lambda).
 // A = U Sigma and B = V^T of the truncated SVD of X, up to the accuracy of the subspace (checked against the exact
 // optimum sum_{i>r} sigma_i^2, never factor by factor: signs and degenerate subspaces are not unique).
@@ -51,12 +51,14 @@ __device__ __forceinline__ bool gemm_wait(uint32_t bar, uint32_t parity) {
 
 // C[m][n] = sum_k A(k, m) B(k, n).  grid = (ceil(N/BN), ceil(M/(128 MB)), K ranges).  TRANS: store C^T (out[n][m]).
 // AK: A is given as [m][k] (K-major), else as [k][m]; BK likewise for B.  K range z covers k_per columns and writes
-// Cf + z * M * ldc.  A may hold a_k < K of the k only (a multiple of 64, K = 2 a_k): it is then gone through twice, for a B
-// that is a sum of two matrices, one below the other.  Out-of-range rows and columns of the operands are zero-filled by the copy engine; stores are guarded.
+// Cf + z * M * ldc.  With two parts B is the sum of the matrices of map_b and map_b2 and A is gone through twice; the k
+// of a part are rounded up to whole blocks of 64.  Cb is the result rounded to bf16, Cl twice what the rounding leaves out
+// (with TRANS).  Out-of-range rows and columns of the operands are zero-filled by the copy engine; stores are guarded.
 template <bool TRANS, bool AK, bool BK, int MB, int BN>
 __global__ void __launch_bounds__(gemm_threads<MB>(), 1)
-clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int M, int N, int K,
-                int a_k, int k_per, float* __restrict__ Cf, __nv_bfloat16* __restrict__ Cb, long long ldc, unsigned int* __restrict__ flags) {
+clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                const __grid_constant__ CUtensorMap map_b2, int M, int N, int k_part, int k_all, int k_per, float* __restrict__ Cf,
+                __nv_bfloat16* __restrict__ Cb, __nv_bfloat16* __restrict__ Cl, long long ldc, unsigned int* __restrict__ flags) {
   extern __shared__ uint8_t gemm_smem[];
   constexpr int kGemmStages = gemm_stages<MB, BN>(), kGemmStageBytes = gemm_stage_bytes<MB, BN>();
   constexpr uint32_t kAccCols = BN <= 128 ? 128u : 256u, kCols = MB * kAccCols;      // tensor-memory columns
@@ -67,7 +69,7 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   const uint32_t base = (smem_u32(gemm_smem) + 1023u) & ~1023u;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n0 = blockIdx.x * BN, m0 = blockIdx.y * (128 * MB);
-  const int k_first = blockIdx.z * k_per, KB = (min(K - k_first, k_per) + 63) / 64;
+  const int k_first = blockIdx.z * k_per, KB = (min(k_all - k_first, k_per) + 63) / 64;
   if (Cf) Cf += (size_t)blockIdx.z * M * ldc;
   const uint32_t bar0 = smem_u32(bars);
   auto FULL = [&](int s) { return bar0 + 8u * (uint32_t)s; };
@@ -96,19 +98,22 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         if (kb >= kGemmStages && !gemm_wait(EMPTY(s), (uint32_t)((kb / kGemmStages - 1) & 1))) { ok = false; break; }
         const uint32_t st = base + (uint32_t)s * kGemmStageBytes;
         mbar_expect_tx(FULL(s), kGemmStageBytes);
-        const int k = k_first + kb * 64, ka = k < a_k ? k : k - a_k;
+        const int kt = k_first + kb * 64;
+        const bool second = kt >= k_part;
+        const int k = second ? kt - k_part : kt;
+        const CUtensorMap* mb = second ? &map_b2 : &map_b;
         // K-major: one box of 64 k by all rows; MN-major: slabs of 64 columns by 64 k, 8 KB each
         if (AK) {
-          tma_load_2d(st, &map_a, ka, m0, FULL(s));
+          tma_load_2d(st, &map_a, k, m0, FULL(s));
         } else {
 #pragma unroll
-          for (int i = 0; i < 2 * MB; ++i) tma_load_2d(st + i * 8192, &map_a, m0 + i * 64, ka, FULL(s));
+          for (int i = 0; i < 2 * MB; ++i) tma_load_2d(st + i * 8192, &map_a, m0 + i * 64, k, FULL(s));
         }
         if (BK) {
-          tma_load_2d(st + kOffB, &map_b, k, n0, FULL(s));
+          tma_load_2d(st + kOffB, mb, k, n0, FULL(s));
         } else {
 #pragma unroll
-          for (int i = 0; i < BN / 64; ++i) tma_load_2d(st + kOffB + i * 8192, &map_b, n0 + i * 64, k, FULL(s));
+          for (int i = 0; i < BN / 64; ++i) tma_load_2d(st + kOffB + i * 8192, mb, n0 + i * 64, k, FULL(s));
         }
       }
     }
@@ -185,7 +190,11 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
               if (n < N) {
                 const long long at = TRANS ? (long long)n * ldc + m : (long long)m * ldc + n;
                 if (Cf) Cf[at] = v[i];
-                if (Cb) Cb[at] = __float2bfloat16(v[i]);
+                if (Cb) {
+                  const __nv_bfloat16 hi = __float2bfloat16(v[i]);
+                  Cb[at] = hi;
+                  if (TRANS && Cl) Cl[at] = __float2bfloat16(2.0f * (v[i] - __bfloat162float(hi)));
+                }
               }
             }
           }
@@ -1009,13 +1018,15 @@ __global__ void symmetrize_kernel(const float* __restrict__ part, int n_part, fl
   M[(size_t)j * l + i] = v;
 }
 
+// k of a product, all parts: whole blocks of 64 per part
+int gemm_k(int K, int parts) { return parts == 1 ? K : parts * ((K + 63) & ~63); }
 int gemm_splits(int M, int N, int K, int most);
 
 struct ClfPlan {
   int T, Tp, N, r, l, q;
   int gram_split, gram_rows;                                 // row ranges of a Gram matrix and rows of each
   int u_split, ritz_split;                                   // K ranges of U = X^T Y and of the Ritz matrix
-  size_t off_flags, off_zb, off_yt, off_up, off_u, off_z, off_part, off_g, off_rt, off_w, off_iv, off_m, off_p, off_ps, off_vb, off_cs, off_m2,
+  size_t off_flags, off_zb, off_yt, off_yl, off_up, off_u, off_z, off_part, off_g, off_rt, off_w, off_iv, off_m, off_p, off_ps, off_vb, off_cs, off_m2,
       off_q, total;
 };
 
@@ -1031,6 +1042,7 @@ bool make_plan(const xkv_clf_config* c, ClfPlan* p) {
   p->off_flags = o; o = align_up(o + 256);
   p->off_zb = o; o = align_up(o + (size_t)2 * p->N * p->l * 2);  // Z as two bf16 matrices, one below the other
   p->off_yt = o; o = align_up(o + (size_t)p->l * p->Tp * 2);
+  p->off_yl = o; o = align_up(o + (size_t)p->l * p->Tp * 2);        // twice what the rounding of W leaves out
   p->u_split = gemm_splits(p->N, p->l, p->T, 8);
   p->off_up = o; if (p->u_split > 1) o = align_up(o + (size_t)p->u_split * p->N * p->l * 4);   // partial sums of U
   p->off_u = o; o = align_up(o + (size_t)p->N * p->l * 4);
@@ -1041,7 +1053,7 @@ bool make_plan(const xkv_clf_config* c, ClfPlan* p) {
   p->gram_split = fill < 1 ? 1 : fill > 8 ? 8 : fill;
   p->gram_rows = ((p->N + p->gram_split - 1) / p->gram_split + 31) & ~31;
   p->gram_split = (p->N + p->gram_rows - 1) / p->gram_rows;
-  p->ritz_split = gemm_splits(p->l, p->l, p->T, 16);
+  p->ritz_split = gemm_splits(p->l, p->l, gemm_k(p->T, 2), 16);
   const size_t part_words = p->gram_split * 2 > p->ritz_split ? p->gram_split * 2 : p->ritz_split;
   p->off_part = o; o = align_up(o + part_words * p->l * p->l * 4);   // partial Gram matrices (fp64) / Ritz matrices (fp32)
   p->off_g = o; o = align_up(o + (size_t)p->l * p->l * 8);      // the Gram matrix, factorised in place of its tiles, fp64
@@ -1079,21 +1091,26 @@ struct GemmOut {
   float* f;                 // either may be null
   __nv_bfloat16* b;
   long long ld;
+  __nv_bfloat16* lo = nullptr;   // transposed results only: twice what b's rounding leaves out
 };
 
 template <bool TRANS, bool AK, bool BK, int MB, int BN>
-cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, int splits, GemmOut c, unsigned int* flags, int device, cudaStream_t s) {
-  const int M = AK ? a.rows : a.cols, N = BK ? b.rows : b.cols, K = BK ? b.cols : b.rows, a_k = AK ? a.cols : a.rows;
-  CUtensorMap ma, mb;
+cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, const void* b2, int splits, GemmOut c, unsigned int* flags, int device,
+                           cudaStream_t s) {
+  const int M = AK ? a.rows : a.cols, N = BK ? b.rows : b.cols, K = AK ? a.cols : a.rows;
+  const int k_all = gemm_k(K, b2 ? 2 : 1), k_part = b2 ? k_all / 2 : k_all;
+  CUtensorMap ma, mb, mb2;
   if (!encode_bf16_map(&ma, a.p, (uint64_t)a.rows, (uint64_t)a.cols, (uint64_t)a.pitch, AK ? 128 * MB : 64) ||
-      !encode_bf16_map(&mb, b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BK ? BN : 64))
+      !encode_bf16_map(&mb, b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BK ? BN : 64) ||
+      !encode_bf16_map(&mb2, b2 ? b2 : b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BK ? BN : 64))
     return cudaErrorInvalidValue;
   const size_t smem = 1024 + (size_t)gemm_stages<MB, BN>() * gemm_stage_bytes<MB, BN>();
   cudaError_t e = ensure_dyn_smem<clf_gemm_kernel<TRANS, AK, BK, MB, BN>>(smem, device);
   if (e != cudaSuccess) return e;
-  const int k_per = ((K + splits - 1) / splits + 63) & ~63;
+  const int k_per = ((k_all + splits - 1) / splits + 63) & ~63;
   const dim3 grid((N + BN - 1) / BN, (M + 128 * MB - 1) / (128 * MB), splits);
-  clf_gemm_kernel<TRANS, AK, BK, MB, BN><<<grid, gemm_threads<MB>(), smem, s>>>(ma, mb, M, N, K, a_k, k_per, c.f, c.b, c.ld, flags);
+  clf_gemm_kernel<TRANS, AK, BK, MB, BN><<<grid, gemm_threads<MB>(), smem, s>>>(ma, mb, mb2, M, N, k_part, k_all, k_per, c.f, c.b, c.lo, c.ld,
+                                                                               flags);
   count_launch(kFamClf);
   return cudaGetLastError();
 }
@@ -1110,16 +1127,17 @@ int gemm_bn(int N) {
 int gemm_mb(int M) { return ((M + 255) & ~255) * 8LL <= ((M + 127) & ~127) * 9LL ? 2 : 1; }
 
 template <bool TRANS, bool AK, bool BK>
-cudaError_t launch_gemm(GemmOperand a, GemmOperand b, int splits, GemmOut c, unsigned int* flags, int device, cudaStream_t s) {
+cudaError_t launch_gemm(GemmOperand a, GemmOperand b, int splits, GemmOut c, unsigned int* flags, int device, cudaStream_t s,
+                        const void* b2 = nullptr) {      // b2: the second part of B, laid out like b
   const int bn = gemm_bn(BK ? b.rows : b.cols);
   if (gemm_mb(AK ? a.rows : a.cols) == 2) {
-    if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, 2, 256>(a, b, splits, c, flags, device, s);
-    if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, 2, 192>(a, b, splits, c, flags, device, s);
-    return launch_gemm_bn<TRANS, AK, BK, 2, 128>(a, b, splits, c, flags, device, s);
+    if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, 2, 256>(a, b, b2, splits, c, flags, device, s);
+    if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, 2, 192>(a, b, b2, splits, c, flags, device, s);
+    return launch_gemm_bn<TRANS, AK, BK, 2, 128>(a, b, b2, splits, c, flags, device, s);
   }
-  if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, 1, 256>(a, b, splits, c, flags, device, s);
-  if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, 1, 192>(a, b, splits, c, flags, device, s);
-  return launch_gemm_bn<TRANS, AK, BK, 1, 128>(a, b, splits, c, flags, device, s);
+  if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, 1, 256>(a, b, b2, splits, c, flags, device, s);
+  if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, 1, 192>(a, b, b2, splits, c, flags, device, s);
+  return launch_gemm_bn<TRANS, AK, BK, 1, 128>(a, b, b2, splits, c, flags, device, s);
 }
 
 // K ranges that bring a product's tiles to about one per SM, none of them empty or shorter than 1024.
@@ -1197,10 +1215,8 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
   cudaError_t e = device_sms(device, &sms);
   if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 256, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(Zb, omega, (size_t)N * l * 2, cudaMemcpyDeviceToDevice, s);
-  // Y = X Z (stored as Y^T), Z rounded to bf16 or as both of its parts,  and  U = X^T Y
-  auto product_y = [&](int parts) {
-    return launch_gemm<true, true, false>({X, T, N, N}, {Zb, parts * N, l, l}, 1, {nullptr, Yt, p.Tp}, flags, device, s);
-  };
+  // Y = X Z (stored as Y^T)  and  U = X^T Y
+  auto product_y = [&]() { return launch_gemm<true, true, false>({X, T, N, N}, {Zb, N, l, l}, 1, {nullptr, Yt, p.Tp}, flags, device, s); };
   auto product_u = [&]() -> cudaError_t {
     float* out = p.u_split > 1 ? (float*)(w + p.off_up) : U;
     cudaError_t e2 = launch_gemm<false, false, true>({X, T, N, N}, {Yt, l, T, p.Tp}, p.u_split, {out, nullptr, l}, flags, device, s);
@@ -1245,16 +1261,19 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
     return cudaGetLastError();
   };
   for (int it = 0; it <= p.q && e == cudaSuccess; ++it) {
-    e = product_y(1);
+    e = product_y();
     if (e == cudaSuccess) e = product_u();
     if (e == cudaSuccess) e = cholqr(it == p.q ? 3 : 1);
   }
   // Rayleigh-Ritz: W = X Z, M = W^T W (= Z^T X^T X Z), its eigenvectors by Jacobi.  M is that of the fp32 Z whose
-  // combinations become V, so Z's rounding to bf16 must not enter: a column in the noise floor, rounded, holds a part of
-  // 2^-9 of the largest singular values (error of M_ij relative to sqrt(M_ii M_jj), rms: 1e-2 with the rounded Z on both
-  // sides, 3e-3 as Z^T X^T (X Z_bf16), 1e-5 to 4e-5 this way; the rounding of W itself averages out over the T rows).
-  if (e == cudaSuccess) e = product_y(2);
-  if (e == cudaSuccess) e = launch_gemm<false, true, true>({Yt, l, T, p.Tp}, {Yt, l, T, p.Tp}, p.ritz_split, {(float*)part, nullptr, l}, flags, device, s);
+  // combinations become V, so neither Z nor W may enter rounded to bf16.  A column of Z in the noise floor, rounded, holds
+  // 2^-9 of the largest singular values: error of M_ij relative to sqrt(M_ii M_jj), rms, 1e-2 with the rounded Z on both
+  // sides, 3e-3 as Z^T X^T (X Z_bf16), 1e-5 this way.  The rounding of W averages out over the rows, unless a few of them
+  // hold most of the weight (sigma_1 of a cache with one row a thousand times the others: off by 3.7e-4 with W rounded on
+  // both sides, 1.5e-4 on one).  With W = H + L the symmetric part of H^T (H + 2 L) is M up to L^T L.
+  __nv_bfloat16* Yl = (__nv_bfloat16*)(w + p.off_yl);
+  if (e == cudaSuccess) e = launch_gemm<true, true, false>({X, T, N, N}, {Zb, N, l, l}, 1, {nullptr, Yt, p.Tp, Yl}, flags, device, s, Zb + (size_t)N * l);
+  if (e == cudaSuccess) e = launch_gemm<false, true, true>({Yt, l, T, p.Tp}, {Yt, l, T, p.Tp}, p.ritz_split, {(float*)part, nullptr, l}, flags, device, s, Yl);
   if (e == cudaSuccess) {
     symmetrize_kernel<<<(l * l + 255) / 256, 256, 0, s>>>((const float*)part, p.ritz_split, Mm, l);
     float* M2 = (float*)(w + p.off_m2);

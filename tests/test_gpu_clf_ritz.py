@@ -17,21 +17,26 @@ def _off_diagonal(H, V):
     return float((M - torch.diag(M.diagonal())).pow(2).mean().sqrt())
 
 
-@pytest.mark.parametrize("T,G,d,r", [(4096, 4, 256, 128), (3001, 2, 320, 200), (20000, 4, 128, 64)])
+@pytest.mark.parametrize("T,G,d,r", [(4096, 4, 256, 128), (3001, 2, 320, 200), (8191, 2, 1024, 256)])
 def test_rows_of_b_are_ritz_vectors_to_bf16(T, G, d, r):
-    g = torch.Generator(device="cuda").manual_seed(T)
+    """Three caches each: one rounding of the same vectors differs from another by up to a quarter in this measure, because a
+    few noise directions with a large entry weigh most."""
     N, rho = G * d, r // 2
-    s = 1.0 / torch.arange(1, rho + 1, device="cuda")
-    signal = (torch.randn(T, rho, generator=g, device="cuda") * s) @ torch.randn(rho, N, generator=g, device="cuda")
-    X = (signal / signal.std() + 0.01 * torch.randn(T, N, generator=g, device="cuda")).to(torch.bfloat16)
-    A, B, sig, _ = _factorize_gpu(X, G, d, r, 32, 2, seed=7)
-    Xd = X.double()
-    H = Xd.T @ Xd
-    V = torch.cat([B[i] for i in range(G)], dim=1).double().T                # (N, r)
-    Q = torch.linalg.qr(V)[0]
-    exact = Q @ torch.linalg.eigh(Q.T @ H @ Q)[1]
-    rounded = exact.to(torch.bfloat16).double()
-    assert _off_diagonal(H, V) <= 1.2 * _off_diagonal(H, rounded)
+    got = want = 0.0
+    for seed in (1, 2, 3):
+        g = torch.Generator(device="cuda").manual_seed(T + seed)
+        s = 1.0 / torch.arange(1, rho + 1, device="cuda")
+        signal = (torch.randn(T, rho, generator=g, device="cuda") * s) @ torch.randn(rho, N, generator=g, device="cuda")
+        X = (signal / signal.std() + 0.01 * torch.randn(T, N, generator=g, device="cuda")).to(torch.bfloat16)
+        A, B, sig, _ = _factorize_gpu(X, G, d, r, 32, 2, seed=7 + seed)
+        Xd = X.double()
+        H = Xd.T @ Xd
+        V = torch.cat([B[i] for i in range(G)], dim=1).double().T            # (N, r)
+        Q = torch.linalg.qr(V)[0]
+        exact = Q @ torch.linalg.eigh(Q.T @ H @ Q)[1]
+        got += _off_diagonal(H, V)
+        want += _off_diagonal(H, exact.to(torch.bfloat16).double())
+    assert got <= 1.25 * want
 
 
 @pytest.mark.parametrize("T,N,r", [(4096, 640, 608), (2500, 192, 136)])
@@ -56,3 +61,19 @@ def test_rotations_keep_the_length(T, N, r):
     sv = torch.linalg.svdvals(X.double())[:r]
     drift = (sig.double() / sv - 1).mean().abs()
     assert drift <= (N - 1) * sweeps * 2.0 ** -26 + 2e-6
+
+
+@pytest.mark.parametrize("T,heavy", [(3000, 1e3), (1200, 30.0), (1, 1.0)])
+def test_one_row_holds_the_weight(T, heavy):
+    """A row a thousand times the others (or the only one): no error averages out over the rows.  The largest singular value
+    is that of X up to the two-part bf16 of Z and W (2^-17 each, on both sides), the length of a vector (see above) and fp32
+    sums."""
+    from paper_2503_18893_b200 import xkv
+    g = torch.Generator(device="cuda").manual_seed(T)
+    X = torch.randn(T, 256, generator=g, device="cuda")
+    X[T // 2] *= heavy
+    X = X.to(torch.bfloat16)
+    A, B, sig, _ = _factorize_gpu(X, 2, 128, 64, 32, 2, seed=11)
+    sv = torch.linalg.svdvals(X.double())
+    l, sweeps = 128, 16
+    assert abs(float(sig[0]) / float(sv[0]) - 1) <= 4 * 2.0 ** -17 + (l - 1) * sweeps * 2.0 ** -26 + 1e-6
