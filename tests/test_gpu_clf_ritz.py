@@ -77,3 +77,22 @@ def test_one_row_holds_the_weight(T, heavy):
     sv = torch.linalg.svdvals(X.double())
     l, sweeps = 128, 16
     assert abs(float(sig[0]) / float(sv[0]) - 1) <= 4 * 2.0 ** -17 + (l - 1) * sweeps * 2.0 ** -26 + 1e-6
+
+
+@pytest.mark.parametrize("which", ["row", "column"])
+def test_directions_are_chosen_where_one_holds_the_weight(which):
+    """An outlier row or column leaves the off-diagonal weight below any fraction of the total; the r best of the l directions
+    have to be found all the same.  Converged, the residual is 1.017 and 1.008 times the optimum here (a sketch of 128 for a
+    flat rest of 64 directions); unrotated directions give 1.049 and 1.039."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    T, N = (3000, 256) if which == "row" else (700, 512)
+    X = torch.randn(T, N, generator=g, device="cuda")
+    if which == "row":
+        X[7] *= 1e3
+    else:
+        X[:, 7] *= 1e4
+    X = X.to(torch.bfloat16)
+    A, B, sig, _ = _factorize_gpu(X, 2, N // 2, 64, 32, 2, seed=13)
+    Xd, V = X.double(), torch.cat([B[0], B[1]], dim=1).double()
+    res = float(((Xd - A.double() @ V) ** 2).sum())
+    assert res <= 1.03 * float((torch.linalg.svdvals(Xd)[64:] ** 2).sum())
