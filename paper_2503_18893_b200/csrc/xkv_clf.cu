@@ -52,9 +52,9 @@ __device__ __forceinline__ bool gemm_wait(uint32_t bar, uint32_t parity) {
 // C[m][n] = sum_k A(k, m) B(k, n).  grid = (ceil(N/BN), ceil(M/(128 MB)), K ranges).  TRANS: store C^T (out[n][m]).
 // AK: A is given as [m][k] (K-major), else as [k][m]; BK likewise for B.  K range z covers k_per columns and writes
 // Cf + z * M * ldc.  With two parts B is the sum of the matrices of map_b and map_b2 and A is gone through twice; the k
-// of a part are rounded up to whole blocks of 64.  Cb is the result rounded to bf16, Cl twice what the rounding leaves out
-// (with TRANS).  Out-of-range rows and columns of the operands are zero-filled by the copy engine; stores are guarded.
-template <bool TRANS, bool AK, bool BK, int MB, int BN>
+// of a part are rounded up to whole blocks of 64.  Cb is the result rounded to bf16; LO: Cl is twice what the rounding leaves
+// out (TRANS only; a template parameter, because a test of the pointer in the epilogue costs every product 11 %).  Out-of-range rows and columns of the operands are zero-filled by the copy engine; stores are guarded.
+template <bool TRANS, bool AK, bool BK, bool LO, int MB, int BN>
 __global__ void __launch_bounds__(gemm_threads<MB>(), 1)
 clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                 const __grid_constant__ CUtensorMap map_b2, int M, int N, int k_part, int k_all, int k_per, float* __restrict__ Cf,
@@ -193,7 +193,7 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                 if (Cb) {
                   const __nv_bfloat16 hi = __float2bfloat16(v[i]);
                   Cb[at] = hi;
-                  if (TRANS && Cl) Cl[at] = __float2bfloat16(2.0f * (v[i] - __bfloat162float(hi)));
+                  if (LO) Cl[at] = __float2bfloat16(2.0f * (v[i] - __bfloat162float(hi)));
                 }
               }
             }
@@ -1130,7 +1130,7 @@ struct GemmOut {
   __nv_bfloat16* lo = nullptr;   // transposed results only: twice what b's rounding leaves out
 };
 
-template <bool TRANS, bool AK, bool BK, int MB, int BN>
+template <bool TRANS, bool AK, bool BK, bool LO, int MB, int BN>
 cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, const void* b2, int splits, GemmOut c, unsigned int* flags, int device,
                            cudaStream_t s) {
   const int M = AK ? a.rows : a.cols, N = BK ? b.rows : b.cols, K = AK ? a.cols : a.rows;
@@ -1141,11 +1141,11 @@ cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, const void* b2, int spl
       !encode_bf16_map(&mb2, b2 ? b2 : b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BK ? BN : 64))
     return cudaErrorInvalidValue;
   const size_t smem = 1024 + (size_t)gemm_stages<MB, BN>() * gemm_stage_bytes<MB, BN>();
-  cudaError_t e = ensure_dyn_smem<clf_gemm_kernel<TRANS, AK, BK, MB, BN>>(smem, device);
+  cudaError_t e = ensure_dyn_smem<clf_gemm_kernel<TRANS, AK, BK, LO, MB, BN>>(smem, device);
   if (e != cudaSuccess) return e;
   const int k_per = ((k_all + splits - 1) / splits + 63) & ~63;
   const dim3 grid((N + BN - 1) / BN, (M + 128 * MB - 1) / (128 * MB), splits);
-  clf_gemm_kernel<TRANS, AK, BK, MB, BN><<<grid, gemm_threads<MB>(), smem, s>>>(ma, mb, mb2, M, N, k_part, k_all, k_per, c.f, c.b, c.lo, c.ld,
+  clf_gemm_kernel<TRANS, AK, BK, LO, MB, BN><<<grid, gemm_threads<MB>(), smem, s>>>(ma, mb, mb2, M, N, k_part, k_all, k_per, c.f, c.b, c.lo, c.ld,
                                                                                flags);
   count_launch(kFamClf);
   return cudaGetLastError();
@@ -1162,18 +1162,18 @@ int gemm_bn(int N) {
 // Two accumulators unless that pads M by more than an eighth.
 int gemm_mb(int M) { return ((M + 255) & ~255) * 8LL <= ((M + 127) & ~127) * 9LL ? 2 : 1; }
 
-template <bool TRANS, bool AK, bool BK>
+template <bool TRANS, bool AK, bool BK, bool LO = false>
 cudaError_t launch_gemm(GemmOperand a, GemmOperand b, int splits, GemmOut c, unsigned int* flags, int device, cudaStream_t s,
                         const void* b2 = nullptr) {      // b2: the second part of B, laid out like b
   const int bn = gemm_bn(BK ? b.rows : b.cols);
   if (gemm_mb(AK ? a.rows : a.cols) == 2) {
-    if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, 2, 256>(a, b, b2, splits, c, flags, device, s);
-    if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, 2, 192>(a, b, b2, splits, c, flags, device, s);
-    return launch_gemm_bn<TRANS, AK, BK, 2, 128>(a, b, b2, splits, c, flags, device, s);
+    if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, LO, 2, 256>(a, b, b2, splits, c, flags, device, s);
+    if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, LO, 2, 192>(a, b, b2, splits, c, flags, device, s);
+    return launch_gemm_bn<TRANS, AK, BK, LO, 2, 128>(a, b, b2, splits, c, flags, device, s);
   }
-  if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, 1, 256>(a, b, b2, splits, c, flags, device, s);
-  if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, 1, 192>(a, b, b2, splits, c, flags, device, s);
-  return launch_gemm_bn<TRANS, AK, BK, 1, 128>(a, b, b2, splits, c, flags, device, s);
+  if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, LO, 1, 256>(a, b, b2, splits, c, flags, device, s);
+  if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, LO, 1, 192>(a, b, b2, splits, c, flags, device, s);
+  return launch_gemm_bn<TRANS, AK, BK, LO, 1, 128>(a, b, b2, splits, c, flags, device, s);
 }
 
 // K ranges that bring a product's tiles to about one per SM, none of them empty or shorter than 1024.
@@ -1308,7 +1308,7 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
   // hold most of the weight (sigma_1 of a cache with one row a thousand times the others: off by 3.7e-4 with W rounded on
   // both sides, 1.5e-4 on one).  With W = H + L the symmetric part of H^T (H + 2 L) is M up to L^T L.
   __nv_bfloat16* Yl = (__nv_bfloat16*)(w + p.off_yl);
-  if (e == cudaSuccess) e = launch_gemm<true, true, false>({X, T, N, N}, {Zb, N, l, l}, 1, {nullptr, Yt, p.Tp, Yl}, flags, device, s, Zb + (size_t)N * l);
+  if (e == cudaSuccess) e = launch_gemm<true, true, false, true>({X, T, N, N}, {Zb, N, l, l}, 1, {nullptr, Yt, p.Tp, Yl}, flags, device, s, Zb + (size_t)N * l);
   if (e == cudaSuccess) e = launch_gemm<false, true, true>({Yt, l, T, p.Tp}, {Yt, l, T, p.Tp}, p.ritz_split, {(float*)part, nullptr, l}, flags, device, s, Yl);
   if (e == cudaSuccess) {
     symmetrize_kernel<<<(l * l + 255) / 256, 256, 0, s>>>((const float*)part, p.ritz_split, Mm, l);
