@@ -23,8 +23,8 @@
 //
 // Diagnostic counters (cycles, per CTA, 64 words; see xkv_debug_read_profile): 0 key-stream producer total, 1-3 its
 // waits (rotary/position buffers, positions, ring), 4 tiles; 48 value-stream producer total, 50-51 its waits
-// (positions, ring); key-phase MMA warp: 8 total, 9 accumulator wait, 10 B ring, 11 row ring, 12 issue;
-// value-phase MMA warp: 40 total, 41 accumulator wait, 43 row ring, 44 issue, 45 weights; 17/18 loader waits;
+// (positions, ring); key-phase MMA warp: 8 total, 9 accumulator wait, 11 rows and B slabs, 12 issue;
+// value-phase MMA warp: 40 total, 41 accumulator wait, 43 row ring, 44 issue, 45 weights; 17 loader wait;
 // 24 key epilogue total, 25 positions, 26 accumulator, 27 group barrier, 28 weights buffer; 32 value epilogue
 // total, 33 accumulator.
 #include <cuda.h>
@@ -40,7 +40,6 @@ using namespace ptx;
 
 constexpr int kTile = 128;                       // selected rows per tile
 constexpr int kSlabBytes = kTile * 128;          // 128 rows x 64 bf16 (one 128-byte swizzle row each)
-constexpr int kNB = 4;                           // slots of the B-slab ring
 // Gather producers: four warps (two per stream) issue asynchronous copies; eight where the rows are dequantised on the way,
 // which is instruction work of the producers (4-bit bases at T = 131072, k = 4096: step 111.8 us with four, 93.7 with eight).
 constexpr int prod_warps(int quant) { return quant ? 8 : 4; }
@@ -64,13 +63,12 @@ struct Sched {
 };
 
 struct Bars {        // offsets (in 8-byte words) into the barrier array
-  int full, fullv, emptyk, emptyv, bfull, kfull, kempty, wfull, wempty, pfull, rfree, posfull, vfree, grp, drain, total;
+  int full, fullv, emptyk, emptyv, kfull, kempty, wfull, wempty, pfull, rfree, posfull, vfree, grp, drain, total;
 };
-__host__ __device__ constexpr Bars bar_layout(int na) {
+__host__ __device__ constexpr Bars bar_layout(int pk, int pv) {   // slot pairs of the key ring, of the value ring
   Bars b{};
-  // one release barrier per slot pair and kind of occupant (key-phase or value-phase slabs): a waiter that knows
-  // the kind it waits for is never confused by the other kind's completions
-  b.full = 0; b.fullv = na; b.emptyk = 2 * na; b.emptyv = 2 * na + na / 2; b.bfull = 3 * na; b.kfull = b.bfull + kNB;
+  // one barrier per slot pair and direction: the issuing warp waits once per pair, for everything the pair holds
+  b.full = 0; b.emptyk = pk; b.fullv = 2 * pk; b.emptyv = b.fullv + pv; b.kfull = b.emptyv + pv;
   b.kempty = b.kfull + 2; b.wfull = b.kempty + 2; b.wempty = b.wfull + 2; b.pfull = b.wempty + 2;
   b.rfree = b.pfull + 2; b.posfull = b.rfree + 2; b.vfree = b.posfull + 4; b.grp = b.vfree + 4; b.drain = b.grp + 1; b.total = b.drain + 2;
   return b;
@@ -223,16 +221,20 @@ __device__ __noinline__ LogitsOut<NR> key_logits_rare(uint32_t acc, const float2
   return o;
 }
 
-// Shared memory besides the two rings: weights, rotary rows, queries, positions, barriers.
+// Slots of the ring of gathered key rows, of the ring of the B_k slabs that go with them (slab pair by slab pair).
+constexpr int kKeySlots = 4;
+constexpr int kBarWords = 48;
+// Shared memory besides the rings: weights, rotary rows, queries, positions, barriers.
 template <int DH, int NR>
 __host__ __device__ constexpr int misc_smem_bytes() {
   return (int)(2 * kPBytes + sizeof(float2) * (2 * 16 + 8) * kRopeStride + sizeof(float) * (NR * DH + 2 * NR + 8 * NR) +
-               sizeof(int) * (4 * kTile + 8) + 8 * (3 * 16 + kNB + 24) + 16);
+               sizeof(int) * (4 * kTile + 8) + 8 * kBarWords + 16);
 }
-// Slots of the gathered-row ring: whatever fits beside the B ring.
+// Slots of the ring of gathered value rows: whatever fits beside those two, at most as many.
 template <int DH, int NR>
-__host__ __device__ constexpr int ring_slots() {
-  return ((kSmemLimit - 1024 - misc_smem_bytes<DH, NR>() - kNB * kSlabBytes) / kSlabBytes) & ~1;   // even: released in pairs
+__host__ __device__ constexpr int value_slots() {
+  const int fit = ((kSmemLimit - 1024 - misc_smem_bytes<DH, NR>() - 2 * kKeySlots * kSlabBytes) / kSlabBytes) & ~1;   // even: released in pairs
+  return fit < kKeySlots ? fit : kKeySlots;
 }
 
 // NR: query heads per KV head rounded up to 4, 8 or 16.  WB: most 128-column blocks of r_v (registers of the
@@ -247,19 +249,17 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   constexpr int HALF = DH / 2;
   constexpr int kThreads = fused_threads(QUANT), PW = prod_warps(QUANT), SPT = PW * 16;   // SPT: producer threads per stream
   constexpr int kWarpK = 8 + PW, kWarpB = kWarpK + 1, kWarpV = kWarpK + 2;                // key MMA, B loader, value MMA
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // (through a shuffle, so that the compiler knows it to be the same in all lanes)
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - smem_u32(smem_raw));
-  constexpr int S = ring_slots<DH, NR>();          // gathered-row slots, all of which may be in flight
-  static_assert(S >= 4 && S <= 16, "ring size");   // slot pairs are tracked in 3 bits by the loader
-  static_assert(kNB <= 8, "loader fifo");
-  // the row slabs are two rings: SK for the key stream, SV for the value stream (both even)
-  constexpr int SK = (S % 4 == 0) ? S / 2 : S / 2 + 1, SV = S - SK;
-  static_assert(SK >= 2 && SV >= 2 && SK % 2 == 0 && SV % 2 == 0, "ring split");
+  // rings of slabs: SK of gathered key rows, SV of gathered value rows, SK of B_k slabs (all even, all may be in flight)
+  constexpr int SK = kKeySlots, SV = value_slots<DH, NR>(), S = SK + SV;
+  static_assert(SK >= 2 && SV >= 2 && SK % 2 == 0 && SV % 2 == 0, "rings");
   const uint32_t bring = base + (uint32_t)S * kSlabBytes;                         // B-slab ring
-  // carve-up after the two rings
-  uint8_t* P_gen = gen + (size_t)(S + kNB) * kSlabBytes;                         // [2][kPBytes] bf16 weights (MMA operand)
-  const uint32_t P_addr = base + (uint32_t)(S + kNB) * kSlabBytes;
+  // carve-up after the rings
+  uint8_t* P_gen = gen + (size_t)(S + SK) * kSlabBytes;                          // [2][kPBytes] bf16 weights (MMA operand)
+  const uint32_t P_addr = base + (uint32_t)(S + SK) * kSlabBytes;
   float2* hi_s = reinterpret_cast<float2*>(P_gen + 2 * kPBytes);                 // [2][16][kRopeStride] coarse rotary rows
   float2* lo_s = hi_s + 2 * 16 * kRopeStride;                                    // [8][kRopeStride]     fine rotary rows
   float* q_s = reinterpret_cast<float*>(lo_s + 8 * kRopeStride);                 // [NR][DH]
@@ -268,7 +268,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   int* pos_s = reinterpret_cast<int*>(red_s + 2 * 4 * NR);                       // [4][128]
   int* algn_s = pos_s + 4 * kTile;                                               // [2][4]
   uint64_t* bars = reinterpret_cast<uint64_t*>(algn_s + 8);
-  constexpr Bars bl = bar_layout(S);
+  constexpr Bars bl = bar_layout(SK / 2, SV / 2);
+  static_assert(bl.total <= kBarWords, "barrier space");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + bl.total);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const uint32_t bar0 = smem_u32(bars);
@@ -284,9 +285,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   const int nst_k = (nks_k + 1) & ~1, nst_v = (nks_v + 1) & ~1;
 
   if (tid == 0) {
-    for (int s = 0; s < S; ++s) { mbar_init(BAR(bl.full + s), SPT); mbar_init(BAR(bl.fullv + s), SPT); }
-    for (int s = 0; s < S / 2; ++s) { mbar_init(BAR(bl.emptyk + s), 1); mbar_init(BAR(bl.emptyv + s), 1); }
-    for (int s = 0; s < kNB; ++s) mbar_init(BAR(bl.bfull + s), 1);
+    for (int s = 0; s < SK / 2; ++s) { mbar_init(BAR(bl.full + s), SPT + 1); mbar_init(BAR(bl.emptyk + s), 1); }
+    for (int s = 0; s < SV / 2; ++s) { mbar_init(BAR(bl.fullv + s), SPT); mbar_init(BAR(bl.emptyv + s), 1); }
     for (int b = 0; b < 2; ++b) {
       mbar_init(BAR(bl.kfull + b), 1); mbar_init(BAR(bl.kempty + b), 128);
       mbar_init(BAR(bl.wfull + b), 1); mbar_init(BAR(bl.wempty + b), 128);
@@ -414,13 +414,11 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
         const uint32_t n0 = in0 ? 16u : 0u, n1 = in1 ? 16u : 0u;
         const char* s0 = Ab + (in0 ? ks * 128 : 0);
         const char* s1 = Ab + (in1 ? ks * 128 + 128 : 0);
-        const uint32_t bar = BAR(bar_full + slot);
 #pragma unroll
         for (int i = 0; i < 16; ++i) cp_async16(st + (uint32_t)i * 1024u, s0 + (size_t)ro[i] * row_bytes, n0);
-        cp_async_arrive_noinc(bar);                        // arrives when this thread's copies have landed
 #pragma unroll
         for (int i = 0; i < 16; ++i) cp_async16(st + kSlabBytes + (uint32_t)i * 1024u, s1 + (size_t)ro[i] * row_bytes, n1);
-        cp_async_arrive_noinc(bar + 8u);
+        cp_async_arrive_noinc(BAR(bar_full + pr));         // arrives when this thread's copies have landed
         slot += 2;
         if (slot == RS) slot = 0;
       }
@@ -476,8 +474,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
         }
         asm volatile("cp.async.wait_all;" ::: "memory");   // the staged rotary rows of this tile (key stream) have landed too
         fence_proxy_async();                               // the tensor core reads these stores
-        mbar_arrive(BAR(bar_full + slot));                 // both slabs of the pair are complete when all threads of the stream are done
-        mbar_arrive(BAR(bar_full + slot + 1));
+        mbar_arrive(BAR(bar_full + pr));                   // the pair is complete when all threads of the stream are done
         slot += 2;
         if (slot == RS) slot = 0;
         return true;
@@ -594,56 +591,56 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     // Two issuing threads, each walking its own ring (one thread spends 70-130 cycles per tcgen05.mma and about
     // 235 per tcgen05.commit).
     const bool kside = warp == kWarpK;
-    // the whole warp walks the loop (all values are warp-uniform); one lane issues the tensor-core instructions
+    // The whole warp walks the loop, one elected lane issues.  The key side is a critical chain of the kernel (of 10.0 k
+    // cycles a tile it waited for data in 2.1 k and issued in 3.8 k; the rest were its own instructions between the two), so
+    // a slot pair costs it one wait (gathered rows and B_k slabs arrive on one barrier) instead of four, and branches
+    // outside the issue are taken on a vote, so that the compiler may keep the descriptors in uniform registers, where the
+    // tensor-core instructions take them from.  The kernel alone: 131072 rows, budget 4096, rank 512 45.1 -> 41.7 us; 65536
+    // rows, budget 16384, rank 1024 255.8 -> 239.7; eight heads, rank 256 75.1 -> 70.2; one tile per CTA 18.1 -> 17.2.
     constexpr uint32_t idesc_k = idesc_bf16_f32(128, 128);                     // keys: both operands K-major
     constexpr uint32_t idesc_v = idesc_bf16_f32(128, 16) | (1u << 15);         // values: A is read along its rows (MN-major)
     const int ps = kside ? 8 : 40;
     const long long role_t0 = clock64();
-    int slot = 0, bslot = 0;                          // positions in the row ring and the B ring
-    uint32_t bring_par = 0;
     // This warp is the only consumer of its ring's `full` barriers and sees every phase of them in order, so one
-    // parity bit per slot is enough.
-    uint32_t seen = 0;
+    // parity bit per pair is enough.
+    uint32_t pr = 0, seen = 0;
     // descriptors differ between slots only in the start-address field (units of 16 bytes)
     const uint64_t desc_hi = smem_desc_sw128(0, 0) & 0xFFFFFFFF00000000ull;
+    constexpr uint32_t kSlab16 = kSlabBytes >> 4;
     const uint32_t rows_lo0 = (uint32_t)(smem_desc_sw128(base, 0) & 0xFFFFFFFFull);
     const uint32_t b_lo0 = (uint32_t)(smem_desc_sw128(bring, 0) & 0xFFFFFFFFull);
     // value phase: A = two adjacent row slabs of the value ring read transposed (64 rank columns each, 16384
     // bytes apart), rows advance in 8-row groups of 1024 bytes; B = the weights of 16 heads x 16 rows
-    const uint32_t rows_t_lo0 = (((rows_lo0 & 0xFFFFu) + (uint32_t)SK * (kSlabBytes >> 4)) & 0xFFFFu) | ((uint32_t)(kSlabBytes >> 4) << 16);
+    const uint32_t rows_t_lo0 = (((rows_lo0 & 0xFFFFu) + (uint32_t)SK * kSlab16) & 0xFFFFu) | (kSlab16 << 16);
     const uint32_t p_lo0 = (uint32_t)(smem_desc_sw128(P_addr, 0) & 0xFFFFFFFFull);
+    auto wait_all = [&](uint32_t bar, uint32_t parity, int word) {
+      return __all_sync(0xffffffffu, wait_bar(ctx, bar, parity, word)) != 0;
+    };
     int it = 0;
     bool ok = true;
     TileIter cur;
     iter_begin(cur);
-    while (ok && iter_next(cur, no_op, no_op)) {
+    while (ok && __all_sync(0xffffffffu, iter_next(cur, no_op, no_op))) {
       const int buf = it & 1;
       const uint32_t par = (uint32_t)((it >> 1) & 1);
       if (kside) {
         // ---- keys: K_hat = A_k[S] B_k
         const int last_kk = (((dev.r_k - 1) & 63) >> 4) + 1;    // 16-column steps in the last real slab
         const uint32_t acc = tmem + (uint32_t)(buf * 128);
-        if (!wait_bar(ctx, BAR(bl.kempty + buf), par ^ 1u, ps + 1)) { ok = false; break; }
+        if (!wait_all(BAR(bl.kempty + buf), par ^ 1u, ps + 1)) { ok = false; break; }
         tc_fence_after();
 #pragma unroll 1
-        for (int ks = 0; ks < nst_k && ok; ks += 2) {
-          // one ring-slot pair per iteration: wait for both slabs and their B slabs, then issue all steps at once
-          const bool real1 = ks + 1 < nks_k;             // the second slab of the last pair may be padding
-          const int bslot1 = (bslot + 1 == kNB) ? 0 : bslot + 1;
-          const uint32_t bpar1 = (bslot + 1 == kNB) ? (bring_par ^ 1u) : bring_par;
-          if (!wait_bar(ctx, BAR(bl.bfull + bslot), bring_par, ps + 2)) { ok = false; break; }
-          if (real1 && !wait_bar(ctx, BAR(bl.bfull + bslot1), bpar1, ps + 2)) { ok = false; break; }
-          if (!wait_bar(ctx, BAR(bl.full + slot), (seen >> slot) & 1u, ps + 3)) { ok = false; break; }
-          if (!wait_bar(ctx, BAR(bl.full + slot + 1), (seen >> (slot + 1)) & 1u, ps + 3)) { ok = false; break; }
-          seen ^= 3u << slot;
+        for (int ks = 0; ks < nst_k; ks += 2) {
+          // one ring-slot pair per iteration: rows and B slabs of both slots, then all steps at once
+          if (!wait_all(BAR(bl.full) + 8u * pr, (seen >> pr) & 1u, ps + 3)) { ok = false; break; }
+          seen ^= 1u << pr;
           tc_fence_after();
           const long long i0 = ctx.prof ? clock64() : 0;
-          if (lane == 0) {
-            const uint64_t a_desc = desc_hi | (rows_lo0 + (uint32_t)slot * (kSlabBytes >> 4));
-            const uint64_t b_desc = desc_hi | (b_lo0 + (uint32_t)bslot * (kSlabBytes >> 4));
-            const uint64_t b_desc1 = desc_hi | (b_lo0 + (uint32_t)bslot1 * (kSlabBytes >> 4));
-            const int nkk0 = (ks == nks_k - 1) ? last_kk : 4;
-            const int nkk1 = !real1 ? 0 : ((ks + 1 == nks_k - 1) ? last_kk : 4);
+          const uint64_t a_desc = desc_hi | (rows_lo0 + pr * (2u * kSlab16));
+          const uint64_t b_desc = desc_hi | (b_lo0 + pr * (2u * kSlab16));
+          const int nkk0 = (ks == nks_k - 1) ? last_kk : 4;
+          const int nkk1 = (ks + 1 >= nks_k) ? 0 : ((ks + 1 == nks_k - 1) ? last_kk : 4);   // the second slab of the last pair may be padding
+          if (elect_one()) {
             tc_mma_bf16(acc, a_desc, b_desc, idesc_k, ks ? 1u : 0u);
 #pragma unroll
             for (int kk = 1; kk < 4; ++kk) {
@@ -651,53 +648,47 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
             }
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
-              if (kk < nkk1) tc_mma_bf16(acc, a_desc + (uint32_t)(kSlabBytes >> 4) + 2u * kk, b_desc1 + 2u * kk, idesc_k, 1u);
+              if (kk < nkk1) tc_mma_bf16(acc, a_desc + kSlab16 + 2u * kk, b_desc + kSlab16 + 2u * kk, idesc_k, 1u);
             }
-            tc_commit(BAR(bl.emptyk + (slot >> 1)));   // releases both slabs of the pair (and their B slabs)
+            tc_commit(BAR(bl.emptyk) + 8u * pr);       // releases both slots of the pair (and their B slabs)
             if (ks + 2 >= nst_k) tc_commit(BAR(bl.kfull + buf));
           }
           __syncwarp();
           if (ctx.prof && lane == 0) atomicAdd(ctx.prof + ps + 4, (unsigned long long)(clock64() - i0));
-          slot += 2;
-          if (slot == SK) slot = 0;
-          bslot = bslot1; bring_par = bpar1;
-          if (real1 && ++bslot == kNB) { bslot = 0; bring_par ^= 1u; }
+          if (++pr == SK / 2) pr = 0;
         }
       } else {
         // ---- values: W += A_v[S]^T P^T, one accumulator of 16 columns per 128 rank columns
-        if (!wait_bar(ctx, BAR(bl.wempty + buf), par ^ 1u, ps + 1)) { ok = false; break; }
-        if (!wait_bar(ctx, BAR(bl.pfull + buf), par, ps + 5)) { ok = false; break; }
+        if (!wait_all(BAR(bl.wempty + buf), par ^ 1u, ps + 1)) { ok = false; break; }
+        if (!wait_all(BAR(bl.pfull + buf), par, ps + 5)) { ok = false; break; }
         tc_fence_after();
         const uint32_t accw = tmem + 256u + (uint32_t)(buf * 128);
-        const uint32_t p_lo = p_lo0 + (uint32_t)buf * (kPBytes >> 4);
+        const uint64_t p_desc = desc_hi | (p_lo0 + (uint32_t)buf * (kPBytes >> 4));
 #pragma unroll 1
-        for (int ks = 0; ks < nst_v && ok; ks += 2) {
-          if (!wait_bar(ctx, BAR(bl.fullv + slot), (seen >> slot) & 1u, ps + 3)) { ok = false; break; }
-          if (!wait_bar(ctx, BAR(bl.fullv + slot + 1), (seen >> (slot + 1)) & 1u, ps + 3)) { ok = false; break; }
-          seen ^= 3u << slot;
+        for (int ks = 0; ks < nst_v; ks += 2) {
+          if (!wait_all(BAR(bl.fullv) + 8u * pr, (seen >> pr) & 1u, ps + 3)) { ok = false; break; }
+          seen ^= 1u << pr;
           tc_fence_after();
           const long long i0 = ctx.prof ? clock64() : 0;
-          if (lane == 0) {
-            const uint64_t a_desc = desc_hi | (rows_t_lo0 + (uint32_t)slot * (kSlabBytes >> 4));
-            const uint32_t acc = accw + (uint32_t)(ks >> 1) * 16u;
+          const uint64_t a_desc = desc_hi | (rows_t_lo0 + pr * (2u * kSlab16));
+          const uint32_t acc = accw + (uint32_t)(ks >> 1) * 16u;
+          if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {   // 16 tile rows per step: 2048 bytes down the slab, 32 bytes along P
-              const uint64_t b_desc = desc_hi | (p_lo + (uint32_t)(kk >> 2) * (2048u >> 4) + (uint32_t)(kk & 3) * 2u);
-              tc_mma_bf16(acc, a_desc + (uint32_t)kk * (2048u >> 4), b_desc, idesc_v, kk ? 1u : 0u);
-            }
-            tc_commit(BAR(bl.emptyv + (slot >> 1)));
+            for (int kk = 0; kk < 8; ++kk)   // 16 tile rows per step: 2048 bytes down the slab, 32 bytes along P
+              tc_mma_bf16(acc, a_desc + (uint32_t)kk * (2048u >> 4), p_desc + (uint32_t)(kk >> 2) * (2048u >> 4) + (uint32_t)(kk & 3) * 2u,
+                          idesc_v, kk ? 1u : 0u);
+            tc_commit(BAR(bl.emptyv) + 8u * pr);
             if (ks + 2 >= nst_v) tc_commit(BAR(bl.wfull + buf));
           }
           __syncwarp();
           if (ctx.prof && lane == 0) atomicAdd(ctx.prof + ps + 4, (unsigned long long)(clock64() - i0));
-          slot += 2;
-          if (slot == SV) slot = 0;
+          if (++pr == SV / 2) pr = 0;
         }
       }
       ++it;
     }
     if (ctx.prof && lane == 0) ctx.prof[ps] = (unsigned long long)(clock64() - role_t0);
-    if (!ok && lane == 0) {
+    if (!ok && elect_one()) {          // (the lane that issued)
       // giving up: the tensor-core operations this thread has issued may still be running and the CTA is about to
       // free its tensor memory; wait (again with a limit) until they have retired
       const uint32_t db = BAR(bl.drain + (kside ? 0 : 1));
@@ -707,59 +698,34 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     __syncwarp();
   } else if (warp == kWarpB) {
     // =============================== B_k slab loader (TMA) ===============================
-    // B slab n goes to slot n % kNB, which held slab n - kNB.  That slab's MMAs are known to be complete
-    //   - if it belongs to an earlier tile: when the previous tile's key accumulator was committed (kfull); with one slab
-    //     per tile, when that of the tile before it was;
-    //   - if it belongs to this tile: when the key-ring pair of its stage was released.
-    // In both cases the barrier's previous phase is already known to be complete and its next phase cannot
-    // complete before the slab being loaded is consumed, so the parity test is unambiguous.
-    // Without padding slabs and with at least kNB slabs per tile the second rule also covers a slab of the previous
-    // tile (the pair after next in the same ring position needs the slab being loaded): then the first slabs of a
-    // tile do not have to wait for the end of the previous tile's key phase.
-    const bool by_pair = nks_k == nst_k && nks_k >= kNB && kNB <= SK;
+    // The slabs of a slot pair of the key ring go to the same pair of their own ring, are released with it and arrive on its
+    // barrier: the loader walks the pairs as the key stream's producers do.
     // fault injection (tests of the give-up path): the slabs are never loaded, so the key-phase warp's wait for
     // them runs into its limit and the CTA winds down
     const bool no_b = (dev.inject & XKV_INJECT_FUSED_NO_B) != 0u;
-    int bslot = 0, it = 0, slot = 0;
-    uint32_t cnt_k = 0;                  // per slot pair: parity of the number of pairs that used it
-    uint32_t fifo = 0;                   // per B slot, 4 bits: slot pair (3) and phase parity (1) of the slab it holds
+    uint32_t pr = 0, used = 0, rel_par = 0;   // per slot pair: filled before; parity of the release to wait for next
     bool ok = true;
     TileIter cur;
     iter_begin(cur);
     while (ok && lane == 0 && iter_next(cur, no_op, no_op)) {
       const int head_row = (int)((((size_t)cur.b * dev.G + cur.l) * dev.H_kv + cur.g) * kDP);
-      uint32_t my = 0;
 #pragma unroll 1
-      for (int ks = 0; ks < nks_k; ++ks) {
-        int sl = slot + ks;
-        while (sl >= SK) sl -= SK;
-        if ((ks & 1) == 0) {             // key stages start on even slots: entering a slot pair
-          const int pr = sl >> 1;
-          my = (uint32_t)pr | (((cnt_k >> pr) & 1u) << 3);
-          cnt_k ^= 1u << pr;
+      for (int ks = 0; ks < nst_k; ks += 2) {
+        const uint32_t bit = 1u << pr;
+        if (used & bit) {
+          if (!wait_bar(ctx, BAR(bl.emptyk) + 8u * pr, (rel_par >> pr) & 1u, 17)) { ok = false; break; }
+          rel_par ^= bit;
         }
-        if (ks >= kNB || (by_pair && it > 0)) {
-          const uint32_t e = (fifo >> (4 * bslot)) & 15u;
-          if (!wait_bar(ctx, BAR(bl.emptyk + (int)(e & 7u)), e >> 3, 17)) { ok = false; break; }
-        } else if (nks_k == 1) {
-          // slab n - kNB belongs to tile it-4.  Tile it-2 is waited for, and at every tile, so that no phase of the barrier
-          // is skipped (a test of a phase too early passes: with a first wait at the fifth tile the loader overwrote slabs in
-          // use)
-          if (it >= 2 && !wait_bar(ctx, BAR(bl.kfull + (it & 1)), (uint32_t)(((it - 2) >> 1) & 1), 18)) { ok = false; break; }
-        } else if (it > 0 && it * nks_k + ks >= kNB) {
-          if (!wait_bar(ctx, BAR(bl.kfull + ((it - 1) & 1)), (uint32_t)(((it - 1) >> 1) & 1), 18)) { ok = false; break; }
-        }
-        fifo = (fifo & ~(15u << (4 * bslot))) | (my << (4 * bslot));
+        used |= bit;
         if (!no_b) {
-          mbar_expect_tx(BAR(bl.bfull + bslot), kSlabBytes);
-          tma_load_2d(bring + (uint32_t)bslot * kSlabBytes, &bk_map, ks * 64, head_row, BAR(bl.bfull + bslot));
+          const uint32_t dst = bring + pr * (2u * kSlabBytes), bar = BAR(bl.full) + 8u * pr;
+          const bool second = ks + 1 < nks_k;          // the second slab of the last pair may be padding: not multiplied
+          mbar_expect_tx(bar, second ? 2u * kSlabBytes : (uint32_t)kSlabBytes);
+          tma_load_2d(dst, &bk_map, ks * 64, head_row, bar);
+          if (second) tma_load_2d(dst + kSlabBytes, &bk_map, ks * 64 + 64, head_row, bar);
         }
-        if (++bslot == kNB) bslot = 0;
+        if (++pr == SK / 2) pr = 0;
       }
-      // (a padding slab after an odd number of real slabs sits in the pair that was entered for the last real one)
-      slot += nst_k;
-      while (slot >= SK) slot -= SK;
-      ++it;
     }
   } else if (warp < 4) {
     // =============================== key epilogue: rope, logits, softmax statistics, weights ===============================
@@ -1311,7 +1277,7 @@ merge_segments_multi_kernel(GroupDev dev, Sched sc, TailParts tail, __nv_bfloat1
 
 template <int DH, int NR>
 constexpr size_t fused_smem_bytes() {
-  return 1024 + (size_t)(ring_slots<DH, NR>() + kNB) * kSlabBytes + misc_smem_bytes<DH, NR>();
+  return 1024 + (size_t)(2 * kKeySlots + value_slots<DH, NR>()) * kSlabBytes + misc_smem_bytes<DH, NR>();
 }
 
 template <int DH, int NR, int WB>
@@ -1327,8 +1293,6 @@ cudaError_t launch_fused_t(const xkv_group* grp, int l0, int l1, const __nv_bflo
   sc.n_slots = fused_slots(grp);
   sc.k_cap = k_cap;
   sc.prof = grp->prof;
-  static_assert(bar_layout(ring_slots<DH, NR>()).total <= 3 * 16 + kNB + 24, "barrier space");
-  static_assert(kNB >= 2 && kNB < ring_slots<DH, NR>(), "B ring must be shorter than the row ring");
   static_assert(NR * WB <= 64 && WB <= kMaxBlocks, "value epilogue registers");
   const size_t smem = fused_smem_bytes<DH, NR>();
   CUtensorMap mk;
