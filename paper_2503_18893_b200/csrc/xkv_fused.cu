@@ -57,11 +57,17 @@ struct Sched {
   int tpp;           // tiles per problem = ceil(k_cap / 128)
   int n_tiles;       // problems * tpp
   int n_ctas;
+  int share, extra;  // tiles of a CTA; the first `extra` CTAs take one more
   int n_slots;       // partial slots per problem
   int k_cap;
   unsigned long long* prof;   // diagnostic counters [n_ctas][64] or nullptr
 };
 
+struct Walk {        // a CTA's tiles: [begin, end), the first problem's part ends at next
+  int begin, end, next;
+  int py, ti, l, b, g;   // the first problem: ordinal, tile in it, layer, sequence, head
+  int seg;           // this CTA's segment of it
+};
 struct Bars {        // offsets (in 8-byte words) into the barrier array
   int full, fullv, emptyk, emptyv, kfull, kempty, wfull, wempty, pfull, rfree, posfull, vfree, grp, drain, total;
 };
@@ -74,8 +80,13 @@ __host__ __device__ constexpr Bars bar_layout(int pk, int pv) {   // slot pairs 
   return b;
 }
 
-// cta that owns global tile t when cta i owns tiles [i*N/C, (i+1)*N/C)
-__host__ __device__ __forceinline__ int cta_of_tile(long long t, int C, int N) { return (int)(((t + 1) * C - 1) / N); }
+// CTA i owns tiles [first_tile(i), first_tile(i + 1)); cta_of_tile is the owner of tile t.  32-bit divisions by numbers of
+// the host: three 64-bit ones behind the dependency wait held a CTA's first gather up.
+__device__ __forceinline__ int first_tile(const Sched& sc, int i) { return i * sc.share + min(i, sc.extra); }
+__device__ __forceinline__ int cta_of_tile(const Sched& sc, int t) {
+  const int split = sc.extra * (sc.share + 1);
+  return t < split ? t / (sc.share + 1) : sc.extra + (t - split) / sc.share;
+}
 
 // PROF = false: `prof` is a compile-time null pointer and every diagnostic branch of the kernel folds away (the
 // loops of the kernel have to stay small: the warps of a scheduler share its instruction cache).
@@ -224,11 +235,13 @@ __device__ __noinline__ LogitsOut<NR> key_logits_rare(uint32_t acc, const float2
 // Slots of the ring of gathered key rows, of the ring of the B_k slabs that go with them (slab pair by slab pair).
 constexpr int kKeySlots = 4;
 constexpr int kBarWords = 48;
+constexpr int kWalkInts = 12;
+static_assert(sizeof(Walk) <= kWalkInts * sizeof(int), "walk");
 // Shared memory besides the rings: weights, rotary rows, queries, positions, barriers.
 template <int DH, int NR>
 __host__ __device__ constexpr int misc_smem_bytes() {
   return (int)(2 * kPBytes + sizeof(float2) * (2 * 16 + 8) * kRopeStride + sizeof(float) * (NR * DH + 2 * NR + 8 * NR) +
-               sizeof(int) * (4 * kTile + 8) + 8 * kBarWords + 16);
+               sizeof(int) * (4 * kTile + 8 + kWalkInts) + 8 * kBarWords + 16);
 }
 // Slots of the ring of gathered value rows: whatever fits beside those two, at most as many.
 template <int DH, int NR>
@@ -267,7 +280,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   float* red_s = alpha_s + 2 * NR;                                               // [2][4][NR]
   int* pos_s = reinterpret_cast<int*>(red_s + 2 * 4 * NR);                       // [4][128]
   int* algn_s = pos_s + 4 * kTile;                                               // [2][4]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(algn_s + 8);
+  Walk* walk_s = reinterpret_cast<Walk*>(algn_s + 8);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(algn_s + 8 + kWalkInts);
   constexpr Bars bl = bar_layout(SK / 2, SV / 2);
   static_assert(bl.total <= kBarWords, "barrier space");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + bl.total);
@@ -283,6 +297,17 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   // both phases are padded to an even number of 64-column slabs so that slabs pair up inside ring-slot pairs
   const int nks_k = (dev.r_k + 63) >> 6, nks_v = (dev.r_v + 63) >> 6;
   const int nst_k = (nks_k + 1) & ~1, nst_v = (nks_v + 1) & ~1;
+
+  const int per_layer = dev.batch * dev.H_kv;
+  const int n_rep = dev.n_rep;
+  if (tid == 64) {     // the CTA's range, once (divisions), to shared memory: only the walk's rare steps look at it again
+    const int first = first_tile(sc, blockIdx.x), py = first / sc.tpp, ti = first - py * sc.tpp;
+    walk_s->begin = first; walk_s->end = first_tile(sc, blockIdx.x + 1);
+    walk_s->next = min(walk_s->end, first - ti + sc.tpp);
+    walk_s->py = py; walk_s->ti = ti;
+    walk_s->g = py % dev.H_kv; walk_s->b = (py / dev.H_kv) % dev.batch; walk_s->l = sc.l0 + py / per_layer;
+    walk_s->seg = (int)blockIdx.x - cta_of_tile(sc, py * sc.tpp);
+  }
 
   if (tid == 0) {
     for (int s = 0; s < SK / 2; ++s) { mbar_init(BAR(bl.full + s), SPT + 1); mbar_init(BAR(bl.emptyk + s), 1); }
@@ -319,11 +344,6 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   grid_dependency_wait();
   grid_dependency_launch();
 
-  const int C = sc.n_ctas, N = sc.n_tiles;
-  const long long t_begin = ((long long)blockIdx.x * N) / C, t_end = ((long long)(blockIdx.x + 1) * N) / C;
-  const int per_layer = dev.batch * dev.H_kv;
-  const int n_rep = dev.n_rep;
-
   // Walks this CTA's tiles, skipping tiles that start at or beyond the problem's row count.
   // The tiles of the range's first problem, which are the end of it wherever the range goes on to another problem, come
   // last: the rows of a selection are ascending, so the CTAs then move through the contexts together (each from the start
@@ -333,18 +353,11 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   struct TileIter {
     int t, stop, py, ti, cnt, l, b, g, pyn; long long prob;   // t: tile ordinal of the call; pyn/ti: problem and tile in it
   };
-  // The problem and tile-in-problem of the first tile, the (layer, sequence, head) of that problem and this CTA's
-  // segment number in it, once (divisions); the walk then only counts.  Later problems of the CTA start inside
-  // its tile range, so the CTA holds their first segment.
-  const int py_first = (int)(t_begin / sc.tpp), ti_first = (int)(t_begin % sc.tpp);
-  const int g_first = py_first % dev.H_kv, b_first = (py_first / dev.H_kv) % dev.batch, l_first = sc.l0 + py_first / per_layer;
-  const int seg_first = (int)blockIdx.x - cta_of_tile((long long)py_first * sc.tpp, C, N);
-  const int t_next = (int)min(t_end, t_begin - ti_first + sc.tpp);       // end of the first problem's part
   auto iter_begin = [&](TileIter& it_) {
-    const bool more = t_next < (int)t_end;
-    it_.t = (more ? t_next : (int)t_begin) - 1; it_.stop = (int)t_end;
-    it_.py = -1; it_.cnt = 0; it_.prob = 0; it_.pyn = py_first; it_.ti = more ? sc.tpp - 1 : ti_first - 1;
-    it_.l = l_first; it_.b = b_first; it_.g = g_first;
+    const bool more = walk_s->next < walk_s->end;
+    it_.t = (more ? walk_s->next : walk_s->begin) - 1; it_.stop = walk_s->end;
+    it_.py = -1; it_.cnt = 0; it_.prob = 0; it_.pyn = walk_s->py; it_.ti = (more ? sc.tpp : walk_s->ti) - 1;
+    it_.l = walk_s->l; it_.b = walk_s->b; it_.g = walk_s->g;
   };
   // advance to the next non-empty tile; returns false at the end of the range.  Whenever the walk moves to a new
   // problem (also one whose tiles are all empty), `on_leave()` runs with the old problem still in `it_` (not before
@@ -352,16 +365,16 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   auto iter_next = [&](TileIter& it_, auto&& on_leave, auto&& on_enter) -> bool {
     for (;;) {
       if (++it_.t >= it_.stop) {
-        if (it_.pyn == py_first) return false;            // (the first problem's part is the last)
-        it_.t = (int)t_begin; it_.stop = t_next; it_.pyn = py_first; it_.ti = ti_first;
+        if (it_.pyn == walk_s->py) return false;          // (the first problem's part is the last)
+        it_.t = walk_s->begin; it_.stop = walk_s->next; it_.pyn = walk_s->py; it_.ti = walk_s->ti;
       } else if (++it_.ti == sc.tpp) {
         it_.ti = 0; ++it_.pyn;
       }
       const int py = it_.pyn;
       if (py != it_.py) {
         if (it_.py >= 0) on_leave();
-        if (py == py_first) {
-          it_.l = l_first; it_.b = b_first; it_.g = g_first;
+        if (py == walk_s->py) {
+          it_.l = walk_s->l; it_.b = walk_s->b; it_.g = walk_s->g;
         } else if (++it_.g == dev.H_kv) {
           it_.g = 0; if (++it_.b == dev.batch) { it_.b = 0; ++it_.l; }
         }
@@ -376,7 +389,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   auto no_op = []() {};
   // partial slot of the segment (this CTA's share) of problem ordinal py
   auto part_of = [&](int py, long long prob) {
-    const int seg = py == py_first ? seg_first : 0;
+    const int seg = py == walk_s->py ? walk_s->seg : 0;   // (later problems of the CTA start inside its range)
     return dev.part + ((size_t)prob * sc.n_slots + seg) * (size_t)n_rep * (dev.r_v + 2);
   };
 
@@ -978,8 +991,8 @@ merge_segments_kernel(GroupDev dev, Sched sc, TailParts tail, __nv_bfloat16* __r
   const int per_layer = dev.batch * dev.H_kv;
   const int g = py % dev.H_kv, b = (py / dev.H_kv) % dev.batch, l = sc.l0 + py / per_layer;
   const long long prob = ((long long)l * dev.batch + b) * dev.H_kv + g;
-  const long long first = (long long)py * sc.tpp;
-  const int c0 = cta_of_tile(first, sc.n_ctas, sc.n_tiles), c1 = cta_of_tile(first + sc.tpp - 1, sc.n_ctas, sc.n_tiles);
+  const int first = py * sc.tpp;
+  const int c0 = cta_of_tile(sc, first), c1 = cta_of_tile(sc, first + sc.tpp - 1);
   const int nseg = min(c1 - c0 + 1, kMergeMaxSeg);
   const size_t stride = (size_t)n_rep * (r + 2);
   // the B_v pieces do not depend on the partials: start those loads before anything else
@@ -1134,8 +1147,8 @@ merge_segments_multi_kernel(GroupDev dev, Sched sc, TailParts tail, __nv_bfloat1
   const int per_layer = dev.batch * dev.H_kv;
   const int g = py % dev.H_kv, b = (py / dev.H_kv) % dev.batch, l = sc.l0 + py / per_layer;
   const long long prob = ((long long)l * dev.batch + b) * dev.H_kv + g;
-  const long long first = (long long)py * sc.tpp;
-  const int c0 = cta_of_tile(first, sc.n_ctas, sc.n_tiles), c1 = cta_of_tile(first + sc.tpp - 1, sc.n_ctas, sc.n_tiles);
+  const int first = py * sc.tpp;
+  const int c0 = cta_of_tile(sc, first), c1 = cta_of_tile(sc, first + sc.tpp - 1);
   const int nseg = min(c1 - c0 + 1, kMergeMaxSeg);
   const size_t stride = (size_t)n_rep * (r + 2);
   const int rg = tid / TPR, dg = tid % TPR;
@@ -1302,6 +1315,8 @@ cudaError_t launch_fused_t(const xkv_group* grp, int l0, int l1, const __nv_bflo
   sc.tpp = (k_cap + kTile - 1) / kTile;
   sc.n_tiles = problems * sc.tpp;
   sc.n_ctas = sc.n_tiles < grp->sm_count ? sc.n_tiles : grp->sm_count;
+  sc.share = sc.n_tiles / sc.n_ctas;
+  sc.extra = sc.n_tiles - sc.share * sc.n_ctas;
   sc.n_slots = fused_slots(grp);
   sc.k_cap = k_cap;
   sc.prof = grp->prof;
