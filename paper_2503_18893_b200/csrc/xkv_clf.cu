@@ -648,7 +648,7 @@ __device__ __forceinline__ int2 tournament_pair(int k, int t, int n) {
 }
 
 // The rotation (c, s) that annihilates a_pq: columns (p, q) become (c p - s q, s p + c q).  The formula is on the chain of
-// every round (a cross round: 1165 cycles, 918 with the formula left out), so each step is one approximate instruction and
+// every round (a cross round with all of the submatrix in shared memory: 1165 cycles, 918 with the formula left out), so each step is one approximate instruction and
 // there is no branch.  |tau| too large to square gives t = 0 and the identity; so does an a_pq next to nothing.
 // An error of t leaves a little of a_pq to the next sweep; an error of c^2 + s^2 stays, and thousands of rotations add theirs
 // up, so the root takes a step of Newton's iteration.  Largest entry of P P^T - I, l = 576, 8 sweeps: 3.0e-4 without the
@@ -694,6 +694,105 @@ __device__ __forceinline__ float piece_sum(const float* __restrict__ red, int o)
   return v;
 }
 
+// The 32 rounds of rotations (i, 32 + (i + t) mod 32) of a pair's 64 x 64 submatrix, in registers.  The matrix is symmetric:
+// kept are its 2 x 2 blocks (a, a + e mod 32), e = 0 .. 16, that is rows a and a' = 32 + (a + t) mod 32 by columns b and b'
+// of b = a + e.  Lane = a; warp w of the first four holds e = 4 w + 1 .. 4 w + 4, warp 0 e = 0 as well.  From round to round
+// a' and b' move one on, so x01 comes from block e + 1 of the same lane, x10 from block e - 1 and x11 from block e of the
+// next lane (across two warps through shared memory).  Warp 0 works the next round's rotations out of its blocks 0 and 1
+// while the others still update theirs: the chain of a round is two rotations, the formula and one barrier.  Warps 4-11 hold
+// Q, eight rows each, lane = columns i and 32 + (i + t) mod 32.
+// (The full submatrix in shared memory, 16 warps and all of them computing the formula: 1165 cycles a round; the same in
+// registers: 973.)
+// A function of its own: it wants the registers that the rest of the kernel would keep.  Called by warps 0-11.
+// X, Q0 [64][64]: submatrix and product so far; buf: room for 2 x 64 + 2 x 4 x 64 floats; Qout [64][64].
+constexpr int kCrossWarps = 12;
+__device__ __noinline__ void cross_rotations(const float* __restrict__ X, float* __restrict__ buf, const float* __restrict__ Q0,
+                                             float* __restrict__ Qout) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, up = (lane + 1) & 31;
+  float2* const cs_s = reinterpret_cast<float2*>(buf);       // [2][32]
+  float* const ex_s = buf + 128;                             // [2][4]: x01 of a warp's first block, x10 of its last
+  if (warp >= 4) {
+    float qu[8], qv[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float* row = Q0 + ((warp - 4) * 8 + k) * kJp;
+      qu[k] = row[lane];
+      qv[k] = row[kJb + lane];
+    }
+#pragma unroll 1
+    for (int t = 0; t < kJb; ++t) {
+      ptx::named_bar_sync(1, kCrossWarps * 32);
+      const float2 cs = cs_s[(t & 1) * 32 + lane];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float u = qu[k], v = qv[k];
+        qu[k] = cs.x * u - cs.y * v;
+        qv[k] = __shfl_sync(0xffffffffu, cs.y * u + cs.x * v, up);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {                            // after 32 moves the columns are back where they began
+      float* row = Qout + ((warp - 4) * 8 + k) * kJp;
+      row[lane] = qu[k];
+      row[kJb + lane] = qv[k];
+    }
+    return;
+  }
+  float x00[5], x01[5], x10[5], x11[5];                      // block e = 4 warp + i (i = 0: warp 0 only)
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const int c = (lane + 4 * warp + i) & 31;
+    x00[i] = X[lane * kJp + c]; x01[i] = X[lane * kJp + kJb + c];
+    x10[i] = X[(kJb + lane) * kJp + c]; x11[i] = X[(kJb + lane) * kJp + kJb + c];
+  }
+  float2 cs = make_float2(1.0f, 0.0f);
+  if (warp == 0) cs_s[lane] = cs = jacobi_rotation(x00[0], x11[0], x01[0]);
+  // block i <- R_a^T block R_b for the rotations (ca, sa) of its rows, (cb, sb) of its columns
+  auto turn = [&](int i, float ca, float sa, float cb, float sb) {
+    const float u00 = cb * x00[i] - sb * x01[i], u01 = sb * x00[i] + cb * x01[i];
+    const float u10 = cb * x10[i] - sb * x11[i], u11 = sb * x10[i] + cb * x11[i];
+    x00[i] = ca * u00 - sa * u10; x01[i] = ca * u01 - sa * u11;
+    x10[i] = sa * u00 + ca * u10; x11[i] = sa * u01 + ca * u11;
+  };
+#pragma unroll 1
+  for (int t = 0; t < kJb; ++t) {
+    ptx::named_bar_sync(1, kCrossWarps * 32);                // this round's rotations, the neighbours' blocks of the last
+    float* const ex = ex_s + (t & 1) * 256;
+    const float* const ex_last = ex_s + ((t + 1) & 1) * 256;
+    if (warp != 0) {
+      cs = cs_s[(t & 1) * 32 + lane];
+      if (t > 0) x10[1] = ex_last[(warp - 1) * 64 + 32 + up];
+    }
+    if (t > 0 && warp < 3) x01[4] = ex_last[(warp + 1) * 64 + lane];
+    const float ca = cs.x, sa = cs.y;
+    auto turn_at = [&](int i) {
+      const int from = (lane + 4 * warp + i) & 31;
+      turn(i, ca, sa, __shfl_sync(0xffffffffu, ca, from), __shfl_sync(0xffffffffu, sa, from));
+    };
+    turn_at(1);
+    if (warp == 0) {
+      turn(0, ca, sa, ca, sa);
+      x11[0] = __shfl_sync(0xffffffffu, x11[0], up);
+      cs = jacobi_rotation(x00[0], x11[0], x01[1]);
+      cs_s[((t + 1) & 1) * 32 + lane] = cs;
+    }
+#pragma unroll
+    for (int i = 2; i < 5; ++i) turn_at(i);
+    ex[warp * 64 + lane] = x01[1];
+    ex[warp * 64 + 32 + lane] = x10[4];
+    const float wrap = __shfl_sync(0xffffffffu, x10[3], (lane + 17) & 31);   // block (a, a + 17) is that of (a + 17, a), transposed
+#pragma unroll
+    for (int i = 4; i >= 2; --i) x10[i] = __shfl_sync(0xffffffffu, x10[i - 1], up);
+    if (warp == 0) x10[1] = __shfl_sync(0xffffffffu, x10[0], up);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x01[i] = x01[i + 1];
+    if (warp == 3) x01[4] = wrap;
+    x10[0] = x01[0];
+#pragma unroll
+    for (int i = 1; i < 5; ++i) x11[i] = __shfl_sync(0xffffffffu, x11[i], up);
+  }
+}
+
 __global__ void __launch_bounds__(kJacobiThreads, 1)
 jacobi_block_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __restrict__ Pt, float* __restrict__ Qg, int l,
                     float4* __restrict__ partial, unsigned arrived, GridSync sy) {
@@ -715,6 +814,7 @@ jacobi_block_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __res
 
   // ---- A: rotations of one pair
   auto solve_pair = [&](const float* M, int2 pq, bool inside, float* Qout) {
+    __syncthreads();
     for (int e = tid; e < kJp * kJp; e += kJacobiThreads) {
       S0[e] = __ldcg(M + (size_t)at(pq, e >> 6) * l + at(pq, e & 63));
       S2[e] = (e >> 6) == (e & 63) ? 1.0f : 0.0f;
@@ -764,41 +864,7 @@ jacobi_block_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __res
       }
     }
     __syncthreads();
-    // the pairs (i, 32 + (i + t) mod 32): warps 16-31 follow one round behind with Q in registers, lane = column i and,
-    // shifted by one lane per round, column 32 + (i + t) mod 32
-    float qu[4], qv[4];
-    if (warp >= 16) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float* row = S2 + ((warp - 16) * 4 + k) * kJp;
-        qu[k] = row[lane];
-        qv[k] = row[kJb + lane];
-      }
-    }
-    for (int t = 0; t <= kJb; ++t) {
-      if (warp < 16) {
-        if (t < kJb)
-          round(lane, kJb + ((lane + t) & (kJb - 1)), t & 1, [&](int a) { return make_int2(a, kJb + ((a + t) & (kJb - 1))); });
-      } else if (t > 0) {
-        const float2 cs = cs_s[((t - 1) & 1) * 32 + lane];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float u = qu[k], v = qv[k];
-          qu[k] = cs.x * u - cs.y * v;
-          qv[k] = __shfl_sync(0xffffffffu, cs.y * u + cs.x * v, (lane + 1) & 31);
-        }
-      }
-      __syncthreads();
-      float* x = X; X = Xn; Xn = x;
-    }
-    if (warp >= 16) {                                        // after 32 shifts the columns are back where they began
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        float* row = Qout + ((warp - 16) * 4 + k) * kJp;
-        row[lane] = qu[k];
-        row[kJb + lane] = qv[k];
-      }
-    }
+    if (warp < kCrossWarps) cross_rotations(X, X == S0 ? S1 : S0, S2, Qout);   // (the other buffer is free)
   };
   // ---- eigenvectors: rows of pair pq, columns c0 .. c0 + 63 of Pt  <-  Q^T times them
   auto rotate_vectors = [&](int2 pq, int c0, const float* Q) {
