@@ -247,14 +247,13 @@ constexpr int kLm8MaxRows = 64;     // rows of a table
 template <int DH, bool ROPE>
 __global__ void __launch_bounds__(kLmThreads, 2)
 landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restrict__ landmarks, float* __restrict__ min_cos,
-                 int G, int batch, int T, int H_kv, int n_c, int n_blocks, double rope_base) {
+                 int G, int batch, int T, int H_kv, int n_c, int CPB, int n_blocks, int two_tables, double rope_base) {
   constexpr int HALF = DH / 2, APH = HALF / 8, NBLK = kLmThreads / HALF;
   extern __shared__ __align__(16) uint4 slots_s[];       // [16][kLmThreads] pieces of the chunk on its way, then the table
   __shared__ double2 rot_s[3][ROPE ? kLmThreads : 1];    // a thread's rotation state: its first row, one row on, one block on
   const int tid = threadIdx.x;
   const int TPR = H_kv * APH, RG = kLmThreads / TPR;     // threads per row of all heads, chunks side by side
-  const int CPB = min(RG, kLm8MaxRows / 8);              // chunks of a row block; the other row groups take other layers
-  const int R = CPB * 8, LG = RG / CPB;
+  const int R = CPB * 8, LG = RG / CPB;                  // rows of a block; beyond CPB chunks the row groups take other layers
   const int rg = tid / TPR, tr = tid % TPR;
   const int g = tr / APH, a = tr % APH;
   const int jc = rg % CPB, lg = rg / CPB;
@@ -276,7 +275,8 @@ landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restri
     rot_s[2][tid] = v;
   }
   float* const tab_f = reinterpret_cast<float*>(tab_s) + ((((ii & 7) >> 1) * APH + (ii >> 3)) * 4 + (ii & 1));
-  const ulonglong2* const tab = reinterpret_cast<const ulonglong2*>(tab_s) + a;
+  const ulonglong2* const tab0 = reinterpret_cast<const ulonglong2*>(tab_s) + a;
+  const int tab_floats = R * HALF * 2;                    // of one table
 
   uint4 u1[8], u2[8];
   uint4* const slot = slots_s + tid;
@@ -285,49 +285,61 @@ landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restri
     const int j = blk * CPB + jc;
     if (j >= n_c) return;
     const int row0 = j * 8, last = min(8, T - row0) - 1;
-    const __nv_bfloat16* kr = keys + ((size_t)lb * T + row0) * d + (size_t)g * DH + a * 8;
+    const __nv_bfloat16* p = keys + ((size_t)lb * T + row0) * d + (size_t)g * DH + a * 8;
+    uint32_t to = slot_addr;
+    auto row = [&]() {
+      ptx::cp_async16(to, p, 16u);
+      ptx::cp_async16(to + kLmThreads * 16, p + HALF, 16u);
+      to += 2 * kLmThreads * 16;
+    };
+    if (last == 7) {                                      // every chunk but a ragged last one: a row is one addition away
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const __nv_bfloat16* p = kr + (size_t)min(r, last) * d;
-      ptx::cp_async16(slot_addr + (uint32_t)(2 * r) * (kLmThreads * 16), p, 16u);
-      ptx::cp_async16(slot_addr + (uint32_t)(2 * r + 1) * (kLmThreads * 16), p + HALF, 16u);
+      for (int r = 0; r < 8; ++r, p += d) row();
+    } else {
+#pragma unroll 1
+      for (int r = 0; r < 8; ++r) { row(); if (r < last) p += d; }
     }
   };
   // (only the lanes of one head take part: the row groups of a warp may be in different chunks)
   const uint32_t hmask = ((1u << APH) - 1u) << ((tid & 31) & ~(APH - 1));
-  // couple e (pairs 2e, 2e + 1) of row r, rotated with table row trow: first half y1, second half y2
-  auto rotated = [&](int r, int trow, int e, u64& y1, u64& y2) {
+  // couple e (pairs 2e, 2e + 1) of row r: first half x1, second half x2
+  auto couple = [&](int r, int e, u64& x1, u64& x2) {
     const uint32_t w1 = e == 0 ? u1[r].x : e == 1 ? u1[r].y : e == 2 ? u1[r].z : u1[r].w;
     const uint32_t w2 = e == 0 ? u2[r].x : e == 1 ? u2[r].y : e == 2 ? u2[r].z : u2[r].w;
-    const u64 x1 = pack2(__uint_as_float(w1 << 16), __uint_as_float(w1 & 0xffff0000u));
-    const u64 x2 = pack2(__uint_as_float(w2 << 16), __uint_as_float(w2 & 0xffff0000u));
-    if (ROPE) {
-      const ulonglong2 t = tab[((size_t)trow * 4 + e) * APH];
-      const float2 s2 = unpack2(mul2(x2, t.y));
-      y1 = fma2(x1, t.x, pack2(-s2.x, -s2.y));
-      y2 = fma2(x2, t.x, mul2(x1, t.y));
-    } else {
-      y1 = x1; y2 = x2;
+    x1 = pack2(__uint_as_float(w1 << 16), __uint_as_float(w1 & 0xffff0000u));
+    x2 = pack2(__uint_as_float(w2 << 16), __uint_as_float(w2 & 0xffff0000u));
+  };
+  // ca - sb with the product sb rounded first (the scalar instruction negates an operand for nothing, the packed one does not)
+  auto fms = [&](u64 c, u64 a, u64 sb) {
+    const float2 cf = unpack2(c), af = unpack2(a), bf = unpack2(sb);
+    return pack2(fmaf(cf.x, af.x, -bf.x), fmaf(cf.y, af.y, -bf.y));
+  };
+  auto fill_table = [&](int buf) {                        // the next block's table, and the state one block on
+    float* to = tab_f + buf * tab_floats;
+    const double2 at = rot_s[0][tid], one = rot_s[1][tid], jump = rot_s[2][tid];
+    double c1 = at.x, s1 = at.y;
+    for (int r = r_begin; r < r_begin + RPB; ++r) {
+      to[(size_t)r * HALF * 2] = (float)c1;
+      to[(size_t)r * HALF * 2 + 2] = (float)s1;
+      const double c2 = c1 * one.x - s1 * one.y, s2 = s1 * one.x + c1 * one.y;
+      c1 = c2; s1 = s2;
     }
+    rot_s[0][tid] = make_double2(at.x * jump.x - at.y * jump.y, at.y * jump.x + at.x * jump.y);
   };
 
   if (b_begin < b_end && lg < n_lb) request_chunk(b_begin, lg);
   for (int blk = b_begin; blk < b_end; ++blk) {
+    const int buf = two_tables ? (blk - b_begin) & 1 : 0;
     if (ROPE) {
-      __syncthreads();                                    // everybody is done with the table of the previous block
-      if (fills) {
-        const double2 at = rot_s[0][tid], one = rot_s[1][tid], jump = rot_s[2][tid];
-        double c1 = at.x, s1 = at.y;
-        for (int r = r_begin; r < r_begin + RPB; ++r) {
-          tab_f[(size_t)r * HALF * 2] = (float)c1;
-          tab_f[(size_t)r * HALF * 2 + 2] = (float)s1;
-          const double c2 = c1 * one.x - s1 * one.y, s2 = s1 * one.x + c1 * one.y;
-          c1 = c2; s1 = s2;
-        }
-        rot_s[0][tid] = make_double2(at.x * jump.x - at.y * jump.y, at.y * jump.x + at.x * jump.y);
+      // With two tables the next block's is written while this one's rows are read: one barrier a block.
+      if (!two_tables || blk == b_begin) {
+        __syncthreads();                                  // everybody is done with the table of the previous block
+        if (fills) fill_table(0);
       }
       __syncthreads();
+      if (two_tables && fills && blk + 1 < b_end) fill_table(buf ^ 1);
     }
+    const ulonglong2* const tab = tab0 + buf * (tab_floats / 4);
     const int j = blk * CPB + jc;
     for (int lb = lg; lb < n_lb; lb += LG) {
       // this thread's own copies have landed; into registers, and the next chunk on its way
@@ -346,10 +358,16 @@ landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restri
         if (r < rows) {
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            u64 y1, y2;
-            rotated(r, jc * 8 + r, e, y1, y2);
-            s1[e] = add2(s1[e], y1);
-            s2[e] = add2(s2[e], y2);
+            u64 x1, x2;
+            couple(r, e, x1, x2);
+            if (ROPE) {
+              const ulonglong2 t = tab[((size_t)(jc * 8 + r) * 4 + e) * APH];
+              const u64 y1 = fms(x1, t.x, mul2(x2, t.y));
+              x2 = fma2(x2, t.x, mul2(x1, t.y));
+              x1 = y1;
+            }
+            s1[e] = add2(s1[e], x1);
+            s2[e] = add2(s2[e], x2);
           }
         }
       }
@@ -367,34 +385,48 @@ landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restri
       *reinterpret_cast<uint4*>(L) = pack8(m1);
       *reinterpret_cast<uint4*>(L + HALF) = pack8(m2);
       if (min_cos) {
-        float v[16], mn2 = 0.0f;                          // per row: dot product with the mean, squared norm
+        // The dot product of a rotated row and the mean is that of the row and the mean rotated back, and a rotation
+        // changes no norm: per two pairs four instructions turn the mean, two and two more are the sums.
+        float v[8], mn2 = 0.0f;                           // per row: dot product with the mean, squared norm
 #pragma unroll
         for (int e = 0; e < 8; ++e) mn2 += m1[e] * m1[e] + m2[e] * m2[e];
 #pragma unroll
         for (int o = 1; o < APH; o <<= 1) mn2 += __shfl_xor_sync(hmask, mn2, o);
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
+        auto row_sums = [&](int r, float& dot, float& nn) {
           const int trow = jc * 8 + min(r, rows - 1);     // a repeated last row changes no minimum
-          float dot = 0.0f, nn = 0.0f;
+          u64 dot2 = 0ull, nn2 = 0ull;
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            u64 y1, y2;
-            rotated(r, trow, e, y1, y2);
-            const float2 p = unpack2(fma2(y1, s1[e], mul2(y2, s2[e]))), q = unpack2(fma2(y1, y1, mul2(y2, y2)));
-            dot = (dot + p.x) + p.y;
-            nn = (nn + q.x) + q.y;
+            u64 x1, x2, b1 = s1[e], b2 = s2[e];
+            couple(r, e, x1, x2);
+            if (ROPE) {
+              const ulonglong2 t = tab[((size_t)trow * 4 + e) * APH];
+              b1 = fma2(s1[e], t.x, mul2(s2[e], t.y));
+              b2 = fms(s2[e], t.x, mul2(s1[e], t.y));
+            }
+            dot2 = fma2(x2, b2, fma2(x1, b1, dot2));
+            nn2 = fma2(x2, x2, fma2(x1, x1, nn2));
           }
-          v[2 * r] = dot; v[2 * r + 1] = nn;
-        }
+          const float2 p = unpack2(dot2), q = unpack2(nn2);
+          dot = p.x + p.y; nn = q.x + q.y;
+        };
         // fold by halving: after the step with distance o a lane keeps the half of the rows its bit selects
-#pragma unroll
-        for (int o = 1, n = 8; o < APH; o <<= 1, n >>= 1) {
+        auto folded = [&](int o, float lo, float hi) {
           const bool up = (a & o) != 0;
+          const float mine = up ? hi : lo, other = up ? lo : hi;
+          return mine + __shfl_xor_sync(hmask, other, o);
+        };
 #pragma unroll
-          for (int i = 0; i < n; ++i) {
-            const float mine = up ? v[n + i] : v[i], other = up ? v[i] : v[n + i];
-            v[i] = mine + __shfl_xor_sync(hmask, other, o);
-          }
+        for (int r = 0; r < 4; ++r) {
+          float dot, nn, dot4, nn4;
+          row_sums(r, dot, nn);
+          row_sums(r + 4, dot4, nn4);
+          v[2 * r] = folded(1, dot, dot4); v[2 * r + 1] = folded(1, nn, nn4);
+        }
+#pragma unroll
+        for (int o = 2, n = 4; o < APH; o <<= 1, n >>= 1) {
+#pragma unroll
+          for (int i = 0; i < n; ++i) v[i] = folded(o, v[i], v[n + i]);
         }
         float best = INFINITY;
 #pragma unroll
@@ -415,21 +447,26 @@ template <int DH>
 cudaError_t launch_landmark8(const __nv_bfloat16* keys, __nv_bfloat16* landmarks, float* min_cos, int G, int batch, int T,
                              int H_kv, float rope_base, cudaStream_t s) {
   const int n_c = (T + 7) / 8, tpr = H_kv * DH / 16;
-  const int cpb = kLmThreads / tpr < kLm8MaxRows / 8 ? kLmThreads / tpr : kLm8MaxRows / 8;
+  const int rg = kLmThreads / tpr;
+  const bool rope = rope_base > 0.0f;
+  int cpb = rg < kLm8MaxRows / 8 ? rg : kLm8MaxRows / 8;
+  // Two CTAs of an SM have room for two tables of 16 KB each: 64 rows of 32 pairs or 32 rows of 64.  Of 64 pairs the
+  // block keeps 64 rows (and one table) only where the row groups beyond 32 rows would find no layer of their own.
+  if (DH == 128 && cpb == 8 && rg / 4 <= G * batch) cpb = 4;
+  const size_t table = rope ? (size_t)cpb * 8 * (DH / 2) * sizeof(float2) : 0;
+  const int two_tables = table <= 16384 ? 1 : 0;
   const int n_blocks = (n_c + cpb - 1) / cpb;
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = device_sms(dev, &sms);
   if (e != cudaSuccess) return e;
   const int grid = n_blocks < 2 * sms ? n_blocks : 2 * sms;           // two CTAs per SM, one wave
-  const bool rope = rope_base > 0.0f;
-  const size_t smem = (size_t)kLmThreads * 256 + (rope ? (size_t)cpb * 8 * (DH / 2) * sizeof(float2) : 0);
+  const size_t smem = (size_t)kLmThreads * 256 + (two_tables ? 2 : 1) * table;
+  auto kernel = rope ? landmark8_kernel<DH, true> : landmark8_kernel<DH, false>;
   e = rope ? ensure_dyn_smem<landmark8_kernel<DH, true>>(smem, dev) : ensure_dyn_smem<landmark8_kernel<DH, false>>(smem, dev);
   if (e != cudaSuccess) return e;
-  if (rope)
-    landmark8_kernel<DH, true><<<grid, kLmThreads, smem, s>>>(keys, landmarks, min_cos, G, batch, T, H_kv, n_c, n_blocks, (double)rope_base);
-  else
-    landmark8_kernel<DH, false><<<grid, kLmThreads, smem, s>>>(keys, landmarks, min_cos, G, batch, T, H_kv, n_c, n_blocks, 1.0);
+  kernel<<<grid, kLmThreads, smem, s>>>(keys, landmarks, min_cos, G, batch, T, H_kv, n_c, cpb, n_blocks, two_tables,
+                                        rope ? (double)rope_base : 1.0);
   return cudaGetLastError();
 }
 
