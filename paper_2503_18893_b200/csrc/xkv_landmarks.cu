@@ -237,19 +237,24 @@ using namespace ptx;                // packed fp32
 // layer) and head, so its fp64 work (an eighth of the fp32 rate here) is divided by batch * G: per CTA and layer, as in
 // the kernel above, it took as long as everything else together.  The rotation is advanced in fp64 from block to block;
 // pow and sincos run once per CTA.
-// A thread holds the 8 rows of its 8 rotary pairs in registers (64 registers), so the cosine pass reads nothing again,
-// while its next chunk is on the way into 256 bytes of shared memory of its own (no barrier: nobody else reads them).
-// The arithmetic is packed fp32 (two pairs per instruction).  The sums of the cosine pass over the threads of a head are
-// folded by halving (a lane ends with one row: 14 shuffles for the 16 sums of a chunk instead of 6 per row).
-// 131072 rows of four layers of eight heads of 128 with cosines: 677 us -> 320 us; what bounds it now is instruction issue
-// and the table loads from shared memory.
+// A thread holds the 8 rows of its 8 rotary pairs in registers, so nothing is read again, while its next chunks are on the
+// way into 256 bytes each of shared memory of its own (no barrier: nobody else reads them).  The arithmetic is packed fp32
+// (two pairs per instruction), the sums of the cosine pass over the threads of a head are folded by halving (a lane ends
+// with one row: 14 shuffles for the 16 sums of a chunk instead of 6 per row).
+// With cosines the rotated rows stay in registers too (128 of them): a 16-byte load for every thread of a warp takes the
+// shared-memory pipe four cycles whether the addresses agree or not, and the second reading of the table, with the second
+// rotation, was a third of the instructions and of that pipe's time.  That leaves room for one CTA per SM, which keeps two
+// chunks per thread on their way.  131072 rows of four layers of eight heads of 128: 296 us with two CTAs rotating twice,
+// 239 with one (5.1 TB/s); 2048 rows 21.4 -> 16.4.  Without cosines two CTAs per SM with the raw rows in registers: 211 us
+// (5.7 TB/s; 197 without rotation).  What is left is the start of a CTA (pow, sincospi) and 64 to 128 KB in flight per SM.
 constexpr int kLm8MaxRows = 64;     // rows of a table
-template <int DH, bool ROPE>
-__global__ void __launch_bounds__(kLmThreads, 2)
+template <int DH, bool ROPE, bool COS>
+__global__ void __launch_bounds__(kLmThreads, COS ? 1 : 2)
 landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restrict__ landmarks, float* __restrict__ min_cos,
                  int G, int batch, int T, int H_kv, int n_c, int CPB, int n_blocks, int two_tables, double rope_base) {
   constexpr int HALF = DH / 2, APH = HALF / 8, NBLK = kLmThreads / HALF;
-  extern __shared__ __align__(16) uint4 slots_s[];       // [16][kLmThreads] pieces of the chunk on its way, then the table
+  constexpr int SLOTS = COS ? 2 : 1;                     // chunks of a thread on their way
+  extern __shared__ __align__(16) uint4 slots_s[];       // [SLOTS][16][kLmThreads] pieces of the chunks on their way, then the tables
   __shared__ double2 rot_s[3][ROPE ? kLmThreads : 1];    // a thread's rotation state: its first row, one row on, one block on
   const int tid = threadIdx.x;
   const int TPR = H_kv * APH, RG = kLmThreads / TPR;     // threads per row of all heads, chunks side by side
@@ -259,7 +264,7 @@ landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restri
   const int jc = rg % CPB, lg = rg / CPB;
   const int d = H_kv * DH, n_lb = G * batch;
   const int b_begin = (int)((long long)blockIdx.x * n_blocks / gridDim.x), b_end = (int)((long long)(blockIdx.x + 1) * n_blocks / gridDim.x);
-  float4* const tab_s = reinterpret_cast<float4*>(slots_s + 16 * kLmThreads);     // [row][4][APH] {cos, cos, sin, sin} of two pairs
+  float4* const tab_s = reinterpret_cast<float4*>(slots_s + SLOTS * 16 * kLmThreads);     // [row][4][APH] {cos, cos, sin, sin} of two pairs
 
   // this thread's share of the table: pair ii, rows [r_begin, r_begin + RPB) of every block
   const int ii = tid % HALF, RPB = max(1, R / NBLK), r_begin = (tid / HALF) * RPB;
@@ -279,14 +284,13 @@ landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restri
   const int tab_floats = R * HALF * 2;                    // of one table
 
   uint4 u1[8], u2[8];
-  uint4* const slot = slots_s + tid;
-  const uint32_t slot_addr = ptx::smem_u32(slot);
-  auto request_chunk = [&](int blk, int lb) {             // lb = sequence * G + layer
+  const uint32_t slot_addr = ptx::smem_u32(slots_s + tid);
+  auto request_chunk = [&](int blk, int lb, int at) {     // lb = sequence * G + layer
     const int j = blk * CPB + jc;
-    if (j >= n_c) return;
+    if (blk >= b_end || j >= n_c || lb >= n_lb) return;
     const int row0 = j * 8, last = min(8, T - row0) - 1;
     const __nv_bfloat16* p = keys + ((size_t)lb * T + row0) * d + (size_t)g * DH + a * 8;
-    uint32_t to = slot_addr;
+    uint32_t to = slot_addr + (uint32_t)at * (16 * kLmThreads * 16);
     auto row = [&]() {
       ptx::cp_async16(to, p, 16u);
       ptx::cp_async16(to + kLmThreads * 16, p + HALF, 16u);
@@ -327,7 +331,16 @@ landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restri
     rot_s[0][tid] = make_double2(at.x * jump.x - at.y * jump.y, at.y * jump.x + at.x * jump.y);
   };
 
-  if (b_begin < b_end && lg < n_lb) request_chunk(b_begin, lg);
+  // the chunk that is requested next: this thread's layers of a block, then the next block
+  int req_blk = b_begin, req_lb = lg, slot = 0;
+  auto request_next = [&](int at) {
+    request_chunk(req_blk, req_lb, at);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    req_lb += LG;
+    if (req_lb >= n_lb) { req_lb = lg; ++req_blk; }
+  };
+#pragma unroll
+  for (int i = 0; i < SLOTS; ++i) request_next(i);
   for (int blk = b_begin; blk < b_end; ++blk) {
     const int buf = two_tables ? (blk - b_begin) & 1 : 0;
     if (ROPE) {
@@ -343,31 +356,35 @@ landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restri
     const int j = blk * CPB + jc;
     for (int lb = lg; lb < n_lb; lb += LG) {
       // this thread's own copies have landed; into registers, and the next chunk on its way
-      asm volatile("cp.async.wait_all;" ::: "memory");
+      asm volatile("cp.async.wait_group %0;" ::"n"(SLOTS - 1) : "memory");
+      const uint4* const from = slots_s + slot * (16 * kLmThreads) + tid;
 #pragma unroll
-      for (int r = 0; r < 8; ++r) { u1[r] = slot[(2 * r) * kLmThreads]; u2[r] = slot[(2 * r + 1) * kLmThreads]; }
-      if (lb + LG < n_lb) request_chunk(blk, lb + LG);
-      else if (blk + 1 < b_end) request_chunk(blk + 1, lg);
+      for (int r = 0; r < 8; ++r) { u1[r] = from[(2 * r) * kLmThreads]; u2[r] = from[(2 * r + 1) * kLmThreads]; }
+      request_next(slot);
+      if (SLOTS == 2) slot ^= 1;
       if (j >= n_c) continue;
       const int rows = min(8, T - j * 8);
       u64 s1[4], s2[4];
+      u64 y1[COS ? 8 : 1][4], y2[COS ? 8 : 1][4];         // the rotated rows
 #pragma unroll
       for (int e = 0; e < 4; ++e) s1[e] = s2[e] = 0ull;
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
-        if (r < rows) {
+        if (COS || r < rows) {
+          const int trow = jc * 8 + min(r, rows - 1), k = COS ? r : 0;
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            u64 x1, x2;
-            couple(r, e, x1, x2);
+            couple(r, e, y1[k][e], y2[k][e]);
             if (ROPE) {
-              const ulonglong2 t = tab[((size_t)(jc * 8 + r) * 4 + e) * APH];
-              const u64 y1 = fms(x1, t.x, mul2(x2, t.y));
-              x2 = fma2(x2, t.x, mul2(x1, t.y));
-              x1 = y1;
+              const ulonglong2 t = tab[((size_t)trow * 4 + e) * APH];
+              const u64 x1 = y1[k][e], x2 = y2[k][e];
+              y1[k][e] = fms(x1, t.x, mul2(x2, t.y));
+              y2[k][e] = fma2(x2, t.x, mul2(x1, t.y));
             }
-            s1[e] = add2(s1[e], x1);
-            s2[e] = add2(s2[e], x2);
+            if (r < rows) {
+              s1[e] = add2(s1[e], y1[k][e]);
+              s2[e] = add2(s2[e], y2[k][e]);
+            }
           }
         }
       }
@@ -384,28 +401,18 @@ landmark8_kernel(const __nv_bfloat16* __restrict__ keys, __nv_bfloat16* __restri
       __nv_bfloat16* L = landmarks + (((size_t)lb * H_kv + g) * n_c + j) * DH + a * 8;
       *reinterpret_cast<uint4*>(L) = pack8(m1);
       *reinterpret_cast<uint4*>(L + HALF) = pack8(m2);
-      if (min_cos) {
-        // The dot product of a rotated row and the mean is that of the row and the mean rotated back, and a rotation
-        // changes no norm: per two pairs four instructions turn the mean, two and two more are the sums.
+      if constexpr (COS) {
         float v[8], mn2 = 0.0f;                           // per row: dot product with the mean, squared norm
 #pragma unroll
         for (int e = 0; e < 8; ++e) mn2 += m1[e] * m1[e] + m2[e] * m2[e];
 #pragma unroll
         for (int o = 1; o < APH; o <<= 1) mn2 += __shfl_xor_sync(hmask, mn2, o);
         auto row_sums = [&](int r, float& dot, float& nn) {
-          const int trow = jc * 8 + min(r, rows - 1);     // a repeated last row changes no minimum
-          u64 dot2 = 0ull, nn2 = 0ull;
+          u64 dot2 = 0ull, nn2 = 0ull;                    // (a repeated last row changes no minimum)
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            u64 x1, x2, b1 = s1[e], b2 = s2[e];
-            couple(r, e, x1, x2);
-            if (ROPE) {
-              const ulonglong2 t = tab[((size_t)trow * 4 + e) * APH];
-              b1 = fma2(s1[e], t.x, mul2(s2[e], t.y));
-              b2 = fms(s2[e], t.x, mul2(s1[e], t.y));
-            }
-            dot2 = fma2(x2, b2, fma2(x1, b1, dot2));
-            nn2 = fma2(x2, x2, fma2(x1, x1, nn2));
+            dot2 = fma2(y2[r][e], s2[e], fma2(y1[r][e], s1[e], dot2));
+            nn2 = fma2(y2[r][e], y2[r][e], fma2(y1[r][e], y1[r][e], nn2));
           }
           const float2 p = unpack2(dot2), q = unpack2(nn2);
           dot = p.x + p.y; nn = q.x + q.y;
@@ -448,25 +455,33 @@ cudaError_t launch_landmark8(const __nv_bfloat16* keys, __nv_bfloat16* landmarks
                              int H_kv, float rope_base, cudaStream_t s) {
   const int n_c = (T + 7) / 8, tpr = H_kv * DH / 16;
   const int rg = kLmThreads / tpr;
-  const bool rope = rope_base > 0.0f;
+  const bool rope = rope_base > 0.0f, cosines = min_cos != nullptr;
   int cpb = rg < kLm8MaxRows / 8 ? rg : kLm8MaxRows / 8;
-  // Two CTAs of an SM have room for two tables of 16 KB each: 64 rows of 32 pairs or 32 rows of 64.  Of 64 pairs the
-  // block keeps 64 rows (and one table) only where the row groups beyond 32 rows would find no layer of their own.
-  if (DH == 128 && cpb == 8 && rg / 4 <= G * batch) cpb = 4;
+  // Two tables, so that a block costs one barrier and its fp64 work runs beside the others' rows (40003 rows of four layers
+  // of four heads, without cosines, 57.3 -> 50.5 us).  One CTA of an SM has room for any two, two CTAs for 16 KB tables: 64
+  // rows of 32 pairs or 32 rows of 64.  Of 64 pairs the block keeps 64 rows (and one table) only where the row groups
+  // beyond 32 rows would find no layer of their own.
+  if (DH == 128 && cpb == 8 && !cosines && rg / 4 <= G * batch) cpb = 4;
   const size_t table = rope ? (size_t)cpb * 8 * (DH / 2) * sizeof(float2) : 0;
-  const int two_tables = table <= 16384 ? 1 : 0;
+  const int two_tables = cosines || table <= 16384 ? 1 : 0;
   const int n_blocks = (n_c + cpb - 1) / cpb;
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = device_sms(dev, &sms);
   if (e != cudaSuccess) return e;
-  const int grid = n_blocks < 2 * sms ? n_blocks : 2 * sms;           // two CTAs per SM, one wave
-  const size_t smem = (size_t)kLmThreads * 256 + (two_tables ? 2 : 1) * table;
-  auto kernel = rope ? landmark8_kernel<DH, true> : landmark8_kernel<DH, false>;
-  e = rope ? ensure_dyn_smem<landmark8_kernel<DH, true>>(smem, dev) : ensure_dyn_smem<landmark8_kernel<DH, false>>(smem, dev);
+  const int ctas = cosines ? sms : 2 * sms;                           // one wave
+  const int grid = n_blocks < ctas ? n_blocks : ctas;
+  const size_t smem = (size_t)kLmThreads * 256 * (cosines ? 2 : 1) + (two_tables ? 2 : 1) * table;
+  const int variant = (rope ? 2 : 0) + (cosines ? 1 : 0);
+  auto launch = [&](auto kernel) {
+    kernel<<<grid, kLmThreads, smem, s>>>(keys, landmarks, min_cos, G, batch, T, H_kv, n_c, cpb, n_blocks, two_tables,
+                                          rope ? (double)rope_base : 1.0);
+  };
+  if (variant == 3 && (e = ensure_dyn_smem<landmark8_kernel<DH, true, true>>(smem, dev)) == cudaSuccess) launch(landmark8_kernel<DH, true, true>);
+  if (variant == 2 && (e = ensure_dyn_smem<landmark8_kernel<DH, true, false>>(smem, dev)) == cudaSuccess) launch(landmark8_kernel<DH, true, false>);
+  if (variant == 1 && (e = ensure_dyn_smem<landmark8_kernel<DH, false, true>>(smem, dev)) == cudaSuccess) launch(landmark8_kernel<DH, false, true>);
+  if (variant == 0 && (e = ensure_dyn_smem<landmark8_kernel<DH, false, false>>(smem, dev)) == cudaSuccess) launch(landmark8_kernel<DH, false, false>);
   if (e != cudaSuccess) return e;
-  kernel<<<grid, kLmThreads, smem, s>>>(keys, landmarks, min_cos, G, batch, T, H_kv, n_c, cpb, n_blocks, two_tables,
-                                        rope ? (double)rope_base : 1.0);
   return cudaGetLastError();
 }
 
