@@ -16,7 +16,7 @@ namespace xkv {
 namespace {
 
 constexpr int kQuantThreads = 256;
-constexpr int kQuantPieces = 4;    // 16-byte pieces per thread, all requested before the first is used
+constexpr int kQuantPieces = 4;    // 16-byte pieces per thread, all requested before the first is used (four: see the quantiser)
 
 __device__ __forceinline__ uint32_t min_bf16x2(uint32_t a, uint32_t b) {
   uint32_t r;
@@ -50,6 +50,10 @@ __device__ __forceinline__ float max_nan(float a, float b) {
 // (differences of bf16 numbers over a bf16 scale): the quotient has to be exact, a test with a fallback diverged in most
 // warps (25 us for 65536 x 384 scalars, with an IEEE division per scalar and one thread per group 38 us; this form 19.5, and 17 with
 // two scalars per packed instruction).
+// A group's scale, offset and reciprocal are some forty instructions, a quarter of the kernel's when all four lanes worked
+// them out for every group, and instruction issue is what bounds it (80 % of the slots): a quad holds four groups, and lane p
+// does that work for group p alone.  A window's token bases and matrices (65536 rows of 384 and 576; six launches):
+// 46.4 -> 41.8 us.
 // Rounding goes through 1.5 * 2^23, whose sum with the quotient holds the integer in its low bits.
 constexpr float kRintMagic = 12582912.0f;
 
@@ -64,6 +68,7 @@ __device__ __forceinline__ uint32_t rtn_code_exact(float f, float scale) {
 template <int BITS>
 __global__ void __launch_bounds__(kQuantThreads)
 quantize_rtn_kernel(const uint4* __restrict__ x, long long n_pieces, uint32_t* __restrict__ codes, uint32_t* __restrict__ meta) {
+  static_assert(kQuantPieces == 4, "a group for every lane of a quad");
   constexpr float kTop = (float)((1 << BITS) - 1);
   const int p = threadIdx.x & 3;                           // piece of the group; n_pieces is a multiple of 4
   const long long first = (long long)blockIdx.x * (kQuantThreads * kQuantPieces) + threadIdx.x;
@@ -75,21 +80,42 @@ quantize_rtn_kernel(const uint4* __restrict__ x, long long n_pieces, uint32_t* _
     const long long i = first + u * kQuantThreads;
     v[u] = i < n_pieces ? __ldcs(x + i) : make_uint4(0u, 0u, 0u, 0u);
   }
+  // The extrema of the quad's four groups, folded by halving: lane p ends with those of its group first + p * kQuantThreads,
+  // works out scale, offset and reciprocal of that group alone, and the quad passes them round.
+  uint32_t lo2[kQuantPieces], hi2[kQuantPieces];
+#pragma unroll
+  for (int u = 0; u < kQuantPieces; ++u) {
+    lo2[u] = min_bf16x2(min_bf16x2(v[u].x, v[u].y), min_bf16x2(v[u].z, v[u].w));
+    hi2[u] = max_nan_bf16x2(max_nan_bf16x2(v[u].x, v[u].y), max_nan_bf16x2(v[u].z, v[u].w));
+  }
+#pragma unroll
+  for (int o = 1; o < kQuantPieces; o <<= 1) {
+    const bool up = (p & o) != 0;
+#pragma unroll
+    for (int i = 0; i + o < kQuantPieces; i += 2 * o) {
+      const uint32_t lo_up = __shfl_xor_sync(0xffffffffu, up ? lo2[i] : lo2[i + o], o);
+      const uint32_t hi_up = __shfl_xor_sync(0xffffffffu, up ? hi2[i] : hi2[i + o], o);
+      lo2[i] = min_bf16x2(up ? lo2[i + o] : lo2[i], lo_up);
+      hi2[i] = max_nan_bf16x2(up ? hi2[i + o] : hi2[i], hi_up);
+    }
+  }
+  uint32_t own_meta;
+  float own_y;                                             // reciprocal of the scale, 0: see below
+  {
+    const float lo = fminf(__uint_as_float(lo2[0] << 16), __uint_as_float(lo2[0] & 0xffff0000u));
+    const float hi = max_nan(__uint_as_float(hi2[0] << 16), __uint_as_float(hi2[0] & 0xffff0000u));
+    const __nv_bfloat16 zb = __float2bfloat16_rn(lo);
+    const __nv_bfloat16 sb = __float2bfloat16_rn(__fdiv_rn(__fsub_rn(hi, lo), kTop));
+    const float scale = __bfloat162float(sb);
+    own_y = scale >= 1e-30f && scale <= 1e30f ? __frcp_rn(scale) : 0.0f;
+    own_meta = (uint32_t)__bfloat16_as_ushort(sb) | ((uint32_t)__bfloat16_as_ushort(zb) << 16);
+  }
 #pragma unroll
   for (int u = 0; u < kQuantPieces; ++u) {
     const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-    uint32_t lo2 = min_bf16x2(min_bf16x2(w[0], w[1]), min_bf16x2(w[2], w[3]));
-    uint32_t hi2 = max_nan_bf16x2(max_nan_bf16x2(w[0], w[1]), max_nan_bf16x2(w[2], w[3]));
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
-      lo2 = min_bf16x2(lo2, __shfl_xor_sync(0xffffffffu, lo2, o));
-      hi2 = max_nan_bf16x2(hi2, __shfl_xor_sync(0xffffffffu, hi2, o));
-    }
-    const float lo = fminf(__uint_as_float(lo2 << 16), __uint_as_float(lo2 & 0xffff0000u));
-    const float hi = max_nan(__uint_as_float(hi2 << 16), __uint_as_float(hi2 & 0xffff0000u));
-    const __nv_bfloat16 zb = __float2bfloat16_rn(lo);
-    __nv_bfloat16 sb = __float2bfloat16_rn(__fdiv_rn(__fsub_rn(hi, lo), kTop));
-    const float zero = __bfloat162float(zb), scale = __bfloat162float(sb);
+    uint32_t mw = __shfl_sync(0xffffffffu, own_meta, u, 4);
+    const float y = __shfl_sync(0xffffffffu, own_y, u, 4);
+    const float scale = __uint_as_float(mw << 16), zero = __uint_as_float(mw & 0xffff0000u);
     // two scalars per packed instruction; m: rint(quotient) + kRintMagic of the pairs (2e, 2e + 1)
     ptx::u64 f[4], m[4];
     const ptx::u64 nz2 = ptx::pack2(-zero, -zero);
@@ -98,16 +124,18 @@ quantize_rtn_kernel(const uint4* __restrict__ x, long long n_pieces, uint32_t* _
     // constant groups, scales with an imprecise or overflowing reciprocal, infinities: the division for every scalar.  A NaN
     // (code 0, no part in the extrema) leads here by way of the maximum, so that it costs the other groups nothing (a
     // clamp of every code took 65536 x 960 scalars from 46.1 to 48.1 us); the maximum is taken again without it.
-    if (!(scale >= 1e-30f && scale <= 1e30f)) {
+    if (y == 0.0f) {
       float step = scale;
       if (isnan(scale)) {
         const unsigned quad = 0xfu << (threadIdx.x & 28u);  // (the same branch in the four lanes of a group)
-        hi2 = max_bf16x2(max_bf16x2(w[0], w[1]), max_bf16x2(w[2], w[3]));
+        uint32_t top2 = max_bf16x2(max_bf16x2(w[0], w[1]), max_bf16x2(w[2], w[3]));
 #pragma unroll
-        for (int o = 1; o < 4; o <<= 1) hi2 = max_bf16x2(hi2, __shfl_xor_sync(quad, hi2, o));
-        const float top = fmaxf(__uint_as_float(hi2 << 16), __uint_as_float(hi2 & 0xffff0000u));
-        sb = __float2bfloat16_rn(__fdiv_rn(__fsub_rn(top, lo), kTop));
+        for (int o = 1; o < 4; o <<= 1) top2 = max_bf16x2(top2, __shfl_xor_sync(quad, top2, o));
+        const float top = fmaxf(__uint_as_float(top2 << 16), __uint_as_float(top2 & 0xffff0000u));
+        const __nv_bfloat16 sb = __float2bfloat16_rn(__fdiv_rn(__fsub_rn(top, zero), kTop));
         step = __bfloat162float(sb);
+        mw = (mw & 0xffff0000u) | (uint32_t)__bfloat16_as_ushort(sb);
+        if (p == u) own_meta = mw;
       }
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -115,7 +143,6 @@ quantize_rtn_kernel(const uint4* __restrict__ x, long long n_pieces, uint32_t* _
         m[e] = ptx::pack2((float)rtn_code_exact<BITS>(x2.x, step) + kRintMagic, (float)rtn_code_exact<BITS>(x2.y, step) + kRintMagic);
       }
     } else {
-      const float y = __frcp_rn(scale);
       const ptx::u64 y2 = ptx::pack2(y, y), ns2 = ptx::pack2(-scale, -scale), magic2 = ptx::pack2(kRintMagic, kRintMagic);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -123,18 +150,17 @@ quantize_rtn_kernel(const uint4* __restrict__ x, long long n_pieces, uint32_t* _
         m[e] = ptx::add2(ptx::fma2(ptx::fma2(t, ns2, f[e]), y2, t), magic2);
       }
     }
-    // a pair of codes as the low and the high half of a word
+    // A pair of codes as the low and the high half of a word: f is at least 0 and at most kTop * scale * (1 + 2^-8), so the
+    // sixteen low bits of m are the code.
     uint32_t c[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const float2 x2 = ptx::unpack2(m[e]);
-      c[e] = __byte_perm(__float_as_uint(x2.x), __float_as_uint(x2.y), 0x5410) & (((1u << BITS) - 1u) * 0x00010001u);
+      c[e] = __byte_perm(__float_as_uint(x2.x), __float_as_uint(x2.y), 0x5410);
     }
-    const uint32_t mw = (uint32_t)__bfloat16_as_ushort(sb) | ((uint32_t)__bfloat16_as_ushort(zb) << 16);
     uint32_t word = 0;
     if constexpr (BITS == 4) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) word |= c[e] << (4 * e);
+      word = (((c[3] << 4) + c[2]) << 8) + ((c[1] << 4) + c[0]);
     } else {
       // the quad's 32 codes as four words of nibbles; lane 0 keeps the scale/offset word, lane j + 1 builds w_j
 #pragma unroll
@@ -154,9 +180,10 @@ quantize_rtn_kernel(const uint4* __restrict__ x, long long n_pieces, uint32_t* _
     const long long i = first + u * kQuantThreads;
     if (i < n_pieces) {
       __stcs(codes + i, word);
-      if (BITS == 4 && p == 0) __stcs(meta + (i >> 2), mw);
     }
   }
+  const long long own = first + p * kQuantThreads;         // a piece of this lane's group
+  if (BITS == 4 && own < n_pieces) __stcs(meta + (own >> 2), own_meta);
 }
 
 // x_hat: bf16(code * scale + zero) with a single rounding (the packed bf16 fused multiply-add rounds the exact value
