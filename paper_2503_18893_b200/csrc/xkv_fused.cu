@@ -459,21 +459,23 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       const uint8_t* Cb = (kstream ? dev.Aq_k : dev.Aq_v) + (size_t)b * dev.T * (size_t)(r >> 1);
       const uint32_t* Mb = (kstream ? dev.Am_k : dev.Am_v) + (size_t)b * dev.T * (size_t)(r >> 5);
       const uint32_t ring_q = base + (kstream ? 0u : (uint32_t)SK * kSlabBytes);
-      auto fetch = [&](int ks, uint4 (&cw)[QP], uint32_t (&mw)[QP]) {
+      uint4 cw[QP];
+      uint32_t mw[QP];
+      auto fetch = [&](int ks, int i) {
         const int col0 = ks * 64 + (int)q4 * 32;           // first column of this lane's group
         const bool in = col0 < r;                          // false in a padding slab: zeros are stored
-#pragma unroll
-        for (int i = 0; i < QP; ++i) {
-          // 4 bits: 16 bytes of codes and a separate scale/offset word; 3 bits: one 16-byte record {meta, w0, w1, w2}
-          cw[i] = in ? __ldg(reinterpret_cast<const uint4*>(Cb + (size_t)rw[i] * (size_t)(r >> 1) + (col0 >> 1))) : make_uint4(0, 0, 0, 0);
-          if (QUANT == 4) mw[i] = in ? __ldg(Mb + (size_t)rw[i] * (size_t)(r >> 5) + (col0 >> 5)) : 0u;
-        }
+        // 4 bits: 16 bytes of codes and a separate scale/offset word; 3 bits: one 16-byte record {meta, w0, w1, w2}
+        cw[i] = in ? __ldg(reinterpret_cast<const uint4*>(Cb + (size_t)rw[i] * (size_t)(r >> 1) + (col0 >> 1))) : make_uint4(0, 0, 0, 0);
+        if (QUANT == 4) mw[i] = in ? __ldg(Mb + (size_t)rw[i] * (size_t)(r >> 5) + (col0 >> 5)) : 0u;
       };
-      auto store = [&](const uint4 (&cw)[QP], const uint32_t (&mw)[QP]) -> bool {
+#pragma unroll
+      for (int i = 0; i < QP; ++i) fetch(0, i);
+#pragma unroll 1
+      for (int ks = 0; ks < nst; ks += 2) {
         const int pr = slot >> 1;
         const uint32_t bit = 1u << pr;
         if (used & bit) {             // wait for the release of the pair's previous occupant
-          if (!wait_bar(ctx, BAR(bar_empty + pr), (rel_par >> pr) & 1u, ps + 3)) { ok = false; return false; }
+          if (!wait_bar(ctx, BAR(bar_empty + pr), (rel_par >> pr) & 1u, ps + 3)) { ok = false; return; }
           rel_par ^= bit;
         }
         used |= bit;
@@ -491,6 +493,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
           } else {
             dequant_group3(w[0], w[1], w[2], w[3], o);
           }
+          if (ks + 2 < nst) fetch(ks + 2, i);              // on its way while the other passes are converted
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
             const uint32_t a = st + j * 128u + (((u0 + (uint32_t)u) ^ (j & 7u)) << 4);
@@ -502,16 +505,6 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
         mbar_arrive(BAR(bar_full + pr));                   // the pair is complete when all threads of the stream are done
         slot += 2;
         if (slot == RS) slot = 0;
-        return true;
-      };
-      // (a second register set, so that the next pair's loads are in flight while this pair is converted, loses: step 98.2
-      // against 94.3 us at the headline size)
-      uint4 ca[QP];
-      uint32_t ma[QP];
-#pragma unroll 1
-      for (int ks = 0; ks < nst; ks += 2) {
-        fetch(ks, ca, ma);
-        if (!store(ca, ma)) return;
       }
     };
     auto load_rows_q = [&](uint32_t (&rw)[QP]) {
