@@ -451,22 +451,36 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     // The same phase from 4-bit codes.  Four consecutive lanes share a tile row: lane q4 fetches the 16 bytes of
     // codes and the scale/offset word of one 32-column group of the slot pair (64 contiguous bytes per row and
     // request), turns them into 32 bf16 values (packed arithmetic, one rounding) and stores them as four 16-byte
-    // units of the swizzled slab; a stream's 128 threads cover 32 rows per pass, 4 passes per pair.  The loads of a
-    // pair are issued before the wait for the pair's release, so their latency overlaps it.
+    // units of the swizzled slab; a stream's 128 threads cover 32 rows per pass, 4 passes per pair.
+    // What bounds it is instructions: every warp of a scheduler issues beside the key epilogue (of 13 k cycles a tile the key
+    // stream waited 0.5 k for its ring).  Addresses are therefore worked out once, as one offset per row and one per
+    // 16-byte unit, and a group's next codes are requested when it is converted, in the same registers.  131072 rows, budget
+    // 4096, rank 512, 4 bits, kernel and merge: 70.7 us with the loads of a pair in front of its conversion, 66.6 behind that
+    // of the pair before, 62.5 with the addresses.  Requesting the next tile's first codes from the last pair of a tile as
+    // well, with its positions published a tile ahead, loses (68.6), and so do prefetches of its rows into L2 (74.7).
     const uint32_t q4 = (uint32_t)(ts & 3), rq = (uint32_t)(ts >> 2);
     constexpr int QP = 4;                                  // passes per slot pair
-    auto issue_phase_q = [&](const uint32_t (&rw)[QP], int b) {
-      const uint8_t* Cb = (kstream ? dev.Aq_k : dev.Aq_v) + (size_t)b * dev.T * (size_t)(r >> 1);
+    // This lane's group lies in slab (q4 >> 1) of the pair, 16-byte units 4*(q4 & 1) .. +3 of the 128-byte row; here of
+    // slot 0 and tile row rq.
+    uint32_t unit[4];
+    if constexpr (QUANT != 0) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        unit[u] = base + (kstream ? 0u : (uint32_t)SK * kSlabBytes) + (q4 >> 1) * kSlabBytes + rq * 128u + ((((q4 & 1u) * 4u + (uint32_t)u) ^ (rq & 7u)) << 4);
+    }
+    // gw: the group of every row in the first slot pair, counted over the sequence (the same for codes and parameters)
+    auto issue_phase_q = [&](const uint32_t (&gw)[QP], int b) {
+      const uint4* Cb = reinterpret_cast<const uint4*>((kstream ? dev.Aq_k : dev.Aq_v) + (size_t)b * dev.T * (size_t)(r >> 1));
       const uint32_t* Mb = (kstream ? dev.Am_k : dev.Am_v) + (size_t)b * dev.T * (size_t)(r >> 5);
-      const uint32_t ring_q = base + (kstream ? 0u : (uint32_t)SK * kSlabBytes);
       uint4 cw[QP];
       uint32_t mw[QP];
       auto fetch = [&](int ks, int i) {
-        const int col0 = ks * 64 + (int)q4 * 32;           // first column of this lane's group
-        const bool in = col0 < r;                          // false in a padding slab: zeros are stored
+        // Beyond the rank the pair's first group is fetched again: no key step reaches those columns, and the value side
+        // keeps none of theirs.
+        const uint32_t at = gw[i] + (ks * 64 + (int)q4 * 32 < r ? 2u * (uint32_t)ks : 0u);
         // 4 bits: 16 bytes of codes and a separate scale/offset word; 3 bits: one 16-byte record {meta, w0, w1, w2}
-        cw[i] = in ? __ldg(reinterpret_cast<const uint4*>(Cb + (size_t)rw[i] * (size_t)(r >> 1) + (col0 >> 1))) : make_uint4(0, 0, 0, 0);
-        if (QUANT == 4) mw[i] = in ? __ldg(Mb + (size_t)rw[i] * (size_t)(r >> 5) + (col0 >> 5)) : 0u;
+        cw[i] = __ldg(Cb + at);
+        if (QUANT == 4) mw[i] = __ldg(Mb + at);
       };
 #pragma unroll
       for (int i = 0; i < QP; ++i) fetch(0, i);
@@ -479,12 +493,11 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
           rel_par ^= bit;
         }
         used |= bit;
-        // this lane's group lies in slab (q4 >> 1) of the pair, 16-byte units 4*(q4 & 1) .. +3 of the 128-byte row
-        const uint32_t st = ring_q + (uint32_t)(slot + (int)(q4 >> 1)) * kSlabBytes;
-        const uint32_t u0 = (q4 & 1u) * 4u;
+        uint32_t to[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) to[u] = unit[u] + (uint32_t)slot * kSlabBytes;
 #pragma unroll
         for (int i = 0; i < QP; ++i) {
-          const uint32_t j = rq + 32u * (uint32_t)i;       // tile row
           const uint32_t w[4] = {cw[i].x, cw[i].y, cw[i].z, cw[i].w};
           uint32_t o[16];
           if (QUANT == 4) {
@@ -495,10 +508,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
           }
           if (ks + 2 < nst) fetch(ks + 2, i);              // on its way while the other passes are converted
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const uint32_t a = st + j * 128u + (((u0 + (uint32_t)u) ^ (j & 7u)) << 4);
-            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(o[4 * u]), "r"(o[4 * u + 1]), "r"(o[4 * u + 2]), "r"(o[4 * u + 3]) : "memory");
-          }
+          for (int u = 0; u < 4; ++u)                      // 32 tile rows on: 4096 bytes (the swizzle repeats every 8)
+            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(to[u] + 4096u * (uint32_t)i), "r"(o[4 * u]), "r"(o[4 * u + 1]), "r"(o[4 * u + 2]), "r"(o[4 * u + 3]) : "memory");
         }
         asm volatile("cp.async.wait_all;" ::: "memory");   // the staged rotary rows of this tile (key stream) have landed too
         fence_proxy_async();                               // the tensor core reads these stores
@@ -507,11 +518,11 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
         if (slot == RS) slot = 0;
       }
     };
-    auto load_rows_q = [&](uint32_t (&rw)[QP]) {
+    auto load_rows_q = [&](uint32_t (&gw)[QP]) {           // (less than 2^24 rows of at most 256 groups)
 #pragma unroll
       for (int i = 0; i < QP; ++i) {
         const int p = pos_s[pb * kTile + (int)rq + 32 * i];
-        rw[i] = p < 0 ? 0u : (uint32_t)p;
+        gw[i] = (p < 0 ? 0u : (uint32_t)p) * (uint32_t)(r >> 5) + q4;
       }
     };
     auto load_rows = [&](uint32_t (&ro)[16]) {             // rows without a selected token read row 0 (weight 0)
@@ -586,10 +597,10 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       }
       if (!wait_bar(ctx, BAR(bl.posfull + pb), (uint32_t)((it >> 2) & 1), ps + 2)) { ok = false; break; }
       if constexpr (QUANT != 0) {
-        uint32_t rw[QP];
-        load_rows_q(rw);
+        uint32_t gw[QP];
+        load_rows_q(gw);
         if (!kstream) mbar_arrive(BAR(bl.vfree + pb));     // this thread is done with the position buffer
-        issue_phase_q(rw, cur.b);
+        issue_phase_q(gw, cur.b);
       } else {
         uint32_t ro[16];
         load_rows(ro);
