@@ -16,6 +16,10 @@ namespace xkv {
 namespace {
 
 constexpr int kQuantThreads = 256;
+// The first blocks, those that may be resident while the kernel before still runs, have their scalars brought into L2 before
+// they wait for it (the second level is where that kernel's writes would land, so nothing stale is read): six launches of a
+// window 41.9 -> 40.6 us.
+constexpr int kQuantAhead = 1184;
 constexpr int kQuantPieces = 4;    // 16-byte pieces per thread, all requested before the first is used (four: see the quantiser)
 
 __device__ __forceinline__ uint32_t min_bf16x2(uint32_t a, uint32_t b) {
@@ -72,6 +76,11 @@ quantize_rtn_kernel(const uint4* __restrict__ x, long long n_pieces, uint32_t* _
   constexpr float kTop = (float)((1 << BITS) - 1);
   const int p = threadIdx.x & 3;                           // piece of the group; n_pieces is a multiple of 4
   const long long first = (long long)blockIdx.x * (kQuantThreads * kQuantPieces) + threadIdx.x;
+  if (blockIdx.x < kQuantAhead && (threadIdx.x & 7) == 0) {
+#pragma unroll
+    for (int u = 0; u < kQuantPieces; ++u)
+      if (first + u * kQuantThreads < n_pieces) asm volatile("prefetch.global.L2 [%0];" ::"l"(x + first + u * kQuantThreads));
+  }
   ptx::grid_dependency_wait();
   ptx::grid_dependency_launch();
   uint4 v[kQuantPieces];
