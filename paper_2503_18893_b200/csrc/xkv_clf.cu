@@ -333,15 +333,16 @@ __device__ __forceinline__ bool grid_barrier(const GridSync& sy, unsigned& arriv
   return *ok_s != 0;
 }
 
-// 1/sqrt(d) for d > 0 by Newton's iteration from the fp32 value (two steps: relative error 2^-22 -> 2^-43 -> rounding).
+// 1/sqrt(d) for d > 0 from the fp32 value y (relative error 2^-22): with e = 1 - d y^2 the binomial series y (1 - e)^-1/2 to
+// its second order leaves 5/16 e^3, below the rounding.  (Four dependent operations; two steps of Newton's iteration are six.)
 // The argument is scaled into [1, 4) by an even power of two first.
-__device__ __forceinline__ double newton_rsqrt(double d) {
+__device__ __forceinline__ double series_rsqrt(double d) {
   const int hi = __double2hiint(d);
   const int e = ((hi >> 20) - 1023) & ~1;                      // even exponent
   const double m = __hiloint2double(hi - (e << 20), __double2loint(d));
   double y = (double)rsqrtf((float)m);
-#pragma unroll
-  for (int i = 0; i < 2; ++i) y = fma(0.5 * y, fma(-m * y, y, 1.0), y);
+  const double err = fma(-m * y, y, 1.0);
+  y = fma(y * err, fma(0.375, err, 0.5), y);
   return __hiloint2double(__double2hiint(y) - ((e >> 1) << 20), __double2loint(y));
 }
 
@@ -352,9 +353,9 @@ __device__ __forceinline__ double newton_rsqrt(double d) {
 //                   one grid barrier per step suffices
 //   i > p, k <= p   the same elimination on the identity, R_ik -= L_ip W_pk (R starts as I), with W_pk = inv(L_pp) R_pk
 //   i == p          W_pk is written
-// A latency chain: 576 columns one after the other in the diagonal blocks, 19 barriers.  (As three launches per panel the
+// A latency chain: 576 columns two by two in the diagonal blocks, 19 barriers.  (As three launches per panel the
 // factorisation of a 576 x 576 matrix was 52 launches of 7 to 16 us; with the inverse formed after it, column by column, the
-// kernel took 321 us, with the inverse carried along 235.)  With W at hand the solve is a product.
+// kernel took 321 us, with the inverse carried along and a column a step 234, now 178.)  With W at hand the solve is a product.
 // Buffers: part [n_part][l][l] partial Gram matrices (lower tiles of 64), Gm [l][l] the working matrix, Rt [l][l] the tiles
 // of R below the diagonal, each transposed, Iv [l/32][32][32] inverses of the diagonal blocks, W [l][l] lower.
 constexpr int kCholNb = 32, kCholThreads = 256, kCholLd = 36;   // 36 doubles per staged row: 4 mod 16, conflict free fragments
@@ -370,8 +371,6 @@ __global__ void __launch_bounds__(kCholThreads, 1)
 chol_inverse_kernel(const double* __restrict__ part, int n_part, double* __restrict__ Gm, double* __restrict__ Rt,
                     double* __restrict__ Iv, double* __restrict__ W, int l, double shift_rel, unsigned arrived, GridSync sy) {
   __shared__ double A_s[kCholNb * kCholLd], B_s[kCholNb * kCholLd], V_s[kCholNb * kCholLd], Li_s[kCholNb * kCholLd], Lk_s[kCholNb * kCholLd];
-  __shared__ __align__(16) double col_s[2][kCholNb];
-  __shared__ double piv_s[2];
   __shared__ double red_s[kCholThreads / 32];
   __shared__ int ok_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = gridDim.x, bid = blockIdx.x;
@@ -416,38 +415,82 @@ chol_inverse_kernel(const double* __restrict__ part, int n_part, double* __restr
       d[0] = acc[j][0]; d[1] = acc[j][1];
     }
   };
-  // ---- factor the diagonal block in A_s and invert the factor.  Warp 0: lane i holds row i; warp 1: lane k holds column k
-  // of the inverse and follows from column to column.  A pivot that is not positive (breakdown) is replaced by a tiny
-  // one and reported.
+  // ---- factor the diagonal block in A_s and invert the factor, two columns a step, which halves the chain of reciprocal
+  // roots: with the pivots a, b, d the second root is that of a d - b^2 and does not wait for the first.  Warps 0-3 hold the
+  // matrix, lane = row, warps 4-7 the inverse, lane = column; the pair of columns (of rows, in the inverse) 2 s, 2 s + 1
+  // belongs to warp s mod 4 of either.  A step is one barrier: the owner brings its pair up to date, works the columns out
+  // and hands them over; the others then take them off their pairs, the owner of the next step after its own barrier.  The
+  // inverse is one step behind.  A pivot that is not positive (breakdown) is replaced by a tiny one and reported.
   auto factor = [&](int p) {
     __syncthreads();
-    if (warp < 2) {
-      double a[kCholNb];
+    double* const col = B_s;                                   // [step & 3][2][32] columns of the factor
+    double* const row = B_s + 4 * 2 * kCholNb;                 // [step & 3][2][32] rows of the inverse
+    double* const piv = row + 4 * 2 * kCholNb;                 // [step & 3][3] 1 / l_11, l_21, 1 / l_22
+    const bool inverse = warp >= 4;
+    const int own = warp & 3;
+    double a[4][2];
 #pragma unroll
-      for (int j = 0; j < kCholNb; ++j) a[j] = warp == 0 ? A_s[lane * kCholLd + j] : (j == lane ? 1.0 : 0.0);
+    for (int k = 0; k < 4; ++k)
 #pragma unroll
-      for (int c = 0; c < kCholNb; ++c) {
-        if (warp == 0) {
-          double d = __shfl_sync(0xffffffffu, a[c], c);
-          if (!(d > 0.0)) { if (lane == 0) atomicOr(sy.flags, XKV_FLAG_CLF_BREAKDOWN); d = 1e-300; }
-          const double y = newton_rsqrt(d);
-          a[c] = lane == c ? d * y : a[c] * y;
-          col_s[c & 1][lane] = a[c];
-          if (lane == 0) piv_s[c & 1] = y;
-        }
-        named_bar_sync(1, 64);
-        if (warp == 0) {
-#pragma unroll
-          for (int j = c + 1; j < kCholNb; ++j) a[j] = fma(-a[c], col_s[c & 1][j], a[j]);   // entries above the diagonal: unused
-        } else {
-          a[c] *= piv_s[c & 1];
-#pragma unroll
-          for (int j = c + 1; j < kCholNb; ++j) a[j] = fma(-a[c], col_s[c & 1][j], a[j]);
-        }
+      for (int x = 0; x < 2; ++x) {
+        const int j = 2 * (4 * k + own) + x;
+        a[k][x] = inverse ? (j == lane ? 1.0 : 0.0) : A_s[lane * kCholLd + j];
       }
-      if (warp == 1) {
+    auto take_off = [&](double (&v)[2], int of, int step) {    // step's columns (and rows) off pair `of`
+      const double* const c = col + (step & 3) * 2 * kCholNb + 2 * of;
+      const double* const m = (inverse ? row : col) + (step & 3) * 2 * kCholNb + lane;
+      const double m0 = m[0], m1 = m[kCholNb];
 #pragma unroll
-        for (int j = 0; j < kCholNb; ++j) Iv[((size_t)p * kCholNb + j) * kCholNb + lane] = j >= lane ? a[j] : 0.0;
+      for (int x = 0; x < 2; ++x) v[x] = fma(-m1, c[kCholNb + x], fma(-m0, c[x], v[x]));
+    };
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll 1
+      for (int w = 0; w < 4; ++w) {
+        const int st = 4 * k + w;
+        double* const my_piv = piv + (st & 3) * 3;
+        if (!inverse && own == w) {
+          if (st > 0) take_off(a[k], st, st - 1);
+          double a0 = __shfl_sync(0xffffffffu, a[k][0], 2 * st);
+          const double b0 = __shfl_sync(0xffffffffu, a[k][0], 2 * st + 1), d0 = __shfl_sync(0xffffffffu, a[k][1], 2 * st + 1);
+          const bool bad_a = !(a0 > 0.0);
+          a0 = bad_a ? 1e-300 : a0;
+          const double det = fma(a0, d0, -(b0 * b0));
+          const bool bad_d = !(det > 0.0);
+          const double y1 = series_rsqrt(a0), y2 = series_rsqrt(bad_d ? 1.0 : det);
+          const double l21 = b0 * y1, i22 = bad_d ? 1e150 : y2 * (a0 * y1), l22 = bad_d ? 1e-150 : det * y2 * y1;
+          const double x1 = (lane == 2 * st ? a0 : a[k][0]) * y1;
+          const double x2 = lane == 2 * st + 1 ? l22 : fma(-x1, l21, a[k][1]) * i22;
+          double* const c = col + (st & 3) * 2 * kCholNb + lane;
+          c[0] = x1; c[kCholNb] = x2;
+          if (lane == 0) {
+            my_piv[0] = y1; my_piv[1] = l21; my_piv[2] = i22;
+            if (bad_a || bad_d) atomicOr(sy.flags, XKV_FLAG_CLF_BREAKDOWN);
+          }
+        }
+        named_bar_sync(1, kCholThreads);
+        if (inverse) {
+          if (st > 0) {
+#pragma unroll
+            for (int j = k; j < 4; ++j)
+              if (j > k || own >= w) take_off(a[j], 4 * j + own, st - 1);
+          }
+          if (own == w) {
+            a[k][0] *= my_piv[0];
+            a[k][1] = fma(-my_piv[1], a[k][0], a[k][1]) * my_piv[2];
+            double* const c = row + (st & 3) * 2 * kCholNb + lane;
+            c[0] = a[k][0]; c[kCholNb] = a[k][1];
+#pragma unroll
+            for (int x = 0; x < 2; ++x) Iv[((size_t)p * kCholNb + 2 * st + x) * kCholNb + lane] = 2 * st + x >= lane ? a[k][x] : 0.0;
+          }
+        } else if (own != ((w + 1) & 3)) {
+#pragma unroll
+          for (int j = k; j < 4; ++j)
+            if (j > k || own > w) {
+              if (own == w && st > 0) take_off(a[j], 4 * j + own, st - 1);
+              take_off(a[j], 4 * j + own, st);
+            }
+        }
       }
     }
   };
