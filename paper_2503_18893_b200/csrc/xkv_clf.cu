@@ -33,7 +33,7 @@ using namespace ptx;
 // Tiles are (128 MB) x BN, MB accumulators of 128 rows in tensor memory sharing the B operand; one stage of the operand
 // ring holds 64 k.  What bounds the products is the rate at which L2 feeds the SMs (about 53 bytes per cycle and SM when
 // all of them ask): a 128 x 256 tile wants 96, a 256 x 192 tile 73 and a 256 x 256 tile 64 at the full rate of the tensor
-// core.  X Z at 131072 x 4096 x 576: 0.87 ms with 128 x 256 tiles, 0.50 with 256 x 192;
+// core.  X Z at 131072 x 4096 x 576, a CTA per tile: 0.87 ms with 128 x 256 tiles, 0.50 with 256 x 192;
 // X^T Y 0.65 ms with 96 tiles of 128 x 192, 0.40 with 48 of 256 x 192 over three K ranges.
 constexpr int kGemmEpiWarps = 4;                  // per 128 rows; then one TMA producer warp, one MMA issue warp
 template <int MB> constexpr int gemm_threads() { return (MB * kGemmEpiWarps + 2) * 32; }
@@ -49,7 +49,11 @@ __device__ __forceinline__ bool gemm_wait(uint32_t bar, uint32_t parity) {
   return false;
 }
 
-// C[m][n] = sum_k A(k, m) B(k, n).  grid = (ceil(N/BN), ceil(M/(128 MB)), K ranges).  TRANS: store C^T (out[n][m]).
+// C[m][n] = sum_k A(k, m) B(k, n).  tiles = (ceil(N/BN), ceil(M/(128 MB)), K ranges), the first fastest; a CTA takes every
+// gridDim.x-th of them.  The operand ring runs on from tile to tile, and a result in bf16 alone leaves tensor memory for
+// registers before it is stored, so that the next tile's products run beside its stores.  131072 x 4096 x 576: 495 us with a
+// CTA per tile, 429 now; with two parts of B and of the result 930 -> 866.
+// TRANS: store C^T (out[n][m]).
 // AK: A is given as [m][k] (K-major), else as [k][m]; BK likewise for B.  K range z covers k_per columns and writes
 // Cf + z * M * ldc.  With two parts B is the sum of the matrices of map_b and map_b2 and A is gone through twice; the k
 // of a part are rounded up to whole blocks of 64.  Cb is the result rounded to bf16; LO: Cl is twice what the rounding leaves
@@ -58,26 +62,32 @@ template <bool TRANS, bool AK, bool BK, bool LO, int MB, int BN>
 __global__ void __launch_bounds__(gemm_threads<MB>(), 1)
 clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                 const __grid_constant__ CUtensorMap map_b2, int M, int N, int k_part, int k_all, int k_per, float* __restrict__ Cf,
-                __nv_bfloat16* __restrict__ Cb, __nv_bfloat16* __restrict__ Cl, long long ldc, unsigned int* __restrict__ flags) {
+                __nv_bfloat16* __restrict__ Cb, __nv_bfloat16* __restrict__ Cl, long long ldc, dim3 tiles, unsigned int* __restrict__ flags) {
   extern __shared__ uint8_t gemm_smem[];
   constexpr int kGemmStages = gemm_stages<MB, BN>(), kGemmStageBytes = gemm_stage_bytes<MB, BN>();
   constexpr uint32_t kAccCols = BN <= 128 ? 128u : 256u, kCols = MB * kAccCols;      // tensor-memory columns
   constexpr int kWarpLoad = MB * kGemmEpiWarps, kWarpMma = kWarpLoad + 1;
-  __shared__ __align__(8) uint64_t bars[2 * kGemmMaxStages + 1];
+  __shared__ __align__(8) uint64_t bars[2 * kGemmMaxStages + 2];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_s;
   const uint32_t base = (smem_u32(gemm_smem) + 1023u) & ~1023u;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * (128 * MB);
-  const int k_first = blockIdx.z * k_per, KB = (min(k_all - k_first, k_per) + 63) / 64;
-  if (Cf) Cf += (size_t)blockIdx.z * M * ldc;
+  struct Tile { int n0, m0, z, k_first, KB; };
+  const unsigned n_tiles = tiles.x * tiles.y * tiles.z;
+  auto tile_at = [&](unsigned t) {
+    Tile c;
+    c.n0 = (int)(t % tiles.x) * BN; c.m0 = (int)(t / tiles.x % tiles.y) * (128 * MB); c.z = (int)(t / (tiles.x * tiles.y));
+    c.k_first = c.z * k_per; c.KB = (min(k_all - c.k_first, k_per) + 63) / 64;
+    return c;
+  };
   const uint32_t bar0 = smem_u32(bars);
   auto FULL = [&](int s) { return bar0 + 8u * (uint32_t)s; };
   auto EMPTY = [&](int s) { return bar0 + 8u * (uint32_t)(kGemmStages + s); };
-  const uint32_t ACC = bar0 + 8u * (uint32_t)(2 * kGemmStages);
+  const uint32_t ACC = bar0 + 8u * (uint32_t)(2 * kGemmStages), FREE = ACC + 8u;   // accumulators complete; read out
   if (tid == 0) {
     for (int s = 0; s < kGemmStages; ++s) { mbar_init(FULL(s), 1); mbar_init(EMPTY(s), 1); }
     mbar_init(ACC, 1);
+    mbar_init(FREE, MB * kGemmEpiWarps * 32);
     abort_s = 0;
     fence_mbar_init();
   }
@@ -93,27 +103,31 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   constexpr uint32_t kOffB = MB * 16384u;
   if (warp == kWarpLoad) {
     if (lane == 0) {
-      for (int kb = 0; kb < KB; ++kb) {
-        const int s = kb % kGemmStages;
-        if (kb >= kGemmStages && !gemm_wait(EMPTY(s), (uint32_t)((kb / kGemmStages - 1) & 1))) { ok = false; break; }
-        const uint32_t st = base + (uint32_t)s * kGemmStageBytes;
-        mbar_expect_tx(FULL(s), kGemmStageBytes);
-        const int kt = k_first + kb * 64;
-        const bool second = kt >= k_part;
-        const int k = second ? kt - k_part : kt;
-        const CUtensorMap* mb = second ? &map_b2 : &map_b;
-        // K-major: one box of 64 k by all rows; MN-major: slabs of 64 columns by 64 k, 8 KB each
-        if (AK) {
-          tma_load_2d(st, &map_a, k, m0, FULL(s));
-        } else {
+      int it = 0;                                          // blocks of 64 k so far
+      for (unsigned t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
+        const Tile c = tile_at(t);
+        for (int kb = 0; kb < c.KB; ++kb, ++it) {
+          const int s = it % kGemmStages;
+          if (it >= kGemmStages && !gemm_wait(EMPTY(s), (uint32_t)((it / kGemmStages - 1) & 1))) { ok = false; break; }
+          const uint32_t st = base + (uint32_t)s * kGemmStageBytes;
+          mbar_expect_tx(FULL(s), kGemmStageBytes);
+          const int kt = c.k_first + kb * 64;
+          const bool second = kt >= k_part;
+          const int k = second ? kt - k_part : kt;
+          const CUtensorMap* mb = second ? &map_b2 : &map_b;
+          // K-major: one box of 64 k by all rows; MN-major: slabs of 64 columns by 64 k, 8 KB each
+          if (AK) {
+            tma_load_2d(st, &map_a, k, c.m0, FULL(s));
+          } else {
 #pragma unroll
-          for (int i = 0; i < 2 * MB; ++i) tma_load_2d(st + i * 8192, &map_a, m0 + i * 64, k, FULL(s));
-        }
-        if (BK) {
-          tma_load_2d(st + kOffB, mb, k, n0, FULL(s));
-        } else {
+            for (int i = 0; i < 2 * MB; ++i) tma_load_2d(st + i * 8192, &map_a, c.m0 + i * 64, k, FULL(s));
+          }
+          if (BK) {
+            tma_load_2d(st + kOffB, mb, k, c.n0, FULL(s));
+          } else {
 #pragma unroll
-          for (int i = 0; i < BN / 64; ++i) tma_load_2d(st + kOffB + i * 8192, mb, n0 + i * 64, k, FULL(s));
+            for (int i = 0; i < BN / 64; ++i) tma_load_2d(st + kOffB + i * 8192, mb, c.n0 + i * 64, k, FULL(s));
+          }
         }
       }
     }
@@ -128,80 +142,138 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       auto lo = [&](uint32_t at, bool kmajor) {
         return kmajor ? (uint32_t)(smem_desc_sw128(at, 0) & 0xFFFFFFFFull) : ((at & 0x3FFFFu) >> 4) | kSlab;
       };
-      for (int kb = 0; kb < KB; ++kb) {
-        const int s = kb % kGemmStages;
-        if (!gemm_wait(FULL(s), (uint32_t)((kb / kGemmStages) & 1))) { ok = false; break; }
+      int it = 0;
+      uint32_t done = 0;                                   // tiles issued
+      for (unsigned t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++done) {
+        if (done > 0 && !gemm_wait(FREE, (done - 1) & 1u)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t st = base + (uint32_t)s * kGemmStageBytes;
-        const uint32_t b_lo = lo(st + kOffB, BK);
+        const int KB = tile_at(t).KB;
+        for (int kb = 0; kb < KB; ++kb, ++it) {
+          const int s = it % kGemmStages;
+          if (!gemm_wait(FULL(s), (uint32_t)((it / kGemmStages) & 1))) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t st = base + (uint32_t)s * kGemmStageBytes;
+          const uint32_t b_lo = lo(st + kOffB, BK);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
+          for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
-          for (int mb = 0; mb < MB; ++mb)
-            tc_mma_bf16(tmem + (uint32_t)mb * kAccCols, desc_hi | (lo(st + mb * 16384u, AK) + (uint32_t)kk * a_step),
-                        desc_hi | (b_lo + (uint32_t)kk * b_step), idesc, (kb | kk) ? 1u : 0u);
-        tc_commit(EMPTY(s));
+            for (int mb = 0; mb < MB; ++mb)
+              tc_mma_bf16(tmem + (uint32_t)mb * kAccCols, desc_hi | (lo(st + mb * 16384u, AK) + (uint32_t)kk * a_step),
+                          desc_hi | (b_lo + (uint32_t)kk * b_step), idesc, (kb | kk) ? 1u : 0u);
+          tc_commit(EMPTY(s));
+        }
+        tc_commit(ACC);
       }
-      tc_commit(ACC);
     }
   }
   if (warp >= kWarpLoad) {          // a producer or issuer that gave up tells the epilogue not to wait for ever
     if (!ok && lane == 0) { abort_s = 1; atomicOr(flags, XKV_FLAG_TIMEOUT); }
   } else {
     // ---- epilogue: thread = accumulator lane = row m0 + tid
-    bool done = false;
-    for (uint32_t i = 0; i < kGemmWaitLimit && !done; ++i) {
-      done = mbar_try_wait(ACC, 0);
-      if (!done && (i & 1023u) == 1023u && *(volatile int*)&abort_s) break;
-    }
-    if (done) {
+    uint32_t par = 0;
+    for (unsigned t = blockIdx.x; t < n_tiles; t += gridDim.x, par ^= 1u) {
+      const Tile c = tile_at(t);
+      float* const Cz = Cf ? Cf + (size_t)c.z * M * ldc : nullptr;
+      bool done = false;
+      for (uint32_t i = 0; i < kGemmWaitLimit && !done; ++i) {
+        done = mbar_try_wait(ACC, par);
+        if (!done && (i & 1023u) == 1023u && *(volatile int*)&abort_s) break;
+      }
+      if (!done) {
+        if (tid == 0) atomicOr(flags, XKV_FLAG_TIMEOUT);
+        break;
+      }
       tc_fence_after();
-      const int m = m0 + tid;
+      const int m = c.m0 + tid;
       const uint32_t lane_base = ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * kAccCols;
+      if (!Cf && c.n0 + BN <= N && (TRANS || (ldc & 7) == 0)) {
+        // bf16 alone: to registers, the accumulators handed back, then the stores; as many columns at a time as registers hold
+        constexpr int kPart = LO ? (BN == 192 ? 96 : 64) : BN == 256 ? 128 : BN;
 #pragma unroll 1
-      for (int cb = 0; cb < BN / 32; ++cb) {
-        float v[32];
-        tmem_ld32(tmem + lane_base + (uint32_t)(cb * 32), v);
-        tc_wait_ld();
-        if (m < M) {
-          const int nb = n0 + cb * 32;
-          if (!TRANS && nb + 32 <= N && (ldc & 7) == 0) {
-            // a whole run of 32 columns of one row: 16-byte stores (the row pitch keeps them aligned)
-            const long long at = (long long)m * ldc + nb;
-            if (Cf) {
+        for (int n = 0; n < BN; n += kPart) {
+          uint32_t h[kPart / 2], rest[LO ? kPart / 2 : 1];
 #pragma unroll
-              for (int i = 0; i < 32; i += 4) *reinterpret_cast<float4*>(Cf + at + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-            }
-            if (Cb) {
+          for (int cb = 0; cb < kPart / 32; ++cb) {
+            float v[32];
+            tmem_ld32(tmem + lane_base + (uint32_t)(n + cb * 32), v);
+            tc_wait_ld();
 #pragma unroll
-              for (int i = 0; i < 32; i += 8) {
-                __nv_bfloat162 h0 = __floats2bfloat162_rn(v[i], v[i + 1]), h1 = __floats2bfloat162_rn(v[i + 2], v[i + 3]);
-                __nv_bfloat162 h2 = __floats2bfloat162_rn(v[i + 4], v[i + 5]), h3 = __floats2bfloat162_rn(v[i + 6], v[i + 7]);
-                uint4 u;
-                u.x = *reinterpret_cast<uint32_t*>(&h0); u.y = *reinterpret_cast<uint32_t*>(&h1);
-                u.z = *reinterpret_cast<uint32_t*>(&h2); u.w = *reinterpret_cast<uint32_t*>(&h3);
-                *reinterpret_cast<uint4*>(Cb + at + i) = u;
+            for (int i = 0; i < 16; ++i) {
+              const __nv_bfloat162 two = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+              h[cb * 16 + i] = *reinterpret_cast<const uint32_t*>(&two);
+              if (LO) {
+                const __nv_bfloat162 out = __floats2bfloat162_rn(2.0f * (v[2 * i] - __low2float(two)), 2.0f * (v[2 * i + 1] - __high2float(two)));
+                rest[cb * 16 + i] = *reinterpret_cast<const uint32_t*>(&out);
               }
             }
-          } else {
+          }
+          if (n + kPart == BN) {
+            tc_fence_before();
+            mbar_arrive(FREE);
+          }
+          if (m < M) {
+            if (TRANS) {
+              uint16_t* to = reinterpret_cast<uint16_t*>(Cb) + (long long)(c.n0 + n) * ldc + m;
+              const long long to_rest = LO ? Cl - Cb : 0;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              const int n = nb + i;
-              if (n < N) {
-                const long long at = TRANS ? (long long)n * ldc + m : (long long)m * ldc + n;
-                if (Cf) Cf[at] = v[i];
+              for (int i = 0; i < kPart; ++i, to += ldc) {
+                asm volatile("" : "+l"(to));               // one address at a time, not all of them in registers
+                *to = (uint16_t)((i & 1) ? h[i >> 1] >> 16 : h[i >> 1]);
+                if (LO) to[to_rest] = (uint16_t)((i & 1) ? rest[i >> 1] >> 16 : rest[i >> 1]);
+              }
+            } else {
+              uint4* to = reinterpret_cast<uint4*>(Cb + (long long)m * ldc + c.n0 + n);
+#pragma unroll
+              for (int i = 0; i < kPart / 8; ++i) to[i] = make_uint4(h[4 * i], h[4 * i + 1], h[4 * i + 2], h[4 * i + 3]);
+            }
+          }
+        }
+      } else {
+#pragma unroll 1
+          for (int cb = 0; cb < BN / 32; ++cb) {
+            float v[32];
+            tmem_ld32(tmem + lane_base + (uint32_t)(cb * 32), v);
+            tc_wait_ld();
+            if (m < M) {
+              const int nb = c.n0 + cb * 32;
+              if (!TRANS && nb + 32 <= N && (ldc & 7) == 0) {
+                // a whole run of 32 columns of one row: 16-byte stores (the row pitch keeps them aligned)
+                const long long at = (long long)m * ldc + nb;
+                if (Cz) {
+#pragma unroll
+                  for (int i = 0; i < 32; i += 4) *reinterpret_cast<float4*>(Cz + at + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                }
                 if (Cb) {
-                  const __nv_bfloat16 hi = __float2bfloat16(v[i]);
-                  Cb[at] = hi;
-                  if (LO) Cl[at] = __float2bfloat16(2.0f * (v[i] - __bfloat162float(hi)));
+#pragma unroll
+                  for (int i = 0; i < 32; i += 8) {
+                    __nv_bfloat162 h0 = __floats2bfloat162_rn(v[i], v[i + 1]), h1 = __floats2bfloat162_rn(v[i + 2], v[i + 3]);
+                    __nv_bfloat162 h2 = __floats2bfloat162_rn(v[i + 4], v[i + 5]), h3 = __floats2bfloat162_rn(v[i + 6], v[i + 7]);
+                    uint4 u;
+                    u.x = *reinterpret_cast<uint32_t*>(&h0); u.y = *reinterpret_cast<uint32_t*>(&h1);
+                    u.z = *reinterpret_cast<uint32_t*>(&h2); u.w = *reinterpret_cast<uint32_t*>(&h3);
+                    *reinterpret_cast<uint4*>(Cb + at + i) = u;
+                  }
+                }
+              } else {
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                  const int n = nb + i;
+                  if (n < N) {
+                    const long long at = TRANS ? (long long)n * ldc + m : (long long)m * ldc + n;
+                    if (Cz) Cz[at] = v[i];
+                    if (Cb) {
+                      const __nv_bfloat16 hi = __float2bfloat16(v[i]);
+                      Cb[at] = hi;
+                      if (LO) Cl[at] = __float2bfloat16(2.0f * (v[i] - __bfloat162float(hi)));
+                    }
+                  }
                 }
               }
             }
           }
-        }
+        tc_fence_before();
+        mbar_arrive(FREE);
       }
-    } else if (tid == 0) {
-      atomicOr(flags, XKV_FLAG_TIMEOUT);
     }
   }
   tc_fence_before();
@@ -1253,8 +1325,12 @@ cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, const void* b2, int spl
   cudaError_t e = ensure_dyn_smem<clf_gemm_kernel<TRANS, AK, BK, LO, MB, BN>>(smem, device);
   if (e != cudaSuccess) return e;
   const int k_per = ((k_all + splits - 1) / splits + 63) & ~63;
-  const dim3 grid((N + BN - 1) / BN, (M + 128 * MB - 1) / (128 * MB), splits);
-  clf_gemm_kernel<TRANS, AK, BK, LO, MB, BN><<<grid, gemm_threads<MB>(), smem, s>>>(ma, mb, mb2, M, N, k_part, k_all, k_per, c.f, c.b, c.lo, c.ld,
+  const dim3 tiles((N + BN - 1) / BN, (M + 128 * MB - 1) / (128 * MB), splits);
+  int sms = 0;
+  if ((e = device_sms(device, &sms)) != cudaSuccess) return e;
+  const long long n_tiles = (long long)tiles.x * tiles.y * tiles.z;
+  const unsigned grid = (unsigned)(n_tiles < sms ? n_tiles : sms);        // one CTA per SM (shared and tensor memory)
+  clf_gemm_kernel<TRANS, AK, BK, LO, MB, BN><<<grid, gemm_threads<MB>(), smem, s>>>(ma, mb, mb2, M, N, k_part, k_all, k_per, c.f, c.b, c.lo, c.ld, tiles,
                                                                                flags);
   count_launch(kFamClf);
   return cudaGetLastError();
