@@ -52,7 +52,7 @@ __device__ __forceinline__ bool gemm_wait(uint32_t bar, uint32_t parity) {
 // C[m][n] = sum_k A(k, m) B(k, n).  tiles = (ceil(N/BN), ceil(M/(128 MB)), K ranges), the first fastest; a CTA takes every
 // gridDim.x-th of them.  The operand ring runs on from tile to tile, and a result in bf16 alone leaves tensor memory for
 // registers before it is stored, so that the next tile's products run beside its stores.  131072 x 4096 x 576: 495 us with a
-// CTA per tile, 429 now; with two parts of B and of the result 930 -> 866.
+// CTA per tile, 421 now; with two parts of B and of the result 930 -> 855.
 // TRANS: store C^T (out[n][m]).
 // AK: A is given as [m][k] (K-major), else as [k][m]; BK likewise for B.  K range z covers k_per columns and writes
 // Cf + z * M * ldc.  With two parts B is the sum of the matrices of map_b and map_b2 and A is gone through twice; the k
@@ -188,7 +188,7 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       const uint32_t lane_base = ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * kAccCols;
       if (!Cf && c.n0 + BN <= N && (TRANS || (ldc & 7) == 0)) {
         // bf16 alone: to registers, the accumulators handed back, then the stores; as many columns at a time as registers hold
-        constexpr int kPart = LO ? (BN == 192 ? 96 : 64) : BN == 256 ? 128 : BN;
+        constexpr int kPart = BN == 192 ? 96 : LO ? 64 : 128;
 #pragma unroll 1
         for (int n = 0; n < BN; n += kPart) {
           uint32_t h[kPart / 2], rest[LO ? kPart / 2 : 1];
