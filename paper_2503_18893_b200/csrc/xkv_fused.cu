@@ -499,16 +499,16 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       for (int u = 0; u < 4; ++u)
         unit[u] = base + (kstream ? 0u : (uint32_t)SK * kSlabBytes) + (q4 >> 1) * kSlabBytes + rq * 128u + ((((q4 & 1u) * 4u + (uint32_t)u) ^ (rq & 7u)) << 4);
     }
-    // gw: the group of every row in the first slot pair, counted over the sequence (the same for codes and parameters)
+    // gw: the first group of every row, counted over the sequence (the same for codes and parameters)
     auto issue_phase_q = [&](const uint32_t (&gw)[QP], int b) {
       const uint4* Cb = reinterpret_cast<const uint4*>((kstream ? dev.Aq_k : dev.Aq_v) + (size_t)b * dev.T * (size_t)(r >> 1));
       const uint32_t* Mb = (kstream ? dev.Am_k : dev.Am_v) + (size_t)b * dev.T * (size_t)(r >> 5);
       uint4 cw[QP];
       uint32_t mw[QP];
       auto fetch = [&](int ks, int i) {
-        // Beyond the rank the pair's first group is fetched again: no key step reaches those columns, and the value side
-        // keeps none of theirs.
-        const uint32_t at = gw[i] + (ks * 64 + (int)q4 * 32 < r ? 2u * (uint32_t)ks : 0u);
+        // Beyond the rank the row's first group is fetched instead (inside the row also where the rank has fewer than four
+        // groups): no key step reaches those columns, and the value side keeps none of theirs.
+        const uint32_t at = gw[i] + (ks * 64 + (int)q4 * 32 < r ? 2u * (uint32_t)ks + q4 : 0u);
         // 4 bits: 16 bytes of codes and a separate scale/offset word; 3 bits: one 16-byte record {meta, w0, w1, w2}
         cw[i] = __ldg(Cb + at);
         if (QUANT == 4) mw[i] = __ldg(Mb + at);
@@ -553,7 +553,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
 #pragma unroll
       for (int i = 0; i < QP; ++i) {
         const int p = pos_s[pb * kTile + (int)rq + 32 * i];
-        gw[i] = (p < 0 ? 0u : (uint32_t)p) * (uint32_t)(r >> 5) + q4;
+        gw[i] = (p < 0 ? 0u : (uint32_t)p) * (uint32_t)(r >> 5);
       }
     };
     auto load_rows = [&](uint32_t (&ro)[16]) {             // rows without a selected token read row 0 (weight 0)
