@@ -676,6 +676,16 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     auto wait_all = [&](uint32_t bar, uint32_t parity, int word) {
       return __all_sync(0xffffffffu, wait_bar(ctx, bar, parity, word)) != 0;
     };
+    // Rows that were copied asynchronously are writes of the generic proxy, and their threads go on without waiting for them:
+    // the fence towards the tensor core's reads is this warp's, behind the wait.  (The quantised streams store their rows
+    // and fence themselves, before they arrive.)  It costs 0.2 to 0.6 % of a step: 131072 rows, budget 4096, 79.3 -> 79.8 us;
+    // 65536 rows, budget 16384, 321.1 -> 321.8.
+    auto wait_rows = [&](uint32_t bar, uint32_t parity, int word) {
+      const bool landed = wait_all(bar, parity, word);
+      if constexpr (QUANT == 0) fence_proxy_async();
+      tc_fence_after();
+      return landed;
+    };
     int it = 0;
     bool ok = true;
     TileIter cur;
@@ -692,9 +702,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
 #pragma unroll 1
         for (int ks = 0; ks < nst_k; ks += 2) {
           // one ring-slot pair per iteration: rows and B slabs of both slots, then all steps at once
-          if (!wait_all(BAR(bl.full) + 8u * pr, (seen >> pr) & 1u, ps + 3)) { ok = false; break; }
+          if (!wait_rows(BAR(bl.full) + 8u * pr, (seen >> pr) & 1u, ps + 3)) { ok = false; break; }
           seen ^= 1u << pr;
-          tc_fence_after();
           const long long i0 = ctx.prof ? clock64() : 0;
           const uint64_t a_desc = desc_hi | (rows_lo0 + pr * (2u * kSlab16));
           const uint64_t b_desc = desc_hi | (b_lo0 + pr * (2u * kSlab16));
@@ -726,9 +735,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
         const uint64_t p_desc = desc_hi | (p_lo0 + (uint32_t)buf * (kPBytes >> 4));
 #pragma unroll 1
         for (int ks = 0; ks < nst_v; ks += 2) {
-          if (!wait_all(BAR(bl.fullv) + 8u * pr, (seen >> pr) & 1u, ps + 3)) { ok = false; break; }
+          if (!wait_rows(BAR(bl.fullv) + 8u * pr, (seen >> pr) & 1u, ps + 3)) { ok = false; break; }
           seen ^= 1u << pr;
-          tc_fence_after();
           const long long i0 = ctx.prof ? clock64() : 0;
           const uint64_t a_desc = desc_hi | (rows_t_lo0 + pr * (2u * kSlab16));
           const uint32_t acc = accw + (uint32_t)(ks >> 1) * 16u;
