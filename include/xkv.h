@@ -352,10 +352,13 @@ XKV_API int xkv_debug_launch_counts(uint64_t* counts);
  *                             (but in range).
  *   XKV_INJECT_FUSED_NO_B     the reconstruct+attend kernel does not load the reconstruction matrices and
  *                             waits only briefly; its output for that call is unspecified.
+ *   XKV_INJECT_FUSED_NO_ROWS  the same, with the matrices loaded and no rows of A_k (nor their positions) to go with them:
+ *                             the kernel gives up while copies of its own are outstanding.
  * mask = 0 restores normal operation; later calls on the handle are then correct again.
  */
 #define XKV_INJECT_SCAN_NO_LOAD 1u
 #define XKV_INJECT_FUSED_NO_B 2u
+#define XKV_INJECT_FUSED_NO_ROWS 16u
 XKV_API int xkv_debug_set_fault_injection(xkv_group* grp, uint32_t mask);
 /*
  * The same for xkv_clf_factorize, which has no handle: the mask applies to every later call of the process until it

@@ -144,7 +144,7 @@ int xkv_debug_launch_counts(uint64_t* counts) {
   return XKV_OK;
 }
 int xkv_debug_set_fault_injection(xkv_group* g, uint32_t mask) {
-  if (!g || (mask & ~(XKV_INJECT_SCAN_NO_LOAD | XKV_INJECT_FUSED_NO_B))) return XKV_ERR_INVALID_ARG;
+  if (!g || (mask & ~(XKV_INJECT_SCAN_NO_LOAD | XKV_INJECT_FUSED_NO_B | XKV_INJECT_FUSED_NO_ROWS))) return XKV_ERR_INVALID_ARG;
   g->dev.inject = mask;
   return XKV_OK;
 }

@@ -67,6 +67,7 @@ struct Walk {        // a CTA's tiles: [begin, end), the first problem's part en
   int begin, end, next;
   int py, ti, l, b, g;   // the first problem: ordinal, tile in it, layer, sequence, head
   int seg;           // this CTA's segment of it
+  unsigned loaded;   // pairs of B_k slabs that the loader has requested, for the wind-down
 };
 struct Bars {        // offsets (in 8-byte words) into the barrier array
   int full, fullv, emptyk, emptyv, kfull, kempty, wfull, wempty, pfull, rfree, posfull, vfree, grp, drain, total;
@@ -353,7 +354,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     mbar_init(BAR(bl.grp), 128);
     mbar_init(BAR(bl.drain), 1); mbar_init(BAR(bl.drain + 1), 1);
     abort_flag[0] = 0;
-    abort_flag[1] = (dev.inject & XKV_INJECT_FUSED_NO_B) ? 16 : 0;   // injected fault: give up after about a millisecond
+    // an injected fault: give up after about a millisecond
+    abort_flag[1] = (dev.inject & (XKV_INJECT_FUSED_NO_B | XKV_INJECT_FUSED_NO_ROWS)) ? 16 : 0;
     fence_mbar_init();
   }
   if (rope_smem) {
@@ -424,6 +426,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     return dev.part + ((size_t)prob * sc.n_slots + seg) * (size_t)n_rep * (dev.r_v + 2);
   };
 
+  uint32_t pairs = 0;   // slot pairs that this thread (a producer, the loader) has begun to fill
   if (warp >= 8 && warp < kWarpK) {
     // =============================== producers: gather rows of A ===============================
     // Two independent streams with a ring of their own each: the first half of the producer warps (8-9, with quantised
@@ -475,6 +478,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
 #pragma unroll
         for (int i = 0; i < 16; ++i) cp_async16(st + kSlabBytes + (uint32_t)i * 1024u, s1 + (size_t)ro[i] * row_bytes, n1);
         cp_async_arrive_noinc(BAR(bar_full + pr));         // arrives when this thread's copies have landed
+        ++pairs;
         slot += 2;
         if (slot == RS) slot = 0;
       }
@@ -545,6 +549,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
         asm volatile("cp.async.wait_all;" ::: "memory");   // the staged rotary rows of this tile (key stream) have landed too
         fence_proxy_async();                               // the tensor core reads these stores
         mbar_arrive(BAR(bar_full + pr));                   // the pair is complete when all threads of the stream are done
+        ++pairs;
         slot += 2;
         if (slot == RS) slot = 0;
       }
@@ -569,6 +574,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     TileIter cur, nxt;
     iter_begin(nxt);
     bool have = iter_next(nxt, no_op, no_op);
+    if (kstream && (dev.inject & XKV_INJECT_FUSED_NO_ROWS)) have = false;   // fault injection: no positions, no rows of A_k
     auto load_pos = [&](const TileIter& x, int row) {
       return (x.ti * kTile + row < x.cnt) ? sel_idx[x.prob * sc.k_cap + x.ti * kTile + row] : -1;
     };
@@ -791,10 +797,12 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
           mbar_expect_tx(bar, second ? 2u * kSlabBytes : (uint32_t)kSlabBytes);
           tma_load_2d(dst, &bk_map, ks * 64, head_row, bar);
           if (second) tma_load_2d(dst + kSlabBytes, &bk_map, ks * 64 + 64, head_row, bar);
+          ++pairs;
         }
         if (++pr == SK / 2) pr = 0;
       }
     }
+    if (lane == 0) walk_s->loaded = pairs;
   } else if (warp < 4) {
     // =============================== key epilogue: rope, logits, softmax statistics, weights ===============================
     const int j = tid;                                  // tile row = TMEM lane
@@ -1009,6 +1017,18 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   if (warp == kWarpK) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
+  }
+  if (*abort_flag) {
+    // Given up: slabs of B_k may still be on their way into this CTA's shared memory, which the next CTA on the SM would
+    // inherit.  They arrive on barriers that count the key stream's threads too: those make up the arrivals that they owe
+    // the pairs requested, so that a pair's phase ends with its last byte, and the loader stays (again with a limit) for it.
+    const uint32_t loaded = walk_s->loaded;
+    if (warp >= 8 && warp < 8 + PW / 2) {
+      for (uint32_t n = pairs; n < loaded; ++n) mbar_arrive(BAR(bl.full) + 8u * (n % (SK / 2)));
+    } else if (warp == kWarpB && lane == 0) {
+      for (uint32_t n = loaded > SK / 2 ? loaded - SK / 2 : 0u; n < loaded; ++n)
+        for (uint32_t i = 0; i < (1u << 22); ++i) if (mbar_try_wait(BAR(bl.full) + 8u * (n % (SK / 2)), (n / (SK / 2)) & 1u)) break;
+    }
   }
 }
 

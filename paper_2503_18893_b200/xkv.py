@@ -132,6 +132,7 @@ XKV_INJECT_SCAN_NO_LOAD = 1
 XKV_INJECT_FUSED_NO_B = 2
 XKV_INJECT_CLF_BARRIER = 4
 XKV_INJECT_CLF_CHOLESKY = 8
+XKV_INJECT_FUSED_NO_ROWS = 16
 _lib.xkv_debug_set_clf_fault_injection.argtypes = [ctypes.c_uint32]
 _lib.xkv_debug_set_clf_fault_injection.restype = ctypes.c_int
 
