@@ -8,6 +8,7 @@
 #include <atomic>
 
 #include "xkv.h"
+#include "xkv_grow.h"
 
 namespace xkv {
 
@@ -102,7 +103,7 @@ void count_launch(KernelFamily family, int n = 1);
 
 // cudaFuncAttributeMaxDynamicSharedMemorySize of one kernel, set once per device instead of on every launch (the
 // attribute is sticky; re-issuing it costs host time on the launch path).  `Kernel` is the kernel's address, so
-// every instantiation keeps its own record.
+// every instantiation keeps its own record.  The attribute is per kernel and device, not per thread: see xkv_grow.h.
 constexpr int kMaxDevices = 64;
 template <auto Kernel>
 inline cudaError_t ensure_dyn_smem(size_t bytes, int device) {
@@ -120,9 +121,8 @@ inline cudaError_t ensure_dyn_smem(size_t bytes, int device) {
     static_bytes.store(st, std::memory_order_release);
   }
   if (bytes + (size_t)st <= 48 * 1024) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) have[device].store(bytes, std::memory_order_release);
-  return e;
+  static std::mutex lock;
+  return grow(have[device], lock, bytes, [](size_t to) { return cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)to); });
 }
 
 // SMs of a device, looked up once per device.
