@@ -29,6 +29,7 @@
 // total, 33 accumulator.
 #include <cuda.h>
 
+#include "xkv_gather.h"
 #include "xkv_internal.cuh"
 #include "xkv_ptx.cuh"
 
@@ -510,9 +511,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       uint4 cw[QP];
       uint32_t mw[QP];
       auto fetch = [&](int ks, int i) {
-        // Beyond the rank the row's first group is fetched instead (inside the row also where the rank has fewer than four
-        // groups): no key step reaches those columns, and the value side keeps none of theirs.
-        const uint32_t at = gw[i] + (ks * 64 + (int)q4 * 32 < r ? 2u * (uint32_t)ks + q4 : 0u);
+        const uint32_t at = gw[i] + quant_group(ks, q4, r);
         // 4 bits: 16 bytes of codes and a separate scale/offset word; 3 bits: one 16-byte record {meta, w0, w1, w2}
         cw[i] = __ldg(Cb + at);
         if (QUANT == 4) mw[i] = __ldg(Mb + at);

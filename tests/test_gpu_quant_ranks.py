@@ -1,5 +1,6 @@
 """The gather from codes at ranks of fewer groups than a slot pair has lanes for (a row of one to three groups), over whole
-contexts, so that the last rows of the bases are read."""
+contexts: results only.  (What a lane beyond the rank fetches is never used, so a read past the row would not show here; that
+every lane stays inside the row is checked in test_host_headers.py.)"""
 import pytest
 
 from tests.test_gpu_quant import test_decode_step_from_quantised_bases as check

@@ -48,3 +48,26 @@ int main() {
   return 0;
 }
 """)
+
+
+def test_the_gather_from_codes_stays_inside_the_row(run_cpp):
+    """Every rank up to 8192, the largest of a handle, every pair of slabs, every lane; and every group
+    of the row is fetched, by the lane whose columns it holds."""
+    run_cpp(r"""
+#include <cstdio>
+#include "xkv_gather.h"
+int main() {
+  for (int rank = 32; rank <= 8192; rank += 32) {
+    const int groups = rank / 32, slabs = ((rank + 63) / 64 + 1) & ~1;     // slabs are padded to pairs
+    int fetched[256] = {};
+    for (int ks = 0; ks < slabs; ks += 2)
+      for (uint32_t lane = 0; lane < 4; ++lane) {
+        const uint32_t at = xkv::quant_group(ks, lane, rank);
+        if (at >= (uint32_t)groups) { printf("rank %d, slab %d, lane %u: group %u\n", rank, ks, lane, at); return 1; }
+        if (ks * 64 + (int)lane * 32 == (int)at * 32) ++fetched[at];
+      }
+    for (int i = 0; i < groups; ++i) if (fetched[i] != 1) { printf("rank %d: group %d fetched %d times\n", rank, i, fetched[i]); return 1; }
+  }
+  return 0;
+}
+""")
