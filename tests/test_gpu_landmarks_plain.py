@@ -1,5 +1,10 @@
-"""Landmarks of the default chunk with and without cosines come from two kernels with the same arithmetic: the same bits, also
-where a CTA walks many row blocks, keeps one table or two, or has row groups without a layer of their own."""
+"""Landmarks of the default chunk with and without cosines come from two kernels with the same arithmetic on a row, also where
+a CTA walks many row blocks, keeps one table or two, or has row groups without a layer of their own: the same bits where
+nothing is rotated.  With rotation the two reach a table entry from other fp64 starts by other numbers of steps: after n steps
+(at most T) the angles agree to n 2^-53, so a share of n 2^-28 of the fp32 entries is rounded the other way, off by 2^-24.  A
+sum of eight such rows then moves by 2^-24 of its terms and changes its bf16 (a spacing of 2^-8) once in 2^15 times, to the
+neighbour unless the terms cancel: 8 T 2^-28 2^-15, below 1e-7 of the entries, are expected to differ, and ten times that is
+allowed."""
 import pytest
 import torch
 
@@ -23,7 +28,12 @@ def test_same_landmarks(T, G, H_kv, d_h, base):
     mc = torch.empty((G, 1, H_kv, n_c), dtype=torch.float32, device="cuda")
     xkv.xkv_build_landmarks(keys, lm[0], G=G, batch=1, T=T, H_kv=H_kv, d_h=d_h, rope_base=base)
     xkv.xkv_build_landmarks(keys, lm[1], G=G, batch=1, T=T, H_kv=H_kv, d_h=d_h, rope_base=base, min_cos=mc)
-    assert torch.equal(lm[0].view(torch.int16), lm[1].view(torch.int16))
+    if base == 0:
+        assert torch.equal(lm[0].view(torch.int16), lm[1].view(torch.int16))
+    else:
+        a, b = lm[0].double(), lm[1].double()
+        assert int((a != b).sum()) <= 1e-6 * a.numel()
+        assert ((a - b).abs() <= 2.0 ** -7 * a.abs() + 2.0 ** -20 * a.abs().max()).all()
     # the last chunk of one head, which may be ragged: its mean and its cosines in fp64
     x = keys[0, G - 1, 8 * (n_c - 1):, :d_h].double()
     if base > 0:
