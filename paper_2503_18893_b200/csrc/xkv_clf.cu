@@ -187,8 +187,9 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       const int m = c.m0 + tid;
       const uint32_t lane_base = ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * kAccCols;
       if (!Cf && c.n0 + BN <= N && (TRANS || (ldc & 7) == 0)) {
-        // bf16 alone: to registers, the accumulators handed back, then the stores; as many columns at a time as registers hold
-        constexpr int kPart = BN == 192 ? 96 : LO ? 64 : 128;
+        // bf16 alone: to registers, the accumulators handed back, then the stores; as many columns at a time as registers
+        // hold without spills (two parts of 192 columns, 96 at a time: 48 bytes of them, and the same time)
+        constexpr int kPart = LO ? 64 : BN == 192 ? 96 : 128;
 #pragma unroll 1
         for (int n = 0; n < BN; n += kPart) {
           uint32_t h[kPart / 2], rest[LO ? kPart / 2 : 1];
@@ -230,47 +231,47 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         }
       } else {
 #pragma unroll 1
-          for (int cb = 0; cb < BN / 32; ++cb) {
-            float v[32];
-            tmem_ld32(tmem + lane_base + (uint32_t)(cb * 32), v);
-            tc_wait_ld();
-            if (m < M) {
-              const int nb = c.n0 + cb * 32;
-              if (!TRANS && nb + 32 <= N && (ldc & 7) == 0) {
-                // a whole run of 32 columns of one row: 16-byte stores (the row pitch keeps them aligned)
-                const long long at = (long long)m * ldc + nb;
-                if (Cz) {
+        for (int cb = 0; cb < BN / 32; ++cb) {
+          float v[32];
+          tmem_ld32(tmem + lane_base + (uint32_t)(cb * 32), v);
+          tc_wait_ld();
+          if (m < M) {
+            const int nb = c.n0 + cb * 32;
+            if (!TRANS && nb + 32 <= N && (ldc & 7) == 0) {
+              // a whole run of 32 columns of one row: 16-byte stores (the row pitch keeps them aligned)
+              const long long at = (long long)m * ldc + nb;
+              if (Cz) {
 #pragma unroll
-                  for (int i = 0; i < 32; i += 4) *reinterpret_cast<float4*>(Cz + at + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                for (int i = 0; i < 32; i += 4) *reinterpret_cast<float4*>(Cz + at + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+              }
+              if (Cb) {
+#pragma unroll
+                for (int i = 0; i < 32; i += 8) {
+                  __nv_bfloat162 h0 = __floats2bfloat162_rn(v[i], v[i + 1]), h1 = __floats2bfloat162_rn(v[i + 2], v[i + 3]);
+                  __nv_bfloat162 h2 = __floats2bfloat162_rn(v[i + 4], v[i + 5]), h3 = __floats2bfloat162_rn(v[i + 6], v[i + 7]);
+                  uint4 u;
+                  u.x = *reinterpret_cast<uint32_t*>(&h0); u.y = *reinterpret_cast<uint32_t*>(&h1);
+                  u.z = *reinterpret_cast<uint32_t*>(&h2); u.w = *reinterpret_cast<uint32_t*>(&h3);
+                  *reinterpret_cast<uint4*>(Cb + at + i) = u;
                 }
-                if (Cb) {
+              }
+            } else {
 #pragma unroll
-                  for (int i = 0; i < 32; i += 8) {
-                    __nv_bfloat162 h0 = __floats2bfloat162_rn(v[i], v[i + 1]), h1 = __floats2bfloat162_rn(v[i + 2], v[i + 3]);
-                    __nv_bfloat162 h2 = __floats2bfloat162_rn(v[i + 4], v[i + 5]), h3 = __floats2bfloat162_rn(v[i + 6], v[i + 7]);
-                    uint4 u;
-                    u.x = *reinterpret_cast<uint32_t*>(&h0); u.y = *reinterpret_cast<uint32_t*>(&h1);
-                    u.z = *reinterpret_cast<uint32_t*>(&h2); u.w = *reinterpret_cast<uint32_t*>(&h3);
-                    *reinterpret_cast<uint4*>(Cb + at + i) = u;
-                  }
-                }
-              } else {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                  const int n = nb + i;
-                  if (n < N) {
-                    const long long at = TRANS ? (long long)n * ldc + m : (long long)m * ldc + n;
-                    if (Cz) Cz[at] = v[i];
-                    if (Cb) {
-                      const __nv_bfloat16 hi = __float2bfloat16(v[i]);
-                      Cb[at] = hi;
-                      if (LO) Cl[at] = __float2bfloat16(2.0f * (v[i] - __bfloat162float(hi)));
-                    }
+              for (int i = 0; i < 32; ++i) {
+                const int n = nb + i;
+                if (n < N) {
+                  const long long at = TRANS ? (long long)n * ldc + m : (long long)m * ldc + n;
+                  if (Cz) Cz[at] = v[i];
+                  if (Cb) {
+                    const __nv_bfloat16 hi = __float2bfloat16(v[i]);
+                    Cb[at] = hi;
+                    if (LO) Cl[at] = __float2bfloat16(2.0f * (v[i] - __bfloat162float(hi)));
                   }
                 }
               }
             }
           }
+        }
         tc_fence_before();
         mbar_arrive(FREE);
       }
@@ -730,8 +731,8 @@ namespace {
 //   B  the grid applies M <- Q^T M Q, 64 x 32 pieces, from one buffer to the other.
 // Two grid barriers per 32 rounds of rotations.  (Applying every round of l/2 rotations to the whole matrix takes a
 // barrier per round: 575 per sweep of a 576 x 576 matrix, 4.9 us each, 8.5 ms for three sweeps; taking the 64 x 64
-// problems to convergence before they are applied was slower still.  This form takes 1.5 ms for the same three sweeps; the
-// factorisation of a 131072 x 4096 cache went from 26.2 to 17.2 ms.)  A check per sweep ends the sweeps once the
+// problems to convergence before they are applied was slower still.  This form took 1.5 ms for
+// the same three sweeps and takes 1.22 with the cross rounds in registers.)  A check per sweep ends the sweeps once the
 // off-diagonal weight is below kJacobiTol.  On return the eigenvalues are on the diagonal of M (buffer 0), the
 // eigenvectors the rows of Pt.
 constexpr int kJacobiMaxPairs = 1024;              // l <= 2048
