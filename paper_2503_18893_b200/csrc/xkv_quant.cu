@@ -16,10 +16,11 @@ namespace xkv {
 namespace {
 
 constexpr int kQuantThreads = 256;
-// The first blocks, those that may be resident while the kernel before still runs, have their scalars brought into L2 before
+// The first blocks, those that may start while the kernel before still runs, have their scalars brought into L2 before
 // they wait for it (the second level is where that kernel's writes would land, so nothing stale is read): six launches of a
-// window 41.9 -> 40.6 us.
-constexpr int kQuantAhead = 1184;
+// window 41.9 -> 40.6 us.  As many as an SM's 2048 threads hold of them; its registers hold five at a time, but the others
+// follow before those have finished (five per SM: 41.2 us).  A device with another number of SMs only prefetches more or less.
+constexpr int kQuantAhead = 2048 / kQuantThreads * kPlanSms;
 constexpr int kQuantPieces = 4;    // 16-byte pieces per thread, all requested before the first is used (four: see the quantiser)
 
 __device__ __forceinline__ uint32_t min_bf16x2(uint32_t a, uint32_t b) {
@@ -45,8 +46,8 @@ __device__ __forceinline__ float max_nan(float a, float b) {
 }
 
 // HBM bound: 2 bytes read and (bits + 1) / 8 written per scalar.  Four consecutive lanes share a group of 32 scalars, a
-// lane holds one 16-byte piece (8 scalars): loads and stores of a warp are contiguous, extrema are packed bf16 minima
-// folded by two shuffles.
+// lane holds one 16-byte piece (8 scalars) of four groups: loads and stores of a warp are contiguous, extrema are packed
+// bf16 minima and maxima, folded by halving so that a lane ends with those of one group.
 // The codes are rint(fl(f / scale)), f = x - zero.  The correctly rounded quotient comes from the correctly rounded
 // reciprocal y by q = f y, q + (f - q scale) y with fused multiply-adds (Markstein, IBM J. Res. Dev. 34(1), 1990); the
 // exact quotient of a 24-bit by an 8-bit number is never closer than 2^-33 to a rounding boundary and the value that is
@@ -55,7 +56,7 @@ __device__ __forceinline__ float max_nan(float a, float b) {
 // warps (25 us for 65536 x 384 scalars, with an IEEE division per scalar and one thread per group 38 us; this form 19.5, and 17 with
 // two scalars per packed instruction).
 // A group's scale, offset and reciprocal are some forty instructions, a quarter of the kernel's when all four lanes worked
-// them out for every group, and instruction issue is what bounds it (80 % of the slots): a quad holds four groups, and lane p
+// them out for every group, and instruction issue is what bounds it (71 % of the slots now): a quad holds four groups, and lane p
 // does that work for group p alone.  A window's token bases and matrices (65536 rows of 384 and 576; six launches):
 // 46.4 -> 41.8 us.
 // Rounding goes through 1.5 * 2^23, whose sum with the quotient holds the integer in its low bits.
