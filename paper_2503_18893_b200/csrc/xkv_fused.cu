@@ -661,7 +661,9 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     // a slot pair costs it one wait (gathered rows and B_k slabs arrive on one barrier) instead of four, and branches
     // outside the issue are taken on a vote, so that the compiler may keep the descriptors in uniform registers, where the
     // tensor-core instructions take them from.  The kernel alone: 131072 rows, budget 4096, rank 512 45.1 -> 41.7 us; 65536
-    // rows, budget 16384, rank 1024 255.8 -> 239.7; eight heads, rank 256 75.1 -> 70.2; one tile per CTA 18.1 -> 17.2.
+    // rows, budget 16384, rank 1024 255.8 -> 239.7; eight heads, rank 256 75.1 -> 70.2; one tile per CTA 18.1 -> 17.2.  (Of
+    // the first a step shows little: kernel and merge back to back over eight windows 45.4 -> 41.2 us with the order of the
+    // tiles, behind the selections 76.8 -> 75.9.)
     constexpr uint32_t idesc_k = idesc_bf16_f32(128, 128);                     // keys: both operands K-major
     constexpr uint32_t idesc_v = idesc_bf16_f32(128, 16) | (1u << 15);         // values: A is read along its rows (MN-major)
     const int ps = kside ? 8 : 40;
