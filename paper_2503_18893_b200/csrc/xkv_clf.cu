@@ -188,8 +188,9 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       const uint32_t lane_base = ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(warp >> 2) * kAccCols;
       if (!Cf && c.n0 + BN <= N && (TRANS || (ldc & 7) == 0)) {
         // bf16 alone: to registers, the accumulators handed back, then the stores; as many columns at a time as registers
-        // hold without spills (two parts of 192 columns, 96 at a time: 48 bytes of them, and the same time)
-        constexpr int kPart = LO ? 64 : BN == 192 ? 96 : 128;
+        // hold.  (Two parts of 192 columns spill 48 bytes at 96; 64 at a time spill nothing and hand the accumulators back
+        // later: X Z in two parts, 131072 x 4096 x 576, 844 -> 849 us.)
+        constexpr int kPart = BN == 192 ? 96 : LO ? 64 : 128;
 #pragma unroll 1
         for (int n = 0; n < BN; n += kPart) {
           uint32_t h[kPart / 2], rest[LO ? kPart / 2 : 1];
