@@ -656,14 +656,14 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     // Two issuing threads, each walking its own ring (one thread spends 70-130 cycles per tcgen05.mma and about
     // 235 per tcgen05.commit).
     const bool kside = warp == kWarpK;
-    // The whole warp walks the loop, one elected lane issues.  The key side is a critical chain of the kernel (of 10.0 k
-    // cycles a tile it waited for data in 2.1 k and issued in 3.8 k; the rest were its own instructions between the two), so
-    // a slot pair costs it one wait (gathered rows and B_k slabs arrive on one barrier) instead of four, and branches
-    // outside the issue are taken on a vote, so that the compiler may keep the descriptors in uniform registers, where the
-    // tensor-core instructions take them from.  The kernel alone: 131072 rows, budget 4096, rank 512 45.1 -> 41.7 us; 65536
-    // rows, budget 16384, rank 1024 255.8 -> 239.7; eight heads, rank 256 75.1 -> 70.2; one tile per CTA 18.1 -> 17.2.  (Of
-    // the first a step shows little: kernel and merge back to back over eight windows 45.4 -> 41.2 us with the order of the
-    // tiles, behind the selections 76.8 -> 75.9.)
+    // The whole warp walks the loop, one elected lane issues.  The key side is a critical chain of the kernel (with four
+    // waits per slot pair, of 10.0 k cycles a tile it waited for data in 2.1 k and issued in 3.8 k; the rest were its own
+    // instructions between the two; of 7.6 k now 1.9, 3.0 and 2.6), so a slot pair costs it one wait (gathered rows and B_k
+    // slabs arrive on one barrier), and branches outside the issue are taken on a vote, so that the compiler may keep the
+    // descriptors in uniform registers, where the tensor-core instructions take them from.  The kernel alone: 131072 rows,
+    // budget 4096, rank 512 45.1 -> 41.7 us; 65536 rows, budget 16384, rank 1024 255.8 -> 239.7; eight heads, rank 256 75.1
+    // -> 70.2; one tile per CTA 18.1 -> 17.2.  (Of the first a step shows little: kernel and merge back to back over eight
+    // windows 45.4 -> 41.2 us with the order of the tiles, behind the selections 76.8 -> 75.9.)
     constexpr uint32_t idesc_k = idesc_bf16_f32(128, 128);                     // keys: both operands K-major
     constexpr uint32_t idesc_v = idesc_bf16_f32(128, 16) | (1u << 15);         // values: A is read along its rows (MN-major)
     const int ps = kside ? 8 : 40;
@@ -685,8 +685,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     };
     // Rows that were copied asynchronously are writes of the generic proxy, and their threads go on without waiting for them:
     // the fence towards the tensor core's reads is this warp's, behind the wait.  (The quantised streams store their rows
-    // and fence themselves, before they arrive.)  It costs 0.2 to 0.6 % of a step: 131072 rows, budget 4096, 79.3 -> 79.8 us;
-    // 65536 rows, budget 16384, 321.1 -> 321.8.
+    // and fence themselves, before they arrive.)  It costs 0.2 to 0.9 % of a step: 131072 rows, budget 4096, 78.3 -> 78.7 us;
+    // 65536 rows, budget 16384, 318.7 -> 319.6; 32768 rows by layer 113.4 -> 114.1.
     auto wait_rows = [&](uint32_t bar, uint32_t parity, int word) {
       const bool landed = wait_all(bar, parity, word);
       if constexpr (QUANT == 0) fence_proxy_async();
