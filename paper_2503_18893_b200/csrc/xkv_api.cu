@@ -201,6 +201,7 @@ int xkv_group_create(const xkv_group_config* cfg, void* stream, xkv_group** out)
     const size_t btk = heads * kDP * c.r_k * sizeof(__nv_bfloat16);
     const size_t btv = heads * kDP * c.r_v * sizeof(__nv_bfloat16);
     const size_t pooled = c.landmarks ? heads * d.n_c * sizeof(float) : 0;
+    const size_t tiles = c.landmarks && d.n_rep > 4 ? heads * ((d.n_c + kLandmarkBoxRows - 1) / kLandmarkBoxRows) * sizeof(uint32_t) : 0;
     const size_t hi = (size_t)d.n_hi * (c.d_h / 2) * sizeof(float2);
     const size_t lo = ((size_t)1 << d.rope_shift) * (c.d_h / 2) * sizeof(float2);
     const size_t pf0 = attend_part_floats(g), pf1 = fused_part_floats(g);
@@ -218,6 +219,7 @@ int xkv_group_create(const xkv_group_config* cfg, void* stream, xkv_group** out)
     XKV_ALLOC(Bt_v, __nv_bfloat16*, btv);
     XKV_ALLOC(Bv_copy, __nv_bfloat16*, (size_t)c.batch * c.G * c.r_v * c.H_kv * c.d_h * sizeof(__nv_bfloat16));
     XKV_ALLOC(d.pooled, float*, pooled);
+    if (tiles) XKV_ALLOC(d.tile_max, uint32_t*, tiles);
     XKV_ALLOC(rhi, float2*, hi);
     XKV_ALLOC(rlo, float2*, lo);
     XKV_ALLOC(d.part, float*, part);

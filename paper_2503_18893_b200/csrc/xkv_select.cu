@@ -193,6 +193,139 @@ score_pool_kernel(const __grid_constant__ CUtensorMap tmap, GroupDev dev, const 
   if (j0 + row0 + kScoreThreads < dev.n_c) dst[j0 + row0 + kScoreThreads] = score_key(best1);
 }
 
+// ---- The scan with more than four query heads per KV head: tensor-core scores and their error bound.
+// Only the index sets leave the selection, so a score has to be the canonical one only where it decides something: the
+// scores here carry an error of at most E, and topk_pivot_kernel scores the few chunks within 2 E of the cut again in the
+// canonical order.  score_pool_kernel is bound by the shared-memory pipe with that many heads (14 query loads of four cycles
+// for 112 multiply-adds per 8 dimensions at seven); here a landmark leaves shared memory once, as the fragments of
+// mma.sync.m16n8k16, whose eight columns are the heads, and the queries stay in registers.  What bounds it is the landmarks.
+// mma.sync and not tcgen05: 0.1 TFLOP in all, and a warp keeps its own tile without tensor memory or a second barrier.
+//
+// The bound.  The products are exact in fp32.  With S = sum_i |q_i l_i| the canonical chain of d_h <= 128 multiply-adds is
+// off by at most 128 2^-24 S, d_h / 16 steps of at most 17 truncated terms each by at most 136 2^-23 S, and scaling adds one
+// rounding to either: less than 2^-15 S together.  S <= |q|_1 max |l|, both maxima over the problem: the largest landmark
+// element of every tile is written beside the scores.
+constexpr float kScoreBound = 1.0f / 32768.0f;
+
+__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t max_u16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+
+// grid as above.  NT: groups of eight heads.  tile_max [problem][tile]: bits of the largest |element| as a bf16 number (a NaN
+// above everything).
+template <int DH, int NT>
+__global__ void __launch_bounds__(kScoreThreads)
+score_bound_kernel(const __grid_constant__ CUtensorMap tmap, GroupDev dev, const __nv_bfloat16* __restrict__ q, int l0) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t bar_storage;
+  constexpr int KS = DH / 16;
+  const uint32_t tile = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t bar = smem_u32(&bar_storage);
+  const int lane = threadIdx.x, g8 = lane >> 2, t = lane & 3;
+
+  const int g = blockIdx.y % dev.H_kv;
+  const int b = (blockIdx.y / dev.H_kv) % dev.batch;
+  const int l = l0 + blockIdx.y / (dev.H_kv * dev.batch);
+  const int j0 = blockIdx.x * kScoreRows;
+  const long long prob_lm = ((long long)b * dev.G + l) * dev.H_kv + g;       // landmark order
+  const long long prob_out = ((long long)l * dev.batch + b) * dev.H_kv + g;  // [G][batch][H_kv] order
+
+  // loads ahead of the dependency wait, fault injection, limits: as in score_pool_kernel
+  const bool no_load = (dev.inject & XKV_INJECT_SCAN_NO_LOAD) != 0u;
+  const bool early = dev.lm_const != 0;
+  if (!early) grid_dependency_wait();
+  if (lane == 0) {
+    mbar_init(bar, 1);
+    fence_mbar_init();
+    if (!no_load) {
+      mbar_expect_tx(bar, (uint32_t)((DH / 64) * kScoreRows * 128));
+      const int y = (int)(prob_lm * dev.n_c + j0);
+      const uint64_t pol = l2_policy_evict_first();
+#pragma unroll
+      for (int bx = 0; bx < DH / 64; ++bx) tma_load_2d_hint(tile + bx * kScoreRows * 128, &tmap, bx * 64, y, bar, pol);
+    }
+  }
+  if (early) grid_dependency_wait();
+  grid_dependency_launch();
+  // this lane's fragments of the queries: head 8 n + g8, dimensions 16 ks + 2 t, + 1 and those 8 on (heads beyond n_rep: zero)
+  const __nv_bfloat16* qg = q + (((long long)l * dev.batch + b) * dev.H_q + (long long)g * dev.n_rep) * DH;
+  uint32_t qf[NT][KS][2];
+#pragma unroll
+  for (int n = 0; n < NT; ++n) {
+    const int h = 8 * n + g8;
+    const uint32_t* qh = reinterpret_cast<const uint32_t*>(qg + (size_t)h * DH) + t;
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+      for (int x = 0; x < 2; ++x) qf[n][ks][x] = h < dev.n_rep ? qh[ks * 8 + x * 4] : 0u;
+  }
+  __syncwarp();
+
+  if (!mbar_wait_bounded(bar, 0, no_load ? 1024u : kWaitLimit)) {
+    if (lane == 0) atomicOr(dev.flags, XKV_FLAG_TIMEOUT);
+    if (!no_load) (void)mbar_wait_bounded(bar, 0);
+    return;
+  }
+  // lane i hands ldmatrix the address of row i % 16, dimensions 8 (i / 16) of a 16 x 16 piece
+  const uint32_t arow = (uint32_t)(lane & 15), ahalf = (uint32_t)(lane >> 4);
+  float keep[2] = {0.0f, 0.0f};                            // rows 16 t + g8 and 16 t + 8 + g8
+  uint32_t big0 = 0u, big1 = 0u;
+#pragma unroll
+  for (int m = 0; m < kScoreRows / 16; ++m) {
+    const uint32_t row = (uint32_t)(16 * m) + arow, sw = row & 7u;
+    float acc[NT][4];
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[n][i] = 0.0f;
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) {
+      uint32_t a[4];
+      ldmatrix_x4(a, tile + (uint32_t)(ks >> 2) * (kScoreRows * 128u) + row * 128u + ((((uint32_t)(ks & 3) * 2u + ahalf) ^ sw) << 4));
+      big0 = max_u16x2(big0, max_u16x2(a[0] & 0x7fff7fffu, a[1] & 0x7fff7fffu));
+      big1 = max_u16x2(big1, max_u16x2(a[2] & 0x7fff7fffu, a[3] & 0x7fff7fffu));
+#pragma unroll
+      for (int n = 0; n < NT; ++n) mma_16816(acc[n], a, qf[n][ks][0], qf[n][ks][1]);
+    }
+    // columns 2 t, 2 t + 1 of rows g8 (acc 0, 1) and g8 + 8 (acc 2, 3): maximum over the heads that exist
+    float best[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int x = 0; x < 2; ++x)
+        if (8 * n + 2 * t + x < dev.n_rep) {
+          best[0] = fmaxf(best[0], acc[n][x] * dev.sel_scale);
+          best[1] = fmaxf(best[1], acc[n][2 + x] * dev.sel_scale);
+        }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      best[0] = fmaxf(best[0], __shfl_xor_sync(0xffffffffu, best[0], o));
+      best[1] = fmaxf(best[1], __shfl_xor_sync(0xffffffffu, best[1], o));
+    }
+    if (t == m) { keep[0] = best[0]; keep[1] = best[1]; }
+  }
+  static_assert(kScoreRows == 64, "four lanes of a row, four pieces of 16 rows");
+  uint32_t* dst = reinterpret_cast<uint32_t*>(dev.pooled) + prob_out * dev.n_c;
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int j = j0 + 16 * t + 8 * x + g8;
+    if (j < dev.n_c) dst[j] = score_key(keep[x]);
+  }
+  big0 = max_u16x2(big0, big1);
+  const uint32_t big = __reduce_max_sync(0xffffffffu, max(big0 & 0xffffu, big0 >> 16));
+  if (lane == 0) dev.tile_max[prob_out * gridDim.x + blockIdx.x] = big;
+}
+
 // ---------------------------------------------------------------------------------------------
 
 constexpr int kTopkThreads = 1024;
@@ -573,6 +706,12 @@ topk_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __restrict
 // second bitmap.  GPT = 0 disables the filter (P = the smallest key): chosen by the host when there are fewer groups than
 // k_ch.  ITEMS = 16 keys per thread serve n_c <= 16384 chunks, ITEMS = 32 (keys read twice instead of held in registers)
 // n_c <= 32768.  The result is identical to topk_kernel's for every input.
+//
+// BOUND: the keys are those of score_bound_kernel, off by at most E (see there).  The k_ch-th largest canonical score then
+// lies within E of the k_ch-th largest key, so chunks more than 2 E above the bin of step 4 are taken and those more than 2 E
+// below it are not; the band between is scored again in the canonical order, a warp per chunk, a lane per head, and its keys
+// take the place of the bin's.  Step 3 lists down to P - 2 E.  A band of more than kTopkCand chunks (ties, or an infinity or
+// NaN somewhere, where E is infinite and the band is everything) goes through the bins again.
 // (With consecutive keys per thread, extrema by shuffles, a thread per candidate and separate scans for ties and
 // positions, about 25 barriers: 32768 rows decoded layer by layer 129.4 us, 122.4 us with this form; 121873 rows 212.6 ->
 // 193.6; 2048 rows 19.3 -> 17.6.)
@@ -614,10 +753,38 @@ __device__ __forceinline__ void find_bin(const uint32_t* hist, uint32_t need, ui
   __syncthreads();
 }
 
-template <int GPT, int ITEMS, int TH>
+// float of a key (score_key's inverse but for -0)
+__device__ __forceinline__ float key_score(uint32_t k) { return __uint_as_float((k & 0x80000000u) ? k ^ 0x80000000u : ~k); }
+
+// The canonical pooled score of one landmark row, by a warp: lane h takes query head h.  q_s: bf16 queries in shared memory,
+// 16-byte units, qu units to a head.
+template <int DH>
+__device__ __forceinline__ uint32_t canonical_key(const __nv_bfloat16* __restrict__ row, const uint4* __restrict__ q_s, int qu,
+                                                  int n_rep, float scale, int lane) {
+  const uint4* rv = reinterpret_cast<const uint4*>(row);
+  uint4 v[DH / 8];
+#pragma unroll
+  for (int i = 0; i < DH / 8; ++i) v[i] = __ldg(rv + i);
+  const uint4* qh = q_s + min(lane, n_rep - 1) * qu;
+  float acc = 0.0f;
+#pragma unroll
+  for (int i = 0; i < DH / 8; ++i) {
+    const uint4 qv = qh[i];
+    const uint32_t lw[4] = {v[i].x, v[i].y, v[i].z, v[i].w}, qw[4] = {qv.x, qv.y, qv.z, qv.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      acc = fmaf(__uint_as_float(qw[e] << 16), __uint_as_float(lw[e] << 16), acc);
+      acc = fmaf(__uint_as_float(qw[e] & 0xffff0000u), __uint_as_float(lw[e] & 0xffff0000u), acc);
+    }
+  }
+  // (the maximum of order-preserving keys is the key of the maximum; a NaN takes no part, as in fmaxf)
+  return __reduce_max_sync(0xffffffffu, score_key(fmaxf(-INFINITY, acc * scale)));
+}
+
+template <int GPT, int ITEMS, int TH, bool BOUND>
 __global__ void __launch_bounds__(TH, 1)
 topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __restrict__ outliers, int n_out, float sign,
-                  int32_t* __restrict__ sel_idx, int32_t* __restrict__ sel_cnt) {
+                  const __nv_bfloat16* __restrict__ q, int32_t* __restrict__ sel_idx, int32_t* __restrict__ sel_cnt) {
   extern __shared__ __align__(16) uint8_t pivot_smem[];
   constexpr int kPivotListMax = TH * ITEMS;                              // every key may pass (all keys equal)
   constexpr int NW = kPivotListMax / 32;                                 // words of a bitmap
@@ -631,6 +798,8 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
   __shared__ unsigned long long cand_s[kTopkCand];                                 // (key, ~chunk index): larger = earlier
   __shared__ uint32_t sh[3];
   __shared__ uint32_t sh_n, sh_cand;
+  __shared__ uint32_t warp_l[TH / 32], warp_q[TH / 32];                            // BOUND: largest landmark element, largest |q|_1
+  __shared__ uint32_t sh_sure;                                                     // BOUND: chunks taken without their canonical score
 
   constexpr int NWARP = TH / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -651,9 +820,16 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
     take_w[w] = !all ? 0u : first + 32 <= n_c ? 0xffffffffu : (first < n_c ? ((1u << (n_c - first)) - 1u) : 0u);
     eq_w[w] = 0u;
   }
-  if (tid == 0) { sh_n = 0; sh_cand = 0; sh[0] = sh[1] = sh[2] = 0; }
+  if (tid == 0) { sh_n = 0; sh_cand = 0; sh[0] = sh[1] = sh[2] = 0; sh_sure = 0; }
   grid_dependency_wait();                      // the pooled scores come from the kernel launched before
   grid_dependency_launch();
+  const int pieces = dev.d_h / 8;              // 16-byte pieces of a query
+  const long long head0 = (prob / dev.H_kv) * dev.H_q + (prob % dev.H_kv) * dev.n_rep;    // of this problem's queries
+  uint4 q_piece = make_uint4(0u, 0u, 0u, 0u);
+  if constexpr (BOUND) {
+    static_assert(TH >= kMaxRep * 16, "a thread per piece of the queries");
+    if (tid < dev.n_rep * pieces) q_piece = __ldg(reinterpret_cast<const uint4*>(q + head0 * dev.d_h) + tid);
+  }
   bool ties = false;                           // the bin of the k_ch-th largest key holds equal keys only, and many of them
   uint32_t need = (uint32_t)k_ch;
   if (!all) {
@@ -680,6 +856,23 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
       }
     };
     load();
+    if constexpr (BOUND) {
+      const int n_t = (n_c + kScoreRows - 1) / kScoreRows;
+      uint32_t big = 0u;
+      for (int i = tid; i < n_t; i += TH) big = max(big, __ldcg(dev.tile_max + prob * n_t + i));
+      const uint32_t w[4] = {q_piece.x, q_piece.y, q_piece.z, q_piece.w};
+      float l1 = 0.0f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) l1 += __uint_as_float((w[e] << 16) & 0x7fffffffu) + __uint_as_float(w[e] & 0x7fff0000u);
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const float other = __shfl_xor_sync(0xffffffffu, l1, o);
+        if (o < pieces) l1 += other;
+      }
+      big = __reduce_max_sync(0xffffffffu, big);
+      const uint32_t lq = __reduce_max_sync(0xffffffffu, __float_as_uint(l1));
+      if (lane == 0) { warp_l[warp] = big; warp_q[warp] = lq; }
+    }
     // ---- 1: maxima of the groups that hold a chunk, and their range (keys beyond the last chunk are 0)
     uint32_t gmax[NG], kmin = 0xffffffffu, kmax = 0u;
 #pragma unroll
@@ -701,6 +894,13 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
     __syncthreads();
     kmin = __reduce_min_sync(0xffffffffu, lane < NWARP ? warp_min[lane] : 0xffffffffu);
     kmax = __reduce_max_sync(0xffffffffu, lane < NWARP ? warp_max[lane] : 0u);
+    float E2 = 0.0f;                                       // BOUND: 2 E
+    if constexpr (BOUND) {
+      const float big = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < NWARP ? warp_l[lane] : 0u) << 16);
+      const float l1 = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < NWARP ? warp_q[lane] : 0u));
+      const float S = l1 * big;
+      E2 = S < 1e36f ? fmaf(2.0f * kScoreBound * dev.sel_scale, S, 1e-37f) : INFINITY;    // (also where S is NaN)
+    }
     // ---- 2: pivot: lower edge of the bin that holds the k_ch-th largest group maximum
     uint32_t P = kmin;
     if (GPT != 0) {
@@ -712,12 +912,21 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
       find_bin<TH>(hist0, (uint32_t)k_ch, warp_tot, sh, tid);
       P = kmin + (sh[0] << sh1);
     }
+    uint32_t Pl = P;                                       // what is listed
+    if constexpr (BOUND) {
+      Pl = E2 < INFINITY ? min(P, score_key(__fadd_rd(key_score(P), -E2))) : 0u;
+      if (tid < dev.n_rep * pieces) {                      // the queries, into the first histogram, whose work is done
+        const int h = tid / pieces, u = tid - h * pieces;
+        reinterpret_cast<uint4*>(hist0)[h * (pieces + 1) + u] = q_piece;
+      }
+      static_assert(kMaxRep * (16 + 1) * 4 <= kTopkBins, "queries in a histogram");
+    }
     // ---- 3: the keys >= P, with their chunk index, to the list (one shared-memory atomic per warp)
     {
       if (ITEMS > 16) load();                              // 32 keys are not held across the barriers above: read them again
       uint32_t cm = 0;
 #pragma unroll
-      for (int i = 0; i < ITEMS; ++i) if (key[i] >= P && chunk_of(i) < n_c) cm |= 1u << i;
+      for (int i = 0; i < ITEMS; ++i) if (key[i] >= Pl && chunk_of(i) < n_c) cm |= 1u << i;
       const uint32_t mine_c = (uint32_t)__popc(cm);
       uint32_t inc = mine_c;
 #pragma unroll
@@ -739,30 +948,79 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
     const int n_list = (int)sh_n;                                      // >= k_ch
     // ---- 4: bins subdivide the window [lo, lo + span] that holds the k_ch-th largest key
     uint32_t lo = P, span = kmax - P, in_bin;
-    for (bool again = false;; again = true) {
-      const int bits = 32 - __clz(span);                               // span < 2^bits
-      const int shb = bits > 11 ? bits - 11 : 0;
-      if (again) {
-        for (int i = tid; i < kTopkBins; i += TH) hist1[i] = 0;
+    auto narrow = [&](uint32_t most, bool again) {         // down to `most` keys, or equal ones
+      for (;; again = true) {
+        const int bits = 32 - __clz(span);                             // span < 2^bits
+        const int shb = bits > 11 ? bits - 11 : 0;
+        if (again) {
+          for (int i = tid; i < kTopkBins; i += TH) hist1[i] = 0;
+          __syncthreads();
+        }
+        for (int e = tid; e < n_list; e += TH) {
+          const uint32_t rel = list_key[e] - lo;                       // keys below lo wrap to huge values
+          if (rel <= span) atomicAdd(&hist1[rel >> shb], 1u);
+        }
         __syncthreads();
+        find_bin<TH>(hist1, need, warp_tot, sh, tid);
+        const uint32_t bsel = sh[0];
+        need = sh[1];
+        in_bin = sh[2];
+        lo += bsel << shb;
+        span = min(span - (bsel << shb), (shb ? (1u << shb) : 1u) - 1u);
+        if (shb == 0 || in_bin <= most) break;
+        __syncthreads();                                               // sh is read before the next pass writes it
       }
+    };
+    narrow(BOUND ? (uint32_t)NWARP : (uint32_t)kTopkCand, false);
+    bool ranked = false;                                   // the candidates are in cand_s already
+    if constexpr (BOUND) {
+      // chunks above the band are taken; those in it keep their entry and are listed (the first kTopkCand of them)
+      // (at least the bin is in the band, whatever the keys are: fewer than k_ch chunks are above it, k_ch at or above its foot)
+      const uint32_t above = E2 < INFINITY ? max(lo + span, score_key(__fadd_ru(key_score(lo + span), E2))) : 0xffffffffu;
+      const uint32_t below = E2 < INFINITY ? min(lo, score_key(__fadd_rd(key_score(lo), -E2))) : 0u;
+      const __nv_bfloat16* rows = dev.landmarks + ((prob / dev.H_kv % dev.batch * dev.G + prob / per_layer) * dev.H_kv + prob % dev.H_kv) * n_c * dev.d_h;
+      auto exact_key = [&](uint32_t j) {
+        const __nv_bfloat16* row = rows + (size_t)j * dev.d_h;
+        const uint4* q_s = reinterpret_cast<const uint4*>(hist0);
+        return dev.d_h == 128 ? canonical_key<128>(row, q_s, pieces + 1, dev.n_rep, dev.sel_scale, lane)
+                              : canonical_key<64>(row, q_s, pieces + 1, dev.n_rep, dev.sel_scale, lane);
+      };
       for (int e = tid; e < n_list; e += TH) {
-        const uint32_t rel = list_key[e] - lo;                         // keys below lo wrap to huge values
-        if (rel <= span) atomicAdd(&hist1[rel >> shb], 1u);
+        const uint32_t kk = list_key[e], j = list_idx[e];
+        const bool sure = kk > above, band = !sure && kk >= below;
+        if (sure) { atomicOr(&take_w[j >> 5], 1u << (j & 31u)); atomicAdd(&sh_sure, 1u); }
+        if (band) {
+          const uint32_t at = atomicAdd(&sh_cand, 1u);
+          if (at < (uint32_t)kTopkCand) cand_s[at] = j;
+        } else {
+          list_key[e] = 0u;                                // below the key of every score
+        }
       }
       __syncthreads();
-      find_bin<TH>(hist1, need, warp_tot, sh, tid);
-      const uint32_t bsel = sh[0];
-      need = sh[1];
-      in_bin = sh[2];
-      lo += bsel << shb;
-      span = min(span - (bsel << shb), (shb ? (1u << shb) : 1u) - 1u);
-      if (shb == 0 || in_bin <= (uint32_t)kTopkCand) break;
-      __syncthreads();                                                 // sh is read before the next pass writes it
+      in_bin = sh_cand;
+      need = (uint32_t)k_ch - sh_sure;
+      ranked = in_bin <= (uint32_t)kTopkCand;
+      if (ranked) {
+        for (uint32_t e = (uint32_t)warp; e < in_bin; e += NWARP) {
+          const uint32_t j = (uint32_t)cand_s[e], kk = exact_key(j);
+          if (lane == 0) cand_s[e] = ((unsigned long long)kk << 32) | (0xffffffffu - j);
+        }
+      } else {
+        for (int e = warp; e < n_list; e += NWARP) {
+          if (list_key[e] == 0u) continue;                 // (the same in all lanes)
+          const uint32_t kk = exact_key(list_idx[e]);
+          __syncwarp();
+          if (lane == 0) list_key[e] = kk;
+        }
+        __syncthreads();
+        if (tid == 0) sh_cand = 0;
+        lo = 1u; span = 0xfffffffeu;
+        narrow((uint32_t)kTopkCand, true);
+      }
     }
     ties = in_bin > (uint32_t)kTopkCand;
     // ---- 5: keys above the bin are taken; the keys of the bin become candidates (or, all equal and many, a bitmap)
-    for (int e = tid; e < n_list; e += TH) {
+    for (int e = tid; e < n_list && !ranked; e += TH) {
       const uint32_t kk = list_key[e], j = list_idx[e];
       if (kk >= lo) {
         if (kk - lo > span) atomicOr(&take_w[j >> 5], 1u << (j & 31u));
@@ -852,8 +1110,8 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
 
 // Top-k of `problems` rows of dev.pooled (sign == 0: keys; else floats compared as sign * value).
 static cudaError_t launch_topk(const GroupDev& dev, int device, int problems, int l0, int k_ch, int k_cap,
-                               const int32_t* outliers, int n_out, float sign, int32_t* sel_idx, int32_t* sel_cnt,
-                               cudaStream_t s) {
+                               const int32_t* outliers, int n_out, float sign, const __nv_bfloat16* q, int32_t* sel_idx,
+                               int32_t* sel_cnt, cudaStream_t s) {   // q: not null if the keys are score_bound_kernel's
   if (dev.n_c > kTopkThreads * 32)
     return launch_pdl(topk_kernel, dim3(problems), dim3(kTopkThreads), 0, s, dev, l0, k_ch, k_cap, outliers, n_out,
                       sign, sel_idx, sel_cnt);
@@ -872,27 +1130,32 @@ static cudaError_t launch_topk(const GroupDev& dev, int device, int problems, in
   // problems 38.6 -> 38.2); with 256 problems 2048 rows lose (9.0 -> 10.0).  From 512 to 1024 threads the barriers cost
   // more than the threads bring (65536 rows, 8 problems, budget 2048: 8.9 -> 9.7 us), unless the lists are long (4
   // problems, budget 8192: 10.5 -> 10.1) or the problems many (window of 128: 158.2 -> 157.5 us).
+  if (q && th < 512) th = 512;                     // (a thread per piece of the queries, a warp per chunk of the band)
   if (problems <= sms && (th < 512 || (th == 512 && (problems > sms / 4 || groups(1) < k_ch)))) th *= 2;
   const size_t smem = (size_t)th * items * (sizeof(uint32_t) + sizeof(uint16_t));
-#define XKV_PIVOT(GPT, ITEMS, TH)                                                                                     \
+#define XKV_PIVOT(GPT, ITEMS, TH, BOUND)                                                                              \
   do {                                                                                                                \
-    e = ensure_dyn_smem<topk_pivot_kernel<GPT, ITEMS, TH>>(smem, device);                                             \
+    e = ensure_dyn_smem<topk_pivot_kernel<GPT, ITEMS, TH, BOUND>>(smem, device);                                      \
     if (e == cudaSuccess)                                                                                             \
-      e = launch_pdl(topk_pivot_kernel<GPT, ITEMS, TH>, dim3(problems), dim3(TH), smem, s, dev, l0, k_ch, k_cap,      \
-                     outliers, n_out, sign, sel_idx, sel_cnt);                                                        \
+      e = launch_pdl(topk_pivot_kernel<GPT, ITEMS, TH, BOUND>, dim3(problems), dim3(TH), smem, s, dev, l0, k_ch, k_cap, \
+                     outliers, n_out, sign, q, sel_idx, sel_cnt);                                                     \
   } while (0)
-#define XKV_PIVOT_G(ITEMS, TH)                                                                                        \
+#define XKV_PIVOT_G(ITEMS, TH, BOUND)                                                                                 \
   do {                                                                                                                \
-    if (groups(1) >= k_ch) XKV_PIVOT(1, ITEMS, TH);                                                                   \
-    else if (groups(2) >= k_ch) XKV_PIVOT(2, ITEMS, TH);                                                              \
-    else if (groups(4) >= k_ch) XKV_PIVOT(4, ITEMS, TH);                                                              \
-    else XKV_PIVOT(0, ITEMS, TH);                                                                                     \
+    if (groups(1) >= k_ch) XKV_PIVOT(1, ITEMS, TH, BOUND);                                                            \
+    else if (groups(2) >= k_ch) XKV_PIVOT(2, ITEMS, TH, BOUND);                                                       \
+    else if (groups(4) >= k_ch) XKV_PIVOT(4, ITEMS, TH, BOUND);                                                       \
+    else XKV_PIVOT(0, ITEMS, TH, BOUND);                                                                              \
   } while (0)
-  if (items == 32) XKV_PIVOT_G(32, 1024);
-  else if (th == 128) XKV_PIVOT_G(16, 128);
-  else if (th == 256) XKV_PIVOT_G(16, 256);
-  else if (th == 512) XKV_PIVOT_G(16, 512);
-  else XKV_PIVOT_G(16, 1024);
+  if (q) {
+    if (items == 32) XKV_PIVOT_G(32, 1024, true);
+    else if (th == 512) XKV_PIVOT_G(16, 512, true);
+    else XKV_PIVOT_G(16, 1024, true);
+  } else if (items == 32) XKV_PIVOT_G(32, 1024, false);
+  else if (th == 128) XKV_PIVOT_G(16, 128, false);
+  else if (th == 256) XKV_PIVOT_G(16, 256, false);
+  else if (th == 512) XKV_PIVOT_G(16, 512, false);
+  else XKV_PIVOT_G(16, 1024, false);
 #undef XKV_PIVOT_G
 #undef XKV_PIVOT
   return e;
@@ -908,24 +1171,42 @@ static cudaError_t launch_select_dev(const GroupDev& dev, const CUtensorMap& tma
   const int k_ch_raw = (int)(((int64_t)k + c - 1) / c);
   const int k_ch = k_ch_raw < dev.n_c ? k_ch_raw : dev.n_c;
   const int k_cap = (k_ch_raw + dev.n_out) * c;      // room for the union with the outlier chunks
-  const size_t smem = 1024 + (size_t)(dev.d_h / 64) * kScoreRows * 128 + (size_t)dev.n_rep * dev.d_h * 4;
   dim3 grid(tiles, problems);
   cudaError_t e;
+  // Tensor-core scores with a bound pay where the scan is more than a few microseconds of work: the band costs the top-k 1.5
+  // to 3 us.  Selections, canonical scan -> bound: 7 heads, 65536 rows, 128 problems 67.3 -> 46.4 us, 64 problems 37.8 -> 26.9,
+  // 16 problems 15.7 -> 12.7, 8192 rows and 128 problems 16.5 -> 14.7, 32768 rows and 16 problems 10.2 -> 10.6, 2048 rows and
+  // 128 problems 9.7 -> 12.4; 5 heads, 16384 rows, 64 problems 14.4 -> 14.0, 32768 rows and 16 problems 9.3 -> 10.4; 16 heads,
+  // 131072 rows, 64 problems 135.8 -> 47.3, 32768 rows and 16 problems 14.9 -> 11.6, 16384 rows and 16 problems 11.9 -> 12.0.
+  // Without a handle there is no room for the tiles' largest elements.
+  const bool bound = dev.tile_max != nullptr && dev.n_rep > 4 && k_ch < dev.n_c && dev.n_c <= kTopkThreads * 32 &&
+                     (int64_t)problems * dev.n_c * dev.n_rep >= 5 << 17;
+  const size_t smem = 1024 + (size_t)(dev.d_h / 64) * kScoreRows * 128 + (bound ? 0 : (size_t)dev.n_rep * dev.d_h * 4);
+#define XKV_SCAN_BOUND(DH, NT)                                                                          \
+  do {                                                                                                  \
+    e = ensure_dyn_smem<score_bound_kernel<DH, NT>>(smem, device);                                      \
+    if (e != cudaSuccess) return e;                                                                     \
+    e = launch_pdl(score_bound_kernel<DH, NT>, grid, dim3(kScoreThreads), smem, s, tmap, dev, q, l0);   \
+  } while (0)
 #define XKV_SCAN(DH, HMAX)                                                                              \
   do {                                                                                                  \
     e = ensure_dyn_smem<score_pool_kernel<DH, HMAX>>(smem, device);                                     \
     if (e != cudaSuccess) return e;                                                                     \
     e = launch_pdl(score_pool_kernel<DH, HMAX>, grid, dim3(kScoreThreads), smem, s, tmap, dev, q, l0); \
   } while (0)
-  if (dev.d_h == 128) {
+  if (bound) {
+    if (dev.d_h == 128) { if (dev.n_rep <= 8) XKV_SCAN_BOUND(128, 1); else XKV_SCAN_BOUND(128, 2); }
+    else { if (dev.n_rep <= 8) XKV_SCAN_BOUND(64, 1); else XKV_SCAN_BOUND(64, 2); }
+  } else if (dev.d_h == 128) {
     if (dev.n_rep <= 4) XKV_SCAN(128, 4); else XKV_SCAN(128, 8);
   } else {
     if (dev.n_rep <= 4) XKV_SCAN(64, 4); else XKV_SCAN(64, 8);
   }
 #undef XKV_SCAN
+#undef XKV_SCAN_BOUND
   count_launch(kFamScan);
   if (e != cudaSuccess) return e;
-  e = launch_topk(dev, device, problems, l0, k_ch, k_cap, dev.outliers, dev.n_out, 0.0f, sel_idx, sel_cnt, s);
+  e = launch_topk(dev, device, problems, l0, k_ch, k_cap, dev.outliers, dev.n_out, 0.0f, bound ? q : nullptr, sel_idx, sel_cnt, s);
   count_launch(kFamTopk);
   return e;
 }
@@ -943,7 +1224,7 @@ cudaError_t launch_topk_rows(const float* scores, int problems, int n, int k, fl
   dev.G = 1; dev.batch = problems; dev.H_kv = 1; dev.T = n; dev.c = 1; dev.n_c = n;
   dev.pooled = const_cast<float*>(scores);
   const int k_ch = k < n ? k : n;
-  cudaError_t e = launch_topk(dev, device, problems, 0, k_ch, k, nullptr, 0, sign, out, nullptr, s);
+  cudaError_t e = launch_topk(dev, device, problems, 0, k_ch, k, nullptr, 0, sign, nullptr, out, nullptr, s);
   count_launch(kFamTopk);
   return e;
 }
