@@ -9,7 +9,7 @@
 //                               iteration, three for the last iterate, which has to be orthonormal)
 //   Rayleigh-Ritz:        W^T = Z^T X^T,  M = W^T W (= Z^T X^T X Z, l x l),  M = P Lambda P^T (Jacobi); Z and W as sums of
 //                         two bf16 matrices here
-//   V = Z P_r (N x r);    B_l = rows of V^T (bf16);   A = X V_bf16 (T x r, tensor core);   sigma = sqrt(Lambda).
+//   V = Z P_r (N x r);    B_l = rows of V^T (bf16);   A = X V = W P_r (T x r, tensor core);   sigma = sqrt(Lambda).
 // A = U Sigma and B = V^T of the truncated SVD of X, up to the accuracy of the subspace (checked against the exact
 // optimum sum_{i>r} sigma_i^2, never factor by factor: signs and degenerate subspaces are not unique).
 //
@@ -17,7 +17,8 @@
 // along k) or MN-major (its rows run along m or n), which the shared-memory descriptors cover, so no matrix is ever
 // transposed in memory:
 //   Y = X Z (X K-major, Z MN-major), stored transposed as Y^T;    U = X^T Y (X MN-major, Y^T K-major);
-//   M = W^T W (W^T K-major twice);                                 A = X V (X K-major, V MN-major).
+//   M = W^T W (W^T K-major twice);                                 A = W P (W^T MN-major, P^T K-major) or
+//                                                                  A = X V (X K-major, V MN-major).
 #include <cuda.h>
 #include <math.h>
 
@@ -55,13 +56,14 @@ __device__ __forceinline__ bool gemm_wait(uint32_t bar, uint32_t parity) {
 // CTA per tile, 421 now; with two parts of B and of the result 930 -> 855.
 // TRANS: store C^T (out[n][m]).
 // AK: A is given as [m][k] (K-major), else as [k][m]; BK likewise for B.  K range z covers k_per columns and writes
-// Cf + z * M * ldc.  With two parts B is the sum of the matrices of map_b and map_b2 and A is gone through twice; the k
-// of a part are rounded up to whole blocks of 64.  Cb is the result rounded to bf16; LO: Cl is twice what the rounding leaves
+// Cf + z * M * ldc.  With two parts B is the sum of the matrices of map_b and map_b2 and A is gone through twice, a third
+// adds the product of those of map_a3 and map_b3; the k of a part are rounded up to whole blocks of 64.  Cb is the result rounded to bf16; LO: Cl is twice what the rounding leaves
 // out (TRANS only; a template parameter, because a test of the pointer in the epilogue costs every product 11 %).  Out-of-range rows and columns of the operands are zero-filled by the copy engine; stores are guarded.
 template <bool TRANS, bool AK, bool BK, bool LO, int MB, int BN>
 __global__ void __launch_bounds__(gemm_threads<MB>(), 1)
 clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                const __grid_constant__ CUtensorMap map_b2, int M, int N, int k_part, int k_all, int k_per, float* __restrict__ Cf,
+                const __grid_constant__ CUtensorMap map_b2, const __grid_constant__ CUtensorMap map_a3,
+                const __grid_constant__ CUtensorMap map_b3, int M, int N, int k_part, int k_all, int k_per, float* __restrict__ Cf,
                 __nv_bfloat16* __restrict__ Cb, __nv_bfloat16* __restrict__ Cl, long long ldc, dim3 tiles, unsigned int* __restrict__ flags) {
   extern __shared__ uint8_t gemm_smem[];
   constexpr int kGemmStages = gemm_stages<MB, BN>(), kGemmStageBytes = gemm_stage_bytes<MB, BN>();
@@ -112,15 +114,15 @@ clf_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           const uint32_t st = base + (uint32_t)s * kGemmStageBytes;
           mbar_expect_tx(FULL(s), kGemmStageBytes);
           const int kt = c.k_first + kb * 64;
-          const bool second = kt >= k_part;
-          const int k = second ? kt - k_part : kt;
-          const CUtensorMap* mb = second ? &map_b2 : &map_b;
+          const int part = kt >= k_part ? kt >= 2 * k_part ? 2 : 1 : 0;
+          const int k = kt - part * k_part;
+          const CUtensorMap *ma = part == 2 ? &map_a3 : &map_a, *mb = part == 2 ? &map_b3 : part == 1 ? &map_b2 : &map_b;
           // K-major: one box of 64 k by all rows; MN-major: slabs of 64 columns by 64 k, 8 KB each
           if (AK) {
-            tma_load_2d(st, &map_a, k, c.m0, FULL(s));
+            tma_load_2d(st, ma, k, c.m0, FULL(s));
           } else {
 #pragma unroll
-            for (int i = 0; i < 2 * MB; ++i) tma_load_2d(st + i * 8192, &map_a, c.m0 + i * 64, k, FULL(s));
+            for (int i = 0; i < 2 * MB; ++i) tma_load_2d(st + i * 8192, ma, c.m0 + i * 64, k, FULL(s));
           }
           if (BK) {
             tma_load_2d(st + kOffB, mb, k, c.n0, FULL(s));
@@ -1133,11 +1135,12 @@ jacobi_block_kernel(float* __restrict__ M0, float* __restrict__ M1, float* __res
 }
 
 // The r largest eigenvalues (ties to the lower index) and their eigenvectors as the rows of Ps (r x l); sigma =
-// sqrt(lambda).  One warp per eigenvalue.
+// sqrt(lambda).  One warp per eigenvalue.  Pb, if wanted: the rows again as bf16, what that rounding leaves out, and half of
+// the first.
 constexpr int kSelectWarps = 8;
 __global__ void __launch_bounds__(kSelectWarps * 32)
 eig_select_kernel(const float* __restrict__ M, const float* __restrict__ Pt, int l, int r, float* __restrict__ Ps,
-                  float* __restrict__ sigma) {
+                  __nv_bfloat16* __restrict__ Pb, float* __restrict__ sigma) {
   const int lane = threadIdx.x & 31, i = blockIdx.x * kSelectWarps + (threadIdx.x >> 5);
   if (i >= l) return;
   const float li = M[(size_t)i * l + i];
@@ -1149,10 +1152,20 @@ eig_select_kernel(const float* __restrict__ M, const float* __restrict__ Pt, int
   rk = __reduce_add_sync(0xffffffffu, rk);
   if (rk >= r) return;
   if (lane == 0 && sigma) sigma[rk] = sqrtf(fmaxf(li, 0.0f));
-  for (int j = lane; j < l; j += 32) Ps[(size_t)rk * l + j] = Pt[(size_t)i * l + j];
+  for (int j = lane; j < l; j += 32) {
+    const float v = Pt[(size_t)i * l + j];
+    const size_t at = (size_t)rk * l + j;
+    Ps[at] = v;
+    if (Pb) {
+      const __nv_bfloat16 hi = __float2bfloat16(v);
+      Pb[at] = hi;
+      Pb[(size_t)r * l + at] = __float2bfloat16(v - __bfloat162float(hi));
+      Pb[(size_t)2 * r * l + at] = __float2bfloat16(0.5f * __bfloat162float(hi));
+    }
+  }
 }
 
-// V = Z Ps^T (N x r, fp32), rounded to bf16: row-major, and as the per-layer matrices B [G][r][d], B[g][m][j] = V[g d + j][m].
+// V = Z Ps^T (N x r, fp32), rounded to bf16: row-major (if Vb is not null), and as the per-layer matrices B [G][r][d], B[g][m][j] = V[g d + j][m].
 // 64 x 64 tiles, 256 threads, 4 x 4 outputs per thread, chunks of 32 k.
 __global__ void __launch_bounds__(256)
 ritz_vectors_kernel(const float* __restrict__ Z, const float* __restrict__ Ps, int l, int r, int d, __nv_bfloat16* __restrict__ Vb,
@@ -1200,7 +1213,7 @@ ritz_vectors_kernel(const float* __restrict__ Z, const float* __restrict__ Ps, i
       const int m = m0 + tx * 4 + x;
       if (m < r) {
         const __nv_bfloat16 v = __float2bfloat16(acc[i][x]);
-        Vb[(size_t)n * r + m] = v;
+        if (Vb) Vb[(size_t)n * r + m] = v;
         B[((size_t)g * r + m) * d + j] = v;
       }
     }
@@ -1313,15 +1326,22 @@ struct GemmOut {
   __nv_bfloat16* lo = nullptr;   // transposed results only: twice what b's rounding leaves out
 };
 
+// Further parts of a product, laid out like the first: a (b + b2) + a3 b3.
+struct GemmParts {
+  const void *b2 = nullptr, *a3 = nullptr, *b3 = nullptr;
+};
+
 template <bool TRANS, bool AK, bool BK, bool LO, int MB, int BN>
-cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, const void* b2, int splits, GemmOut c, unsigned int* flags, int device,
+cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, const GemmParts& more, int splits, GemmOut c, unsigned int* flags, int device,
                            cudaStream_t s) {
   const int M = AK ? a.rows : a.cols, N = BK ? b.rows : b.cols, K = AK ? a.cols : a.rows;
-  const int k_all = gemm_k(K, b2 ? 2 : 1), k_part = b2 ? k_all / 2 : k_all;
-  CUtensorMap ma, mb, mb2;
+  const int parts = more.a3 ? 3 : more.b2 ? 2 : 1, k_all = gemm_k(K, parts), k_part = k_all / parts;
+  CUtensorMap ma, mb, mb2, ma3, mb3;
   if (!encode_bf16_map(&ma, a.p, (uint64_t)a.rows, (uint64_t)a.cols, (uint64_t)a.pitch, AK ? 128 * MB : 64) ||
       !encode_bf16_map(&mb, b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BK ? BN : 64) ||
-      !encode_bf16_map(&mb2, b2 ? b2 : b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BK ? BN : 64))
+      !encode_bf16_map(&mb2, parts > 1 ? more.b2 : b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BK ? BN : 64) ||
+      !encode_bf16_map(&ma3, parts > 2 ? more.a3 : a.p, (uint64_t)a.rows, (uint64_t)a.cols, (uint64_t)a.pitch, AK ? 128 * MB : 64) ||
+      !encode_bf16_map(&mb3, parts > 2 ? more.b3 : b.p, (uint64_t)b.rows, (uint64_t)b.cols, (uint64_t)b.pitch, BK ? BN : 64))
     return cudaErrorInvalidValue;
   const size_t smem = 1024 + (size_t)gemm_stages<MB, BN>() * gemm_stage_bytes<MB, BN>();
   cudaError_t e = ensure_dyn_smem<clf_gemm_kernel<TRANS, AK, BK, LO, MB, BN>>(smem, device);
@@ -1332,7 +1352,7 @@ cudaError_t launch_gemm_bn(GemmOperand a, GemmOperand b, const void* b2, int spl
   if ((e = device_sms(device, &sms)) != cudaSuccess) return e;
   const long long n_tiles = (long long)tiles.x * tiles.y * tiles.z;
   const unsigned grid = (unsigned)(n_tiles < sms ? n_tiles : sms);        // one CTA per SM (shared and tensor memory)
-  clf_gemm_kernel<TRANS, AK, BK, LO, MB, BN><<<grid, gemm_threads<MB>(), smem, s>>>(ma, mb, mb2, M, N, k_part, k_all, k_per, c.f, c.b, c.lo, c.ld, tiles,
+  clf_gemm_kernel<TRANS, AK, BK, LO, MB, BN><<<grid, gemm_threads<MB>(), smem, s>>>(ma, mb, mb2, ma3, mb3, M, N, k_part, k_all, k_per, c.f, c.b, c.lo, c.ld, tiles,
                                                                                flags);
   count_launch(kFamClf);
   return cudaGetLastError();
@@ -1351,16 +1371,16 @@ int gemm_mb(int M) { return ((M + 255) & ~255) * 8LL <= ((M + 127) & ~127) * 9LL
 
 template <bool TRANS, bool AK, bool BK, bool LO = false>
 cudaError_t launch_gemm(GemmOperand a, GemmOperand b, int splits, GemmOut c, unsigned int* flags, int device, cudaStream_t s,
-                        const void* b2 = nullptr) {      // b2: the second part of B, laid out like b
+                        GemmParts more = {}) {
   const int bn = gemm_bn(BK ? b.rows : b.cols);
   if (gemm_mb(AK ? a.rows : a.cols) == 2) {
-    if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, LO, 2, 256>(a, b, b2, splits, c, flags, device, s);
-    if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, LO, 2, 192>(a, b, b2, splits, c, flags, device, s);
-    return launch_gemm_bn<TRANS, AK, BK, LO, 2, 128>(a, b, b2, splits, c, flags, device, s);
+    if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, LO, 2, 256>(a, b, more, splits, c, flags, device, s);
+    if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, LO, 2, 192>(a, b, more, splits, c, flags, device, s);
+    return launch_gemm_bn<TRANS, AK, BK, LO, 2, 128>(a, b, more, splits, c, flags, device, s);
   }
-  if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, LO, 1, 256>(a, b, b2, splits, c, flags, device, s);
-  if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, LO, 1, 192>(a, b, b2, splits, c, flags, device, s);
-  return launch_gemm_bn<TRANS, AK, BK, LO, 1, 128>(a, b, b2, splits, c, flags, device, s);
+  if (bn == 256) return launch_gemm_bn<TRANS, AK, BK, LO, 1, 256>(a, b, more, splits, c, flags, device, s);
+  if (bn == 192) return launch_gemm_bn<TRANS, AK, BK, LO, 1, 192>(a, b, more, splits, c, flags, device, s);
+  return launch_gemm_bn<TRANS, AK, BK, LO, 1, 128>(a, b, more, splits, c, flags, device, s);
 }
 
 // K ranges that bring a product's tiles to about one per SM, none of them empty or shorter than 1024.
@@ -1495,8 +1515,14 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
   // hold most of the weight (sigma_1 of a cache with one row a thousand times the others: off by 3.7e-4 with W rounded on
   // both sides, 1.5e-4 on one).  With W = H + L the symmetric part of H^T (H + 2 L) is M up to L^T L.
   __nv_bfloat16* Yl = (__nv_bfloat16*)(w + p.off_yl);
-  if (e == cudaSuccess) e = launch_gemm<true, true, false, true>({X, T, N, N}, {Zb, N, l, l}, 1, {nullptr, Yt, p.Tp, Yl}, flags, device, s, Zb + (size_t)N * l);
-  if (e == cudaSuccess) e = launch_gemm<false, true, true>({Yt, l, T, p.Tp}, {Yt, l, T, p.Tp}, p.ritz_split, {(float*)part, nullptr, l}, flags, device, s, Yl);
+  // A = X V = W P from the W that is there already, H (P1 + P2) + (2 L) (P1 / 2) with P = P1 + P2 in bf16 too (they take the
+  // place of V_bf16 in the workspace): 3 l instead of N terms a sum, and without the rounding of V in them (what P1 + P2
+  // leaves out is 2^-17).  131072 x 4096, r = 512, the call and the reconstruction behind it 7554 -> 7338 us.  Residual over
+  // the optimum of that rank, 2048 to 20000 rows, five shapes: 1.0299-1.0456 -> 1.0293-1.0432; with an outlier row or column
+  // 1.17-7.7 -> 1.16-7.1.  Where 3 l is not less than N the product with V_bf16 is the shorter one.
+  const bool from_w = 3 * l < N;
+  if (e == cudaSuccess) e = launch_gemm<true, true, false, true>({X, T, N, N}, {Zb, N, l, l}, 1, {nullptr, Yt, p.Tp, Yl}, flags, device, s, {Zb + (size_t)N * l});
+  if (e == cudaSuccess) e = launch_gemm<false, true, true>({Yt, l, T, p.Tp}, {Yt, l, T, p.Tp}, p.ritz_split, {(float*)part, nullptr, l}, flags, device, s, {Yl});
   if (e == cudaSuccess) {
     symmetrize_kernel<<<(l * l + 255) / 256, 256, 0, s>>>((const float*)part, p.ritz_split, Mm, l);
     float* M2 = (float*)(w + p.off_m2);
@@ -1508,13 +1534,17 @@ int clf_factorize(const xkv_clf_config* c, const void* X, const void* omega, voi
     e = launch_cooperative<jacobi_block_kernel>(sms, kJacobiThreads, kJacobiSmem, args, device, s);
   }
   if (e == cudaSuccess) {
-    eig_select_kernel<<<(l + kSelectWarps - 1) / kSelectWarps, kSelectWarps * 32, 0, s>>>(Mm, Pm, l, r, Ps, sigma);
-    ritz_vectors_kernel<<<dim3((r + 63) / 64, N / 64), 256, 0, s>>>(Z, Ps, l, r, c->d, Vb, (__nv_bfloat16*)B_out);
+    eig_select_kernel<<<(l + kSelectWarps - 1) / kSelectWarps, kSelectWarps * 32, 0, s>>>(Mm, Pm, l, r, Ps, from_w ? Vb : nullptr, sigma);
+    ritz_vectors_kernel<<<dim3((r + 63) / 64, N / 64), 256, 0, s>>>(Z, Ps, l, r, c->d, from_w ? nullptr : Vb, (__nv_bfloat16*)B_out);
     count_launch(kFamClf, 3);
     e = cudaGetLastError();
   }
-  // A = X V_bf16, stored [T][r]
-  if (e == cudaSuccess) e = launch_gemm<false, true, false>({X, T, N, N}, {Vb, N, r, r}, 1, {nullptr, (__nv_bfloat16*)A_out, r}, flags, device, s);
+  // A = X V, stored [T][r]
+  if (e == cudaSuccess && from_w)
+    e = launch_gemm<false, false, true>({Yt, l, T, p.Tp}, {Vb, r, l, l}, 1, {nullptr, (__nv_bfloat16*)A_out, r}, flags, device, s,
+                                        {Vb + (size_t)r * l, Yl, Vb + (size_t)2 * r * l});
+  else if (e == cudaSuccess)
+    e = launch_gemm<false, true, false>({X, T, N, N}, {Vb, N, r, r}, 1, {nullptr, (__nv_bfloat16*)A_out, r}, flags, device, s);
   if (e != cudaSuccess) { set_cuda_error(e); (void)cudaGetLastError(); return XKV_ERR_CUDA; }
   return XKV_OK;
 }
