@@ -214,14 +214,14 @@ int xkv_group_create(const xkv_group_config* cfg, void* stream, xkv_group** out)
       dst = (type)p;                                       \
       g->workspace_bytes += (bytes);                       \
     } while (0)
-    __nv_bfloat16 *Bt_k, *Bt_v, *Bv_copy; float2 *rhi, *rlo;
+    __nv_bfloat16 *Bt_k, *Bt_v, *Bv_copy; float4 *rhi, *rlo;
     XKV_ALLOC(Bt_k, __nv_bfloat16*, btk);
     XKV_ALLOC(Bt_v, __nv_bfloat16*, btv);
     XKV_ALLOC(Bv_copy, __nv_bfloat16*, (size_t)c.batch * c.G * c.r_v * c.H_kv * c.d_h * sizeof(__nv_bfloat16));
     XKV_ALLOC(d.pooled, float*, pooled);
     if (tiles) XKV_ALLOC(d.tile_max, uint32_t*, tiles);
-    XKV_ALLOC(rhi, float2*, hi);
-    XKV_ALLOC(rlo, float2*, lo);
+    XKV_ALLOC(rhi, float4*, hi);
+    XKV_ALLOC(rlo, float4*, lo);
     XKV_ALLOC(d.part, float*, part);
     XKV_ALLOC(d.flags, unsigned int*, 256);
 #undef XKV_ALLOC

@@ -46,7 +46,6 @@ constexpr int kSlabBytes = kTile * 128;          // 128 rows x 64 bf16 (one 128-
 constexpr int prod_warps(int quant) { return quant ? 8 : 4; }
 constexpr int fused_threads(int quant) { return (11 + prod_warps(quant)) * 32; }
 constexpr int kSmemLimit = 227 * 1024;
-constexpr int kRopeStride = 66;                  // float2 per staged rotary row (64 + pad against bank conflicts)
 constexpr int kPBytes = 2 * 16 * 128;            // softmax weights of a tile as a bf16 MMA operand: [2][16 heads][64 rows]
 constexpr int kMaxBlocks = 8;                    // 128-column blocks of r_v that fit the TMEM accumulators
 constexpr unsigned long long kWaitLimitNs = 250000000ull;    // a wait that lasts a quarter of a second has failed
@@ -143,127 +142,181 @@ __device__ __forceinline__ bool wait_bar(const Ctx& c, uint32_t bar, uint32_t pa
   return r;
 }
 
-// Logits of one rebuilt key row against NR query heads: rotate the (i, i+HALF) pairs, accumulate q . k.
-// hi/lo point at this row's coarse/fine rotary entries (cos, sin), in shared (SMEM) or global memory.
-template <int DH, int NR, bool ROPE, bool SMEM>
-__device__ __forceinline__ void key_logits(uint32_t acc, const float2* __restrict__ hi, const float2* __restrict__ lo,
-                                           const float* __restrict__ q_s, float (&z)[NR]) {
-  constexpr int HALF = DH / 2;
-  u64 z2[NR == 8 ? NR : 1];
+// The queries in shared memory, fp32: [head][d_h / 4] units of 16 bytes, unit u = dimensions {2u, 2u + 1, d_h/2 + 2u,
+// d_h/2 + 2u + 1}, which is what two rotary pairs (i, i + d_h/2) are multiplied with.
+
+__device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// Logits of the 32 rebuilt key rows of a warp against NR query heads (rounded up to eights): rotate the (i, i + HALF)
+// pairs, then mma.sync.  One warp per scheduler issues a multiply-add every two cycles at best, so what bounds this is
+// their number: 8 a pair for the angles and the rotation, and 2 for every head if the heads are multiplied one by one.
+// Four lanes share a row: lane 4g + t reads rows g, g + 8, g + 16, g + 24 and of every eight dimensions 2t and 2t + 1 (the
+// 16x256b form of tcgen05.ld), two dimensions side by side are the operands of one packed instruction, and the rotated
+// values are where an operand of m16n8k8 wants them.  The queries are bf16 and thus exact as tf32; a key element goes in as
+// two parts, its upper 11 bits and the rest, of which the tensor core drops less than 2^-21 of the element, the size of
+// the rounding errors of the rotation; the products are exact and a sum takes 32 steps instead of 128.  (Against fp64 on the
+// same bases, thirteen shapes: outputs 1.72e-3 to 2.10e-3 rms and log-sums 6.7e-5 to 1.5e-4, the same to three digits as with
+// fp32 multiply-adds throughout: the weights' and outputs' rounding to bf16.)
+// Against a row per lane, every head a chain of multiply-adds: seven heads, eight sequences of 65536 rows 129.4 -> 123.3 us a
+// step, 4-bit bases (whose producers share the schedulers) 88.4 -> 85.9, 32768 rows by layer 114.6 -> 113.0, rank 1024 with a
+// budget of 16384 307.7 -> 304.1; four heads in the steady state are bound elsewhere (131072 rows 76.8 -> 76.8, on GPUs that
+// run at lower clocks up to 80.3 -> 77.5).  Four lanes a row with the heads as packed multiply-adds: 64 registers of sums for
+// eight heads, 157.4 where a row per lane took 151.9.
+// hi: the coarse rotary entries of the warp's four 8-row chunks, 16-byte units; lo: the fine ones of position g of a
+// chunk, units swizzled by `swz`; q_s: the queries.  On return a lane holds the logits of row g + 8t.
+template <int DH, int NR>
+__device__ __forceinline__ void quad_logits(uint32_t acc, const ulonglong2* __restrict__ hi, const ulonglong2* __restrict__ lo,
+                                            int swz, const uint4* __restrict__ q_s, int lane, float (&z)[NR]) {
+  constexpr int HALF = DH / 2, UN = HALF / 2;            // units of a rotary row, of a head
+  constexpr int NT = (NR + 7) / 8;                       // groups of eight heads
+  constexpr unsigned long long kNeg2 = 0x8000000080000000ull;
+  const int t = lane & 3, g = lane >> 2;
+  float c[NT][2][4];                                     // [.][rows g, g + 8 | g + 16, g + 24][heads 2t, 2t + 1 of either]
 #pragma unroll
-  for (int h = 0; h < (NR == 8 ? NR : 1); ++h) z2[h] = 0ull;
-  // 4 rotary pairs per pass: the loop body has to stay small, the four warps of a scheduler run four different
-  // loops and share its instruction cache (32 pairs per pass: 77 us per call, 8: 73 us, 4: 71 us)
+  for (int n = 0; n < NT; ++n)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) c[n][i >> 2][i & 3] = 0.0f;
 #pragma unroll 1
-  for (int pass = 0; pass < HALF / 4; ++pass) {
-    uint32_t xa[4], xb[4];
-    tmem_ld4_nb(acc + (uint32_t)(pass * 4), xa);
-    tmem_ld4_nb(acc + (uint32_t)(HALF + pass * 4), xb);
-    tc_wait_ld_nb(xa, xb);            // the table and query loads below do not depend on it and may be issued above it
-    float x1[4], x2[4];
+  for (int jj = 0; jj < HALF / 8; ++jj) {
+    uint32_t xa[2][4], xb[2][4];                         // [16 rows][row g: 2 dimensions, row g + 8: 2]
 #pragma unroll
-    for (int e = 0; e < 4; ++e) { x1[e] = __uint_as_float(xa[e]); x2[e] = __uint_as_float(xb[e]); }
+    for (int i = 0; i < 2; ++i) {
+      const uint32_t at = acc + ((uint32_t)i << 20) + (uint32_t)(jj * 8);
+      tmem_ld_quad(at, xa[i]);
+      tmem_ld_quad(at + (uint32_t)HALF, xb[i]);
+    }
+    const int u = jj * 4 + t;
+    const ulonglong2 f = lo[u ^ swz];                    // {cosines, sines} of two pairs
+    ulonglong2 a[4];
 #pragma unroll
-    for (int i4 = 0; i4 < 1; ++i4) {
-      float r1[4], r2[4];
-      const int ii = pass * 4 + i4 * 4;
-      if (ROPE) {
-        float2 a[4], c2[4];
-        if (SMEM) {
-          const float4 a01 = *reinterpret_cast<const float4*>(hi + ii), a23 = *reinterpret_cast<const float4*>(hi + ii + 2);
-          const float4 c01 = *reinterpret_cast<const float4*>(lo + ii), c23 = *reinterpret_cast<const float4*>(lo + ii + 2);
-          a[0] = make_float2(a01.x, a01.y); a[1] = make_float2(a01.z, a01.w);
-          a[2] = make_float2(a23.x, a23.y); a[3] = make_float2(a23.z, a23.w);
-          c2[0] = make_float2(c01.x, c01.y); c2[1] = make_float2(c01.z, c01.w);
-          c2[2] = make_float2(c23.x, c23.y); c2[3] = make_float2(c23.z, c23.w);
-        } else {
+    for (int r = 0; r < 4; ++r) a[r] = hi[r * UN + u];
+    uint4 qv[NT];                                        // head 8 n + g (heads beyond NR: whatever, their columns are not read)
 #pragma unroll
-          for (int e = 0; e < 4; ++e) { a[e] = __ldg(hi + ii + e); c2[e] = __ldg(lo + ii + e); }
-        }
+    for (int n = 0; n < NT; ++n) qv[n] = q_s[(8 * n + (NR < 8 ? g & (NR - 1) : g)) * UN + u];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) tc_wait_ld_nb(xa[i], xb[i]);
+    const u64 fn = f.y ^ kNeg2;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      uint32_t h1[4], h2[4], l1[4], l2[4];               // [row g: 2 dimensions, row g + 8: 2], either half; upper and lower parts
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const ulonglong2 ar = a[2 * i + k];
+        const u64 cs = fma2(ar.y, fn, mul2(ar.x, f.x));              // cos(x + y)
+        const u64 sn = fma2(ar.x, f.y, mul2(ar.y, f.x));             // sin(x + y)
+        const u64 x1 = pack2u(xa[i][2 * k], xa[i][2 * k + 1]), x2 = pack2u(xb[i][2 * k], xb[i][2 * k + 1]);
+        const float2 r1 = unpack2(fma2(x2, sn ^ kNeg2, mul2(x1, cs))), r2 = unpack2(fma2(x1, sn, mul2(x2, cs)));
+        const float v[4] = {r1.x, r1.y, r2.x, r2.y};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float cs = a[e].x * c2[e].x - a[e].y * c2[e].y;      // cos(x + y)
-          const float sn = a[e].y * c2[e].x + a[e].x * c2[e].y;      // sin(x + y)
-          const float u = x1[i4 * 4 + e], v = x2[i4 * 4 + e];
-          r1[e] = u * cs - v * sn;
-          r2[e] = v * cs + u * sn;
+          const uint32_t up = __float_as_uint(v[e]) & 0xffffe000u, rest = __float_as_uint(v[e] - __uint_as_float(up));
+          if (e < 2) { h1[2 * k + e] = up; l1[2 * k + e] = rest; } else { h2[2 * k + e - 2] = up; l2[2 * k + e - 2] = rest; }
         }
-      } else {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) { r1[e] = x1[i4 * 4 + e]; r2[e] = x2[i4 * 4 + e]; }
       }
-      if constexpr (NR == 8) {
-        // two dimensions per instruction, the even and the odd ones in sums of their own: half the instructions, and chains
-        // of four multiply-adds a pass instead of eight (seven heads, eight sequences of 65536 rows: 153.3 -> 151.7 us; with
-        // four heads no change: 79.5 and 79.3 at 131072 rows, 166.3 and 166.9 by layer with a tail)
-        const u64 r1a = pack2(r1[0], r1[1]), r1b = pack2(r1[2], r1[3]), r2a = pack2(r2[0], r2[1]), r2b = pack2(r2[2], r2[3]);
 #pragma unroll
-        for (int h0 = 0; h0 < NR; h0 += 4) {
-          ulonglong2 qa[4], qb[4];
-#pragma unroll
-          for (int h = 0; h < 4; ++h) {
-            qa[h] = *reinterpret_cast<const ulonglong2*>(q_s + (h0 + h) * DH + ii);
-            qb[h] = *reinterpret_cast<const ulonglong2*>(q_s + (h0 + h) * DH + HALF + ii);
-          }
-#pragma unroll
-          for (int h = 0; h < 4; ++h) z2[h0 + h] = fma2(qa[h].x, r1a, z2[h0 + h]);
-#pragma unroll
-          for (int h = 0; h < 4; ++h) z2[h0 + h] = fma2(qb[h].x, r2a, z2[h0 + h]);
-#pragma unroll
-          for (int h = 0; h < 4; ++h) z2[h0 + h] = fma2(qa[h].y, r1b, z2[h0 + h]);
-#pragma unroll
-          for (int h = 0; h < 4; ++h) z2[h0 + h] = fma2(qb[h].y, r2b, z2[h0 + h]);
-        }
-        continue;
-      }
-      // heads in groups of four, element by element inside a group: the four multiply-adds of an element are
-      // independent (one head after the other is a chain of eight dependent ones)
-#pragma unroll
-      for (int h0 = 0; h0 < NR; h0 += 4) {
-        float4 qa[4], qb[4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          qa[h] = *reinterpret_cast<const float4*>(q_s + (h0 + h) * DH + ii);
-          qb[h] = *reinterpret_cast<const float4*>(q_s + (h0 + h) * DH + HALF + ii);
-        }
-#pragma unroll
-        for (int h = 0; h < 4; ++h) z[h0 + h] = fmaf(qa[h].x, r1[0], z[h0 + h]);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) z[h0 + h] = fmaf(qb[h].x, r2[0], z[h0 + h]);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) z[h0 + h] = fmaf(qa[h].y, r1[1], z[h0 + h]);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) z[h0 + h] = fmaf(qb[h].y, r2[1], z[h0 + h]);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) z[h0 + h] = fmaf(qa[h].z, r1[2], z[h0 + h]);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) z[h0 + h] = fmaf(qb[h].z, r2[2], z[h0 + h]);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) z[h0 + h] = fmaf(qa[h].w, r1[3], z[h0 + h]);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) z[h0 + h] = fmaf(qb[h].w, r2[3], z[h0 + h]);
+      for (int n = 0; n < NT; ++n) {
+        mma_tf32(c[n][i], l1[0], l1[2], l1[1], l1[3], qv[n].x, qv[n].y);
+        mma_tf32(c[n][i], l2[0], l2[2], l2[1], l2[3], qv[n].z, qv[n].w);
+        mma_tf32(c[n][i], h1[0], h1[2], h1[1], h1[3], qv[n].x, qv[n].y);
+        mma_tf32(c[n][i], h2[0], h2[2], h2[1], h2[3], qv[n].z, qv[n].w);
       }
     }
   }
-  if constexpr (NR == 8) {
+  // transpose among the four lanes of a row: from heads 2t, 2t + 1 of four rows to all heads of row g + 8t
+  const bool up1 = (t & 1) != 0, up2 = (t & 2) != 0;
 #pragma unroll
-    for (int h = 0; h < NR; ++h) { const float2 t = unpack2(z2[h]); z[h] = t.x + t.y; }
+  for (int n = 0; n < NT; ++n) {
+    float w[2][2][2];                                    // [heads 2 (t & 1), + 1 | those and 4][row][head of the pair]
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const float low = c[n][0][2 * k + x], high = c[n][1][2 * k + x];         // rows k, k + 2
+        const float mine = up2 ? high : low, got = __shfl_xor_sync(0xffffffffu, up2 ? low : high, 2);
+        w[0][k][x] = up2 ? got : mine;
+        w[1][k][x] = up2 ? mine : got;
+      }
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        if (8 * n + 4 * p >= NR) continue;
+        const float mine = up1 ? w[p][1][x] : w[p][0][x], got = __shfl_xor_sync(0xffffffffu, up1 ? w[p][0][x] : w[p][1][x], 1);
+        z[8 * n + 4 * p + x] = up1 ? got : mine;
+        z[8 * n + 4 * p + 2 + x] = up1 ? mine : got;
+      }
   }
 }
 
-// The variants that ordinary tiles do not take (no RoPE; a tile whose 8-row groups are not whole landmark chunks, or
-// a rotary table that is not staged) are kept out of line: the key epilogue's loop has to stay small.
+// The same for the variants that ordinary tiles do not take (no RoPE; a tile whose 8-row groups are not whole landmark
+// chunks, or a rotary table that is not staged), a thread per row, the tables in global memory; out of line, because the
+// key epilogue's loop has to stay small (the four warps of a scheduler run four different loops and share its instruction
+// cache: 32 pairs unrolled in it took 77 us a call, 8 pairs 73, 4 pairs 71).  On return a lane holds the logits of the row
+// of its own TMEM lane.
 template <int NR>
 struct LogitsOut { float z[NR]; };
 template <int DH, int NR, bool ROPE>
-__device__ __noinline__ LogitsOut<NR> key_logits_rare(uint32_t acc, const float2* __restrict__ hi, const float2* __restrict__ lo,
-                                                      const float* __restrict__ q_s) {
+__device__ __noinline__ LogitsOut<NR> key_logits_rare(uint32_t acc, const float4* __restrict__ hi, const float4* __restrict__ lo,
+                                                      const float4* __restrict__ q_s) {
+  constexpr int HALF = DH / 2;
   LogitsOut<NR> o;
 #pragma unroll
   for (int h = 0; h < NR; ++h) o.z[h] = 0.0f;
-  key_logits<DH, NR, ROPE, false>(acc, hi, lo, q_s, o.z);
+#pragma unroll 1
+  for (int u = 0; u < HALF / 2; u += 2) {                // four rotary pairs per pass
+    uint32_t xa[4], xb[4];
+    tmem_ld4_nb(acc + (uint32_t)(2 * u), xa);
+    tmem_ld4_nb(acc + (uint32_t)(HALF + 2 * u), xb);
+    tc_wait_ld_nb(xa, xb);
+    float r1[4], r2[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { r1[e] = __uint_as_float(xa[e]); r2[e] = __uint_as_float(xb[e]); }
+    if (ROPE) {
+      const float4 a0 = __ldg(hi + u), a1 = __ldg(hi + u + 1), c0 = __ldg(lo + u), c1 = __ldg(lo + u + 1);
+      const float ac[4] = {a0.x, a0.y, a1.x, a1.y}, as[4] = {a0.z, a0.w, a1.z, a1.w};
+      const float cc[4] = {c0.x, c0.y, c1.x, c1.y}, cn[4] = {c0.z, c0.w, c1.z, c1.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float cs = ac[e] * cc[e] - as[e] * cn[e];              // cos(x + y)
+        const float sn = as[e] * cc[e] + ac[e] * cn[e];              // sin(x + y)
+        const float x1 = r1[e], x2 = r2[e];
+        r1[e] = x1 * cs - x2 * sn;
+        r2[e] = x2 * cs + x1 * sn;
+      }
+    }
+    // heads in groups of four, element by element inside a group: the four multiply-adds of an element are
+    // independent (one head after the other is a chain of eight dependent ones)
+#pragma unroll
+    for (int h0 = 0; h0 < NR; h0 += 4) {
+      float4 q0[4], q1[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) { q0[h] = q_s[(h0 + h) * (DH / 4) + u]; q1[h] = q_s[(h0 + h) * (DH / 4) + u + 1]; }
+#pragma unroll
+      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q0[h].x, r1[0], o.z[h0 + h]);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q0[h].z, r2[0], o.z[h0 + h]);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q0[h].y, r1[1], o.z[h0 + h]);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q0[h].w, r2[1], o.z[h0 + h]);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q1[h].x, r1[2], o.z[h0 + h]);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q1[h].z, r2[2], o.z[h0 + h]);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q1[h].y, r1[3], o.z[h0 + h]);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q1[h].w, r2[3], o.z[h0 + h]);
+    }
+  }
   return o;
 }
+
+// Rotary rows are multiples of 128 bytes: odd fine rows swap the halves of every 128 bytes, so that the eight lanes of a
+// quarter warp, two rows of 64 bytes each, hit all banks once.
+__host__ __device__ constexpr int lo_swz(int row) { return (row & 1) << 2; }
 
 // Slots of the ring of gathered key rows, of the ring of the B_k slabs that go with them (slab pair by slab pair).
 constexpr int kKeySlots = 4;
@@ -273,7 +326,7 @@ static_assert(sizeof(Walk) <= kWalkInts * sizeof(int), "walk");
 // Shared memory besides the rings: weights, rotary rows, queries, positions, barriers.
 template <int DH, int NR>
 __host__ __device__ constexpr int misc_smem_bytes() {
-  return (int)(2 * kPBytes + sizeof(float2) * (2 * 16 + 8) * kRopeStride + sizeof(float) * (NR * DH + 2 * NR + 8 * NR) +
+  return (int)(2 * kPBytes + sizeof(float2) * (2 * 16 + 8) * (DH / 2) + sizeof(float) * (NR * DH + 2 * NR + 8 * NR) +
                sizeof(int) * (4 * kTile + 8 + kWalkInts) + 8 * kBarWords + 16);
 }
 // Slots of the ring of gathered value rows: whatever fits beside those two, at most as many.
@@ -306,9 +359,10 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
   // carve-up after the rings
   uint8_t* P_gen = gen + (size_t)(S + SK) * kSlabBytes;                          // [2][kPBytes] bf16 weights (MMA operand)
   const uint32_t P_addr = base + (uint32_t)(S + SK) * kSlabBytes;
-  float2* hi_s = reinterpret_cast<float2*>(P_gen + 2 * kPBytes);                 // [2][16][kRopeStride] coarse rotary rows
-  float2* lo_s = hi_s + 2 * 16 * kRopeStride;                                    // [8][kRopeStride]     fine rotary rows
-  float* q_s = reinterpret_cast<float*>(lo_s + 8 * kRopeStride);                 // [NR][DH]
+  constexpr int UN = HALF / 2;                                                   // 16-byte units {cos, cos, sin, sin} of a rotary row
+  float4* hi_s = reinterpret_cast<float4*>(P_gen + 2 * kPBytes);                 // [2][16][UN] coarse rotary rows
+  float4* lo_s = hi_s + 2 * 16 * UN;                                             // [8][UN]     fine rotary rows, unit u of row i at u ^ lo_swz(i)
+  float* q_s = reinterpret_cast<float*>(lo_s + 8 * UN);                          // [NR][DH], see quad_logits
   float* alpha_s = q_s + NR * DH;                                                // [2][NR]
   float* red_s = alpha_s + 2 * NR;                                               // [2][4][NR]
   int* pos_s = reinterpret_cast<int*>(red_s + 2 * 4 * NR);                       // [4][128]
@@ -360,7 +414,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     fence_mbar_init();
   }
   if (rope_smem) {
-    for (int i = tid; i < 8 * HALF; i += kThreads) lo_s[(i / HALF) * kRopeStride + (i % HALF)] = dev.rope_lo[i];
+    for (int i = tid; i < 8 * UN; i += kThreads) lo_s[(i / UN) * UN + ((i % UN) ^ lo_swz(i / UN))] = dev.rope_lo[i];
   }
   // weights of heads that do not exist stay zero for the whole kernel
   for (int i = tid; i < 2 * kPBytes / 4; i += kThreads) reinterpret_cast<uint32_t*>(P_gen)[i] = 0u;
@@ -604,7 +658,7 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
 #pragma unroll
         for (int i = 0; i < PP; ++i) pos_s[pb * kTile + ts + SPT * i] = pq[i];
         if (rope_smem) {
-          // rows 8a..8a+7 of the tile usually share one coarse rotary row (a landmark chunk): stage it once.
+          // rows 8a..8a+7 of the tile are usually the eight positions of one coarse rotary row (a landmark chunk): stage it once.
           // Warp pw handles the 32-row blocks pw, pw + PW / 2, ... (lane = row inside the block).
 #pragma unroll
           for (int hb = 0; hb < PP; ++hb) {
@@ -614,15 +668,15 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
             gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, 1));
             gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, 2));
             gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, 4));
-            const bool aligned = __all_sync(0xffffffffu, p < 0 || hidx == gmax);
+            const bool aligned = __all_sync(0xffffffffu, p < 0 || (hidx == gmax && (p & 7) == (lane & 7)));
             if (lane == 0) algn_s[buf * 4 + blk] = aligned ? 1 : 0;
             if (aligned) {
 #pragma unroll
               for (int a = 0; a < 4; ++a) {
                 const int gm = __shfl_sync(0xffffffffu, gmax, a * 8);
-                if (lane * 2 < HALF) {
-                  cp_async16(smem_u32(hi_s + (size_t)(buf * 16 + blk * 4 + a) * kRopeStride + lane * 2),
-                             dev.rope_hi + (size_t)(gm < 0 ? 0 : gm) * HALF + lane * 2, 16u);
+                if (lane < UN) {
+                  cp_async16(smem_u32(hi_s + (size_t)(buf * 16 + blk * 4 + a) * UN + lane),
+                             dev.rope_hi + (size_t)(gm < 0 ? 0 : gm) * UN + lane, 16u);
                 }
               }
             }
@@ -806,7 +860,9 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
     if (lane == 0) walk_s->loaded = pairs;
   } else if (warp < 4) {
     // =============================== key epilogue: rope, logits, softmax statistics, weights ===============================
-    const int j = tid;                                  // tile row = TMEM lane
+    // tile row whose softmax terms this thread works on (quad_logits leaves the logits there)
+    const int quad_t = lane & 3, quad_g = lane >> 2;
+    const int j = warp * 32 + quad_t * 8 + quad_g;
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
     const float scale2 = dev.att_scale * kLog2e;
     const int rmask = (1 << dev.rope_shift) - 1;
@@ -873,13 +929,13 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
         for (int i = 0; i < kPer; ++i) {
           const int pc = j + 128 * i;
           if (pc < kPieces) {
-            float4 a, b;
-            a.x = __uint_as_float(u[i].x << 16); a.y = __uint_as_float(u[i].x & 0xffff0000u);
-            a.z = __uint_as_float(u[i].y << 16); a.w = __uint_as_float(u[i].y & 0xffff0000u);
-            b.x = __uint_as_float(u[i].z << 16); b.y = __uint_as_float(u[i].z & 0xffff0000u);
-            b.z = __uint_as_float(u[i].w << 16); b.w = __uint_as_float(u[i].w & 0xffff0000u);
-            *reinterpret_cast<float4*>(q_s + pc * 8) = a;
-            *reinterpret_cast<float4*>(q_s + pc * 8 + 4) = b;
+            // eight dimensions: half of four units
+            const int h = pc / (DH / 8), m = pc % (DH / 8);
+            float* to = q_s + h * DH + (m % (HALF / 8)) * 16 + (m / (HALF / 8)) * 2;
+            const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              *reinterpret_cast<float2*>(to + 4 * e) = make_float2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u));
           }
         }
       }
@@ -891,23 +947,23 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       if (!wait_bar(ctx, BAR(bl.posfull + pbuf), (uint32_t)((it >> 2) & 1), ps + 1)) { ok = false; break; }   // positions published
       if (!wait_bar(ctx, BAR(bl.kfull + buf), par, ps + 2)) { ok = false; break; }
       tc_fence_after();
-      const int pos = pos_s[pbuf * kTile + j];
+      const int pos = pos_s[pbuf * kTile + j], own = pos_s[pbuf * kTile + tid];   // own: of the row in this thread's TMEM lane
       if (++pbuf == 4) pbuf = 0;
-      const int pp = pos < 0 ? 0 : pos;
       float z[NR];
-#pragma unroll
-      for (int h = 0; h < NR; ++h) z[h] = 0.0f;
       const uint32_t acc = tmem + lane_base + (uint32_t)(buf * 128);
       if (rope_smem && algn_s[buf * 4 + warp]) {
-        key_logits<DH, NR, true, true>(acc, hi_s + (size_t)(buf * 16 + (j >> 3)) * kRopeStride,
-                                       lo_s + (size_t)(pp & 7) * kRopeStride, q_s, z);
+        quad_logits<DH, NR>(acc, reinterpret_cast<const ulonglong2*>(hi_s + (buf * 16 + warp * 4) * UN),
+                            reinterpret_cast<const ulonglong2*>(lo_s + quad_g * UN), lo_swz(quad_g),
+                            reinterpret_cast<const uint4*>(q_s), lane, z);
       } else {
+        const int pp = own < 0 ? 0 : own;
+        const float4* qv = reinterpret_cast<const float4*>(q_s);
         const LogitsOut<NR> o = dev.use_rope
-            ? key_logits_rare<DH, NR, true>(acc, dev.rope_hi + (size_t)(pp >> dev.rope_shift) * HALF,
-                                            dev.rope_lo + (size_t)(pp & rmask) * HALF, q_s)
-            : key_logits_rare<DH, NR, false>(acc, nullptr, nullptr, q_s);
+            ? key_logits_rare<DH, NR, true>(acc, dev.rope_hi + (size_t)(pp >> dev.rope_shift) * UN,
+                                            dev.rope_lo + (size_t)(pp & rmask) * UN, qv)
+            : key_logits_rare<DH, NR, false>(acc, nullptr, nullptr, qv);
 #pragma unroll
-        for (int h = 0; h < NR; ++h) z[h] = o.z[h];
+        for (int h = 0; h < NR; ++h) z[h] = __shfl_sync(0xffffffffu, o.z[h], quad_t * 8 + quad_g);
       }
       tc_fence_before();
       mbar_arrive(BAR(bl.kempty + buf));                // accumulator may be overwritten

@@ -35,8 +35,8 @@ struct GroupDev {
   const __nv_bfloat16* Bt_k;        // [batch][G][H_kv][kDP][r_k]  transposed head blocks, zero padded
   const __nv_bfloat16* Bt_v;        // [batch][G][H_kv][kDP][r_v]
   const __nv_bfloat16* B_v;         // [batch][G][r_v][H_kv*d_h]   owned copy in the caller's layout
-  const float2* rope_hi;            // [n_hi][d_h/2]          (cos, sin) of (p_hi << rope_shift) * theta_i
-  const float2* rope_lo;            // [2^rope_shift][d_h/2]  (cos, sin) of p_lo * theta_i
+  const float4* rope_hi;            // [n_hi][d_h/4]          {cos, cos, sin, sin} of (p_hi << rope_shift) * theta_i, i = 2u, 2u + 1
+  const float4* rope_lo;            // [2^rope_shift][d_h/4]  the same of p_lo * theta_i
   float* pooled;                    // [G][batch][H_kv][n_c] pooled landmark scores
   uint32_t* tile_max;               // [G][batch][H_kv][ceil(n_c / kLandmarkBoxRows)] largest landmark element of every tile of the scan, or nullptr
   float* part;                      // attention partials, see xkv_attend.cu
@@ -76,6 +76,13 @@ struct xkv_group {
 namespace xkv {
 
 void set_cuda_error(cudaError_t e);
+
+// (cos, sin) of rotary pair i in a row of the tables: a pair of frequencies is four floats {cos, cos, sin, sin}, so that
+// packed fp32 arithmetic finds its operands side by side.
+__device__ __forceinline__ float2 rope_entry(const float4* __restrict__ row, int i) {
+  const float* f = reinterpret_cast<const float*>(row + (i >> 1)) + (i & 1);
+  return make_float2(__ldg(f), __ldg(f + 2));
+}
 
 // Launch with programmatic stream serialization: the kernel may begin while the previous kernel of the stream
 // drains; it must execute griddepcontrol.wait before it reads anything an earlier kernel may have written.
@@ -140,7 +147,7 @@ inline cudaError_t device_sms(int device, int* sms) {
 // xkv_prep.cu
 cudaError_t launch_repack_b(const __nv_bfloat16* B, __nv_bfloat16* Bt, int batch, int G, int r, int H_kv,
                             int d_h, cudaStream_t s);
-cudaError_t launch_rope_tables(float2* hi, float2* lo, int n_hi, int rope_shift, int d_h, double base,
+cudaError_t launch_rope_tables(float4* hi, float4* lo, int n_hi, int rope_shift, int d_h, double base,
                                cudaStream_t s);
 
 // xkv_select.cu

@@ -35,9 +35,9 @@ cudaError_t launch_repack_b(const __nv_bfloat16* B, __nv_bfloat16* Bt, int batch
 }
 
 // theta_i = base^(-2i/d_h); position p = (p_hi << shift) + p_lo.  hi[p_hi][i] = (cos, sin)((p_hi << shift) * theta_i),
-// lo[p_lo][i] = (cos, sin)(p_lo * theta_i), evaluated in fp64 so that combining the two by the angle-addition
+// lo[p_lo][i] = (cos, sin)(p_lo * theta_i) (stored as rope_entry reads them), evaluated in fp64 so that combining the two by the angle-addition
 // formulas carries fp32 rounding only.  Position-major layout: the d_h/2 entries of one position are contiguous.
-__global__ void rope_tables_kernel(float2* hi, float2* lo, int n_hi, int shift, int half, double base) {
+__global__ void rope_tables_kernel(float4* hi, float4* lo, int n_hi, int shift, int half, double base) {
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int n_lo = 1 << shift;
   const long long total = (long long)(n_hi + n_lo) * half;
@@ -48,11 +48,13 @@ __global__ void rope_tables_kernel(float2* hi, float2* lo, int n_hi, int shift, 
   const double p = col < n_hi ? (double)((long long)col << shift) : (double)(col - n_hi);
   double sn, cs;
   sincos(p * theta, &sn, &cs);
-  const float2 v = make_float2((float)cs, (float)sn);
-  if (col < n_hi) hi[(size_t)col * half + i] = v; else lo[(size_t)(col - n_hi) * half + i] = v;
+  float4* row = col < n_hi ? hi + (size_t)col * (half / 2) : lo + (size_t)(col - n_hi) * (half / 2);
+  float* f = reinterpret_cast<float*>(row + (i >> 1)) + (i & 1);
+  f[0] = (float)cs;
+  f[2] = (float)sn;
 }
 
-cudaError_t launch_rope_tables(float2* hi, float2* lo, int n_hi, int rope_shift, int d_h, double base,
+cudaError_t launch_rope_tables(float4* hi, float4* lo, int n_hi, int rope_shift, int d_h, double base,
                                cudaStream_t s) {
   const int half = d_h / 2;
   const long long total = (long long)(n_hi + (1 << rope_shift)) * half;

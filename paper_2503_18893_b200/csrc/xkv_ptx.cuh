@@ -146,6 +146,11 @@ __device__ __forceinline__ void tmem_ld4_nb(uint32_t taddr, uint32_t (&r)[4]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr));
 }
+// 16 lanes x 8 columns: thread i of the warp receives columns 2(i%4), +1 of lane i/4 (r[0], r[1]) and of lane i/4 + 8.
+__device__ __forceinline__ void tmem_ld_quad(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr));
+}
 __device__ __forceinline__ void tc_wait_ld_nb(uint32_t (&a)[4], uint32_t (&b)[4]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]));
@@ -180,6 +185,11 @@ using u64 = unsigned long long;
 __device__ __forceinline__ u64 pack2(float a, float b) {
   u64 r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ u64 pack2u(uint32_t a, uint32_t b) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
   return r;
 }
 __device__ __forceinline__ float2 unpack2(u64 v) {
