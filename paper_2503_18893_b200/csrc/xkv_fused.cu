@@ -149,35 +149,42 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1
   asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// Logits of the 32 rebuilt key rows of a warp against NR query heads (rounded up to eights): rotate the (i, i + HALF)
-// pairs, then mma.sync.  One warp per scheduler issues a multiply-add every two cycles at best, so what bounds this is
-// their number: 8 a pair for the angles and the rotation, and 2 for every head if the heads are multiplied one by one.
+// Logits of the 32 rebuilt key rows of a warp against NR query heads: rotate the (i, i + HALF) pairs, multiply.
 // Four lanes share a row: lane 4g + t reads rows g, g + 8, g + 16, g + 24 and of every eight dimensions 2t and 2t + 1 (the
-// 16x256b form of tcgen05.ld), two dimensions side by side are the operands of one packed instruction, and the rotated
-// values are where an operand of m16n8k8 wants them.  The queries are bf16 and thus exact as tf32; a key element goes in as
-// two parts, its upper 11 bits and the rest, of which the tensor core drops less than 2^-21 of the element, the size of
-// the rounding errors of the rotation; the products are exact and a sum takes 32 steps instead of 128.  (Against fp64 on the
-// same bases, thirteen shapes: outputs 1.72e-3 to 2.10e-3 rms and log-sums 6.7e-5 to 1.5e-4, the same to three digits as with
-// fp32 multiply-adds throughout: the weights' and outputs' rounding to bf16.)
-// Against a row per lane, every head a chain of multiply-adds: seven heads, eight sequences of 65536 rows 129.4 -> 123.3 us a
-// step, 4-bit bases (whose producers share the schedulers) 88.4 -> 85.9, 32768 rows by layer 114.6 -> 113.0, rank 1024 with a
-// budget of 16384 307.7 -> 304.1; four heads in the steady state are bound elsewhere (131072 rows 76.8 -> 76.8, on GPUs that
-// run at lower clocks up to 80.3 -> 77.5).  Four lanes a row with the heads as packed multiply-adds: 64 registers of sums for
-// eight heads, 157.4 where a row per lane took 151.9.
+// 16x256b form of tcgen05.ld), so that a query or table entry it loads serves four rows, and two dimensions side by side are
+// the operands of one packed instruction.  One warp per scheduler issues a multiply-add every two cycles at best, so what
+// bounds this is their number: 8 a pair for the angles and the rotation, and 2 for every head.
+// MMA: the heads (rounded up to eights) are multiplied by mma.sync instead: the rotated values are where an operand of
+// m16n8k8 wants them.  The queries are bf16 and thus exact as tf32; a key element goes in as two parts, its upper 11 bits and
+// the rest, of which the tensor core drops less than 2^-21 of the element, the size of the rounding errors of the rotation;
+// the products are exact and a sum takes 32 steps instead of 128.  (Against fp64 on the same bases, thirteen shapes: outputs
+// 1.72e-3 to 2.10e-3 rms and log-sums 6.7e-5 to 1.5e-4, the same to three digits as with fp32 multiply-adds: the weights' and
+// outputs' rounding to bf16.)
+// Which one: without MMA only four heads and bf16 bases have registers for the sums (eight heads 157.4 us a step of eight
+// sequences of 65536 rows where a row per lane takes 151.9, 4-bit bases 92.5 where it takes 88.3), and there it is the
+// better one in the steady state, where shared memory and the tensor pipe are all but busy (131072 rows 78.3 -> 75.4 us a step
+// from a row per lane, with MMA 78.6 -> 79.2; four sequences of them 268.3 -> 252.4, with MMA 270.4 -> 268.7; rank 1024, budget
+// 16384 316.5 -> 311.9).  MMA: seven heads 129.4 -> 123.5, 4-bit bases 88.2 -> 86.8, one tile per CTA (32768 rows by layer)
+// 114.3 -> 113.0 where the other gives 114.
 // hi: the coarse rotary entries of the warp's four 8-row chunks, 16-byte units; lo: the fine ones of position g of a
 // chunk, units swizzled by `swz`; q_s: the queries.  On return a lane holds the logits of row g + 8t.
-template <int DH, int NR>
+template <int DH, int NR, bool MMA>
 __device__ __forceinline__ void quad_logits(uint32_t acc, const ulonglong2* __restrict__ hi, const ulonglong2* __restrict__ lo,
                                             int swz, const uint4* __restrict__ q_s, int lane, float (&z)[NR]) {
   constexpr int HALF = DH / 2, UN = HALF / 2;            // units of a rotary row, of a head
   constexpr int NT = (NR + 7) / 8;                       // groups of eight heads
   constexpr unsigned long long kNeg2 = 0x8000000080000000ull;
   const int t = lane & 3, g = lane >> 2;
-  float c[NT][2][4];                                     // [.][rows g, g + 8 | g + 16, g + 24][heads 2t, 2t + 1 of either]
+  float c[NT][2][4];                                     // MMA: [.][rows g, g + 8 | g + 16, g + 24][heads 2t, 2t + 1 of either]
+  u64 s[MMA ? 1 : 4][NR];                                // else: [row][head], sums of the even and of the odd dimensions
 #pragma unroll
   for (int n = 0; n < NT; ++n)
 #pragma unroll
     for (int i = 0; i < 8; ++i) c[n][i >> 2][i & 3] = 0.0f;
+#pragma unroll
+  for (int r = 0; r < (MMA ? 1 : 4); ++r)
+#pragma unroll
+    for (int h = 0; h < NR; ++h) s[r][h] = 0ull;
 #pragma unroll 1
   for (int jj = 0; jj < HALF / 8; ++jj) {
     uint32_t xa[2][4], xb[2][4];                         // [16 rows][row g: 2 dimensions, row g + 8: 2]
@@ -194,21 +201,38 @@ __device__ __forceinline__ void quad_logits(uint32_t acc, const ulonglong2* __re
     for (int r = 0; r < 4; ++r) a[r] = hi[r * UN + u];
     uint4 qv[NT];                                        // head 8 n + g (heads beyond NR: whatever, their columns are not read)
 #pragma unroll
-    for (int n = 0; n < NT; ++n) qv[n] = q_s[(8 * n + (NR < 8 ? g & (NR - 1) : g)) * UN + u];
+    for (int n = 0; n < NT && MMA; ++n) qv[n] = q_s[(8 * n + (NR < 8 ? g & (NR - 1) : g)) * UN + u];
 #pragma unroll
     for (int i = 0; i < 2; ++i) tc_wait_ld_nb(xa[i], xb[i]);
     const u64 fn = f.y ^ kNeg2;
+    u64 r1[4], r2[4];                                    // the rotated pairs, either half
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const u64 cs = fma2(a[r].y, fn, mul2(a[r].x, f.x));            // cos(x + y)
+      const u64 sn = fma2(a[r].x, f.y, mul2(a[r].y, f.x));           // sin(x + y)
+      const u64 x1 = pack2u(xa[r >> 1][2 * (r & 1)], xa[r >> 1][2 * (r & 1) + 1]);
+      const u64 x2 = pack2u(xb[r >> 1][2 * (r & 1)], xb[r >> 1][2 * (r & 1) + 1]);
+      r1[r] = fma2(x2, sn ^ kNeg2, mul2(x1, cs));
+      r2[r] = fma2(x1, sn, mul2(x2, cs));
+    }
+    if constexpr (!MMA) {
+#pragma unroll
+      for (int h = 0; h < NR; ++h) {
+        const ulonglong2 qh = reinterpret_cast<const ulonglong2*>(q_s)[h * UN + u];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) s[r][h] = fma2(qh.x, r1[r], s[r][h]);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) s[r][h] = fma2(qh.y, r2[r], s[r][h]);
+      }
+      continue;
+    }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       uint32_t h1[4], h2[4], l1[4], l2[4];               // [row g: 2 dimensions, row g + 8: 2], either half; upper and lower parts
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const ulonglong2 ar = a[2 * i + k];
-        const u64 cs = fma2(ar.y, fn, mul2(ar.x, f.x));              // cos(x + y)
-        const u64 sn = fma2(ar.x, f.y, mul2(ar.y, f.x));             // sin(x + y)
-        const u64 x1 = pack2u(xa[i][2 * k], xa[i][2 * k + 1]), x2 = pack2u(xb[i][2 * k], xb[i][2 * k + 1]);
-        const float2 r1 = unpack2(fma2(x2, sn ^ kNeg2, mul2(x1, cs))), r2 = unpack2(fma2(x1, sn, mul2(x2, cs)));
-        const float v[4] = {r1.x, r1.y, r2.x, r2.y};
+        const float2 p1 = unpack2(r1[2 * i + k]), p2 = unpack2(r2[2 * i + k]);
+        const float v[4] = {p1.x, p1.y, p2.x, p2.y};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const uint32_t up = __float_as_uint(v[e]) & 0xffffe000u, rest = __float_as_uint(v[e] - __uint_as_float(up));
@@ -224,8 +248,21 @@ __device__ __forceinline__ void quad_logits(uint32_t acc, const ulonglong2* __re
       }
     }
   }
-  // transpose among the four lanes of a row: from heads 2t, 2t + 1 of four rows to all heads of row g + 8t
   const bool up1 = (t & 1) != 0, up2 = (t & 2) != 0;
+  if constexpr (!MMA) {
+    // sums over the four lanes of a row, folded by halving: a lane ends with one row
+#pragma unroll
+    for (int h = 0; h < NR; ++h) {
+      float v[4], w[2];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) { const float2 p = unpack2(s[r][h]); v[r] = p.x + p.y; }
+#pragma unroll
+      for (int r = 0; r < 2; ++r) w[r] = (up2 ? v[r + 2] : v[r]) + __shfl_xor_sync(0xffffffffu, up2 ? v[r] : v[r + 2], 2);
+      z[h] = (up1 ? w[1] : w[0]) + __shfl_xor_sync(0xffffffffu, up1 ? w[0] : w[1], 1);
+    }
+    return;
+  }
+  // transpose among the four lanes of a row: from heads 2t, 2t + 1 of four rows to all heads of row g + 8t
 #pragma unroll
   for (int n = 0; n < NT; ++n) {
     float w[2][2][2];                                    // [heads 2 (t & 1), + 1 | those and 4][row][head of the pair]
@@ -290,25 +327,20 @@ __device__ __noinline__ LogitsOut<NR> key_logits_rare(uint32_t acc, const float4
     // independent (one head after the other is a chain of eight dependent ones)
 #pragma unroll
     for (int h0 = 0; h0 < NR; h0 += 4) {
-      float4 q0[4], q1[4];
 #pragma unroll
-      for (int h = 0; h < 4; ++h) { q0[h] = q_s[(h0 + h) * (DH / 4) + u]; q1[h] = q_s[(h0 + h) * (DH / 4) + u + 1]; }
+      for (int v = 0; v < 2; ++v) {
+        float4 qv[4];
 #pragma unroll
-      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q0[h].x, r1[0], o.z[h0 + h]);
+        for (int h = 0; h < 4; ++h) qv[h] = q_s[(h0 + h) * (DH / 4) + u + v];
 #pragma unroll
-      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q0[h].z, r2[0], o.z[h0 + h]);
+        for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(qv[h].x, r1[2 * v], o.z[h0 + h]);
 #pragma unroll
-      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q0[h].y, r1[1], o.z[h0 + h]);
+        for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(qv[h].z, r2[2 * v], o.z[h0 + h]);
 #pragma unroll
-      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q0[h].w, r2[1], o.z[h0 + h]);
+        for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(qv[h].y, r1[2 * v + 1], o.z[h0 + h]);
 #pragma unroll
-      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q1[h].x, r1[2], o.z[h0 + h]);
-#pragma unroll
-      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q1[h].z, r2[2], o.z[h0 + h]);
-#pragma unroll
-      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q1[h].y, r1[3], o.z[h0 + h]);
-#pragma unroll
-      for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(q1[h].w, r2[3], o.z[h0 + h]);
+        for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(qv[h].w, r2[2 * v + 1], o.z[h0 + h]);
+      }
     }
   }
   return o;
@@ -338,9 +370,10 @@ __host__ __device__ constexpr int value_slots() {
 
 // NR: query heads per KV head rounded up to 4, 8 or 16.  WB: most 128-column blocks of r_v (registers of the
 // value epilogue): NR * WB <= 64.
+// MMA: how the key epilogue multiplies (quad_logits).
 // QUANT = 4 or 3: the token bases are gathered from 4-bit or 3-bit codes (xkv_group_set_quantized_bases) and
 // dequantised by the producer warps on their way into the rings; 0: bf16 bases.
-template <int DH, int NR, int WB, bool PROF, int QUANT>
+template <int DH, int NR, int WB, bool PROF, int QUANT, bool MMA>
 __global__ void __launch_bounds__(fused_threads(QUANT), 1)
 sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched sc, const __nv_bfloat16* __restrict__ q,
                 const int32_t* __restrict__ sel_idx, const int32_t* __restrict__ sel_cnt) {
@@ -952,9 +985,9 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       float z[NR];
       const uint32_t acc = tmem + lane_base + (uint32_t)(buf * 128);
       if (rope_smem && algn_s[buf * 4 + warp]) {
-        quad_logits<DH, NR>(acc, reinterpret_cast<const ulonglong2*>(hi_s + (buf * 16 + warp * 4) * UN),
-                            reinterpret_cast<const ulonglong2*>(lo_s + quad_g * UN), lo_swz(quad_g),
-                            reinterpret_cast<const uint4*>(q_s), lane, z);
+        quad_logits<DH, NR, MMA>(acc, reinterpret_cast<const ulonglong2*>(hi_s + (buf * 16 + warp * 4) * UN),
+                                 reinterpret_cast<const ulonglong2*>(lo_s + quad_g * UN), lo_swz(quad_g),
+                                 reinterpret_cast<const uint4*>(q_s), lane, z);
       } else {
         const int pp = own < 0 ? 0 : own;
         const float4* qv = reinterpret_cast<const float4*>(q_s);
@@ -1445,26 +1478,28 @@ cudaError_t launch_fused_t(const xkv_group* grp, int l0, int l1, const __nv_bflo
   CUtensorMap mk;
   memcpy(&mk, grp->bk_tmap, sizeof(mk));
   cudaError_t e;
+  auto launch = [&](auto kernel_smem, auto kernel, int quant) {
+    e = kernel_smem(smem, grp->device);
+    if (e == cudaSuccess) e = launch_pdl(kernel, dim3(sc.n_ctas), dim3(fused_threads(quant)), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
+  };
+#define XKV_FUSED(PROF, QUANT, MMA) launch(ensure_dyn_smem<sr_fused_kernel<DH, NR, WB, PROF, QUANT, MMA>>, sr_fused_kernel<DH, NR, WB, PROF, QUANT, MMA>, QUANT)
+  // four heads in the steady state, bf16 bases: packed multiply-adds (see quad_logits)
+  const bool fma = NR == 4 && sc.n_tiles >= 2 * sc.n_ctas;
   if (grp->prof) {     // the variant with the diagnostic counters compiled in
     if (dev.Aq_k) return cudaErrorNotSupported;        // no diagnostic variant of the quantised gather
-    e = ensure_dyn_smem<sr_fused_kernel<DH, NR, WB, true, 0>>(smem, grp->device);
-    if (e != cudaSuccess) return e;
-    e = launch_pdl(sr_fused_kernel<DH, NR, WB, true, 0>, dim3(sc.n_ctas), dim3(fused_threads(0)), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
+    if (fma) XKV_FUSED(true, 0, NR != 4); else XKV_FUSED(true, 0, true);
   } else if (dev.Aq_k && dev.quant_bits == 3) {
-    e = ensure_dyn_smem<sr_fused_kernel<DH, NR, WB, false, 3>>(smem, grp->device);
-    if (e != cudaSuccess) return e;
-    e = launch_pdl(sr_fused_kernel<DH, NR, WB, false, 3>, dim3(sc.n_ctas), dim3(fused_threads(3)), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
+    XKV_FUSED(false, 3, true);
   } else if (dev.Aq_k) {
-    e = ensure_dyn_smem<sr_fused_kernel<DH, NR, WB, false, 4>>(smem, grp->device);
-    if (e != cudaSuccess) return e;
-    e = launch_pdl(sr_fused_kernel<DH, NR, WB, false, 4>, dim3(sc.n_ctas), dim3(fused_threads(4)), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
+    XKV_FUSED(false, 4, true);
+  } else if (fma) {
+    XKV_FUSED(false, 0, NR != 4);
   } else {
-    e = ensure_dyn_smem<sr_fused_kernel<DH, NR, WB, false, 0>>(smem, grp->device);
-    if (e != cudaSuccess) return e;
-    e = launch_pdl(sr_fused_kernel<DH, NR, WB, false, 0>, dim3(sc.n_ctas), dim3(fused_threads(0)), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
+    XKV_FUSED(false, 0, true);
   }
-  count_launch(kFamFused);
+#undef XKV_FUSED
   if (e != cudaSuccess) return e;
+  count_launch(kFamFused);
   TailParts tail{nullptr, 0};
   if (tc.k) {
     e = launch_tail_partials(grp, l0, l1, q, tc.k, tc.v, tc.len, tc.cap, tc.part, true, s);

@@ -27,15 +27,13 @@ def _rows(mode, rng):
     return mixed
 
 
-@pytest.mark.parametrize("d_h,n_rep", [(128, 1), (128, 4), (128, 5), (128, 8), (128, 9), (128, 16), (64, 3), (64, 7), (64, 16)])
-@pytest.mark.parametrize("mode", ["whole", "shifted", "shuffled", "repeated", "mixed"])
-def test_rows_in_and_out_of_chunk_order(mode, d_h, n_rep):
+def _check(mode, d_h, n_rep, G, H_kv, batch):
     rng = np.random.default_rng(4100 + n_rep + d_h)
-    s = synth.config(1, T=T, k=512, G=2, H_kv=2, H_q=2 * n_rep, d_h=d_h, batch=1, r_k=96, r_v=72, seed=4100 + n_rep)
+    s = synth.config(1, T=T, k=512, G=G, H_kv=H_kv, H_q=H_kv * n_rep, d_h=d_h, batch=batch, r_k=96, r_v=72, seed=4100 + n_rep)
     inp = C.case_from_factors(s)
-    lists = [_rows(mode, rng) for _ in range(4)]
-    idx = np.stack([np.pad(r, (0, ROWS - len(r)), constant_values=-1) for r in lists]).reshape(2, 1, 2, ROWS).astype(np.int32)
-    cnt = np.array([len(r) for r in lists], dtype=np.int32).reshape(2, 1, 2)
+    lists = [_rows(mode, rng) for _ in range(G * batch * H_kv)]
+    idx = np.stack([np.pad(r, (0, ROWS - len(r)), constant_values=-1) for r in lists]).reshape(G, batch, H_kv, ROWS).astype(np.int32)
+    cnt = np.array([len(r) for r in lists], dtype=np.int32).reshape(G, batch, H_kv)
     g = C.GpuCase(s, inp)
     gout, glse = g.attend(idx, cnt, 0)
     assert g.status() == (0, 0)
@@ -44,3 +42,15 @@ def test_rows_in_and_out_of_chunk_order(mode, d_h, n_rep):
     # the weights are bf16 in the sum as in the product: 2^-9 of it at most, and as much again for the logits
     np.testing.assert_allclose(glse, olse, atol=2.0 ** -8)
     g.close()
+
+
+@pytest.mark.parametrize("d_h,n_rep", [(128, 1), (128, 4), (128, 5), (128, 8), (128, 9), (128, 16), (64, 3), (64, 7), (64, 16)])
+@pytest.mark.parametrize("mode", ["whole", "shifted", "shuffled", "repeated", "mixed"])
+def test_rows_in_and_out_of_chunk_order(mode, d_h, n_rep):
+    _check(mode, d_h, n_rep, G=2, H_kv=2, batch=1)
+
+
+@pytest.mark.parametrize("d_h,n_rep", [(128, 2), (128, 4), (64, 1), (64, 4)])
+@pytest.mark.parametrize("mode", ["whole", "mixed"])
+def test_two_tiles_and_more_per_sm(mode, d_h, n_rep):
+    _check(mode, d_h, n_rep, G=4, H_kv=8, batch=4)         # 384 tiles
