@@ -4,7 +4,7 @@
 //
 // Per tile (128 selected rows S_t of one problem, j indexes the tile's rows, m the rank dimension):
 //   keys    K_hat[j][d] = sum_m A_k[S_t[j]][m] B_k[m][d]       tcgen05.mma, M = rows, N = d_h, fp32 in TMEM
-//           z[h][j]     = scale * <q_h, rope(K_hat[j])>          thread j owns TMEM lane j (one rebuilt key row)
+//           z[h][j]     = scale * <q_h, rope(K_hat[j])>          four lanes of a warp share a rebuilt key row
 //           p[h][j]     = exp(z - running max)                   online softmax; p is handed on as bf16
 //   values  W[m][h]    += sum_j A_v[S_t[j]][m] p[h][j]           tcgen05.mma, M = 128 rank columns, N = heads
 // and once per problem, after the segments have been merged,  out_h = (W[:, h] / l_h)^T B_v.
