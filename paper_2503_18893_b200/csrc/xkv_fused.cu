@@ -984,11 +984,21 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       if (++pbuf == 4) pbuf = 0;
       float z[NR];
       const uint32_t acc = tmem + lane_base + (uint32_t)(buf * 128);
-      if (rope_smem && algn_s[buf * 4 + warp]) {
+      bool by_row = !(rope_smem && algn_s[buf * 4 + warp]);
+      if (!by_row) {
         quad_logits<DH, NR, MMA>(acc, reinterpret_cast<const ulonglong2*>(hi_s + (buf * 16 + warp * 4) * UN),
                                  reinterpret_cast<const ulonglong2*>(lo_s + quad_g * UN), lo_swz(quad_g),
                                  reinterpret_cast<const uint4*>(q_s), lane, z);
-      } else {
+        if constexpr (MMA) {
+          // an infinite key element has no upper part and rest: such a row's logits come out as NaN there, also one that is
+          // minus infinity and takes no part in the softmax
+          bool nan = false;
+#pragma unroll
+          for (int h = 0; h < NR; ++h) nan |= h < n_rep && z[h] != z[h];
+          by_row = __any_sync(0xffffffffu, nan && pos >= 0);
+        }
+      }
+      if (by_row) {
         const int pp = own < 0 ? 0 : own;
         const float4* qv = reinterpret_cast<const float4*>(q_s);
         const LogitsOut<NR> o = dev.use_rope
