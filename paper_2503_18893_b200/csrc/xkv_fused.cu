@@ -155,11 +155,12 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1
 // the operands of one packed instruction.  One warp per scheduler issues a multiply-add every two cycles at best, so what
 // bounds this is their number: 8 a pair for the angles and the rotation, and 2 for every head.
 // MMA: the heads (rounded up to eights) are multiplied by mma.sync instead: the rotated values are where an operand of
-// m16n8k8 wants them.  The queries are bf16 and thus exact as tf32; a key element goes in as two parts, its upper 11 bits and
-// the rest, of which the tensor core drops less than 2^-21 of the element, the size of the rounding errors of the rotation;
-// the products are exact and a sum takes 32 steps instead of 128.  (Against fp64 on the same bases, thirteen shapes: outputs
-// 1.72e-3 to 2.10e-3 rms and log-sums 6.7e-5 to 1.5e-4, the same to three digits as with fp32 multiply-adds: the weights' and
-// outputs' rounding to bf16.)
+// m16n8k8 wants them.  The queries are bf16 and thus exact as tf32; a key element goes in as two parts, its nearest value of 11
+// bits and the rest, 12 bits and a sign, of which the tensor core keeps 11: at most 2^-23 of the element is lost.  The tensor
+// core cuts its sums off instead of rounding them, so a sum runs over sixteen dimensions only and is added on in fp32: one sum
+// over all of them (32 steps), and an upper part that was cut off too, had logits of single rows off by 1.2 to 1.5 (rms,
+// in 2^-24 of sum |q k|; d_h 64 and 128); now 0.24 to 0.33, a multiply-add per element and head in fp32 0.36 to 0.51, the
+// packed form 0.24.  It costs nothing (seven heads 123.2 -> 123.1 us a step, 32768 rows by layer 111.7 -> 111.7).
 // Which one: without MMA only four heads and bf16 bases have registers for the sums (eight heads 157.4 us a step of eight
 // sequences of 65536 rows where a row per lane takes 151.9, 4-bit bases 92.5 where it takes 88.3), and there it is the
 // better one in the steady state, where shared memory and the tensor pipe are all but busy (131072 rows 78.3 -> 75.4 us a step
@@ -235,16 +236,20 @@ __device__ __forceinline__ void quad_logits(uint32_t acc, const ulonglong2* __re
         const float v[4] = {p1.x, p1.y, p2.x, p2.y};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const uint32_t up = __float_as_uint(v[e]) & 0xffffe000u, rest = __float_as_uint(v[e] - __uint_as_float(up));
+          const uint32_t up = (__float_as_uint(v[e]) + 0x1000u) & 0xffffe000u, rest = __float_as_uint(v[e] - __uint_as_float(up));
           if (e < 2) { h1[2 * k + e] = up; l1[2 * k + e] = rest; } else { h2[2 * k + e - 2] = up; l2[2 * k + e - 2] = rest; }
         }
       }
 #pragma unroll
       for (int n = 0; n < NT; ++n) {
-        mma_tf32(c[n][i], l1[0], l1[2], l1[1], l1[3], qv[n].x, qv[n].y);
-        mma_tf32(c[n][i], l2[0], l2[2], l2[1], l2[3], qv[n].z, qv[n].w);
-        mma_tf32(c[n][i], h1[0], h1[2], h1[1], h1[3], qv[n].x, qv[n].y);
-        mma_tf32(c[n][i], h2[0], h2[2], h2[1], h2[3], qv[n].z, qv[n].w);
+        // sums of sixteen dimensions, lower parts first, added in fp32
+        float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        mma_tf32(d, l1[0], l1[2], l1[1], l1[3], qv[n].x, qv[n].y);
+        mma_tf32(d, l2[0], l2[2], l2[1], l2[3], qv[n].z, qv[n].w);
+        mma_tf32(d, h1[0], h1[2], h1[1], h1[3], qv[n].x, qv[n].y);
+        mma_tf32(d, h2[0], h2[2], h2[1], h2[3], qv[n].z, qv[n].w);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) c[n][i][e] += d[e];
       }
     }
   }
