@@ -992,12 +992,13 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
         if (band) {
           const uint32_t at = atomicAdd(&sh_cand, 1u);
           if (at < (uint32_t)kTopkCand) cand_s[at] = j;
-        } else {
-          list_key[e] = 0u;                                // below the key of every score
         }
+        // out of the band: 0, in it: not 0, whatever the key (the key of a score never is 0, but a scan that gave up leaves
+        // what was there before)
+        list_key[e] = band ? max(kk, 1u) : 0u;
       }
       __syncthreads();
-      in_bin = sh_cand;
+      in_bin = sh_cand;                                    // with the chunks taken, at least k_ch
       need = (uint32_t)k_ch - sh_sure;
       ranked = in_bin <= (uint32_t)kTopkCand;
       if (ranked) {
@@ -1032,6 +1033,7 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
       }
     }
     __syncthreads();
+    in_bin = min(in_bin, sh_cand);                         // what cand_s holds
     if (!ties && (uint32_t)warp < in_bin) {
       constexpr int CL = kTopkCand / 32;
       unsigned long long held[CL];                         // this lane's share of the candidates
