@@ -219,7 +219,7 @@ int xkv_group_create(const xkv_group_config* cfg, void* stream, xkv_group** out)
     XKV_ALLOC(Bt_v, __nv_bfloat16*, btv);
     XKV_ALLOC(Bv_copy, __nv_bfloat16*, (size_t)c.batch * c.G * c.r_v * c.H_kv * c.d_h * sizeof(__nv_bfloat16));
     XKV_ALLOC(d.pooled, float*, pooled);
-    if (tiles) XKV_ALLOC(d.tile_max, uint32_t*, tiles);
+    if (tiles) XKV_ALLOC(d.tile_sum, uint32_t*, tiles);
     XKV_ALLOC(rhi, float4*, hi);
     XKV_ALLOC(rlo, float4*, lo);
     XKV_ALLOC(d.part, float*, part);

@@ -38,7 +38,7 @@ struct GroupDev {
   const float4* rope_hi;            // [n_hi][d_h/4]          {cos, cos, sin, sin} of (p_hi << rope_shift) * theta_i, i = 2u, 2u + 1
   const float4* rope_lo;            // [2^rope_shift][d_h/4]  the same of p_lo * theta_i
   float* pooled;                    // [G][batch][H_kv][n_c] pooled landmark scores
-  uint32_t* tile_max;               // [G][batch][H_kv][ceil(n_c / kLandmarkBoxRows)] largest landmark element of every tile of the scan, or nullptr
+  uint32_t* tile_sum;               // [G][batch][H_kv][ceil(n_c / kLandmarkBoxRows)] largest sum_i |q_i l_i| of every tile of the scan, or nullptr
   float* part;                      // attention partials, see xkv_attend.cu
   unsigned int* flags;              // device flag word
   const int32_t* outliers;          // [G][batch][H_kv][n_out] static outlier chunk ids (Algorithm 2 line 5), or nullptr

@@ -201,10 +201,14 @@ score_pool_kernel(const __grid_constant__ CUtensorMap tmap, GroupDev dev, const 
 // mma.sync.m16n8k16, whose eight columns are the heads, and the queries stay in registers.  What bounds it is the landmarks.
 // mma.sync and not tcgen05: 0.1 TFLOP in all, and a warp keeps its own tile without tensor memory or a second barrier.
 //
-// The bound.  The products are exact in fp32.  With S = sum_i |q_i l_i| the canonical chain of d_h <= 128 multiply-adds is
-// off by at most 128 2^-24 S, d_h / 16 steps of at most 17 truncated terms each by at most 136 2^-23 S, and scaling adds one
-// rounding to either: less than 2^-15 S together.  S <= |q|_1 max |l|, both maxima over the problem: the largest landmark
-// element of every tile is written beside the scores.
+// The bound.  The products are exact in fp32.  With S = sum_i |q_i l_i| of a row and a head the canonical chain of d_h <= 128
+// multiply-adds is off by at most 128 2^-24 S, d_h / 16 steps of 17 terms and a sum, each cut off below 2^-23 of the largest
+// at worst, by at most 144 2^-23 S, and scaling adds one rounding to either: less than 0.82 2^-15 S together (S itself, from
+// the tensor core too, is short by less than 2^-15 of it).  S comes from the same fragments without their signs, its largest
+// value in a tile is written beside the scores, and E is that of the largest of the problem.  (|q|_1 max |l| in its place needs no
+// further products, but is a hundred times larger where one channel or row stands out, and the band with it.  Selections of
+// 65536 rows, seven heads, 128 problems, with that -> with S: Gaussian landmarks 47.0 -> 46.5 us, a channel of 300 72 -> 49, one
+// row in a hundred a hundred times as long 75 -> 52, one element of 1000 144 -> 48, of 3000 575 -> 53; canonical scan 68.)
 constexpr float kScoreBound = 1.0f / 32768.0f;
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
@@ -215,14 +219,8 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4],
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ uint32_t max_u16x2(uint32_t a, uint32_t b) {
-  uint32_t r;
-  asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-  return r;
-}
-
-// grid as above.  NT: groups of eight heads.  tile_max [problem][tile]: bits of the largest |element| as a bf16 number (a NaN
-// above everything).
+// grid as above.  NT: groups of eight heads.  tile_sum [problem][tile]: bits of the tile's largest S (a NaN above everything;
+// 0: all its rows or all the queries are zero, and so is every score).
 template <int DH, int NT>
 __global__ void __launch_bounds__(kScoreThreads)
 score_bound_kernel(const __grid_constant__ CUtensorMap tmap, GroupDev dev, const __nv_bfloat16* __restrict__ q, int l0) {
@@ -279,24 +277,33 @@ score_bound_kernel(const __grid_constant__ CUtensorMap tmap, GroupDev dev, const
   // lane i hands ldmatrix the address of row i % 16, dimensions 8 (i / 16) of a 16 x 16 piece
   const uint32_t arow = (uint32_t)(lane & 15), ahalf = (uint32_t)(lane >> 4);
   float keep[2] = {0.0f, 0.0f};                            // rows 16 t + g8 and 16 t + 8 + g8
-  uint32_t big0 = 0u, big1 = 0u;
+  uint32_t big = 0u;                                       // largest S
 #pragma unroll
   for (int m = 0; m < kScoreRows / 16; ++m) {
     const uint32_t row = (uint32_t)(16 * m) + arow, sw = row & 7u;
-    float acc[NT][4];
+    float acc[NT][4], sum[NT][4];
 #pragma unroll
     for (int n = 0; n < NT; ++n)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) acc[n][i] = 0.0f;
+      for (int i = 0; i < 4; ++i) acc[n][i] = sum[n][i] = 0.0f;
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) {
-      uint32_t a[4];
+      uint32_t a[4], mag[4];
       ldmatrix_x4(a, tile + (uint32_t)(ks >> 2) * (kScoreRows * 128u) + row * 128u + ((((uint32_t)(ks & 3) * 2u + ahalf) ^ sw) << 4));
-      big0 = max_u16x2(big0, max_u16x2(a[0] & 0x7fff7fffu, a[1] & 0x7fff7fffu));
-      big1 = max_u16x2(big1, max_u16x2(a[2] & 0x7fff7fffu, a[3] & 0x7fff7fffu));
 #pragma unroll
-      for (int n = 0; n < NT; ++n) mma_16816(acc[n], a, qf[n][ks][0], qf[n][ks][1]);
+      for (int i = 0; i < 4; ++i) mag[i] = a[i] & 0x7fff7fffu;
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        mma_16816(acc[n], a, qf[n][ks][0], qf[n][ks][1]);
+        mma_16816(sum[n], mag, qf[n][ks][0] & 0x7fff7fffu, qf[n][ks][1] & 0x7fff7fffu);
+      }
     }
+    // (the box runs on beyond the last chunk, into the next problem's rows: they do not count)
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (j0 + 16 * m + 8 * (i >> 1) + g8 < dev.n_c) big = max(big, __float_as_uint(sum[n][i]) & 0x7fffffffu);
     // columns 2 t, 2 t + 1 of rows g8 (acc 0, 1) and g8 + 8 (acc 2, 3): maximum over the heads that exist
     float best[2] = {-INFINITY, -INFINITY};
 #pragma unroll
@@ -321,9 +328,22 @@ score_bound_kernel(const __grid_constant__ CUtensorMap tmap, GroupDev dev, const
     const int j = j0 + 16 * t + 8 * x + g8;
     if (j < dev.n_c) dst[j] = score_key(keep[x]);
   }
-  big0 = max_u16x2(big0, big1);
-  const uint32_t big = __reduce_max_sync(0xffffffffu, max(big0 & 0xffffu, big0 >> 16));
-  if (lane == 0) dev.tile_max[prob_out * gridDim.x + blockIdx.x] = big;
+  big = __reduce_max_sync(0xffffffffu, big);
+  if (big == 0u) {
+    // zero, or so small that the products are lost: only the first is exact (all rows of the box are looked at)
+    uint32_t any_l = 0u, any_q = 0u;
+    for (uint32_t off = (uint32_t)lane * 16u; off < (uint32_t)((DH / 64) * kScoreRows * 128); off += 512u) {
+      const uint4 v = lds128(tile + off);
+      any_l |= v.x | v.y | v.z | v.w;
+    }
+    any_l &= 0x7fff7fffu;
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks) any_q |= (qf[n][ks][0] | qf[n][ks][1]) & 0x7fff7fffu;
+    if (__any_sync(0xffffffffu, any_l != 0u) && __any_sync(0xffffffffu, any_q != 0u)) big = 1u;
+  }
+  if (lane == 0) dev.tile_sum[prob_out * gridDim.x + blockIdx.x] = big;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -709,9 +729,12 @@ topk_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __restrict
 //
 // BOUND: the keys are those of score_bound_kernel, off by at most E (see there).  The k_ch-th largest canonical score then
 // lies within E of the k_ch-th largest key, so chunks more than 2 E above the bin of step 4 are taken and those more than 2 E
-// below it are not; the band between is scored again in the canonical order, a warp per chunk, a lane per head, and its keys
-// take the place of the bin's.  Step 3 lists down to P - 2 E.  A band of more than kTopkCand chunks (ties, or an infinity or
-// NaN somewhere, where E is infinite and the band is everything) goes through the bins again.
+// below it are not; the band between is scored again in the canonical order and its keys take the place of the bin's.  Step 3
+// lists down to P - 2 E.  With E = 0 (nothing but zeros) the keys are the canonical ones.  A band of more than kTopkCand chunks
+// (that many scores equal to 2^-14 of S, or a score that is not finite somewhere, where E is infinite and the band everything)
+// goes through the bins again, a chunk per thread on the problem's one SM (8192 chunks of one and the same score, 128 problems of
+// seven heads: 201 us, a warp per chunk 663, the canonical scan with its top-k 75; 64 problems of sixteen heads and 16384 chunks
+// 635, 1270 and 154).  Tiles of zeros are left out of that: the unused end of a context, 98 % zeros: 72 us, canonical 79.
 // (With consecutive keys per thread, extrema by shuffles, a thread per candidate and separate scans for ties and
 // positions, about 25 barriers: 32768 rows decoded layer by layer 129.4 us, 122.4 us with this form; 121873 rows 212.6 ->
 // 193.6; 2048 rows 19.3 -> 17.6.)
@@ -781,6 +804,61 @@ __device__ __forceinline__ uint32_t canonical_key(const __nv_bfloat16* __restric
   return __reduce_max_sync(0xffffffffu, score_key(fmaxf(-INFINITY, acc * scale)));
 }
 
+// The same of one row by one thread: an element is loaded and widened once for eight heads.  q_f: fp32 queries in shared memory,
+// dh to a head.
+__device__ __forceinline__ uint32_t canonical_key_thread(const uint4* __restrict__ row, const float* __restrict__ q_f, int dh,
+                                                      int n_rep, float scale) {
+  float best = -INFINITY;
+#pragma unroll 1
+  for (int h0 = 0; h0 < n_rep; h0 += 8) {
+    float acc[8];
+#pragma unroll
+    for (int h = 0; h < 8; ++h) acc[h] = 0.0f;
+#pragma unroll 1
+    for (int i = 0; i < dh / 8; i += 2) {
+      const uint4 v0 = __ldg(row + i), v1 = __ldg(row + i + 1);
+      const uint32_t lw[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+      float x[16];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) { x[2 * e] = __uint_as_float(lw[e] << 16); x[2 * e + 1] = __uint_as_float(lw[e] & 0xffff0000u); }
+#pragma unroll
+      for (int h = 0; h < 8; ++h) {
+        if (h0 + h < n_rep) {
+          const float4* qh = reinterpret_cast<const float4*>(q_f + (h0 + h) * dh + i * 8);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float4 qv = qh[e];
+            acc[h] = fmaf(qv.w, x[4 * e + 3], fmaf(qv.z, x[4 * e + 2], fmaf(qv.y, x[4 * e + 1], fmaf(qv.x, x[4 * e], acc[h]))));
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 8; ++h) if (h0 + h < n_rep) best = fmaxf(best, acc[h] * scale);
+  }
+  return score_key(best);
+}
+
+// The listed chunks of a wide band (those with an entry other than 0) scored again, a thread per chunk, out of line: it is
+// seldom taken.  q_s as above; q_f: room for them in fp32.  Chunks of a tile of zeros, the unused end of a context, have their
+// key already.
+__device__ __noinline__ void rescore_wide(uint32_t* __restrict__ list_key, const uint16_t* __restrict__ list_idx, int n_list,
+                                          const __nv_bfloat16* __restrict__ rows, const uint32_t* __restrict__ tile_sum,
+                                          const uint4* __restrict__ q_s, float* __restrict__ q_f, int n_rep, int dh, float scale) {
+  const int pieces = dh / 8;
+  if ((int)threadIdx.x < n_rep * pieces) {
+    const uint4 v = q_s[threadIdx.x / pieces * (pieces + 1) + threadIdx.x % pieces];
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    float* to = q_f + threadIdx.x * 8;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { to[2 * e] = __uint_as_float(w[e] << 16); to[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u); }
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < n_list; e += blockDim.x)
+    if (list_key[e] != 0u && __ldcg(tile_sum + list_idx[e] / kScoreRows) != 0u)
+      list_key[e] = canonical_key_thread(reinterpret_cast<const uint4*>(rows + (size_t)list_idx[e] * dh), q_f, dh, n_rep, scale);
+}
+
 template <int GPT, int ITEMS, int TH, bool BOUND>
 __global__ void __launch_bounds__(TH, 1)
 topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __restrict__ outliers, int n_out, float sign,
@@ -798,7 +876,7 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
   __shared__ unsigned long long cand_s[kTopkCand];                                 // (key, ~chunk index): larger = earlier
   __shared__ uint32_t sh[3];
   __shared__ uint32_t sh_n, sh_cand;
-  __shared__ uint32_t warp_l[TH / 32], warp_q[TH / 32];                            // BOUND: largest landmark element, largest |q|_1
+  __shared__ uint32_t warp_s[TH / 32];                                             // BOUND: largest S
   __shared__ uint32_t sh_sure;                                                     // BOUND: chunks taken without their canonical score
 
   constexpr int NWARP = TH / 32;
@@ -859,19 +937,9 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
     if constexpr (BOUND) {
       const int n_t = (n_c + kScoreRows - 1) / kScoreRows;
       uint32_t big = 0u;
-      for (int i = tid; i < n_t; i += TH) big = max(big, __ldcg(dev.tile_max + prob * n_t + i));
-      const uint32_t w[4] = {q_piece.x, q_piece.y, q_piece.z, q_piece.w};
-      float l1 = 0.0f;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) l1 += __uint_as_float((w[e] << 16) & 0x7fffffffu) + __uint_as_float(w[e] & 0x7fff0000u);
-#pragma unroll
-      for (int o = 1; o < 16; o <<= 1) {
-        const float other = __shfl_xor_sync(0xffffffffu, l1, o);
-        if (o < pieces) l1 += other;
-      }
+      for (int i = tid; i < n_t; i += TH) big = max(big, __ldcg(dev.tile_sum + prob * n_t + i));
       big = __reduce_max_sync(0xffffffffu, big);
-      const uint32_t lq = __reduce_max_sync(0xffffffffu, __float_as_uint(l1));
-      if (lane == 0) { warp_l[warp] = big; warp_q[warp] = lq; }
+      if (lane == 0) warp_s[warp] = big;
     }
     // ---- 1: maxima of the groups that hold a chunk, and their range (keys beyond the last chunk are 0)
     uint32_t gmax[NG], kmin = 0xffffffffu, kmax = 0u;
@@ -896,10 +964,8 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
     kmax = __reduce_max_sync(0xffffffffu, lane < NWARP ? warp_max[lane] : 0u);
     float E2 = 0.0f;                                       // BOUND: 2 E
     if constexpr (BOUND) {
-      const float big = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < NWARP ? warp_l[lane] : 0u) << 16);
-      const float l1 = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < NWARP ? warp_q[lane] : 0u));
-      const float S = l1 * big;
-      E2 = S < 1e36f ? fmaf(2.0f * kScoreBound * dev.sel_scale, S, 1e-37f) : INFINITY;    // (also where S is NaN)
+      const float S = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < NWARP ? warp_s[lane] : 0u));
+      E2 = S == 0.0f ? 0.0f : S < 1e36f ? fmaf(2.0f * kScoreBound * dev.sel_scale, S, 1e-37f) : INFINITY;    // (also where S is NaN)
     }
     // ---- 2: pivot: lower edge of the bin that holds the k_ch-th largest group maximum
     uint32_t P = kmin;
@@ -971,9 +1037,10 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
         __syncthreads();                                               // sh is read before the next pass writes it
       }
     };
-    narrow(BOUND ? (uint32_t)NWARP : (uint32_t)kTopkCand, false);
+    const bool exact = !BOUND || E2 == 0.0f;
+    narrow(exact ? (uint32_t)kTopkCand : (uint32_t)NWARP, false);
     bool ranked = false;                                   // the candidates are in cand_s already
-    if constexpr (BOUND) {
+    if (BOUND && !exact) {
       // chunks above the band are taken; those in it keep their entry and are listed (the first kTopkCand of them)
       // (at least the bin is in the band, whatever the keys are: fewer than k_ch chunks are above it, k_ch at or above its foot)
       const uint32_t above = E2 < INFINITY ? max(lo + span, score_key(__fadd_ru(key_score(lo + span), E2))) : 0xffffffffu;
@@ -1007,12 +1074,9 @@ topk_pivot_kernel(GroupDev dev, int l0, int k_ch, int k_cap, const int32_t* __re
           if (lane == 0) cand_s[e] = ((unsigned long long)kk << 32) | (0xffffffffu - j);
         }
       } else {
-        for (int e = warp; e < n_list; e += NWARP) {
-          if (list_key[e] == 0u) continue;                 // (the same in all lanes)
-          const uint32_t kk = exact_key(list_idx[e]);
-          __syncwarp();
-          if (lane == 0) list_key[e] = kk;
-        }
+        static_assert(kMaxRep * 128 <= kTopkBins, "fp32 queries in a histogram");
+        rescore_wide(list_key, list_idx, n_list, rows, dev.tile_sum + prob * ((n_c + kScoreRows - 1) / kScoreRows),
+                     reinterpret_cast<const uint4*>(hist0), reinterpret_cast<float*>(hist1), dev.n_rep, dev.d_h, dev.sel_scale);
         __syncthreads();
         if (tid == 0) sh_cand = 0;
         lo = 1u; span = 0xfffffffeu;
@@ -1180,8 +1244,8 @@ static cudaError_t launch_select_dev(const GroupDev& dev, const CUtensorMap& tma
   // 16 problems 15.7 -> 12.7, 8192 rows and 128 problems 16.5 -> 14.7, 32768 rows and 16 problems 10.2 -> 10.6, 2048 rows and
   // 128 problems 9.7 -> 12.4; 5 heads, 16384 rows, 64 problems 14.4 -> 14.0, 32768 rows and 16 problems 9.3 -> 10.4; 16 heads,
   // 131072 rows, 64 problems 135.8 -> 47.3, 32768 rows and 16 problems 14.9 -> 11.6, 16384 rows and 16 problems 11.9 -> 12.0.
-  // Without a handle there is no room for the tiles' largest elements.
-  const bool bound = dev.tile_max != nullptr && dev.n_rep > 4 && k_ch < dev.n_c && dev.n_c <= kTopkThreads * 32 &&
+  // Without a handle there is no room for the tiles' sums.
+  const bool bound = dev.tile_sum != nullptr && dev.n_rep > 4 && k_ch < dev.n_c && dev.n_c <= kTopkThreads * 32 &&
                      (int64_t)problems * dev.n_c * dev.n_rep >= 5 << 17;
   const size_t smem = 1024 + (size_t)(dev.d_h / 64) * kScoreRows * 128 + (bound ? 0 : (size_t)dev.n_rep * dev.d_h * 4);
 #define XKV_SCAN_BOUND(DH, NT)                                                                          \
