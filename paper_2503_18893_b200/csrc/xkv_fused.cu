@@ -293,60 +293,79 @@ __device__ __forceinline__ void quad_logits(uint32_t acc, const ulonglong2* __re
 }
 
 // The same for the variants that ordinary tiles do not take (no RoPE; a tile whose 8-row groups are not whole landmark
-// chunks, or a rotary table that is not staged), a thread per row, the tables in global memory; out of line, because the
-// key epilogue's loop has to stay small (the four warps of a scheduler run four different loops and share its instruction
-// cache: 32 pairs unrolled in it took 77 us a call, 8 pairs 73, 4 pairs 71).  On return a lane holds the logits of the row
-// of its own TMEM lane.
+// chunks, or a rotary table that is not staged), a thread per row, the tables (hi, lo: addresses) in global memory; out of line,
+// because the key epilogue's loop has to stay small (the four warps of a scheduler run four different loops and share its
+// instruction cache: 32 pairs unrolled in it took 77 us a call, 8 pairs 73, 4 pairs 71).  On return a lane holds the logits of
+// the row of its own TMEM lane.
+enum RowTables { kNoTables, kHandleTables };
 template <int NR>
 struct LogitsOut { float z[NR]; };
-template <int DH, int NR, bool ROPE>
-__device__ __noinline__ LogitsOut<NR> key_logits_rare(uint32_t acc, const float4* __restrict__ hi, const float4* __restrict__ lo,
-                                                      const float4* __restrict__ q_s) {
+template <int DH, int NR, int QUANT, int TABLES>
+__device__ __noinline__ LogitsOut<NR> key_logits_rows(uint32_t acc, u64 hi, u64 lo, const ulonglong2* __restrict__ q_s) {
   constexpr int HALF = DH / 2;
+  constexpr unsigned long long kNeg2 = 0x8000000080000000ull;
+  // Two dimensions per instruction where the sums have registers: not with sixteen heads, and with eight over codes (96 registers
+  // a thread) only without tables.  One by one -> packed: 4-bit bases, seven heads, no RoPE 83.0 -> 80.3 us; rows of no chunk,
+  // four heads 70.7 -> 69.9, over codes 78.0 -> 75.7; seven heads 133.3 -> 132.4, but over codes 145 -> 157.
+  constexpr bool PACKED = NR <= 8 && !(NR == 8 && QUANT != 0 && TABLES != kNoTables);
   LogitsOut<NR> o;
+  u64 s[PACKED ? NR : 1];
 #pragma unroll
   for (int h = 0; h < NR; ++h) o.z[h] = 0.0f;
+#pragma unroll
+  for (int h = 0; h < (PACKED ? NR : 1); ++h) s[h] = 0ull;
 #pragma unroll 1
   for (int u = 0; u < HALF / 2; u += 2) {                // four rotary pairs per pass
     uint32_t xa[4], xb[4];
     tmem_ld4_nb(acc + (uint32_t)(2 * u), xa);
     tmem_ld4_nb(acc + (uint32_t)(HALF + 2 * u), xb);
-    tc_wait_ld_nb(xa, xb);
-    float r1[4], r2[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) { r1[e] = __uint_as_float(xa[e]); r2[e] = __uint_as_float(xb[e]); }
-    if (ROPE) {
-      const float4 a0 = __ldg(hi + u), a1 = __ldg(hi + u + 1), c0 = __ldg(lo + u), c1 = __ldg(lo + u + 1);
-      const float ac[4] = {a0.x, a0.y, a1.x, a1.y}, as[4] = {a0.z, a0.w, a1.z, a1.w};
-      const float cc[4] = {c0.x, c0.y, c1.x, c1.y}, cn[4] = {c0.z, c0.w, c1.z, c1.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float cs = ac[e] * cc[e] - as[e] * cn[e];              // cos(x + y)
-        const float sn = as[e] * cc[e] + ac[e] * cn[e];              // sin(x + y)
-        const float x1 = r1[e], x2 = r2[e];
-        r1[e] = x1 * cs - x2 * sn;
-        r2[e] = x2 * cs + x1 * sn;
-      }
-    }
-    // heads in groups of four, element by element inside a group: the four multiply-adds of an element are
-    // independent (one head after the other is a chain of eight dependent ones)
-#pragma unroll
-    for (int h0 = 0; h0 < NR; h0 += 4) {
+    ulonglong2 a[2], f[2];
+    if (TABLES == kHandleTables) {
 #pragma unroll
       for (int v = 0; v < 2; ++v) {
-        float4 qv[4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) qv[h] = q_s[(h0 + h) * (DH / 4) + u + v];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(qv[h].x, r1[2 * v], o.z[h0 + h]);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(qv[h].z, r2[2 * v], o.z[h0 + h]);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(qv[h].y, r1[2 * v + 1], o.z[h0 + h]);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(qv[h].w, r2[2 * v + 1], o.z[h0 + h]);
+        a[v] = __ldg(reinterpret_cast<const ulonglong2*>(hi) + u + v);
+        f[v] = __ldg(reinterpret_cast<const ulonglong2*>(lo) + u + v);
       }
     }
+    tc_wait_ld_nb(xa, xb);
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      u64 r1 = pack2u(xa[2 * v], xa[2 * v + 1]), r2 = pack2u(xb[2 * v], xb[2 * v + 1]);
+      if (TABLES != kNoTables) {
+        const u64 cs = fma2(a[v].y, f[v].y ^ kNeg2, mul2(a[v].x, f[v].x));       // cos(x + y)
+        const u64 sn = fma2(a[v].x, f[v].y, mul2(a[v].y, f[v].x));               // sin(x + y)
+        const u64 x1 = r1, x2 = r2;
+        r1 = fma2(x2, sn ^ kNeg2, mul2(x1, cs));
+        r2 = fma2(x1, sn, mul2(x2, cs));
+      }
+      // heads in groups of four: their multiply-adds are independent (one head after the other is a chain)
+#pragma unroll
+      for (int h0 = 0; h0 < NR; h0 += 4) {
+        ulonglong2 qv[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) qv[h] = q_s[(h0 + h) * (DH / 4) + u + v];
+        if constexpr (PACKED) {
+#pragma unroll
+          for (int h = 0; h < 4; ++h) s[h0 + h] = fma2(qv[h].x, r1, s[h0 + h]);
+#pragma unroll
+          for (int h = 0; h < 4; ++h) s[h0 + h] = fma2(qv[h].y, r2, s[h0 + h]);
+        } else {
+          const float2 p1 = unpack2(r1), p2 = unpack2(r2);
+#pragma unroll
+          for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(unpack2(qv[h].x).x, p1.x, o.z[h0 + h]);
+#pragma unroll
+          for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(unpack2(qv[h].y).x, p2.x, o.z[h0 + h]);
+#pragma unroll
+          for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(unpack2(qv[h].x).y, p1.y, o.z[h0 + h]);
+#pragma unroll
+          for (int h = 0; h < 4; ++h) o.z[h0 + h] = fmaf(unpack2(qv[h].y).y, p2.y, o.z[h0 + h]);
+        }
+      }
+    }
+  }
+  if constexpr (PACKED) {
+#pragma unroll
+    for (int h = 0; h < NR; ++h) { const float2 p = unpack2(s[h]); o.z[h] = p.x + p.y; }
   }
   return o;
 }
@@ -1005,11 +1024,11 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       }
       if (by_row) {
         const int pp = own < 0 ? 0 : own;
-        const float4* qv = reinterpret_cast<const float4*>(q_s);
+        const ulonglong2* qv = reinterpret_cast<const ulonglong2*>(q_s);
         const LogitsOut<NR> o = dev.use_rope
-            ? key_logits_rare<DH, NR, true>(acc, dev.rope_hi + (size_t)(pp >> dev.rope_shift) * UN,
-                                            dev.rope_lo + (size_t)(pp & rmask) * UN, qv)
-            : key_logits_rare<DH, NR, false>(acc, nullptr, nullptr, qv);
+            ? key_logits_rows<DH, NR, QUANT, kHandleTables>(acc, (u64)(dev.rope_hi + (size_t)(pp >> dev.rope_shift) * UN),
+                                                            (u64)(dev.rope_lo + (size_t)(pp & rmask) * UN), qv)
+            : key_logits_rows<DH, NR, QUANT, kNoTables>(acc, 0, 0, qv);
 #pragma unroll
         for (int h = 0; h < NR; ++h) z[h] = __shfl_sync(0xffffffffu, o.z[h], quad_t * 8 + quad_g);
       }

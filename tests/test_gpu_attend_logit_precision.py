@@ -12,11 +12,12 @@ G, T, R, K = 4, 16384, 64, 128
 
 
 @pytest.mark.parametrize("bits", [16, 4])
+@pytest.mark.parametrize("rows", ["in order", "out of order", "not rotated"])
 @pytest.mark.parametrize("d_h,H_kv,n_rep,batch", [
     (128, 8, 1, 1), (128, 8, 4, 1), (128, 4, 7, 4), (128, 4, 16, 2), (64, 8, 4, 1), (64, 8, 8, 2),
     (128, 8, 4, 16), (64, 8, 3, 16),            # two tiles and more per CTA
 ])
-def test_logits_of_single_rows(d_h, H_kv, n_rep, batch, bits):
+def test_logits_of_single_rows(d_h, H_kv, n_rep, batch, rows, bits):
     g = torch.Generator(device="cuda").manual_seed(4400 + d_h + n_rep)
     H_q, half = H_kv * n_rep, d_h // 2
     rn = lambda *shape: torch.randn(shape, generator=g, device="cuda").to(torch.bfloat16)
@@ -24,7 +25,8 @@ def test_logits_of_single_rows(d_h, H_kv, n_rep, batch, bits):
     A = torch.zeros((batch, T, R), dtype=torch.bfloat16, device="cuda")
     A[:, t, t // 8 % R] = 1.0
     B, q = rn(batch, G, R, H_kv * d_h), rn(G, batch, H_q, d_h)
-    grp = xkv.create_from_tensors(A, A, B, B, None, H_kv=H_kv, H_q=H_q, k_max=K)
+    rope_base = 0.0 if rows == "not rotated" else 10000.0
+    grp = xkv.create_from_tensors(A, A, B, B, None, H_kv=H_kv, H_q=H_q, k_max=K, rope_base=rope_base)
     if bits != 16:
         codes, meta = xkv.xkv_quantize_rtn(A, bits)
         assert torch.equal(xkv.xkv_dequantize_rtn(codes, meta, bits), A)
@@ -35,12 +37,14 @@ def test_logits_of_single_rows(d_h, H_kv, n_rep, batch, bits):
     err = []
     for _ in range(8):
         row = torch.randint(0, T // 8, (G, batch, H_kv, 1), generator=g, device="cuda", dtype=torch.int32) * 8
+        row += 3 if rows == "out of order" else 0          # position 0 of a tile is not position 0 of a chunk then
         idx = torch.full((G, batch, H_kv, K), -1, dtype=torch.int32, device="cuda")
         idx[..., :1] = row
         xkv.xkv_sr_reconstruct_attend(grp, 0, G, q, idx, torch.ones((G, batch, H_kv), dtype=torch.int32, device="cuda"), K, out, lse)
         p = row.long()
         keys = B.view(batch, G, R, H_kv, d_h).permute(1, 0, 3, 2, 4)                        # G, batch, H_kv, R, d_h
         x = keys.gather(3, (p // 8 % R)[..., None].expand(-1, -1, -1, 1, d_h))[..., 0, :].double()
+        p = p if rope_base > 0.0 else 0 * p
         cs, sn = (p.double() * theta).cos(), (p.double() * theta).sin()
         k = torch.cat([x[..., :half] * cs - x[..., half:] * sn, x[..., half:] * cs + x[..., :half] * sn], -1)
         terms = q.view(G, batch, H_kv, n_rep, d_h).double() * k[..., None, :] / math.sqrt(d_h)
