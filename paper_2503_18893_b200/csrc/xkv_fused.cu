@@ -292,16 +292,29 @@ __device__ __forceinline__ void quad_logits(uint32_t acc, const ulonglong2* __re
   }
 }
 
-// The same for the variants that ordinary tiles do not take (no RoPE; a tile whose 8-row groups are not whole landmark
-// chunks, or a rotary table that is not staged), a thread per row, the tables (hi, lo: addresses) in global memory; out of line,
-// because the key epilogue's loop has to stay small (the four warps of a scheduler run four different loops and share its
-// instruction cache: 32 pairs unrolled in it took 77 us a call, 8 pairs 73, 4 pairs 71).  On return a lane holds the logits of
-// the row of its own TMEM lane.
-enum RowTables { kNoTables, kHandleTables };
+// Rotary rows are multiples of 128 bytes.  Unit u of a fine row is kept at u ^ lo_swz(row): the eight lanes of a quarter warp
+// hit all banks once, be they two neighbouring rows of four units (quad_logits) or the same unit of eight rows (key_logits_rows).
+__host__ __device__ constexpr int lo_swz(int row) { return ((row & 1) << 2) | (row >> 1); }
+
+// The same for the variants that ordinary tiles do not take, a row per lane, out of line, because the key epilogue's loop has to
+// stay small (the four warps of a scheduler run four different loops and share its instruction cache: 32 pairs unrolled in it
+// took 77 us a call, 8 pairs 73, 4 pairs 71).  Rotary rows: none; the staged ones (hi, lo: shared-memory addresses, units of lo
+// swizzled by swz), where 8-row groups share a coarse row, in whatever order; the handle's (hi, lo: addresses) where they share
+// none, or the fine table is not staged.  (Rows of whole chunks in any order, from the handle's tables -> from the staged ones: four
+// heads, 131072 rows, budget 4096 69.4 -> 40.8 us, in order 40.0; seven heads, eight sequences of 65536 rows 135.8 -> 73.0, in
+// order 67.5; sixteen heads 109.3 -> 82.4, in order 74.4; 4-bit bases, four heads 73.1 -> 53.2, in order 50.8.)
+// On return a lane holds the logits of the row of its own TMEM lane.
+enum RowTables { kNoTables, kHandleTables, kStagedTables };
 template <int NR>
 struct LogitsOut { float z[NR]; };
+__device__ __forceinline__ ulonglong2 lds_u64x2(uint32_t addr) {
+  ulonglong2 v;
+  asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(addr));
+  return v;
+}
 template <int DH, int NR, int QUANT, int TABLES>
-__device__ __noinline__ LogitsOut<NR> key_logits_rows(uint32_t acc, u64 hi, u64 lo, const ulonglong2* __restrict__ q_s) {
+__device__ __noinline__ LogitsOut<NR> key_logits_rows(uint32_t acc, unsigned long long hi, unsigned long long lo, int swz,
+                                                      const ulonglong2* __restrict__ q_s) {
   constexpr int HALF = DH / 2;
   constexpr unsigned long long kNeg2 = 0x8000000080000000ull;
   // Two dimensions per instruction where the sums have registers: not with sixteen heads, and with eight over codes (96 registers
@@ -325,6 +338,13 @@ __device__ __noinline__ LogitsOut<NR> key_logits_rows(uint32_t acc, u64 hi, u64 
       for (int v = 0; v < 2; ++v) {
         a[v] = __ldg(reinterpret_cast<const ulonglong2*>(hi) + u + v);
         f[v] = __ldg(reinterpret_cast<const ulonglong2*>(lo) + u + v);
+      }
+    }
+    if (TABLES == kStagedTables) {
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        a[v] = lds_u64x2((uint32_t)hi + (uint32_t)(u + v) * 16u);
+        f[v] = lds_u64x2((uint32_t)lo + (uint32_t)((u + v) ^ swz) * 16u);
       }
     }
     tc_wait_ld_nb(xa, xb);
@@ -369,10 +389,6 @@ __device__ __noinline__ LogitsOut<NR> key_logits_rows(uint32_t acc, u64 hi, u64 
   }
   return o;
 }
-
-// Rotary rows are multiples of 128 bytes: odd fine rows swap the halves of every 128 bytes, so that the eight lanes of a
-// quarter warp, two rows of 64 bytes each, hit all banks once.
-__host__ __device__ constexpr int lo_swz(int row) { return (row & 1) << 2; }
 
 // Slots of the ring of gathered key rows, of the ring of the B_k slabs that go with them (slab pair by slab pair).
 constexpr int kKeySlots = 4;
@@ -725,8 +741,9 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
             gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, 1));
             gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, 2));
             gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, 4));
-            const bool aligned = __all_sync(0xffffffffu, p < 0 || (hidx == gmax && (p & 7) == (lane & 7)));
-            if (lane == 0) algn_s[buf * 4 + blk] = aligned ? 1 : 0;
+            const bool aligned = __all_sync(0xffffffffu, p < 0 || hidx == gmax);
+            const bool in_order = __all_sync(0xffffffffu, p < 0 || (p & 7) == (lane & 7));
+            if (lane == 0) algn_s[buf * 4 + blk] = aligned ? in_order ? 1 : 2 : 0;
             if (aligned) {
 #pragma unroll
               for (int a = 0; a < 4; ++a) {
@@ -1008,7 +1025,8 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       if (++pbuf == 4) pbuf = 0;
       float z[NR];
       const uint32_t acc = tmem + lane_base + (uint32_t)(buf * 128);
-      bool by_row = !(rope_smem && algn_s[buf * 4 + warp]);
+      const int staged = rope_smem ? algn_s[buf * 4 + warp] : 0;      // 1: whole chunks in order, 2: in another order
+      bool by_row = staged != 1;
       if (!by_row) {
         quad_logits<DH, NR, MMA>(acc, reinterpret_cast<const ulonglong2*>(hi_s + (buf * 16 + warp * 4) * UN),
                                  reinterpret_cast<const ulonglong2*>(lo_s + quad_g * UN), lo_swz(quad_g),
@@ -1025,10 +1043,12 @@ sr_fused_kernel(const __grid_constant__ CUtensorMap bk_map, GroupDev dev, Sched 
       if (by_row) {
         const int pp = own < 0 ? 0 : own;
         const ulonglong2* qv = reinterpret_cast<const ulonglong2*>(q_s);
-        const LogitsOut<NR> o = dev.use_rope
-            ? key_logits_rows<DH, NR, QUANT, kHandleTables>(acc, (u64)(dev.rope_hi + (size_t)(pp >> dev.rope_shift) * UN),
-                                                            (u64)(dev.rope_lo + (size_t)(pp & rmask) * UN), qv)
-            : key_logits_rows<DH, NR, QUANT, kNoTables>(acc, 0, 0, qv);
+        const LogitsOut<NR> o =
+            staged ? key_logits_rows<DH, NR, QUANT, kStagedTables>(acc, smem_u32(hi_s + (buf * 16 + (tid >> 3)) * UN),
+                                                               smem_u32(lo_s + (pp & 7) * UN), lo_swz(pp & 7), qv)
+            : dev.use_rope ? key_logits_rows<DH, NR, QUANT, kHandleTables>(acc, (u64)(dev.rope_hi + (size_t)(pp >> dev.rope_shift) * UN),
+                                                                       (u64)(dev.rope_lo + (size_t)(pp & rmask) * UN), 0, qv)
+                           : key_logits_rows<DH, NR, QUANT, kNoTables>(acc, 0, 0, 0, qv);
 #pragma unroll
         for (int h = 0; h < NR; ++h) z[h] = __shfl_sync(0xffffffffu, o.z[h], quad_t * 8 + quad_g);
       }
