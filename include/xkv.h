@@ -180,8 +180,12 @@ XKV_API int xkv_sr_reconstruct_attend_tail(xkv_group* grp, int layer_begin, int 
  * Y = X Z, U = X^T Y, Z = orth(U) (one pass of Cholesky QR with a relative diagonal shift, three for the last
  * iterate; Gram matrix, factor and solve in fp64); then the
  * Rayleigh-Ritz step on span(Z): M = Z^T X^T X Z = P Lambda P^T (Jacobi), V = Z P_r, B = V^T rounded to bf16,
- * A = X bf16(V), sigma = sqrt(Lambda).  The result approximates the optimum of Eq. 1 (it is not unique up to signs and
- * rotations inside equal singular values: compare residuals, never factors).
+ * A = X V rounded to bf16, sigma = sqrt(Lambda).  V is not rounded in that product if 3 l < G d (it is then formed from X Z
+ * and P_r, each in two 16-bit parts); else it is X bf16(V).  So A is not the product of X with the B that is handed back to the
+ * last bit: the two differ by the rounding of B, 2^-9 / sqrt(3) of an entry of V at random, which the residual is better off
+ * without.  Rows that a caller adds later as X_new B^T are coefficients to that precision.
+ * The result approximates the optimum of Eq. 1 (it is not unique up to signs and rotations inside equal singular values:
+ * compare residuals, never factors).
  * cfg       host struct: T rows, G layers, d columns per layer (G*d a multiple of 64), rank r (multiple of 8),
  *           oversample p (0 means 32; l = r + p rounded up to a multiple of 64, at most G*d), power_iters q (0..8).
  * X         bf16 [T][G*d] (the layers' caches side by side, layer l in columns l*d .. l*d+d-1), device, 16-byte aligned.
