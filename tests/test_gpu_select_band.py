@@ -17,8 +17,21 @@ SHAPES = [(128, 4, 7, 3, 6, 4097, 256),        # the last tile of a problem hold
           (64, 8, 5, 2, 3, 6000, 700)]
 
 
-def _fill(mode, lm, q):
-    if mode == "element":
+def _fill(mode, lm, q, k_ch=256):
+    if mode == "cluster":                      # two hundred scores around the cut that differ in their last bits only
+        G, B = q.shape[1:3]
+        H_kv, n_c, d_h = lm.shape[2:]
+        g = torch.Generator().manual_seed(5)
+        q[..., :16] = 2.0 ** -10 * torch.sign(q[..., :16])
+        first = q[0].view(G, B, H_kv, -1, d_h)[:, :, :, :1].transpose(0, 1).to(torch.bfloat16).float()     # head 0 of every group
+        lm *= 0.1
+        above, below = k_ch - 100, min(k_ch + 100, n_c)
+        lm[..., :above, :] = first
+        lm[..., above:below, :] = 0.5 * first
+        # one unit in the last place of the first sixteen elements, which weigh 2^-10
+        lm[..., above:below, :16] += 2.0 ** -7 * torch.randint(-1, 2, lm[..., above:below, :16].shape, generator=g)
+        lm[...] = lm[..., torch.randperm(n_c, generator=g), :].clone()
+    elif mode == "element":
         lm[..., 3, 5] = 3000.0
     elif mode == "channel":
         lm[..., 7] = 100.0 + lm[..., 7]
@@ -44,14 +57,15 @@ def _fill(mode, lm, q):
         lm[:, 1] = float("nan")
 
 
-@pytest.mark.parametrize("mode", ["element", "channel", "rows", "zero queries", "zero landmarks", "equal", "tiny", "cancel", "neighbour"])
+@pytest.mark.parametrize("mode", ["cluster", "element", "channel", "rows", "zero queries", "zero landmarks", "equal", "tiny", "cancel",
+                                  "neighbour"])
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "-".join(map(str, s)))
 def test_index_sets_are_those_of_the_canonical_scores(shape, mode):
     d_h, H_kv, n_rep, G, B, n_c, k_ch = shape
     T, k = n_c * 8 - 3, k_ch * 8
     lm = synth.normal(synth.stream_key(8300, 91), (B, G, H_kv, n_c, d_h))
     q = synth.normal(synth.stream_key(8300, 92), (1, G, B, H_kv * n_rep, d_h))
-    _fill(mode, lm, q)
+    _fill(mode, lm, q, k_ch)
     lm, q = lm.to(torch.bfloat16), q.to(torch.bfloat16)
     s = synth.config(1, T=T, k=k, G=G, H_kv=H_kv, H_q=H_kv * n_rep, d_h=d_h, batch=B, c=8, r_k=8, r_v=8, seed=8300)
     A = torch.zeros((B, T, 8), dtype=torch.bfloat16)
