@@ -162,11 +162,14 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1
 // in 2^-24 of sum |q k|; d_h 64 and 128); now 0.24 to 0.33, a multiply-add per element and head in fp32 0.36 to 0.51, the
 // packed form 0.24.  It costs nothing (seven heads 123.2 -> 123.1 us a step, 32768 rows by layer 111.7 -> 111.7).
 // Which one: without MMA only four heads and bf16 bases have registers for the sums (eight heads 157.4 us a step of eight
-// sequences of 65536 rows where a row per lane takes 151.9, 4-bit bases 92.5 where it takes 88.3), and there it is the
-// better one in the steady state, where shared memory and the tensor pipe are all but busy (131072 rows 78.3 -> 75.4 us a step
-// from a row per lane, with MMA 78.6 -> 79.2; four sequences of them 268.3 -> 252.4, with MMA 270.4 -> 268.7; rank 1024, budget
-// 16384 316.5 -> 311.9).  MMA: seven heads 129.4 -> 123.5, 4-bit bases 88.2 -> 86.8, one tile per CTA (32768 rows by layer)
-// 114.3 -> 113.0 where the other gives 114.
+// sequences of 65536 rows where a row per lane takes 151.9, 4-bit bases 92.5 where it takes 88.3; with MMA, seven heads 129.4 ->
+// 122.5 and 4-bit bases 88.2 -> 87.1), and there it is the better one from two tiles per CTA on, where shared memory and the tensor
+// pipe are all but busy: 131072 rows 78.3 -> 75.4 us a step from a row per lane, with MMA 78.6 -> 79.2; four sequences of them 268.3
+// -> 252.4, with MMA 270.4 -> 268.7; rank 1024 and a budget of 16384 316.5 -> 311.9.  A call of 37 problems
+// and 1, 2, 3, 7 tiles per CTA, MMA / without: four heads of 128, rank 512 17.4 / 17.4, 22.0 / 21.0, 26.3 / 24.2, 44.2 /
+// 38.8 us; rank 64 13.2 / 13.2, 16.0 / 16.0, 18.5 / 18.6, 29.1 / 29.3; rank 1024 23.5 / 23.6, 33.4 / 33.0, 41.6 / 41.3, 67.5 /
+// 66.9; one head, rank 512 15.8 / 16.1, 20.4 / 19.4, 24.6 / 22.7, 42.1 / 36.7; four heads of 64, rank 256 14.4 / 14.3, 16.9 / 16.4,
+// 19.6 / 18.4, 29.8 / 26.5.
 // hi: the coarse rotary entries of the warp's four 8-row chunks, 16-byte units; lo: the fine ones of position g of a
 // chunk, units swizzled by `swz`; q_s: the queries.  On return a lane holds the logits of row g + 8t.
 template <int DH, int NR, bool MMA>
@@ -1537,7 +1540,7 @@ cudaError_t launch_fused_t(const xkv_group* grp, int l0, int l1, const __nv_bflo
     if (e == cudaSuccess) e = launch_pdl(kernel, dim3(sc.n_ctas), dim3(fused_threads(quant)), smem, s, mk, dev, sc, q, sel_idx, sel_cnt);
   };
 #define XKV_FUSED(PROF, QUANT, MMA) launch(ensure_dyn_smem<sr_fused_kernel<DH, NR, WB, PROF, QUANT, MMA>>, sr_fused_kernel<DH, NR, WB, PROF, QUANT, MMA>, QUANT)
-  // four heads in the steady state, bf16 bases: packed multiply-adds (see quad_logits)
+  // up to four heads, bf16 bases, two tiles per CTA or more: packed multiply-adds (measured at quad_logits)
   const bool fma = NR == 4 && sc.n_tiles >= 2 * sc.n_ctas;
   if (grp->prof) {     // the variant with the diagnostic counters compiled in
     if (dev.Aq_k) return cudaErrorNotSupported;        // no diagnostic variant of the quantised gather

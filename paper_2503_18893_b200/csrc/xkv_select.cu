@@ -1,9 +1,12 @@
-// Landmark-guided top-k chunk selection (App. B.1, Algorithm 2) in two kernels:
-//   score_pool_kernel  lines 2-3: streams every landmark once (HBM bound), fp32 scores in the canonical
-//                      order, max-pool over the query heads of each KV head;
-//   topk_kernel        lines 1,4: exact k_ch-th largest pooled score by radix select, then an ordered
-//                      compaction (ties to the lowest chunk index, output ascending) and expansion of
-//                      chunk ids to token rows.
+// Landmark-guided top-k chunk selection (App. B.1, Algorithm 2) in two kernels, a scan and a top-k:
+//   score_pool_kernel   lines 2-3: streams every landmark once (HBM bound), fp32 scores in the canonical order, max-pool over the
+//                       query heads of each KV head;
+//   score_bound_kernel  the same with scores by mma.sync and a bound on their error, for more than four heads per KV head and calls
+//                       of some size (launch_select_dev has the line);
+//   topk_pivot_kernel   lines 1, 4, 5: the k_ch largest pooled scores of up to 32768 chunks by a filtered list (ties to the lowest
+//                       chunk index), united with the outlier chunks, ascending, expanded to token rows; of scores with a bound
+//                       those around the cut are worked out again in the canonical order;
+//   topk_kernel         the same for longer contexts, by radix select over all keys.
 #include <cuda.h>
 #include <math.h>
 
