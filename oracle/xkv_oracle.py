@@ -496,7 +496,8 @@ def quantized_compression_ratio(base_ratio: float, bits: int, group: int = RTN_G
 # The paper names the ingredients, not the steps.  The steps taken here are the textbook randomised subspace
 # iteration (Halko, Martinsson, Tropp) run on the right side, because X (T x N, N = G d) is tall:
 #   Z <- Omega (N x l, l = r + p);  repeat q + 1 times: Y = X Z; U = X^T Y; Z = orth(U)
-#   Rayleigh-Ritz on span(Z): M = Z^T X^T X Z = P Lambda P^T; V = Z P_r; B = bf16(V)^T; A = X V; sigma = sqrt(Lambda).
+#   Rayleigh-Ritz on span(Z): M = Z^T X^T X Z = P Lambda P^T; V = Z P_r; B = bf16(V)^T; A = X V if 3 l < N, else X bf16(V);
+#   sigma = sqrt(Lambda).
 # orth = shifted Cholesky QR: G = U^T U + s I, s = shift * max diag(U^T U), G = L L^T, U <- U L^-T, in passes with
 # relative shifts 1e-4, 1e-5 (inside the iteration) and 1e-4, 1e-5, 1e-6, 1e-8, 1e-10 (last iterate).  Matrices that the 16-bit products read are rounded to bf16 first (X is bf16 already).
 # It approximates clf_factorize's optimum; it is compared with it through the residual, never factor by factor.
@@ -536,5 +537,7 @@ def clf_randomized(X_cat: np.ndarray, r: int, omega: np.ndarray, power_iters: in
     lam, P = np.linalg.eigh(M)
     order = np.argsort(-lam)[:r]
     V = Z @ P[:, order]
-    A = bf16_round((X @ V).astype(np.float32))
-    return A, bf16_round(V.astype(np.float32)), np.sqrt(np.maximum(lam[order], 0.0))
+    Vb = bf16_round(V.astype(np.float32))
+    # (three products of l terms instead of N where that is shorter; they need no 16-bit V)
+    A = bf16_round((X @ (V if 3 * omega.shape[1] < X.shape[1] else Vb.astype(np.float64))).astype(np.float32))
+    return A, Vb, np.sqrt(np.maximum(lam[order], 0.0))
