@@ -160,7 +160,9 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1
 // core cuts its sums off instead of rounding them, so a sum runs over sixteen dimensions only and is added on in fp32: one sum
 // over all of them (32 steps), and an upper part that was cut off too, had logits of single rows off by 1.2 to 1.5 (rms,
 // in 2^-24 of sum |q k|; d_h 64 and 128); now 0.24 to 0.33, a multiply-add per element and head in fp32 0.36 to 0.51, the
-// packed form 0.24.  It costs nothing (seven heads 123.2 -> 123.1 us a step, 32768 rows by layer 111.7 -> 111.7).
+// packed form 0.24.  Seven heads 123.9 -> 122.5 us a step with it, 4-bit bases 87.2 -> 87.2, 32768 rows by layer 112.1 -> 112.3; a call
+// with sixteen heads 72.1 -> 75.5 and with 3-bit bases and four heads 50.0 -> 52.2: every pass waits for its four products.  (The
+// sums added a pass later, so that nothing waits: 3-bit 52.6, seven heads 124.0; the rounding by cvt.rna.tf32: 123.9.)
 // Which one: without MMA only four heads and bf16 bases have registers for the sums (eight heads 157.4 us a step of eight
 // sequences of 65536 rows where a row per lane takes 151.9, 4-bit bases 92.5 where it takes 88.3; with MMA, seven heads 129.4 ->
 // 122.5 and 4-bit bases 88.2 -> 87.1), and there it is the better one from two tiles per CTA on, where shared memory and the tensor
